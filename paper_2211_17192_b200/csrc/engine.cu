@@ -141,8 +141,9 @@ struct Pass {
     int n_rows;
     bool tc;
     cudaStream_t st;
-    int pending = 0;      // split count of partial sums not yet added into h
-    int last_splits = 0;  // split count of the last projection
+    bool pending = false;   // partial sums (laid out by `closing`) not yet added into h
+    PartialPlan closing{};  // of the last GEMM that closed a residual branch
+    PartialPlan last{};     // of the last projection
 
     __nv_bfloat16* hi() const { return ctx->x_hi; }
     __nv_bfloat16* lo() const { return ctx->x_lo; }
@@ -150,17 +151,17 @@ struct Pass {
     // a (fp32) or hi/lo = rmsnorm(h[src(i)]) * gain for i < n
     int norm(const float* gain, const int32_t* src_rows, int n) {
         const int d = m.cfg.d_model;
-        const int status = tc ? launch_norm(ctx->h, pending ? ctx->partials : nullptr, pending, n_rows, gain, src_rows, n, d,
+        const int status = tc ? launch_norm(ctx->h, pending ? ctx->partials : nullptr, closing, n_rows, gain, src_rows, n, d,
                                             m.cfg.rms_eps, nullptr, hi(), lo(), st)
-                              : launch_norm(ctx->h, nullptr, 0, n_rows, gain, src_rows, n, d, m.cfg.rms_eps, ctx->a, nullptr,
+                              : launch_norm(ctx->h, nullptr, PartialPlan{}, n_rows, gain, src_rows, n, d, m.cfg.rms_eps, ctx->a, nullptr,
                                             nullptr, st);
-        pending = 0;
+        pending = false;
         return status;
     }
     // y = x . W^T for a consumer that is not the residual stream: partial sums (tc) or `y` (fp32 path, input `x`)
     int proj(const void* w, const void* pw, int n_out, int k, const float* x, float* y) {
         if (tc) {
-            last_splits = gemm_tc_splits(n_out, k, n_rows);
+            last = gemm_tc_plan(n_out, k, n_rows);
             return launch_gemm_tc_partials(hi(), lo(), ctx->hi_rows, pw, true, n_rows, n_out, k, ctx->partials, st);
         }
         return launch_gemm_rows(x, w, m.bf16(), nullptr, nullptr, n_rows, n_out, k, y, st);
@@ -169,7 +170,8 @@ struct Pass {
     int residual(const void* w, const void* pw, int k, const float* x) {
         const int d = m.cfg.d_model;
         if (tc) {
-            pending = gemm_tc_splits(d, k, n_rows);
+            pending = true;
+            closing = gemm_tc_plan(d, k, n_rows);
             return launch_gemm_tc_partials(hi(), lo(), ctx->hi_rows, pw, true, n_rows, d, k, ctx->partials, st);
         }
         return launch_gemm_rows(x, w, m.bf16(), ctx->h, nullptr, n_rows, d, k, ctx->h, st);
@@ -180,7 +182,7 @@ struct Pass {
         const spec_model_cfg& c = m.cfg;
         SPEC_TRY(norm(w.ln2, nullptr, n_rows));
         SPEC_TRY(proj(w.w_in, pw.w_in, m.ffn_in_dim(), c.d_model, ctx->a, ctx->u));
-        SPEC_TRY(launch_ffn_act(tc ? nullptr : ctx->u, partials(), last_splits, n_rows, c.d_ff, c.ffn, tc ? nullptr : ctx->f,
+        SPEC_TRY(launch_ffn_act(tc ? nullptr : ctx->u, partials(), last, n_rows, c.d_ff, c.ffn, tc ? nullptr : ctx->f,
                                 tc ? hi() : nullptr, tc ? lo() : nullptr, st));
         return residual(w.w_out, pw.w_out, c.d_ff, ctx->f);
     }
@@ -192,7 +194,7 @@ struct Pass {
         SPEC_TRY(norm(w.ln1, nullptr, n_rows));
         SPEC_TRY(proj(w.wqkv, pw.wqkv, m.qkv_dim(), c.d_model, ctx->a, ctx->qkv));
         SPEC_TRY(launch_qkv(c.n_heads, c.n_kv_heads, c.d_head, c.arch == SPEC_ARCH_LLAMA ? m.rope_table : nullptr, pool, rows,
-                            n_rows, ctx->qkv, partials(), last_splits, st));
+                            n_rows, ctx->qkv, partials(), last, st));
         const int slices = attention_slices(m, batch, m_rows, max_keys);
         const AttnSource src{ctx->qkv, m.qkv_dim(), pool, kv_len, bias, bias_span, bias_zero};
         SPEC_TRY(launch_attention(m, src, rows, batch, m_rows, slices, max_keys, ctx->attn_part, tc ? nullptr : ctx->att,
@@ -203,8 +205,8 @@ struct Pass {
 
 // Non-zero (and cleared) if a tensor-core GEMM or the persistent pass kernel gave up on a bounded wait.
 int device_gave_up(spec_ctx* ctx) {
-    const int gemm = gemm_tc_take_error(), pass = pass_take_error(), attn = attention_take_error();
-    return gemm ? gemm : pass ? pass : attn;
+    const int gemm = gemm_tc_take_error(), wide = gemm_wide_take_error(), pass = pass_take_error(), attn = attention_take_error();
+    return gemm ? gemm : wide ? wide : pass ? pass : attn;
 }
 
 KvPool layer_pool(const spec_ctx* ctx, const Model& m, int layer) {
@@ -258,7 +260,7 @@ int forward(spec_ctx* ctx, const Model& m, int batch, int m_rows, int n_logit_ro
             SPEC_TRY(pass.proj(w.wq_x, pw.wq_x, m.q_dim(), d, ctx->a, ctx->qkv));
             if (pass.tc)  // the partial sums become the query rows
                 SPEC_TRY(launch_qkv(c.n_heads, 0, c.d_head, nullptr, KvPool{}, rows, n_rows, ctx->qkv, ctx->partials,
-                                    pass.last_splits, ctx->stream));
+                                    pass.last, ctx->stream));
             const KvPool pool = source_pool(ctx, m, static_cast<char*>(m.cross_kv) + static_cast<size_t>(l) * m.cross_stride);
             const int slices = attention_slices(m, batch, m_rows, ctx->rt.max_src_len);
             const AttnSource src{ctx->qkv, m.q_dim(), pool, ctx->src_len, nullptr, 0, 0};
@@ -303,7 +305,7 @@ int encode(spec_ctx* ctx, const Model& m, int batch, int m_rows) {
         SPEC_TRY(pass.proj(w.wkv_x, pw.wkv_x, 2 * m.kv_dim(), c.d_model, ctx->a, ctx->qkv));
         const KvPool pool = source_pool(ctx, m, static_cast<char*>(m.cross_kv) + static_cast<size_t>(l) * m.cross_stride);
         SPEC_TRY(launch_qkv(0, c.n_kv_heads, c.d_head, nullptr, pool, rows, n_rows, ctx->qkv, pass.partials(),
-                            pass.last_splits, ctx->stream));
+                            pass.last, ctx->stream));
     }
     return SPEC_OK;
 }

@@ -23,48 +23,18 @@
 #include <tuple>
 
 #include "model.cuh"
+#include "tc_util.cuh"
 
 namespace spec {
 namespace {
 
-constexpr int kTileM = 128;     // output features per CTA (MMA M)
-constexpr int kTileK = 64;      // bf16 elements per k-block: one 128-byte swizzle row
-constexpr int kMmaK = 16;       // K of one tcgen05.mma.kind::f16
+using namespace tc;
+
 constexpr int kThreads = 128;
-constexpr uint32_t kSpinLimit = 1u << 22;
 
 __device__ int g_gemm_error;  // first device-side time-out (0 = none)
 
-// ---- PTX wrappers ----------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-
-// Bounded wait for the phase with the given parity; false on time-out.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit = kSpinLimit) {
-    const uint32_t addr = smem_u32(bar);
-    for (uint32_t spin = 0; spin < limit; ++spin) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t"
-            ".reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t"
-            "}"
-            : "=r"(done)
-            : "r"(addr), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-
+// ---- PTX wrappers (the shared ones: tc_util.cuh) ----
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
@@ -79,24 +49,6 @@ __device__ __forceinline__ void tma_load_2d_hint(void* dst, const CUtensorMap* m
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;"
         ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(policy)
         : "memory");
-}
-
-// Shared-memory matrix descriptor of a K-major tile whose rows are 128 bytes
-// long and 128-byte swizzled: 8-row groups are 1024 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
-    uint64_t d = 0;
-    d |= static_cast<uint64_t>((addr & 0x3FFFF) >> 4);   // start address, 16-byte units
-    d |= static_cast<uint64_t>(1) << 16;                 // leading byte offset (unused with swizzle)
-    d |= static_cast<uint64_t>(1024 >> 4) << 32;         // stride byte offset between 8-row groups
-    d |= static_cast<uint64_t>(1) << 46;                 // descriptor version of this architecture
-    d |= static_cast<uint64_t>(2) << 61;                 // 128-byte swizzle
-    return d;
-}
-
-// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = 128.
-__host__ __device__ constexpr uint32_t instr_desc(int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) |
-           (static_cast<uint32_t>(kTileM >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
@@ -117,29 +69,17 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                  : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 template <int N_TOK>
 struct Smem {
-    // two CTAs per SM up to 128 rows; wider tiles fill the SM alone
-    static constexpr int kStages = N_TOK <= 16 ? 5 : N_TOK <= 32 ? 4 : N_TOK <= 80 ? 3 : N_TOK <= 128 ? 2 : 3;
+    // two CTAs per SM
+    static constexpr int kStages = N_TOK <= 16 ? 5 : N_TOK <= 32 ? 4 : N_TOK <= 80 ? 3 : 2;
     static constexpr int kABytes = kTileM * kTileK * 2;   // 16 KB
     static constexpr int kBBytes = N_TOK * kTileK * 2;     // one of hi / lo
     static constexpr int kStageBytes = kABytes + 2 * kBBytes;
     static constexpr int kTotal = kStages * kStageBytes + 1024 /* alignment slack */ + 256 /* barriers */;
 };
 
-// grid = (tiles of 128 features x token tiles, splits), block = 128.
+// grid = (tiles of 128 features, splits), block = 128.
 template <int N_TOK>
 __global__ void __launch_bounds__(kThreads)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_hi,
@@ -149,7 +89,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     // up after `drill` polls: the path a lost copy would take, with no copy in flight when the CTA leaves
     using S = Smem<N_TOK>;
     const uint32_t limit = drill > 0 ? static_cast<uint32_t>(drill) : kSpinLimit;
-    constexpr int kTmemCols = N_TOK <= 32 ? 32 : N_TOK <= 64 ? 64 : N_TOK <= 128 ? 128 : 256;  // a power of two that holds N_TOK columns
+    constexpr int kTmemCols = N_TOK <= 32 ? 32 : N_TOK <= 64 ? 64 : 128;  // a power of two that holds N_TOK columns
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + S::kStages * S::kStageBytes);
@@ -157,12 +97,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     uint64_t* acc_bar = empty_bar + S::kStages;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_bar + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // (the token tiles of one weight tile are neighbours in launch order: they run side by side and the second
-    // finds the weights in L2 - with the token tile as the slowest grid dimension a 224-row launch read every
-    // weight from HBM twice)
-    const int token_tiles = (n_rows + N_TOK - 1) / N_TOK;
-    const int tile = blockIdx.x / token_tiles, split = blockIdx.y, splits = gridDim.y, tok0 = (blockIdx.x % token_tiles) * N_TOK;
+    const int warp = __shfl_sync(kFullMask, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // (uniform for the compiler)
+    const int tile = blockIdx.x, split = blockIdx.y, splits = gridDim.y;
     const int kb0 = static_cast<int>(static_cast<long long>(k_blocks) * split / splits);
     const int kb1 = static_cast<int>(static_cast<long long>(k_blocks) * (split + 1) / splits);
 
@@ -185,59 +121,65 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     const uint32_t tmem_acc = *tmem_slot;
     bool ok = true;
 
-    if (warp == 0 && lane == 0 && drill <= 0) {
+    if (warp == 0 && drill <= 0) {
         // ---- producer: weights and both activation terms of one k-block per stage ----
         // The weights do not depend on the kernel before this one: the first
         // ring of weight tiles is already streaming while that kernel finishes.
         // Weight tile of k-block kb: in the row-major matrix the box at (kb*64, tile*128);
         // in the tile-major copy the 128 consecutive 128-byte rows of tile (tile, kb).
+        const bool leader = elect_one();
         uint64_t stream_once;
         asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream_once));
-        auto load_w = [&](void* dst, int kb, uint64_t* bar) {
-            if (packed) tma_load_2d_hint(dst, &map_w, 0, (tile * k_blocks + kb) * kTileM, bar, stream_once);
-            else tma_load_2d_hint(dst, &map_w, kb * kTileK, tile * kTileM, bar, stream_once);
+        auto load_w = [&](int s, int kb) {
+            if (!leader) return;
+            mbar_expect_tx(&full_bar[s], S::kStageBytes);
+            if (packed) tma_load_2d_hint(smem + s * S::kStageBytes, &map_w, 0, (tile * k_blocks + kb) * kTileM, &full_bar[s], stream_once);
+            else tma_load_2d_hint(smem + s * S::kStageBytes, &map_w, kb * kTileK, tile * kTileM, &full_bar[s], stream_once);
+        };
+        auto load_x = [&](int s, int kb) {
+            if (!leader) return;
+            uint8_t* stage = smem + s * S::kStageBytes;
+            tma_load_2d(stage + S::kABytes, &map_hi, kb * kTileK, 0, &full_bar[s]);
+            tma_load_2d(stage + S::kABytes + S::kBBytes, &map_lo, kb * kTileK, 0, &full_bar[s]);
         };
         const int total = kb1 - kb0;
         const int ahead = min(total, S::kStages);
-        for (int it = 0; it < ahead; ++it) {
-            mbar_expect_tx(&full_bar[it], S::kStageBytes);
-            load_w(smem + it * S::kStageBytes, kb0 + it, &full_bar[it]);
-        }
+        for (int it = 0; it < ahead; ++it) load_w(it, kb0 + it);
         pdl_wait();  // the activations are written by the previous kernel
-        for (int it = 0; it < ahead; ++it) {
-            uint8_t* stage = smem + it * S::kStageBytes;
-            tma_load_2d(stage + S::kABytes, &map_hi, (kb0 + it) * kTileK, tok0, &full_bar[it]);
-            tma_load_2d(stage + S::kABytes + S::kBBytes, &map_lo, (kb0 + it) * kTileK, tok0, &full_bar[it]);
-        }
+        for (int it = 0; it < ahead; ++it) load_x(it, kb0 + it);
+        int s = 0, use = 1;  // stage of block `it` and how often the ring has gone round
         for (int it = ahead; it < total; ++it) {
-            const int kb = kb0 + it, s = it % S::kStages;
-            if (!mbar_wait(&empty_bar[s], ((it / S::kStages) - 1) & 1, limit)) { ok = false; break; }
-            uint8_t* stage = smem + s * S::kStageBytes;
-            mbar_expect_tx(&full_bar[s], S::kStageBytes);
-            load_w(stage, kb, &full_bar[s]);
-            tma_load_2d(stage + S::kABytes, &map_hi, kb * kTileK, tok0, &full_bar[s]);
-            tma_load_2d(stage + S::kABytes + S::kBBytes, &map_lo, kb * kTileK, tok0, &full_bar[s]);
+            if (!mbar_wait_warp(&empty_bar[s], (use - 1) & 1, limit)) { ok = false; break; }
+            load_w(s, kb0 + it);
+            load_x(s, kb0 + it);
+            if (++s == S::kStages) { s = 0; ++use; }
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // ---- MMA issuer ----
-        constexpr uint32_t idesc = instr_desc(N_TOK);
+        constexpr uint32_t idesc = instr_desc(kTileM, N_TOK);
+        const bool leader = elect_one();
+        const uint32_t base = smem_u32(smem);
+        int s = 0, use = 0;
         for (int kb = kb0; kb < kb1; ++kb) {
-            const int it = kb - kb0, s = it % S::kStages;
-            if (!mbar_wait(&full_bar[s], (it / S::kStages) & 1, limit)) { ok = false; break; }
+            if (!mbar_wait_warp(&full_bar[s], use & 1, limit)) { ok = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a_addr = smem_u32(smem + s * S::kStageBytes);
+            const uint32_t a_addr = base + s * S::kStageBytes;
             const uint64_t a_desc = smem_desc_sw128(a_addr);
             const uint64_t hi_desc = smem_desc_sw128(a_addr + S::kABytes);
             const uint64_t lo_desc = smem_desc_sw128(a_addr + S::kABytes + S::kBBytes);
+            if (leader) {
 #pragma unroll
-            for (int k = 0; k < kTileK / kMmaK; ++k) {
-                const uint64_t step = static_cast<uint64_t>((k * kMmaK * 2) >> 4);  // 32 bytes along K, in 16-byte units
-                mma_f16(tmem_acc, a_desc + step, hi_desc + step, idesc, (it > 0 || k > 0) ? 1u : 0u);
-                mma_f16(tmem_acc, a_desc + step, lo_desc + step, idesc, 1u);
+                for (int k = 0; k < kTileK / kMmaK; ++k) {
+                    const uint64_t step = static_cast<uint64_t>((k * kMmaK * 2) >> 4);  // 32 bytes along K, in 16-byte units
+                    mma_f16(tmem_acc, a_desc + step, hi_desc + step, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+                    mma_f16(tmem_acc, a_desc + step, lo_desc + step, idesc, 1u);
+                }
+                mma_commit(&empty_bar[s]);  // the stage may be refilled once these MMAs have read it
             }
-            mma_commit(&empty_bar[s]);  // the stage may be refilled once these MMAs have read it
+            __syncwarp();
+            if (++s == S::kStages) { s = 0; ++use; }
         }
-        if (ok) mma_commit(acc_bar);  // accumulator complete
+        if (ok && leader) mma_commit(acc_bar);  // accumulator complete
     }
     __syncwarp();
     pdl_wait();  // (already satisfied for the producer) nothing below may overtake the previous kernel
@@ -261,19 +203,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     if (ok) {
 #pragma unroll
         for (int c0 = 0; c0 < N_TOK; c0 += 16) {
-            if (tok0 + c0 < n_rows) {  // uniform across the warp
-                float v[16];
+            if (c0 < n_rows) {  // uniform across the warp
+                uint32_t v[16];
                 if (kb1 > kb0) {
                     tmem_ld16(tmem_acc + (static_cast<uint32_t>(warp * 32) << 16) + c0, v);
+                    tmem_ld_wait();
                 } else {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] = 0.0f;
+                    for (int i = 0; i < 16; ++i) v[i] = 0u;
                 }
                 if (feature < n_out) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        const int r = tok0 + c0 + i;
-                        if (r < n_rows) out[static_cast<size_t>(r) * n_out] = v[i];
+                        const int r = c0 + i;
+                        if (r < n_rows) out[static_cast<size_t>(r) * n_out] = __uint_as_float(v[i]);
                     }
                 }
             }
@@ -331,13 +274,15 @@ __global__ void split_bf16_kernel(const float* __restrict__ x, size_t n, __nv_bf
 }
 
 // y[dst(r)][n] = sum_s partial[s][r][n] (+ residual[r][n]), splits added in index order
-__global__ void reduce_partials_kernel(const float* __restrict__ partial, int splits, int n_rows, int n_out,
+__global__ void reduce_partials_kernel(const float* __restrict__ partial, const PartialPlan plan, int n_rows, int n_out,
                                        const float* residual, const int32_t* __restrict__ dst_rows, float* y) {
     pdl_trigger();
     pdl_wait();
     const size_t total = static_cast<size_t>(n_rows) * n_out;
     for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < total;
          i += static_cast<size_t>(gridDim.x) * blockDim.x) {
+        const size_t r = i / n_out, n = i % n_out;
+        const int splits = partial_count(plan, static_cast<int>(r), static_cast<int>(n));
         float acc = 0.0f;
         for (int s0 = 0; s0 < splits; s0 += 8) {  // eight loads in flight at a time, added in split order
             float p[8];
@@ -348,7 +293,6 @@ __global__ void reduce_partials_kernel(const float* __restrict__ partial, int sp
                 if (s0 + k < splits) acc = (s0 + k == 0) ? p[k] : acc + p[k];
         }
         if (residual) acc += residual[i];
-        const size_t r = i / n_out, n = i % n_out;
         y[(dst_rows ? static_cast<size_t>(dst_rows[r]) : r) * n_out + n] = acc;
     }
 }
@@ -395,8 +339,10 @@ struct MapKey {
     }
 };
 
+}  // namespace
+
 // Tensor maps are pure functions of (address, shape, box): cached process-wide.
-int cached_map(const void* base, int rows, int cols, int box_rows, bool swizzle, CUtensorMap* out) {
+int cached_bf16_map(const void* base, int rows, int cols, int box_rows, bool swizzle, CUtensorMap* out) {
     static std::mutex mu;
     static std::map<MapKey, CUtensorMap> cache;
     std::lock_guard<std::mutex> lock(mu);
@@ -412,6 +358,8 @@ int cached_map(const void* base, int rows, int cols, int box_rows, bool swizzle,
     return SPEC_OK;
 }
 
+namespace {
+
 template <int N_TOK>
 int launch_tc(const CUtensorMap& mw, const CUtensorMap& mhi, const CUtensorMap& mlo, float* partial, int n_out,
               int n_rows, int k_blocks, int splits, int packed, cudaStream_t stream, int drill = 0) {
@@ -419,34 +367,17 @@ int launch_tc(const CUtensorMap& mw, const CUtensorMap& mhi, const CUtensorMap& 
     if (first_use_on_this_device(configured))
         SPEC_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<N_TOK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            Smem<N_TOK>::kTotal));
-    const dim3 grid(((n_out + kTileM - 1) / kTileM) * ((n_rows + N_TOK - 1) / N_TOK), splits, 1);
+    const dim3 grid((n_out + kTileM - 1) / kTileM, splits, 1);
     return launch_pdl(gemm_tc_kernel<N_TOK>, grid, dim3(kThreads), Smem<N_TOK>::kTotal, stream, mw, mhi, mlo, partial,
                       n_out, n_rows, k_blocks, packed, drill);
 }
 
 }  // namespace
 
-// Rows per CTA (the MMA's N): the smallest multiple of 16 that holds the rows, so that up to 192 rows
-// the weights are streamed once and no MMA column is padding (the tensor-core work and the activation
-// tiles that every CTA re-reads grow with the padded row count: an 80-row tile for 80 rows instead of
-// a 96-row one took 8 % off the pass at batch 16 x 5 rows); more rows take several tiles, neighbours in
-// launch order (measured: a 256-row tile leaves room for two pipeline stages only and is slower than
-// two passes of 128).
-int gemm_tc_token_tile(int n_rows) {
-    if (n_rows <= 16) return 16;
-    if (n_rows <= 32) return 32;
-    if (n_rows <= 48) return 48;
-    if (n_rows <= 64) return 64;
-    if (n_rows <= 80) return 80;
-    if (n_rows <= 96) return 96;
-    if (n_rows <= 112) return 112;
-    if (n_rows <= 128) return 128;
-    if (n_rows <= 160) return 160;
-    if (n_rows <= 192) return 192;
-    if (n_rows <= 240) return 80;  // three tiles of 80 (three stages each) beat two of 112 or 128: 274 / 302 / 313 us
-                                   // per 7B block at 224 rows
-    return 128;
-}
+// Rows per CTA (the MMA's N): the smallest multiple of 16 that holds the rows, so that no MMA column is padding (the
+// tensor-core work and the activation tiles that every CTA re-reads grow with the padded row count: an 80-row tile for
+// 80 rows instead of a 96-row one took 8 % off the pass at batch 16 x 5 rows).
+int gemm_tc_token_tile(int n_rows) { return (n_rows + 15) / 16 * 16; }
 
 int cached_f16_rows_map(const void* base, unsigned long long rows, int cols, CUtensorMap* out) {
     static std::mutex mu;
@@ -472,13 +403,14 @@ int cached_f16_rows_map(const void* base, unsigned long long rows, int cols, CUt
     return SPEC_OK;
 }
 
+namespace {
+
 // Split-K factor: the smallest one that fills the last wave of CTAs to 85 %, with
 // at least two k-blocks per split.
-int gemm_tc_splits(int n_out, int k, int n_rows) {
-    const int n_tok = gemm_tc_token_tile(n_rows);
-    const int tiles = ((n_out + kTileM - 1) / kTileM) * ((n_rows + n_tok - 1) / n_tok);
+int gemm_tc_splits(int n_out, int k) {
+    const int tiles = (n_out + kTileM - 1) / kTileM;
     const int k_blocks = (k + kTileK - 1) / kTileK;
-    const int resident = 148 * (n_tok <= 128 ? 2 : 1);
+    const int resident = 148 * 2;
     const int max_splits = std::max(1, std::min(k_blocks / 2, 16));
     int best = 1;
     double best_eff = 0.0;
@@ -495,8 +427,23 @@ int gemm_tc_splits(int n_out, int k, int n_rows) {
     return best;
 }
 
+// More than 128 rows go to the CTA-pair kernel (gemm_wide.cu).  Measured back to back, this kernel against that one, us
+// for 22016 x 4096 and for 4096 x 11008: 112 rows 51.3 / 49.4 and 24.8 / 26.3, 128 rows 52.7 / 52.3 and 25.4 / 27.9;
+// above, against the 160- and 192-row and the several-tile launches of this kernel that it replaces: 160 rows
+// 77.1 / 55.5 and 30.5 / 29.3, 224 rows 82.1 / 65.9 and 39.2 / 34.0, 1024 rows 278 / 241 and 146 / 139.
+bool takes_wide(int n_rows) { return n_rows > 128; }
+
+}  // namespace
+
+PartialPlan gemm_tc_plan(int n_out, int k, int n_rows) {
+    if (takes_wide(n_rows)) return gemm_wide_plan(n_out, k, n_rows);
+    PartialPlan p{};
+    p.slots = gemm_tc_splits(n_out, k);
+    return p;
+}
+
 size_t gemm_tc_partial_elems(int n_out, int k, int n_rows) {
-    return static_cast<size_t>(gemm_tc_splits(n_out, k, n_rows)) * n_rows * n_out;
+    return static_cast<size_t>(gemm_tc_plan(n_out, k, n_rows).slots) * n_rows * n_out;
 }
 
 size_t packed_weight_elems(int n_out, int k) {
@@ -519,22 +466,23 @@ int launch_split_bf16(const float* x, size_t n, __nv_bfloat16* hi, __nv_bfloat16
 }
 
 // partial[s][r][n] for x already split into hi + lo (both [hi_rows, k] bf16, the
-// first n_rows rows valid); s < gemm_tc_splits(n_out, k, n_rows).
+// first n_rows rows valid); s < gemm_tc_splits(n_out, k).
 int launch_gemm_tc_partials(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_rows, const void* w, bool packed,
-                            int n_rows, int n_out, int k, float* partial, cudaStream_t stream) {
+                            int n_rows, int n_out, int k, float* partial, cudaStream_t stream, bool fill) {
     if (n_rows <= 0) return SPEC_OK;
     if (k % 8 != 0) return fail(SPEC_ERR_BAD_CONFIG, "gemm: inner dimension %d is not a multiple of 8", k);
+    if (takes_wide(n_rows)) return launch_gemm_wide(hi, lo, hi_rows, w, packed, n_rows, n_out, k, partial, fill, stream);
     const int n_tok = gemm_tc_token_tile(n_rows);
-    const int splits = gemm_tc_splits(n_out, k, n_rows);
+    const int splits = gemm_tc_splits(n_out, k);
     const int k_blocks = (k + kTileK - 1) / kTileK;
     CUtensorMap mw, mhi, mlo;
     const int tiles = (n_out + kTileM - 1) / kTileM;
     // tile-major weights are one long [tiles * k_blocks * 128, 64] matrix of 128-byte rows
     // (stored swizzled already: copied as they are)
-    int status = packed ? cached_map(w, tiles * k_blocks * kTileM, kTileK, kTileM, false, &mw)
-                        : cached_map(w, n_out, k, kTileM, true, &mw);
-    if (status == SPEC_OK) status = cached_map(hi, hi_rows, k, n_tok, true, &mhi);
-    if (status == SPEC_OK) status = cached_map(lo, hi_rows, k, n_tok, true, &mlo);
+    int status = packed ? cached_bf16_map(w, tiles * k_blocks * kTileM, kTileK, kTileM, false, &mw)
+                        : cached_bf16_map(w, n_out, k, kTileM, true, &mw);
+    if (status == SPEC_OK) status = cached_bf16_map(hi, hi_rows, k, n_tok, true, &mhi);
+    if (status == SPEC_OK) status = cached_bf16_map(lo, hi_rows, k, n_tok, true, &mlo);
     if (status != SPEC_OK) return status;
     const int pk = packed ? 1 : 0;
     switch (n_tok) {
@@ -545,9 +493,7 @@ int launch_gemm_tc_partials(const __nv_bfloat16* hi, const __nv_bfloat16* lo, in
         case 80: return launch_tc<80>(mw, mhi, mlo, partial, n_out, n_rows, k_blocks, splits, pk, stream);
         case 96: return launch_tc<96>(mw, mhi, mlo, partial, n_out, n_rows, k_blocks, splits, pk, stream);
         case 112: return launch_tc<112>(mw, mhi, mlo, partial, n_out, n_rows, k_blocks, splits, pk, stream);
-        case 128: return launch_tc<128>(mw, mhi, mlo, partial, n_out, n_rows, k_blocks, splits, pk, stream);
-        case 160: return launch_tc<160>(mw, mhi, mlo, partial, n_out, n_rows, k_blocks, splits, pk, stream);
-        default: return launch_tc<192>(mw, mhi, mlo, partial, n_out, n_rows, k_blocks, splits, pk, stream);
+        default: return launch_tc<128>(mw, mhi, mlo, partial, n_out, n_rows, k_blocks, splits, pk, stream);
     }
 }
 
@@ -558,11 +504,11 @@ int launch_gemm_tc(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_rows
     if (n_rows <= 0) return SPEC_OK;
     const int status = launch_gemm_tc_partials(hi, lo, hi_rows, w, packed, n_rows, n_out, k, partial, stream);
     if (status != SPEC_OK) return status;
-    const int splits = gemm_tc_splits(n_out, k, n_rows);
+    const PartialPlan plan = gemm_tc_plan(n_out, k, n_rows);
     const size_t total = static_cast<size_t>(n_rows) * n_out;
     const int blocks = static_cast<int>(std::min<size_t>((total + 255) / 256, 148 * 8));
     return launch_pdl(reduce_partials_kernel, dim3(blocks), dim3(256), 0, stream, static_cast<const float*>(partial),
-                      splits, n_rows, n_out, residual, dst_rows, y);
+                      plan, n_rows, n_out, residual, dst_rows, y);
 }
 
 // Non-zero if a tensor-core GEMM gave up on a bounded wait since the last call.
@@ -631,8 +577,8 @@ extern "C" int spec_linear_partials(const float* x, const void* w_packed, int ro
         if (status != SPEC_OK) return status;
     }
     if (partial) *partial = sums;
-    if (splits) *splits = gemm_tc_splits(n_out, k, rows);
-    return launch_gemm_tc_partials(hi, lo, padded_rows(rows), w_packed, true, rows, n_out, k, sums, st);
+    if (splits) *splits = gemm_tc_plan(n_out, k, rows).slots;
+    return launch_gemm_tc_partials(hi, lo, padded_rows(rows), w_packed, true, rows, n_out, k, sums, st, true);
 }
 
 extern "C" size_t spec_packed_weight_bytes(int n_out, int k) {
@@ -657,8 +603,8 @@ extern "C" int spec_timeout_drill(void* stream) {
     void* base = nullptr;
     SPEC_CUDA_TRY(cudaGetSymbolAddress(&base, g_drill_tile));
     CUtensorMap mw, mx;
-    int status = cached_map(base, 128, 64, 128, true, &mw);
-    if (status == SPEC_OK) status = cached_map(base, 16, 64, 16, true, &mx);
+    int status = cached_bf16_map(base, 128, 64, 128, true, &mw);
+    if (status == SPEC_OK) status = cached_bf16_map(base, 16, 64, 16, true, &mx);
     if (status != SPEC_OK) return status;
     SPEC_CUDA_TRY(cudaStreamSynchronize(st));
     gemm_tc_take_error();  // (whatever was pending is not this drill's)
@@ -672,6 +618,6 @@ extern "C" int spec_timeout_drill(void* stream) {
 }
 
 extern "C" int spec_device_error(void) {
-    const int gemm = spec::gemm_tc_take_error(), pass = spec::pass_take_error(), attn = spec::attention_take_error();
-    return gemm ? gemm : pass ? pass : attn;
+    const int gemm = spec::gemm_tc_take_error(), wide = spec::gemm_wide_take_error(), pass = spec::pass_take_error(), attn = spec::attention_take_error();
+    return gemm ? gemm : wide ? wide : pass ? pass : attn;
 }

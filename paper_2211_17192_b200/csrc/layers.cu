@@ -86,7 +86,7 @@ constexpr int kNormPerThread = 4;  // rows up to 16384 wide
 
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS)
-norm_kernel(float* h, const float* __restrict__ partial, int splits, int n_rows, const float* __restrict__ gain,
+norm_kernel(float* h, const float* __restrict__ partial, const PartialPlan plan, int n_rows, const float* __restrict__ gain,
             const int32_t* __restrict__ src_rows, int d, float eps, float* __restrict__ out,
             __nv_bfloat16* __restrict__ out_hi, __nv_bfloat16* __restrict__ out_lo) {
     __shared__ float red[THREADS / 32];
@@ -104,7 +104,8 @@ norm_kernel(float* h, const float* __restrict__ partial, int splits, int n_rows,
     // take the places of that GEMM's leaving CTAs and their first weight tiles compete with the tail of its stream
     // (measured per 7B block: 94.5 -> 93.1 us; releasing at the end of this kernel instead: 95.1).
     pdl_trigger();
-    const size_t src = static_cast<size_t>(src_rows ? src_rows[r] : r) * d;
+    const int src_row = src_rows ? src_rows[r] : r;
+    const size_t src = static_cast<size_t>(src_row) * d;
     const size_t stride = static_cast<size_t>(n_rows) * d;
     float4 v[kNormPerThread];
     float ss = 0.0f;
@@ -115,6 +116,7 @@ norm_kernel(float* h, const float* __restrict__ partial, int splits, int n_rows,
         if (g < groups) {
             v[j] = *reinterpret_cast<const float4*>(h + src + 4 * g);
             if (partial) {
+                const int splits = partial_count(plan, src_row, 4 * g);
                 for (int s0 = 0; s0 < splits; s0 += 8) {  // eight loads in flight at a time, added in split order
                     float4 p[8];
 #pragma unroll
@@ -159,7 +161,7 @@ norm_kernel(float* h, const float* __restrict__ partial, int splits, int n_rows,
 // heads; thread j owns the pair j, j + d_head/2), leaves q in `qkv` for the
 // attention kernel, and appends K or V to the paged cache.
 template <typename KV>
-__global__ void qkv_kernel(float* __restrict__ qkv, const float* __restrict__ partial, int splits, int n_rows,
+__global__ void qkv_kernel(float* __restrict__ qkv, const float* __restrict__ partial, const PartialPlan plan, int n_rows,
                            const int32_t* __restrict__ pos, const int32_t* __restrict__ seq, int n_heads,
                            int n_kv_heads, int d_head, const float2* __restrict__ rope_table,
                            KV* __restrict__ kv_layer, const int32_t* __restrict__ page_table, int pages_per_seq,
@@ -174,7 +176,8 @@ __global__ void qkv_kernel(float* __restrict__ qkv, const float* __restrict__ pa
     float x1, x2;
     if (partial) {
         const size_t stride = static_cast<size_t>(n_rows) * width;
-        sum_partials2(partial, splits, stride, at + j, at + j + half, &x1, &x2);
+        // (a head of 64 or 128 columns lies inside one 256-column tile)
+        sum_partials2(partial, partial_count(plan, r, head * d_head), stride, at + j, at + j + half, &x1, &x2);
     } else {
         x1 = qkv[at + j];
         x2 = qkv[at + j + half];
@@ -259,7 +262,7 @@ __device__ __forceinline__ float silu(float x) { return x / (1.0f + expf(-x)); }
 
 // f = gelu(u)  |  gelu(gate) * up  |  silu(gate) * up, with u either given in
 // full or as the partial sums of the FFN-in GEMM.
-__global__ void ffn_act_kernel(const float* __restrict__ u, const float* __restrict__ partial, int splits, int n_rows,
+__global__ void ffn_act_kernel(const float* __restrict__ u, const float* __restrict__ partial, const PartialPlan plan, int n_rows,
                                int d_ff, int ffn, float* __restrict__ f, __nv_bfloat16* __restrict__ f_hi,
                                __nv_bfloat16* __restrict__ f_lo) {
     pdl_trigger();
@@ -273,11 +276,18 @@ __global__ void ffn_act_kernel(const float* __restrict__ u, const float* __restr
         const size_t a = r * width + c;
         float y;
         if (ffn == SPEC_FFN_GELU) {
-            y = gelu_tanh(partial ? sum_partials(partial, splits, stride, a) : u[a]);
+            y = gelu_tanh(partial ? sum_partials(partial, partial_count(plan, static_cast<int>(r), static_cast<int>(c)), stride, a) : u[a]);
         } else {
             float gate, up;
             if (partial) {
-                sum_partials2(partial, splits, stride, a, a + d_ff, &gate, &up);
+                const int n_gate = partial_count(plan, static_cast<int>(r), static_cast<int>(c));
+                const int n_up = partial_count(plan, static_cast<int>(r), static_cast<int>(c) + d_ff);
+                if (n_gate == n_up) {
+                    sum_partials2(partial, n_gate, stride, a, a + d_ff, &gate, &up);
+                } else {
+                    gate = sum_partials(partial, n_gate, stride, a);
+                    up = sum_partials(partial, n_up, stride, a + d_ff);
+                }
             } else {
                 gate = u[a];
                 up = u[a + d_ff];
@@ -312,7 +322,7 @@ int launch_copy_logits(const int32_t* tokens, int max_len, const int32_t* length
                       gamma, rows.pos, rows.seq, src_rows, dst_rows, ngram, vocab, logits);
 }
 
-int launch_norm(float* h, const float* partial, int splits, int rows_total, const float* gain, const int32_t* src_rows,
+int launch_norm(float* h, const float* partial, const PartialPlan& plan, int rows_total, const float* gain, const int32_t* src_rows,
                 int n_rows, int d, float eps, float* out, __nv_bfloat16* out_hi, __nv_bfloat16* out_lo,
                 cudaStream_t stream) {
     if (d % 4 || d > 4 * kNormThreads * kNormPerThread)
@@ -320,37 +330,37 @@ int launch_norm(float* h, const float* partial, int splits, int rows_total, cons
     // a thread per 128-bit group of the row where the row is narrow (fewer warps to reduce over)
     const int groups = d / 4;
     if (groups <= 128)
-        return launch_pdl(norm_kernel<128>, dim3(n_rows), dim3(128), 0, stream, h, partial, splits, rows_total, gain, src_rows, d,
+        return launch_pdl(norm_kernel<128>, dim3(n_rows), dim3(128), 0, stream, h, partial, plan, rows_total, gain, src_rows, d,
                           eps, out, out_hi, out_lo);
     if (groups <= 256)
-        return launch_pdl(norm_kernel<256>, dim3(n_rows), dim3(256), 0, stream, h, partial, splits, rows_total, gain, src_rows, d,
+        return launch_pdl(norm_kernel<256>, dim3(n_rows), dim3(256), 0, stream, h, partial, plan, rows_total, gain, src_rows, d,
                           eps, out, out_hi, out_lo);
-    return launch_pdl(norm_kernel<kNormThreads>, dim3(n_rows), dim3(kNormThreads), 0, stream, h, partial, splits, rows_total,
+    return launch_pdl(norm_kernel<kNormThreads>, dim3(n_rows), dim3(kNormThreads), 0, stream, h, partial, plan, rows_total,
                       gain, src_rows, d, eps, out, out_hi, out_lo);
 }
 
 int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, const KvPool& pool, const RowMeta& rows,
-               int n_rows, float* qkv, const float* partial, int splits, cudaStream_t stream) {
+               int n_rows, float* qkv, const float* partial, const PartialPlan& plan, cudaStream_t stream) {
     const dim3 grid(n_heads + 2 * n_kv_heads, n_rows);
     const dim3 block(d_head / 2);
     if (pool.dtype == SPEC_DTYPE_FP16)
-        return launch_pdl(qkv_kernel<__half>, grid, block, 0, stream, qkv, partial, splits, n_rows, rows.pos, rows.seq, n_heads,
+        return launch_pdl(qkv_kernel<__half>, grid, block, 0, stream, qkv, partial, plan, n_rows, rows.pos, rows.seq, n_heads,
                           n_kv_heads, d_head, rope, static_cast<__half*>(pool.kv), pool.page_table, pool.pages_per_seq,
                           pool.page_size);
     if (pool.dtype == SPEC_DTYPE_BF16)
-        return launch_pdl(qkv_kernel<__nv_bfloat16>, grid, block, 0, stream, qkv, partial, splits, n_rows, rows.pos,
+        return launch_pdl(qkv_kernel<__nv_bfloat16>, grid, block, 0, stream, qkv, partial, plan, n_rows, rows.pos,
                           rows.seq, n_heads, n_kv_heads, d_head, rope, static_cast<__nv_bfloat16*>(pool.kv),
                           pool.page_table, pool.pages_per_seq, pool.page_size);
-    return launch_pdl(qkv_kernel<float>, grid, block, 0, stream, qkv, partial, splits, n_rows, rows.pos, rows.seq,
+    return launch_pdl(qkv_kernel<float>, grid, block, 0, stream, qkv, partial, plan, n_rows, rows.pos, rows.seq,
                       n_heads, n_kv_heads, d_head, rope, static_cast<float*>(pool.kv), pool.page_table,
                       pool.pages_per_seq, pool.page_size);
 }
 
-int launch_ffn_act(const float* u, const float* partial, int splits, int n_rows, int d_ff, int ffn, float* f,
+int launch_ffn_act(const float* u, const float* partial, const PartialPlan& plan, int n_rows, int d_ff, int ffn, float* f,
                    __nv_bfloat16* f_hi, __nv_bfloat16* f_lo, cudaStream_t stream) {
     const size_t total = static_cast<size_t>(n_rows) * d_ff;
     const int blocks = static_cast<int>(std::min<size_t>((total + 255) / 256, 148 * 8));
-    return launch_pdl(ffn_act_kernel, dim3(blocks), dim3(256), 0, stream, u, partial, splits, n_rows, d_ff, ffn, f,
+    return launch_pdl(ffn_act_kernel, dim3(blocks), dim3(256), 0, stream, u, partial, plan, n_rows, d_ff, ffn, f,
                       f_hi, f_lo);
 }
 

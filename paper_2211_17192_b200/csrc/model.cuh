@@ -49,6 +49,27 @@ struct Model {
     bool bf16() const { return cfg.dtype == SPEC_DTYPE_BF16; }
 };
 
+// Where the partial sums of a tensor-core GEMM lie: [slot][row][n_out] fp32, added up by the consumer in slot order.
+// tok_tile == 0: every element has `slots` partial sums.  Otherwise (gemm_wide.cu) the output is cut into tiles of
+// 256 columns by tok_tile rows, the row tiles of a column tile being neighbours in tile order; the first dp_tiles
+// tiles have one sum, the k-blocks of the others (`units` in all, kb per tile) are dealt out to `pairs` CTA pairs in
+// equal contiguous runs and a tile has one sum per pair that takes part in it.
+struct PartialPlan {
+    int slots;  // most partial sums of any element
+    int tok_tile, token_tiles, dp_tiles, kb, units, pairs;
+};
+__host__ __device__ __forceinline__ int partial_owner(const PartialPlan& p, int unit) { return ((unit + 1) * p.pairs - 1) / p.units; }
+__host__ __device__ __forceinline__ int partial_slot(const PartialPlan& p, int tile, int k_block) {
+    if (tile < p.dp_tiles) return 0;
+    const int first = (tile - p.dp_tiles) * p.kb;
+    return partial_owner(p, first + k_block) - partial_owner(p, first);
+}
+__host__ __device__ __forceinline__ int partial_slots_of_tile(const PartialPlan& p, int tile) { return partial_slot(p, tile, p.kb - 1) + 1; }
+// Partial sums of the element in this row and column.
+__host__ __device__ __forceinline__ int partial_count(const PartialPlan& p, int row, int col) {
+    return p.tok_tile == 0 ? p.slots : p.slots == 1 ? 1 : partial_slots_of_tile(p, (col >> 8) * p.token_tiles + row / p.tok_tile);
+}
+
 // Row descriptors of one forward pass (device arrays of `rows` entries).
 // A row with pos < 0 is inactive: it is computed but writes no K,V.
 struct RowMeta {
@@ -73,7 +94,7 @@ int launch_table_logits(const void* table, bool bf16, int vocab, const int32_t* 
 int launch_copy_logits(const int32_t* tokens, int max_len, const int32_t* length, const int32_t* draft_tokens, int gamma,
                        const RowMeta& rows, const int32_t* src_rows, const int32_t* dst_rows, int n_rows, int ngram,
                        int vocab, float* logits, cudaStream_t stream);
-int launch_norm(float* h, const float* partial, int splits, int rows_total, const float* gain, const int32_t* src_rows,
+int launch_norm(float* h, const float* partial, const PartialPlan& plan, int rows_total, const float* gain, const int32_t* src_rows,
                 int n_rows, int d, float eps, float* out, __nv_bfloat16* out_hi, __nv_bfloat16* out_lo,
                 cudaStream_t stream);
 
@@ -85,7 +106,7 @@ int launch_gemm_rows(const float* x, const void* w, bool w_bf16, const float* re
 // Tensor-core path for bf16 weights (gemm_tc.cu): x arrives as two bf16 terms;
 // launch_gemm_tc_partials leaves the split-K partial sums [splits][n_rows][n_out]
 // for the next kernel to add up, launch_gemm_tc adds them up itself.
-int gemm_tc_splits(int n_out, int k, int n_rows);
+PartialPlan gemm_tc_plan(int n_out, int k, int n_rows);
 size_t gemm_tc_partial_elems(int n_out, int k, int n_rows);
 int launch_split_bf16(const float* x, size_t n, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t stream);
 // `packed`: w is the tile-major copy made by launch_pack_weight (every [128 x 64]
@@ -93,7 +114,13 @@ int launch_split_bf16(const float* x, size_t n, __nv_bfloat16* hi, __nv_bfloat16
 size_t packed_weight_elems(int n_out, int k);
 int launch_pack_weight(const void* w, int n_out, int k, void* out, cudaStream_t stream);
 int launch_gemm_tc_partials(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_rows, const void* w, bool packed,
-                            int n_rows, int n_out, int k, float* partial, cudaStream_t stream);
+                            int n_rows, int n_out, int k, float* partial, cudaStream_t stream, bool fill = false);
+// (`fill`: the slots that an element has no sum for are zeroed, so that every element has plan.slots of them)
+// gemm_wide.cu: the same for many rows
+PartialPlan gemm_wide_plan(int n_out, int k, int n_rows);
+int launch_gemm_wide(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_rows, const void* w, bool packed, int n_rows,
+                     int n_out, int k, float* partial, bool fill, cudaStream_t stream);
+int gemm_wide_take_error();
 int launch_gemm_tc(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_rows, const void* w, bool packed,
                    const float* residual, const int32_t* dst_rows, int n_rows, int n_out, int k, float* partial,
                    float* y, cudaStream_t stream);
@@ -118,7 +145,7 @@ struct KvPool {
 // active row appended to the pool.  n_kv_heads = 0: queries only; n_heads = 0:
 // K,V only.
 int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, const KvPool& pool, const RowMeta& rows,
-               int n_rows, float* qkv, const float* partial, int splits, cudaStream_t stream);
+               int n_rows, float* qkv, const float* partial, const PartialPlan& plan, cudaStream_t stream);
 void fill_rope_table(std::vector<float2>& table, int positions, int d_head, double base);
 
 // One attention call: head h of query row r is at q + r * q_stride + h * d_head.
@@ -149,7 +176,7 @@ int launch_attention(const Model& m, const AttnSource& src, const RowMeta& rows,
                      int max_keys, float* part, float* att, __nv_bfloat16* att_hi, __nv_bfloat16* att_lo, cudaStream_t stream);
 
 // f = gelu(u)  |  gelu(u[:, :F]) * u[:, F:]  |  silu(u[:, :F]) * u[:, F:], u given in full or as partial sums.
-int launch_ffn_act(const float* u, const float* partial, int splits, int n_rows, int d_ff, int ffn, float* f,
+int launch_ffn_act(const float* u, const float* partial, const PartialPlan& plan, int n_rows, int d_ff, int ffn, float* f,
                    __nv_bfloat16* f_hi, __nv_bfloat16* f_lo, cudaStream_t stream);
 
 // mega.cu: one forward pass over at most 16 rows as one persistent cooperative kernel

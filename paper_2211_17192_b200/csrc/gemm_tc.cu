@@ -273,27 +273,45 @@ __global__ void split_bf16_kernel(const float* __restrict__ x, size_t n, __nv_bf
     }
 }
 
-// y[dst(r)][n] = sum_s partial[s][r][n] (+ residual[r][n]), splits added in index order
-__global__ void reduce_partials_kernel(const float* __restrict__ partial, const PartialPlan plan, int n_rows, int n_out,
-                                       const float* residual, const int32_t* __restrict__ dst_rows, float* y) {
+// y[dst(r)][n] = sum_s partial[s][r][n] (+ residual[r][n]), splits added in index order.  grid = (column blocks, rows);
+// a thread takes VEC (4 or 1) neighbouring columns at a time.
+template <int VEC>
+__global__ void reduce_partials_kernel(const float* partial, const PartialPlan plan, int n_rows, int n_out,
+                                       const float* residual, const int32_t* dst_rows, float* y) {
     pdl_trigger();
     pdl_wait();
     const size_t total = static_cast<size_t>(n_rows) * n_out;
-    for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < total;
-         i += static_cast<size_t>(gridDim.x) * blockDim.x) {
-        const size_t r = i / n_out, n = i % n_out;
-        const int splits = partial_count(plan, static_cast<int>(r), static_cast<int>(n));
-        float acc = 0.0f;
-        for (int s0 = 0; s0 < splits; s0 += 8) {  // eight loads in flight at a time, added in split order
-            float p[8];
+    const int r = blockIdx.y;
+    const float* in = partial + static_cast<size_t>(r) * n_out;
+    float* out = y + static_cast<size_t>(dst_rows ? dst_rows[r] : r) * n_out;
+    for (int n = VEC * (blockIdx.x * blockDim.x + threadIdx.x); n < n_out; n += VEC * gridDim.x * blockDim.x) {
+        const int splits = partial_count(plan, r, n);
+        float acc[VEC];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) p[k] = s0 + k < splits ? partial[static_cast<size_t>(s0 + k) * total + i] : 0.0f;
+        for (int e = 0; e < VEC; ++e) acc[e] = 0.0f;
+        constexpr int kBatch = VEC == 4 ? 4 : 8;  // loads in flight at a time, added in split order
+        for (int s0 = 0; s0 < splits; s0 += kBatch) {
+            float p[kBatch][VEC];
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (s0 + k < splits) acc = (s0 + k == 0) ? p[k] : acc + p[k];
+            for (int k = 0; k < kBatch; ++k) {
+                if (s0 + k >= splits) continue;
+                const float* src = in + static_cast<size_t>(s0 + k) * total + n;
+                if (VEC == 4) *reinterpret_cast<float4*>(p[k]) = *reinterpret_cast<const float4*>(src);
+                else p[k][0] = *src;
+            }
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k)
+                if (s0 + k < splits) {
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) acc[e] = (s0 + k == 0) ? p[k][e] : acc[e] + p[k][e];
+                }
         }
-        if (residual) acc += residual[i];
-        y[(dst_rows ? static_cast<size_t>(dst_rows[r]) : r) * n_out + n] = acc;
+        if (residual) {
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) acc[e] += residual[static_cast<size_t>(r) * n_out + n + e];
+        }
+        if (VEC == 4) *reinterpret_cast<float4*>(out + n) = make_float4(acc[0], acc[1 % VEC], acc[2 % VEC], acc[3 % VEC]);
+        else out[n] = acc[0];
     }
 }
 
@@ -505,10 +523,11 @@ int launch_gemm_tc(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_rows
     const int status = launch_gemm_tc_partials(hi, lo, hi_rows, w, packed, n_rows, n_out, k, partial, stream);
     if (status != SPEC_OK) return status;
     const PartialPlan plan = gemm_tc_plan(n_out, k, n_rows);
-    const size_t total = static_cast<size_t>(n_rows) * n_out;
-    const int blocks = static_cast<int>(std::min<size_t>((total + 255) / 256, 148 * 8));
-    return launch_pdl(reduce_partials_kernel, dim3(blocks), dim3(256), 0, stream, static_cast<const float*>(partial),
-                      plan, n_rows, n_out, residual, dst_rows, y);
+    const float* sums = partial;
+    const bool vec = n_out % 4 == 0 && (reinterpret_cast<uintptr_t>(y) & 15u) == 0;
+    const dim3 grid((n_out + (vec ? 1023 : 255)) / (vec ? 1024 : 256), n_rows);
+    if (vec) return launch_pdl(reduce_partials_kernel<4>, grid, dim3(256), 0, stream, sums, plan, n_rows, n_out, residual, dst_rows, y);
+    return launch_pdl(reduce_partials_kernel<1>, grid, dim3(256), 0, stream, sums, plan, n_rows, n_out, residual, dst_rows, y);
 }
 
 // Non-zero if a tensor-core GEMM gave up on a bounded wait since the last call.

@@ -11,91 +11,92 @@
 namespace spec {
 namespace {
 
+// No pointer here is __restrict__: a load through a const __restrict__ pointer may be moved in front of pdl_wait(), where
+// what the kernel before writes is not there yet.
+
 __device__ __forceinline__ float load_elem(const void* base, size_t i, bool bf16) {
     return bf16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(base)[i]) : static_cast<const float*>(base)[i];
 }
 
-// x = hi + lo with hi = bf16(x), lo = bf16(x - hi): 16 mantissa bits survive.
-__device__ __forceinline__ void store_split(__nv_bfloat16* hi, __nv_bfloat16* lo, size_t i, float x) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(x);
-    hi[i] = h;
-    lo[i] = __float2bfloat16_rn(x - __bfloat162float(h));
-}
+__device__ __forceinline__ float4 add4(const float4& a, const float4& b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 
-// sum of the split-K partial results of element i, in split order
-__device__ __forceinline__ float sum_partials(const float* __restrict__ partial, int splits, size_t stride, size_t i) {
-    // eight loads in flight at a time (the adds stay in split order, so the sum is the reduction kernels')
-    float acc = 0.0f;
-    for (int s0 = 0; s0 < splits; s0 += 8) {
-        float p[8];
+// Sums of the split-K partial results of the N groups of four elements that start at i[0], .., i[N-1], in split order;
+// BATCH splits' loads of every group are in flight at a time.
+template <int N, int BATCH>
+__device__ __forceinline__ void sum_partials(const float* partial, int splits, size_t stride, const size_t (&i)[N],
+                                             float4 (&out)[N]) {
+    for (int s0 = 0; s0 < splits; s0 += BATCH) {
+        float4 p[BATCH][N];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) p[k] = s0 + k < splits ? partial[static_cast<size_t>(s0 + k) * stride + i] : 0.0f;
+        for (int k = 0; k < BATCH; ++k)
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (s0 + k < splits) acc = (s0 + k == 0) ? p[k] : acc + p[k];
-    }
-    return acc;
-}
-
-// The same for two elements at once (their loads share the flight).
-__device__ __forceinline__ void sum_partials2(const float* __restrict__ partial, int splits, size_t stride, size_t i1,
-                                              size_t i2, float* out1, float* out2) {
-    float a = 0.0f, b = 0.0f;
-    for (int s0 = 0; s0 < splits; s0 += 8) {
-        float p[8], q[8];
+            for (int n = 0; n < N; ++n)
+                p[k][n] = s0 + k < splits ? *reinterpret_cast<const float4*>(partial + static_cast<size_t>(s0 + k) * stride + i[n])
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const bool live = s0 + k < splits;
-            p[k] = live ? partial[static_cast<size_t>(s0 + k) * stride + i1] : 0.0f;
-            q[k] = live ? partial[static_cast<size_t>(s0 + k) * stride + i2] : 0.0f;
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
+        for (int k = 0; k < BATCH; ++k)
             if (s0 + k < splits) {
-                a = (s0 + k == 0) ? p[k] : a + p[k];
-                b = (s0 + k == 0) ? q[k] : b + q[k];
+#pragma unroll
+                for (int n = 0; n < N; ++n) out[n] = (s0 + k == 0) ? p[k][n] : add4(out[n], p[k][n]);
             }
     }
-    *out1 = a;
-    *out2 = b;
 }
 
-// grid = rows, block = 128
-__global__ void embed_kernel(const void* __restrict__ tok_emb, const void* __restrict__ pos_emb, bool bf16,
-                             bool add_pos, const int32_t* __restrict__ token, const int32_t* __restrict__ pos, int d,
-                             int vocab, int max_positions, float* __restrict__ h) {
+// x = hi + lo with hi = bf16(x), lo = bf16(x - hi): 16 mantissa bits survive.  Four elements at once.
+__device__ __forceinline__ void store_split4(__nv_bfloat16* hi, __nv_bfloat16* lo, size_t i, const float4& x) {
+    const float v[4] = {x.x, x.y, x.z, x.w};
+    __align__(8) __nv_bfloat16 h[4], l[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        h[e] = __float2bfloat16_rn(v[e]);
+        l[e] = __float2bfloat16_rn(v[e] - __bfloat162float(h[e]));
+    }
+    *reinterpret_cast<uint2*>(hi + i) = *reinterpret_cast<const uint2*>(h);
+    *reinterpret_cast<uint2*>(lo + i) = *reinterpret_cast<const uint2*>(l);
+}
+
+// four consecutive elements (i a multiple of four) of an fp32 or bf16 array
+__device__ __forceinline__ float4 load_elem4(const void* base, size_t i, bool bf16) {
+    if (!bf16) return *reinterpret_cast<const float4*>(static_cast<const float*>(base) + i);
+    const uint2 t = *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(base) + i);
+    return make_float4(__uint_as_float(t.x << 16), __uint_as_float(t.x & 0xffff0000u), __uint_as_float(t.y << 16),
+                       __uint_as_float(t.y & 0xffff0000u));
+}
+
+// grid = (ceil(d / 512), rows), block = 128: four elements per thread.
+__global__ void embed_kernel(const void* tok_emb, const void* pos_emb, bool bf16,
+                             bool add_pos, const int32_t* token, const int32_t* pos, int d,
+                             int vocab, int max_positions, float* h) {
     pdl_trigger();
     pdl_wait();
-    const int r = blockIdx.x;
+    const int r = blockIdx.y;
     const int t = min(max(token[r], 0), vocab - 1);
     const int p = min(max(pos[r], 0), max_positions - 1);
-    for (int i = threadIdx.x; i < d; i += blockDim.x) {
-        float v = load_elem(tok_emb, static_cast<size_t>(t) * d + i, bf16);
-        if (add_pos) v += load_elem(pos_emb, static_cast<size_t>(p) * d + i, bf16);
-        h[static_cast<size_t>(r) * d + i] = v;
-    }
+    const int i = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (i >= d) return;
+    float4 v = load_elem4(tok_emb, static_cast<size_t>(t) * d + i, bf16);
+    if (add_pos) v = add4(v, load_elem4(pos_emb, static_cast<size_t>(p) * d + i, bf16));
+    *reinterpret_cast<float4*>(h + static_cast<size_t>(r) * d + i) = v;
 }
 
-// grid = rows, block = kNormThreads; d is a multiple of 4.  Row r of the output is
+// grid = rows, block = THREADS; d is a multiple of 4, at most 4 * THREADS * PER.  Row r of the output is
 // RMSNorm(h[src(r)]) * gain.  If `partial` is given, h[r] += sum of the partial
 // results first (the residual add of the GEMM that produced them) and the new h
-// is stored.  A thread holds up to kNormPerThread float4 of the row in registers,
-// so every load of the row and of its partial sums is in flight at once.
-constexpr int kNormThreads = 1024;
-constexpr int kNormPerThread = 4;  // rows up to 16384 wide
+// is stored.  A thread holds up to PER float4 of the row in registers.
+constexpr int kNormMaxWidth = 4 * 1024 * 4;
 
-template <int THREADS>
+template <int THREADS, int PER>
 __global__ void __launch_bounds__(THREADS)
-norm_kernel(float* h, const float* __restrict__ partial, const PartialPlan plan, int n_rows, const float* __restrict__ gain,
-            const int32_t* __restrict__ src_rows, int d, float eps, float* __restrict__ out,
-            __nv_bfloat16* __restrict__ out_hi, __nv_bfloat16* __restrict__ out_lo) {
+norm_kernel(float* h, const float* partial, const PartialPlan plan, int n_rows, const float* gain,
+            const int32_t* src_rows, int d, float eps, float* out,
+            __nv_bfloat16* out_hi, __nv_bfloat16* out_lo) {
     __shared__ float red[THREADS / 32];
     const int r = blockIdx.x;
     const int groups = d / 4;
     // the gains are constants: fetched while the kernel before this one is still finishing
-    float4 gg[kNormPerThread];
+    float4 gg[PER];
 #pragma unroll
-    for (int j = 0; j < kNormPerThread; ++j) {
+    for (int j = 0; j < PER; ++j) {
         const int g = threadIdx.x + j * THREADS;
         gg[j] = g < groups ? *reinterpret_cast<const float4*>(gain + 4 * g) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -107,31 +108,45 @@ norm_kernel(float* h, const float* __restrict__ partial, const PartialPlan plan,
     const int src_row = src_rows ? src_rows[r] : r;
     const size_t src = static_cast<size_t>(src_row) * d;
     const size_t stride = static_cast<size_t>(n_rows) * d;
-    float4 v[kNormPerThread];
-    float ss = 0.0f;
+    float4 v[PER];
 #pragma unroll
-    for (int j = 0; j < kNormPerThread; ++j) {
+    for (int j = 0; j < PER; ++j) {
         const int g = threadIdx.x + j * THREADS;
-        v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (g < groups) {
-            v[j] = *reinterpret_cast<const float4*>(h + src + 4 * g);
-            if (partial) {
-                const int splits = partial_count(plan, src_row, 4 * g);
-                for (int s0 = 0; s0 < splits; s0 += 8) {  // eight loads in flight at a time, added in split order
-                    float4 p[8];
+        v[j] = g < groups ? *reinterpret_cast<const float4*>(h + src + 4 * g) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (partial) {
+        constexpr int kBatch = PER == 1 ? 8 : 2;  // splits in flight at a time, added in split order
+        int splits[PER], most = 0;
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        p[k] = s0 + k < splits ? *reinterpret_cast<const float4*>(partial + (s0 + k) * stride + src + 4 * g)
-                                               : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int j = 0; j < PER; ++j) {
+            const int g = threadIdx.x + j * THREADS;
+            splits[j] = g < groups ? partial_count(plan, src_row, 4 * g) : 0;
+            most = max(most, splits[j]);
+        }
+        for (int s0 = 0; s0 < most; s0 += kBatch) {
+            float4 p[kBatch][PER];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if (s0 + k < splits) { v[j].x += p[k].x; v[j].y += p[k].y; v[j].z += p[k].z; v[j].w += p[k].w; }
-                }
-                *reinterpret_cast<float4*>(h + src + 4 * g) = v[j];
-            }
-            ss += (v[j].x * v[j].x + v[j].y * v[j].y) + (v[j].z * v[j].z + v[j].w * v[j].w);
+            for (int k = 0; k < kBatch; ++k)
+#pragma unroll
+                for (int j = 0; j < PER; ++j)
+                    p[k][j] = s0 + k < splits[j] ? *reinterpret_cast<const float4*>(partial + static_cast<size_t>(s0 + k) * stride + src +
+                                                                                    4 * (threadIdx.x + j * THREADS))
+                                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k)
+#pragma unroll
+                for (int j = 0; j < PER; ++j)
+                    if (s0 + k < splits[j]) v[j] = add4(v[j], p[k][j]);
+        }
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int g = threadIdx.x + j * THREADS;
+            if (g < groups) *reinterpret_cast<float4*>(h + src + 4 * g) = v[j];
         }
     }
+    float ss = 0.0f;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) ss += (v[j].x * v[j].x + v[j].y * v[j].y) + (v[j].z * v[j].z + v[j].w * v[j].w);
     ss = warp_sum(ss);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
     __syncthreads();
@@ -141,72 +156,91 @@ norm_kernel(float* h, const float* __restrict__ partial, const PartialPlan plan,
     const float scale = rsqrtf(total / static_cast<float>(d) + eps);
     const size_t dst = static_cast<size_t>(r) * d;
 #pragma unroll
-    for (int j = 0; j < kNormPerThread; ++j) {
+    for (int j = 0; j < PER; ++j) {
         const int g = threadIdx.x + j * THREADS;
         if (g < groups) {
-            const float y[4] = {v[j].x * scale * gg[j].x, v[j].y * scale * gg[j].y, v[j].z * scale * gg[j].z,
-                                v[j].w * scale * gg[j].w};
-            if (out) *reinterpret_cast<float4*>(out + dst + 4 * g) = make_float4(y[0], y[1], y[2], y[3]);
-            if (out_hi) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) store_split(out_hi, out_lo, dst + 4 * g + e, y[e]);
-            }
+            const float4 y = make_float4(v[j].x * scale * gg[j].x, v[j].y * scale * gg[j].y, v[j].z * scale * gg[j].z,
+                                         v[j].w * scale * gg[j].w);
+            if (out) *reinterpret_cast<float4*>(out + dst + 4 * g) = y;
+            if (out_hi) store_split4(out_hi, out_lo, dst + 4 * g, y);
         }
     }
 }
 
-// grid = (n_heads + 2 n_kv_heads, rows), block = d_head / 2.  qkv row layout:
-// [q heads | k heads | v heads], d_head each.  A CTA finishes one head of one row
-// of the qkv GEMM (optional partial sums), applies rotary positions (q and k
-// heads; thread j owns the pair j, j + d_head/2), leaves q in `qkv` for the
+template <typename KV>
+__device__ __forceinline__ void store_cached4(KV* dst, const float (&v)[4]) {
+    __align__(16) KV t[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) t[e] = to_cached<KV>(v[e]);
+    if (sizeof(KV) == 4) *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(t);
+    else *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(t);
+}
+
+// grid = (ceil(heads * d_head / 8 / block), rows), heads = n_heads + 2 n_kv_heads.  qkv row layout:
+// [q heads | k heads | v heads], d_head each.  A thread finishes elements j .. j+3 and
+// j + d_head/2 .. of one head of one row of the qkv GEMM (optional partial sums), applies
+// rotary positions (q and k heads; they pair j with j + d_head/2), leaves q in `qkv` for the
 // attention kernel, and appends K or V to the paged cache.
 template <typename KV>
-__global__ void qkv_kernel(float* __restrict__ qkv, const float* __restrict__ partial, const PartialPlan plan, int n_rows,
-                           const int32_t* __restrict__ pos, const int32_t* __restrict__ seq, int n_heads,
-                           int n_kv_heads, int d_head, const float2* __restrict__ rope_table,
-                           KV* __restrict__ kv_layer, const int32_t* __restrict__ page_table, int pages_per_seq,
+__global__ void qkv_kernel(float* qkv, const float* partial, const PartialPlan plan, int n_rows,
+                           const int32_t* pos, const int32_t* seq, int n_heads,
+                           int n_kv_heads, int d_head, const float2* rope_table,
+                           KV* kv_layer, const int32_t* page_table, int pages_per_seq,
                            int page_size) {
     pdl_trigger();
     pdl_wait();
-    const int head = blockIdx.x, r = blockIdx.y, j = threadIdx.x;
+    const int half = d_head / 2, per_head = half / 4;
+    const int task = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+    const int head = task / per_head, j = 4 * (task % per_head);
+    if (head >= n_heads + 2 * n_kv_heads) return;
     const int p = pos[r];
-    const int half = d_head / 2;
-    const int width = (n_heads + 2 * n_kv_heads) * d_head;
-    const size_t at = static_cast<size_t>(r) * width + head * d_head;
-    float x1, x2;
-    if (partial) {
-        const size_t stride = static_cast<size_t>(n_rows) * width;
-        // (a head of 64 or 128 columns lies inside one 256-column tile)
-        sum_partials2(partial, partial_count(plan, r, head * d_head), stride, at + j, at + j + half, &x1, &x2);
-    } else {
-        x1 = qkv[at + j];
-        x2 = qkv[at + j + half];
-    }
     const bool is_q = head < n_heads, is_k = !is_q && head < n_heads + n_kv_heads;
-    if (rope_table && p >= 0 && (is_q || is_k)) {
-        const float2 t = rope_table[static_cast<size_t>(p) * half + j];  // (cos, sin) of position p
-        const float y1 = x1 * t.x - x2 * t.y, y2 = x2 * t.x + x1 * t.y;
-        x1 = y1;
-        x2 = y2;
+    const bool rotate = rope_table && p >= 0 && (is_q || is_k);
+    float4 t0, t1;  // (cos, sin) of position p for the four pairs
+    if (rotate) {
+        const float4* t = reinterpret_cast<const float4*>(rope_table + static_cast<size_t>(p) * half + j);
+        t0 = t[0];
+        t1 = t[1];
+    }
+    const int width = (n_heads + 2 * n_kv_heads) * d_head;
+    const size_t at = static_cast<size_t>(r) * width + head * d_head + j;
+    const size_t where[2] = {at, at + half};
+    float4 x[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    if (partial) {
+        // (a head of 64 or 128 columns lies inside one 256-column tile)
+        sum_partials<2, 4>(partial, partial_count(plan, r, head * d_head), static_cast<size_t>(n_rows) * width, where, x);
+    } else {
+        x[0] = *reinterpret_cast<const float4*>(qkv + where[0]);
+        x[1] = *reinterpret_cast<const float4*>(qkv + where[1]);
+    }
+    float a[4] = {x[0].x, x[0].y, x[0].z, x[0].w}, b[4] = {x[1].x, x[1].y, x[1].z, x[1].w};
+    if (rotate) {
+        const float c[4] = {t0.x, t0.z, t1.x, t1.z}, s[4] = {t0.y, t0.w, t1.y, t1.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float y1 = a[e] * c[e] - b[e] * s[e], y2 = b[e] * c[e] + a[e] * s[e];
+            a[e] = y1;
+            b[e] = y2;
+        }
     }
     if (is_q) {
-        qkv[at + j] = x1;
-        qkv[at + j + half] = x2;
+        *reinterpret_cast<float4*>(qkv + where[0]) = make_float4(a[0], a[1], a[2], a[3]);
+        *reinterpret_cast<float4*>(qkv + where[1]) = make_float4(b[0], b[1], b[2], b[3]);
         return;
     }
     if (p < 0) return;  // inactive row: nothing is cached
     const int kv_head = is_k ? head - n_heads : head - n_heads - n_kv_heads;
     const int page = page_table[seq[r] * pages_per_seq + p / page_size];
     const size_t block = (static_cast<size_t>(page) * 2 + (is_k ? 0 : 1)) * n_kv_heads + kv_head;
-    KV* dst = kv_layer + (block * page_size + p % page_size) * d_head;
-    dst[j] = to_cached<KV>(x1);
-    dst[j + half] = to_cached<KV>(x2);
+    KV* dst = kv_layer + (block * page_size + p % page_size) * d_head + j;
+    store_cached4<KV>(dst, a);
+    store_cached4<KV>(dst + half, b);
 }
 
 // logits[dst(i)] = table[token[src(i)]] for a table model: grid = (chunks, rows), block = 256.
-__global__ void table_logits_kernel(const void* __restrict__ table, bool bf16, int vocab, const int32_t* __restrict__ token,
-                                    const int32_t* __restrict__ src_rows, const int32_t* __restrict__ dst_rows,
-                                    float* __restrict__ logits) {
+__global__ void table_logits_kernel(const void* table, bool bf16, int vocab, const int32_t* token,
+                                    const int32_t* src_rows, const int32_t* dst_rows,
+                                    float* logits) {
     pdl_trigger();
     pdl_wait();
     const int i = blockIdx.y;
@@ -222,10 +256,10 @@ __global__ void table_logits_kernel(const void* __restrict__ table, bool bf16, i
 // none.  Positions below length[seq] read the committed tokens, later ones this
 // iteration's guesses.  grid = (chunks, rows): every CTA repeats the search (a few
 // thousand token compares) and writes its share of the row.
-__global__ void copy_logits_kernel(const int32_t* __restrict__ tokens, int max_len, const int32_t* __restrict__ length,
-                                   const int32_t* __restrict__ draft_tokens, int gamma, const int32_t* __restrict__ row_pos,
-                                   const int32_t* __restrict__ row_seq, const int32_t* __restrict__ src_rows,
-                                   const int32_t* __restrict__ dst_rows, int ngram, int vocab, float* __restrict__ logits) {
+__global__ void copy_logits_kernel(const int32_t* tokens, int max_len, const int32_t* length,
+                                   const int32_t* draft_tokens, int gamma, const int32_t* row_pos,
+                                   const int32_t* row_seq, const int32_t* src_rows,
+                                   const int32_t* dst_rows, int ngram, int vocab, float* logits) {
     __shared__ int best[32];
     pdl_trigger();
     pdl_wait();
@@ -261,48 +295,56 @@ __device__ __forceinline__ float gelu_tanh(float x) {
 __device__ __forceinline__ float silu(float x) { return x / (1.0f + expf(-x)); }
 
 // f = gelu(u)  |  gelu(gate) * up  |  silu(gate) * up, with u either given in
-// full or as the partial sums of the FFN-in GEMM.
-__global__ void ffn_act_kernel(const float* __restrict__ u, const float* __restrict__ partial, const PartialPlan plan, int n_rows,
-                               int d_ff, int ffn, float* __restrict__ f, __nv_bfloat16* __restrict__ f_hi,
-                               __nv_bfloat16* __restrict__ f_lo) {
+// full or as the partial sums of the FFN-in GEMM.  grid = (ceil(d_ff / 4 / block), rows): four columns per thread.
+template <int FFN>
+__global__ void ffn_act_kernel(const float* u, const float* partial, const PartialPlan plan, int n_rows,
+                               int d_ff, float* f, __nv_bfloat16* f_hi,
+                               __nv_bfloat16* f_lo) {
     pdl_trigger();
     pdl_wait();
-    const size_t total = static_cast<size_t>(n_rows) * d_ff;
-    const int width = ffn == SPEC_FFN_GELU ? d_ff : 2 * d_ff;
+    const int c = 4 * (blockIdx.x * blockDim.x + threadIdx.x), r = blockIdx.y;
+    if (c >= d_ff) return;
+    constexpr bool kGated = FFN != SPEC_FFN_GELU;
+    const int width = kGated ? 2 * d_ff : d_ff;
     const size_t stride = static_cast<size_t>(n_rows) * width;
-    for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < total;
-         i += static_cast<size_t>(gridDim.x) * blockDim.x) {
-        const size_t r = i / d_ff, c = i % d_ff;
-        const size_t a = r * width + c;
-        float y;
-        if (ffn == SPEC_FFN_GELU) {
-            y = gelu_tanh(partial ? sum_partials(partial, partial_count(plan, static_cast<int>(r), static_cast<int>(c)), stride, a) : u[a]);
+    const size_t at = static_cast<size_t>(r) * width + c;
+    float4 g = make_float4(0.f, 0.f, 0.f, 0.f), up = g;
+    if (!partial) {
+        g = *reinterpret_cast<const float4*>(u + at);
+        if (kGated) up = *reinterpret_cast<const float4*>(u + at + d_ff);
+    } else {
+        const int n_gate = partial_count(plan, r, c), n_up = kGated ? partial_count(plan, r, c + d_ff) : n_gate;
+        if (kGated && n_gate == n_up) {
+            const size_t where[2] = {at, at + d_ff};
+            float4 both[2] = {g, g};
+            sum_partials<2, 4>(partial, n_gate, stride, where, both);
+            g = both[0];
+            up = both[1];
         } else {
-            float gate, up;
-            if (partial) {
-                const int n_gate = partial_count(plan, static_cast<int>(r), static_cast<int>(c));
-                const int n_up = partial_count(plan, static_cast<int>(r), static_cast<int>(c) + d_ff);
-                if (n_gate == n_up) {
-                    sum_partials2(partial, n_gate, stride, a, a + d_ff, &gate, &up);
-                } else {
-                    gate = sum_partials(partial, n_gate, stride, a);
-                    up = sum_partials(partial, n_up, stride, a + d_ff);
-                }
-            } else {
-                gate = u[a];
-                up = u[a + d_ff];
+            const size_t where[1] = {at};
+            float4 one[1] = {g};
+            sum_partials<1, 8>(partial, n_gate, stride, where, one);
+            g = one[0];
+            if (kGated) {
+                const size_t where_up[1] = {at + d_ff};
+                sum_partials<1, 8>(partial, n_up, stride, where_up, one);
+                up = one[0];
             }
-            y = (ffn == SPEC_FFN_SWIGLU ? silu(gate) : gelu_tanh(gate)) * up;
         }
-        if (f) f[i] = y;
-        if (f_hi) store_split(f_hi, f_lo, i, y);
     }
+    float4 y;
+    if (FFN == SPEC_FFN_GELU) y = make_float4(gelu_tanh(g.x), gelu_tanh(g.y), gelu_tanh(g.z), gelu_tanh(g.w));
+    else if (FFN == SPEC_FFN_SWIGLU) y = make_float4(silu(g.x) * up.x, silu(g.y) * up.y, silu(g.z) * up.z, silu(g.w) * up.w);
+    else y = make_float4(gelu_tanh(g.x) * up.x, gelu_tanh(g.y) * up.y, gelu_tanh(g.z) * up.z, gelu_tanh(g.w) * up.w);
+    const size_t i = static_cast<size_t>(r) * d_ff + c;
+    if (f) *reinterpret_cast<float4*>(f + i) = y;
+    if (f_hi) store_split4(f_hi, f_lo, i, y);
 }
 
 }  // namespace
 
 int launch_embed(const Model& m, const RowMeta& rows, int n_rows, float* h, cudaStream_t stream) {
-    return launch_pdl(embed_kernel, dim3(n_rows), dim3(128), 0, stream, m.tok_emb, m.pos_emb, m.bf16(),
+    return launch_pdl(embed_kernel, dim3((m.cfg.d_model / 4 + 127) / 128, n_rows), dim3(128), 0, stream, m.tok_emb, m.pos_emb, m.bf16(),
                       m.cfg.arch == SPEC_ARCH_GPT, rows.token, rows.pos, m.cfg.d_model, m.cfg.vocab,
                       m.cfg.max_positions, h);
 }
@@ -325,24 +367,28 @@ int launch_copy_logits(const int32_t* tokens, int max_len, const int32_t* length
 int launch_norm(float* h, const float* partial, const PartialPlan& plan, int rows_total, const float* gain, const int32_t* src_rows,
                 int n_rows, int d, float eps, float* out, __nv_bfloat16* out_hi, __nv_bfloat16* out_lo,
                 cudaStream_t stream) {
-    if (d % 4 || d > 4 * kNormThreads * kNormPerThread)
-        return fail(SPEC_ERR_BAD_CONFIG, "norm: width %d is not a multiple of 4 or exceeds %d", d, 4 * kNormThreads * kNormPerThread);
-    // a thread per 128-bit group of the row where the row is narrow (fewer warps to reduce over)
+    if (d % 4 || d > kNormMaxWidth)
+        return fail(SPEC_ERR_BAD_CONFIG, "norm: width %d is not a multiple of 4 or exceeds %d", d, kNormMaxWidth);
+#define SPEC_LAUNCH_NORM(T, P)                                                                                              \
+    return launch_pdl(norm_kernel<T, P>, dim3(n_rows), dim3(T), 0, stream, h, partial, plan, rows_total, gain, src_rows, d, \
+                      eps, out, out_hi, out_lo)
+    // a thread per 128-bit group of the row (fewer warps to reduce over where the row is narrow); with more rows than
+    // SMs, small CTAs with several groups per thread, so that the CTAs of an SM wait for memory side by side
     const int groups = d / 4;
-    if (groups <= 128)
-        return launch_pdl(norm_kernel<128>, dim3(n_rows), dim3(128), 0, stream, h, partial, plan, rows_total, gain, src_rows, d,
-                          eps, out, out_hi, out_lo);
-    if (groups <= 256)
-        return launch_pdl(norm_kernel<256>, dim3(n_rows), dim3(256), 0, stream, h, partial, plan, rows_total, gain, src_rows, d,
-                          eps, out, out_hi, out_lo);
-    return launch_pdl(norm_kernel<kNormThreads>, dim3(n_rows), dim3(kNormThreads), 0, stream, h, partial, plan, rows_total,
-                      gain, src_rows, d, eps, out, out_hi, out_lo);
+    if (groups <= 128) SPEC_LAUNCH_NORM(128, 1);
+    if (groups <= 256) SPEC_LAUNCH_NORM(256, 1);
+    if (groups <= 1024 && n_rows > 148) SPEC_LAUNCH_NORM(256, 4);
+    if (groups <= 1024) SPEC_LAUNCH_NORM(1024, 1);
+    SPEC_LAUNCH_NORM(1024, 4);
+#undef SPEC_LAUNCH_NORM
 }
 
 int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, const KvPool& pool, const RowMeta& rows,
                int n_rows, float* qkv, const float* partial, const PartialPlan& plan, cudaStream_t stream) {
-    const dim3 grid(n_heads + 2 * n_kv_heads, n_rows);
-    const dim3 block(d_head / 2);
+    const int tasks = (n_heads + 2 * n_kv_heads) * (d_head / 8);
+    const int threads = n_rows <= 16 ? 64 : 256;
+    const dim3 grid((tasks + threads - 1) / threads, n_rows);
+    const dim3 block(threads);
     if (pool.dtype == SPEC_DTYPE_FP16)
         return launch_pdl(qkv_kernel<__half>, grid, block, 0, stream, qkv, partial, plan, n_rows, rows.pos, rows.seq, n_heads,
                           n_kv_heads, d_head, rope, static_cast<__half*>(pool.kv), pool.page_table, pool.pages_per_seq,
@@ -358,10 +404,14 @@ int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, cons
 
 int launch_ffn_act(const float* u, const float* partial, const PartialPlan& plan, int n_rows, int d_ff, int ffn, float* f,
                    __nv_bfloat16* f_hi, __nv_bfloat16* f_lo, cudaStream_t stream) {
-    const size_t total = static_cast<size_t>(n_rows) * d_ff;
-    const int blocks = static_cast<int>(std::min<size_t>((total + 255) / 256, 148 * 8));
-    return launch_pdl(ffn_act_kernel, dim3(blocks), dim3(256), 0, stream, u, partial, plan, n_rows, d_ff, ffn, f,
-                      f_hi, f_lo);
+    const int threads = n_rows <= 16 ? 64 : 256;
+    const dim3 grid((d_ff / 4 + threads - 1) / threads, n_rows);
+#define SPEC_LAUNCH_ACT(F) \
+    return launch_pdl(ffn_act_kernel<F>, grid, dim3(threads), 0, stream, u, partial, plan, n_rows, d_ff, f, f_hi, f_lo)
+    if (ffn == SPEC_FFN_GELU) SPEC_LAUNCH_ACT(SPEC_FFN_GELU);
+    if (ffn == SPEC_FFN_SWIGLU) SPEC_LAUNCH_ACT(SPEC_FFN_SWIGLU);
+    SPEC_LAUNCH_ACT(SPEC_FFN_GATED_GELU);
+#undef SPEC_LAUNCH_ACT
 }
 
 // (cos, sin) of position * base^(-2j / d_head), evaluated in double precision on

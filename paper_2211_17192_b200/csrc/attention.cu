@@ -573,7 +573,6 @@ attention_f16_kernel(const float* __restrict__ qkv, int q_stride, const int32_t*
     constexpr int KP = kF16Warps / MB;        // key parts of a tile
     constexpr int KW = kF16TileKeys / KP;     // keys of a tile that one warp multiplies (16 MB)
     constexpr int NB = KW / 8;                // 8-key blocks of those
-    constexpr int CH = DH / 8;                // 16-byte chunks of a row
     constexpr int QN = 16 * MB;               // queries of this CTA
     constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
     extern __shared__ __align__(1024) unsigned char smem_raw[];  // (the swizzled boxes want 1024-byte alignment)
@@ -869,6 +868,223 @@ attention_f16_kernel(const float* __restrict__ qkv, int q_stride, const int32_t*
     }
 }
 
+// ---- prompt passes: many rows per sequence over fp16 K,V rows -------------------
+//
+// The rows of a prompt chunk lie sequence after sequence without padding; a segment is one sequence's run of them.
+// A CTA takes 128 queries of one (segment, KV head) - (row, head of the group) pairs, 16 to a warp - and walks the
+// keys from 0 to the last one its last row sees, so every 64-key tile of K and V is fetched once per 128 queries and
+// no key beyond the causal limit is fetched at all.  Tiles, swizzle, fragments and number formats are those of
+// attention_f16_kernel above; there is one key slice, so nothing is merged and the output is written here.  Bound by the
+// mma.sync chains of eight warps per SM.  Against the decode kernels on prompt chunks of 256 rows padded to the longest
+// sequence (7B shape): 16 prompts of 500 .. 1000 tokens 112 -> 22 ms of attention, one of 1024 tokens 19 -> 2 ms.
+constexpr int kPromptWarps = 8;
+constexpr int kPromptQueries = 16 * kPromptWarps;
+constexpr int kPromptStages = 3;
+
+template <int DH>
+struct PromptSmem {
+    static constexpr int kQ = kPromptQueries * DH;
+    static constexpr int kTile = kF16TileKeys * DH;
+    static constexpr int kStage = 2 * kTile;  // K, then V
+    static constexpr size_t kBytes = static_cast<size_t>(kQ + kPromptStages * kStage) * sizeof(__half);
+};
+
+// grid = (query blocks of the longest segment, n_kv_heads, segments), block = 32 * kPromptWarps.
+// segs[i] = (first row, rows, sequence, position of the first row).
+template <int DH>
+__global__ void __launch_bounds__(32 * kPromptWarps, DH == 64 ? 2 : 1)
+attention_prompt_kernel(const float* qkv, int q_stride, const int4* segs, int n_heads, int n_kv_heads,
+                        const __grid_constant__ CUtensorMap kv_map, const int32_t* __restrict__ page_table, int pages_per_seq,
+                        int page_size, float scale, const AttnOut out) {
+    using S = PromptSmem<DH>;
+    constexpr int NB = kF16TileKeys / 8;
+    constexpr float kLog2e = 1.4426950408889634f;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t landed[kPromptStages];
+    __half* Qs = reinterpret_cast<__half*>(smem_raw);
+    __half* stages = Qs + S::kQ;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+#pragma unroll
+        for (int st = 0; st < kPromptStages; ++st)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(&landed[st]))));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    pdl_trigger();
+    pdl_wait();
+    const int4 seg = segs[blockIdx.z];
+    const int row0 = seg.x, pos0 = seg.w;
+    const int kv_head = blockIdx.y, group = n_heads / n_kv_heads;
+    const int queries = group * seg.y;
+    const int q0 = static_cast<int>(gridDim.x - 1 - blockIdx.x) * kPromptQueries;  // (the longest walks are launched first)
+    if (q0 >= queries) return;
+    const int last_row = (min(queries, q0 + kPromptQueries) - 1) / group;
+    const int seq_keys = pos0 + last_row + 1;  // keys that the CTA's last row sees
+    const int tiles = (seq_keys + kF16TileKeys - 1) / kF16TileKeys;
+    const int32_t* pages = page_table + seg.z * pages_per_seq;
+    const int page_shift = __ffs(page_size) - 1;
+
+    auto issue = [&](int i) {  // tile i into stage i % kPromptStages: as in attention_f16_kernel
+        if (tid == 0 && i < tiles) {
+            const int k0 = kF16TileKeys * i;
+            const int st = i % kPromptStages;
+            const uint32_t bar = static_cast<uint32_t>(__cvta_generic_to_shared(&landed[st]));
+            const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(stages + st * S::kStage));
+            int pg[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) pg[h] = pages[min(k0 + 32 * h, seq_keys - 1) >> page_shift];
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the stage was read with ldmatrix before
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(static_cast<uint32_t>(S::kStage * sizeof(__half)))
+                         : "memory");
+#pragma unroll
+            for (int v = 0; v < 2; ++v)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int row = ((2 * pg[h] + v) * n_kv_heads + kv_head) * page_size + ((k0 + 32 * h) & (page_size - 1));
+#pragma unroll
+                    for (int c = 0; c < DH / 64; ++c) {
+                        const uint32_t d = dst + static_cast<uint32_t>((v * S::kTile + c * kF16TileKeys * 64 + h * 32 * 64) * sizeof(__half));
+                        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                                     ::"r"(d), "l"(&kv_map), "r"(c * 64), "r"(row), "r"(bar)
+                                     : "memory");
+                    }
+                }
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < kPromptStages - 1; ++i) issue(i);
+    const float q_scale = scale * kLog2e;
+    for (int i = tid; i < kPromptQueries * (DH / 4); i += 32 * kPromptWarps) {
+        const int qi = i / (DH / 4), e = 4 * (i % (DH / 4)), q = q0 + qi;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (q < queries)
+            v = *reinterpret_cast<const float4*>(qkv + static_cast<size_t>(row0 + q / group) * q_stride + (kv_head * group + q % group) * DH + e);
+        *reinterpret_cast<uint2*>(Qs + f16_at<DH>(qi, e & ~7) + (e & 7)) =
+            make_uint2(pack_half2(v.x * q_scale, v.y * q_scale), pack_half2(v.z * q_scale, v.w * q_scale));
+    }
+    const int g = lane >> 2, t = lane & 3;
+    const int q_lo = q0 + warp * 16 + g, q_hi = q_lo + 8;
+    // (a query beyond the live ones sees what the last one sees; its output is not written)
+    const int keys_lo = pos0 + min(q_lo, queries - 1) / group + 1, keys_hi = pos0 + min(q_hi, queries - 1) / group + 1;
+    const int all_see = __reduce_min_sync(kFullMask, min(keys_lo, keys_hi)), any_sees = __reduce_max_sync(kFullMask, max(keys_lo, keys_hi));
+    float m_lo = -FLT_MAX, m_hi = -FLT_MAX, l_lo = 0.0f, l_hi = 0.0f;  // (the sums are this lane's share until the end)
+    float o[DH / 8][4];
+#pragma unroll
+    for (int n = 0; n < DH / 8; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[n][i] = 0.0f;
+    uint32_t qf[DH / 16][4];
+    const int l7 = lane & 7;
+    const int k_lane = l7 * 64 + ((((lane >> 3) ^ l7) & 7) << 3);
+    const int v_row = (l7 + 8 * ((lane >> 3) & 1)) * 64;
+    int v_chunk[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v_chunk[j] = ((((j << 1) | (lane >> 4)) ^ l7) & 7) << 3;
+
+    for (int i = 0; i < tiles; ++i) {
+        // (a wait that runs out is recorded and the pass goes on: no thread leaves the loop alone)
+        if (!mbar_wait_bounded(&landed[i % kPromptStages], (i / kPromptStages) & 1)) atomicCAS(&g_attn_error, 0, 2);
+        __syncthreads();
+        issue(i + kPromptStages - 1);
+        if (i == 0) {
+#pragma unroll
+            for (int ks = 0; ks < DH / 16; ++ks)
+                ldsm_x4(qf[ks], Qs + f16_at<DH>(warp * 16 + (lane & 7) + 8 * ((lane >> 3) & 1), ks * 16 + 8 * (lane >> 4)));
+        }
+        const int k0 = kF16TileKeys * i;
+        if (k0 >= any_sees) continue;
+        const __half* Kt = stages + (i % kPromptStages) * S::kStage;
+        const __half* Vt = Kt + S::kTile;
+        float s[NB][4];
+#pragma unroll
+        for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[nb][j] = 0.0f;
+#pragma unroll
+        for (int kp = 0; kp < DH / 32; ++kp) {
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb) {
+                uint32_t kf[4];
+                ldsm_x4(kf, Kt + nb * 8 * 64 + (kp >> 1) * (kF16TileKeys * 64) + ((kp & 1) ? (k_lane ^ 32) : k_lane));
+                mma_f16(s[nb], qf[2 * kp], kf[0], kf[1]);
+                mma_f16(s[nb], qf[2 * kp + 1], kf[2], kf[3]);
+            }
+        }
+        if (k0 + kF16TileKeys > all_see) {  // (warp-uniform)
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int key = k0 + nb * 8 + 2 * t + (j & 1);
+                    if (key >= (j >= 2 ? keys_hi : keys_lo)) s[nb][j] = -FLT_MAX;
+                }
+        }
+        float tmax_lo = m_lo, tmax_hi = m_hi;
+#pragma unroll
+        for (int nb = 0; nb < NB; ++nb) {
+            tmax_lo = fmaxf(tmax_lo, fmaxf(s[nb][0], s[nb][1]));
+            tmax_hi = fmaxf(tmax_hi, fmaxf(s[nb][2], s[nb][3]));
+        }
+        tmax_lo = fmaxf(tmax_lo, __shfl_xor_sync(kFullMask, tmax_lo, 1));
+        tmax_lo = fmaxf(tmax_lo, __shfl_xor_sync(kFullMask, tmax_lo, 2));
+        tmax_hi = fmaxf(tmax_hi, __shfl_xor_sync(kFullMask, tmax_hi, 1));
+        tmax_hi = fmaxf(tmax_hi, __shfl_xor_sync(kFullMask, tmax_hi, 2));
+        // (key 0 is in tile 0 and every row sees it: from the first tile on the maxima are real scores)
+        if (__any_sync(kFullMask, tmax_lo != m_lo || tmax_hi != m_hi)) {
+            const float r_lo = exp2_approx(m_lo - tmax_lo), r_hi = exp2_approx(m_hi - tmax_hi);
+            l_lo *= r_lo;
+            l_hi *= r_hi;
+#pragma unroll
+            for (int n = 0; n < DH / 8; ++n) {
+                o[n][0] *= r_lo; o[n][1] *= r_lo; o[n][2] *= r_hi; o[n][3] *= r_hi;
+            }
+            m_lo = tmax_lo;
+            m_hi = tmax_hi;
+        }
+        uint32_t pa[NB / 2][4];
+#pragma unroll
+        for (int nb = 0; nb < NB; ++nb) {
+            const float p0 = exp2_approx(s[nb][0] - m_lo), p1 = exp2_approx(s[nb][1] - m_lo);
+            const float p2 = exp2_approx(s[nb][2] - m_hi), p3 = exp2_approx(s[nb][3] - m_hi);
+            l_lo += p0 + p1;
+            l_hi += p2 + p3;
+            pa[nb / 2][(nb & 1) * 2] = pack_half2(p0, p1);
+            pa[nb / 2][(nb & 1) * 2 + 1] = pack_half2(p2, p3);
+        }
+#pragma unroll
+        for (int n2 = 0; n2 < DH / 16; ++n2) {
+#pragma unroll
+            for (int kk = 0; kk < NB / 2; ++kk) {
+                uint32_t vf[4];
+                ldsm_x4_trans(vf, Vt + kk * 16 * 64 + v_row + (n2 >> 2) * (kF16TileKeys * 64) + v_chunk[n2 & 3]);
+                mma_f16(o[2 * n2], pa[kk], vf[0], vf[1]);
+                mma_f16(o[2 * n2 + 1], pa[kk], vf[2], vf[3]);
+            }
+        }
+    }
+    // (every tile that was asked for has been waited for: nothing is in flight)
+    l_lo += __shfl_xor_sync(kFullMask, l_lo, 1);
+    l_lo += __shfl_xor_sync(kFullMask, l_lo, 2);
+    l_hi += __shfl_xor_sync(kFullMask, l_hi, 1);
+    l_hi += __shfl_xor_sync(kFullMask, l_hi, 2);
+    const float inv[2] = {1.0f / l_lo, 1.0f / l_hi};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int q = h ? q_hi : q_lo;
+        if (q >= queries) continue;
+        const size_t at = (static_cast<size_t>(row0 + q / group) * n_heads + kv_head * group + q % group) * DH + 2 * t;
+#pragma unroll
+        for (int n = 0; n < DH / 8; ++n) {
+            const float y0 = o[n][2 * h] * inv[h], y1 = o[n][2 * h + 1] * inv[h];
+            const __nv_bfloat162 hi = __floats2bfloat162_rn(y0, y1);
+            *reinterpret_cast<__nv_bfloat162*>(out.hi + at + n * 8) = hi;
+            *reinterpret_cast<__nv_bfloat162*>(out.lo + at + n * 8) =
+                __floats2bfloat162_rn(y0 - __low2float(hi), y1 - __high2float(hi));
+        }
+    }
+}
+
 // grid = rows * n_heads, block = DH: merge the key slices of one (row, head).
 template <int DH>
 __global__ void attention_combine_kernel(const float* __restrict__ part, int slices, float* __restrict__ att,
@@ -1147,7 +1363,36 @@ int launch_attention_variant(const Model& m, const AttnSource& src, const RowMet
                       static_cast<const float*>(part), slices, out.att, out.hi, out.lo);
 }
 
+template <int DH>
+int launch_prompt_variant(const Model& m, const AttnSource& src, const PromptSegments& segs, const AttnOut& out, cudaStream_t stream) {
+    const int group = m.cfg.n_heads / m.cfg.n_kv_heads;
+    CUtensorMap kv_map;
+    const int status = cached_f16_rows_map(src.pool.kv, static_cast<unsigned long long>(src.pool.n_pages) * 2 * m.cfg.n_kv_heads *
+                                                            src.pool.page_size, DH, &kv_map);
+    if (status != SPEC_OK) return status;
+    static std::atomic<unsigned long long> configured{0};
+    if (first_use_on_this_device(configured))
+        SPEC_CUDA_TRY(cudaFuncSetAttribute(attention_prompt_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           static_cast<int>(PromptSmem<DH>::kBytes)));
+    const dim3 grid((group * segs.longest + kPromptQueries - 1) / kPromptQueries, m.cfg.n_kv_heads, segs.count);
+    return launch_pdl(attention_prompt_kernel<DH>, grid, dim3(32 * kPromptWarps), PromptSmem<DH>::kBytes, stream, src.q, src.q_stride,
+                      segs.table, m.cfg.n_heads, m.cfg.n_kv_heads, kv_map, src.pool.page_table, src.pool.pages_per_seq,
+                      src.pool.page_size, 1.0f / sqrtf(static_cast<float>(DH)), out);
+}
+
 }  // namespace
+
+// The precision of the f16 products is that of the tensor-core kernels that decode passes of bf16 models take (11
+// significant bits), from the same amount of work on; smaller prompts keep the decode kernels' fp32 products.
+bool prompt_attention_serves(const Model& m, long long query_keys) {
+    return m.bf16() && !m.t5() && m.kv_dtype == SPEC_DTYPE_FP16 && query_keys * m.cfg.n_heads >= 65536;
+}
+
+int launch_prompt_attention(const Model& m, const AttnSource& src, const PromptSegments& segs, __nv_bfloat16* att_hi,
+                            __nv_bfloat16* att_lo, cudaStream_t stream) {
+    const AttnOut out{nullptr, att_hi, att_lo};
+    return m.cfg.d_head == 64 ? launch_prompt_variant<64>(m, src, segs, out, stream) : launch_prompt_variant<128>(m, src, segs, out, stream);
+}
 
 int launch_attention(const Model& m, const AttnSource& src, const RowMeta& rows, int batch, int m_rows, int slices,
                      int max_keys, float* part, float* att, __nv_bfloat16* att_hi, __nv_bfloat16* att_lo, cudaStream_t stream) {

@@ -36,6 +36,7 @@ struct spec_ctx {
     float* attn_part = nullptr;  // per key slice: (max, sum, accumulator) of every (row, head)
     int hi_rows = 0;
     spec::PassScratch pass;  // the persistent pass kernel's scratch (passes of at most 16 rows of a bf16 model)
+    int32_t* row_block = nullptr;  // one allocation: the five row arrays below, a prompt chunk's packed rows and segments
     int32_t *row_token = nullptr, *row_pos = nullptr, *row_seq = nullptr, *logit_src = nullptr, *logit_dst = nullptr;
     int32_t* page_table = nullptr;
 
@@ -189,14 +190,18 @@ struct Pass {
     // h += Wo . attention(projection of rmsnorm(h) * gain) over `pool`
     int self_attention(const spec_layer_weights& w, const spec_layer_weights& pw, const RowMeta& rows, int batch, int m_rows,
                        const KvPool& pool, const int32_t* kv_len, const float* bias, int bias_span, int bias_zero,
-                       int max_keys) {
+                       int max_keys, const PromptSegments* segs = nullptr) {
         const spec_model_cfg& c = m.cfg;
         SPEC_TRY(norm(w.ln1, nullptr, n_rows));
         SPEC_TRY(proj(w.wqkv, pw.wqkv, m.qkv_dim(), c.d_model, ctx->a, ctx->qkv));
         SPEC_TRY(launch_qkv(c.n_heads, c.n_kv_heads, c.d_head, c.arch == SPEC_ARCH_LLAMA ? m.rope_table : nullptr, pool, rows,
                             n_rows, ctx->qkv, partials(), last, st));
-        const int slices = attention_slices(m, batch, m_rows, max_keys);
         const AttnSource src{ctx->qkv, m.qkv_dim(), pool, kv_len, bias, bias_span, bias_zero};
+        if (segs) {
+            SPEC_TRY(launch_prompt_attention(m, src, *segs, hi(), lo(), st));
+            return residual(w.wo, pw.wo, m.q_dim(), ctx->att);
+        }
+        const int slices = attention_slices(m, batch, m_rows, max_keys);
         SPEC_TRY(launch_attention(m, src, rows, batch, m_rows, slices, max_keys, ctx->attn_part, tc ? nullptr : ctx->att,
                                   tc ? hi() : nullptr, tc ? lo() : nullptr, st));
         return residual(w.wo, pw.wo, m.q_dim(), ctx->att);
@@ -208,6 +213,8 @@ int device_gave_up(spec_ctx* ctx) {
     const int gemm = gemm_tc_take_error(), wide = gemm_wide_take_error(), pass = pass_take_error(), attn = attention_take_error();
     return gemm ? gemm : wide ? wide : pass ? pass : attn;
 }
+
+RowMeta row_meta(const spec_ctx* ctx) { return RowMeta{ctx->row_token, ctx->row_pos, ctx->row_seq}; }
 
 KvPool layer_pool(const spec_ctx* ctx, const Model& m, int layer) {
     return KvPool{static_cast<char*>(m.kv) + static_cast<size_t>(layer) * m.layer_stride, m.kv_elem_bytes, m.kv_dtype, ctx->page_table,
@@ -222,12 +229,12 @@ KvPool source_pool(const spec_ctx* ctx, const Model& m, void* base) {
 // One forward pass of `m` over batch * m_rows rows (rows of sequence b are rows
 // b*m_rows .. of ctx->row_*); K,V rows of active rows are appended to the cache.
 // If n_logit_rows > 0 the final norm and LM head run on rows logit_src[i] and
-// write logits rows logit_dst[i] (all rows in order if both are null).
-int forward(spec_ctx* ctx, const Model& m, int batch, int m_rows, int n_logit_rows, const int32_t* logit_src,
-            const int32_t* logit_dst, float* logits) {
+// write logits rows logit_dst[i] (all rows in order if both are null).  With `segs` the rows are a prompt chunk's,
+// m_rows of them in all (batch = 1).
+int forward(spec_ctx* ctx, const Model& m, const RowMeta& rows, int batch, int m_rows, int n_logit_rows, const int32_t* logit_src,
+            const int32_t* logit_dst, float* logits, const PromptSegments* segs = nullptr) {
     const spec_model_cfg& c = m.cfg;
     const int n_rows = batch * m_rows;
-    const RowMeta rows{ctx->row_token, ctx->row_pos, ctx->row_seq};
     if (c.arch == SPEC_ARCH_BIGRAM)  // logits = table[last token]: one gather
         return n_logit_rows > 0 ? launch_table_logits(m.tok_emb, m.bf16(), c.vocab, rows.token, logit_src, logit_dst, n_logit_rows,
                                                        logits, ctx->stream)
@@ -238,7 +245,7 @@ int forward(spec_ctx* ctx, const Model& m, int batch, int m_rows, int n_logit_ro
                                                       n_logit_rows, c.ngram, c.vocab, logits, ctx->stream)
                                 : SPEC_OK;
     const int which = &m == &ctx->model[1] ? 1 : 0;
-    if (ctx->rt.pass_kernel && pass_kernel_serves(ctx->pass, m, which, n_rows, n_logit_rows)) {
+    if (!segs && ctx->rt.pass_kernel && pass_kernel_serves(ctx->pass, m, which, n_rows, n_logit_rows)) {
         // a few rows: the whole pass is one persistent kernel
         const PassTables tables{ctx->page_table, ctx->pages_per_seq, ctx->rt.page_size, ctx->src_page_table,
                                 ctx->src_pages_per_seq, ctx->src_len, ctx->rt.max_len, ctx->rt.max_len - 1};
@@ -254,7 +261,7 @@ int forward(spec_ctx* ctx, const Model& m, int batch, int m_rows, int n_logit_ro
         const spec_layer_weights& w = m.layers[l];
         const spec_layer_weights& pw = pass.tc ? m.packed[l] : w;
         SPEC_TRY(pass.self_attention(w, pw, rows, batch, m_rows, layer_pool(ctx, m, l), nullptr, bias, ctx->rt.max_len,
-                                     ctx->rt.max_len - 1, ctx->rt.max_len));
+                                     ctx->rt.max_len - 1, ctx->rt.max_len, segs));
         if (m.t5()) {  // cross-attention over the source's K,V (every row sees every source position)
             SPEC_TRY(pass.norm(w.lnx, nullptr, n_rows));
             SPEC_TRY(pass.proj(w.wq_x, pw.wq_x, m.q_dim(), d, ctx->a, ctx->qkv));
@@ -439,7 +446,7 @@ int enqueue_iteration(spec_ctx* ctx, int batch, int gamma, float temperature) {
                                 ctx->logit_src, ctx->logit_dst));
             rows = batch;
         }
-        SPEC_TRY(forward(ctx, ctx->model[1], batch, rows / batch, batch, ctx->logit_src, ctx->logit_dst, ctx->draft_logits));
+        SPEC_TRY(forward(ctx, ctx->model[1], row_meta(ctx), batch, rows / batch, batch, ctx->logit_src, ctx->logit_dst, ctx->draft_logits));
         // x_step ~ q_step for every sequence
         SPEC_TRY(launch_sample_strided(ctx->draft_logits + static_cast<size_t>(step - 1) * vocab,
                                        static_cast<size_t>(gamma) * vocab, ctx->draft_u + (step - 1), gamma, batch,
@@ -448,7 +455,7 @@ int enqueue_iteration(spec_ctx* ctx, int batch, int gamma, float temperature) {
     }
     SPEC_TRY(launch_pdl(prep_verify_kernel, dim3(blocks_bg), dim3(threads), 0, st, ctx->tokens, ctx->draft_tokens,
                         ctx->length, batch, gamma, ctx->rt.max_len, ctx->row_token, ctx->row_pos, ctx->row_seq));
-    SPEC_TRY(forward(ctx, ctx->model[0], batch, gamma + 1, batch * (gamma + 1), nullptr, nullptr, ctx->target_logits));
+    SPEC_TRY(forward(ctx, ctx->model[0], row_meta(ctx), batch, gamma + 1, batch * (gamma + 1), nullptr, nullptr, ctx->target_logits));
     SPEC_TRY(launch_verify_sample(ctx->target_logits, ctx->draft_logits, ctx->draft_tokens, ctx->accept_u, ctx->final_u,
                                   batch, gamma, vocab, temperature, ctx->lenience, ctx->top_k, ctx->top_p, ctx->n_accepted,
                                   ctx->next_token, ctx->sampler_ws, st, ctx->nonfinite));
@@ -498,29 +505,76 @@ int build_graph(spec_ctx* ctx, int batch, int gamma, float temperature) {
     return SPEC_OK;
 }
 
-// Feeds, for every sequence, positions [from[b], to[b]) of host tokens through
-// model `which` in chunks (no logits): the prompt pass.
-int feed_host_tokens(spec_ctx* ctx, int which, const int32_t* tokens, int stride, const std::vector<int>& from,
-                     const std::vector<int>& to, int batch) {
+// Feeds positions [0, to[b]) of every sequence's host tokens through model `which` in chunks (no logits): the prompt
+// pass.  The rows of all sequences follow one another without padding; chunks are equal, in whole GEMM row tiles.
+int feed_packed(spec_ctx* ctx, int which, const int32_t* tokens, int stride, const std::vector<int>& to, int batch, int total) {
+    constexpr int kTile = 256;
+    const int chunks = (total + ctx->max_rows - 1) / ctx->max_rows;
+    const int chunk = std::min(ctx->max_rows, ((total + chunks - 1) / chunks + kTile - 1) / kTile * kTile);
+    std::vector<int32_t> block;
+    int b = 0, p = 0;  // the next row's sequence and position
+    for (int done = 0; done < total;) {
+        const int n = std::min(chunk, total - done), n4 = (n + 3) / 4 * 4;
+        block.assign(static_cast<size_t>(3) * n4, 0);  // tokens, positions, sequences; then the segments
+        PromptSegments segs{reinterpret_cast<const int4*>(ctx->row_block + 3 * n4), 0, 0};
+        for (int r = 0; r < n; ++b, p = 0) {
+            const int take = std::min(n - r, to[b] - p);
+            if (take > 0) {
+                const int32_t seg[4] = {r, take, b, p};
+                block.insert(block.end(), seg, seg + 4);
+                ++segs.count;
+                segs.longest = std::max(segs.longest, take);
+                for (int i = 0; i < take; ++i) {
+                    block[r + i] = tokens[static_cast<size_t>(b) * stride + p + i];
+                    block[n4 + r + i] = p + i;
+                    block[2 * n4 + r + i] = b;
+                }
+                r += take;
+                if (p + take < to[b]) {  // (the chunk is full)
+                    p += take;
+                    break;
+                }
+            }
+        }
+        SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_block, block.data(), block.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
+        const RowMeta rows{ctx->row_block, ctx->row_block + n4, ctx->row_block + 2 * n4};
+        SPEC_TRY(forward(ctx, ctx->model[which], rows, 1, n, 0, nullptr, nullptr, nullptr, &segs));
+        SPEC_CUDA_TRY(cudaStreamSynchronize(ctx->stream));  // the host block is reused
+        done += n;
+    }
+    return SPEC_OK;
+}
+
+// The prompt pass of one model: packed where the prompt kernel takes it, otherwise the same number of rows per
+// sequence in every chunk, short prompts padded with inactive rows.
+int feed_host_tokens(spec_ctx* ctx, int which, const int32_t* tokens, int stride, const std::vector<int>& to, int batch) {
+    int longest = 0, total = 0;
+    long long query_keys = 0;
+    for (int b = 0; b < batch; ++b) {
+        longest = std::max(longest, to[b]);
+        total += to[b];
+        query_keys += static_cast<long long>(to[b]) * (to[b] + 1) / 2;
+    }
+    if (total == 0) return SPEC_OK;
+    if (prompt_attention_serves(ctx->model[which], query_keys)) return feed_packed(ctx, which, tokens, stride, to, batch, total);
     const int chunk = std::max(1, ctx->max_rows / batch);
-    int longest = 0;
-    for (int b = 0; b < batch; ++b) longest = std::max(longest, to[b] - from[b]);
     std::vector<int32_t> tok(static_cast<size_t>(batch) * chunk), pos(tok.size()), seq(tok.size());
     for (int c0 = 0; c0 < longest; c0 += chunk) {
+        const int rows = std::min(chunk, longest - c0);
         for (int b = 0; b < batch; ++b)
-            for (int j = 0; j < chunk; ++j) {
-                const int p = from[b] + c0 + j;
-                const size_t r = static_cast<size_t>(b) * chunk + j;
+            for (int j = 0; j < rows; ++j) {
+                const int p = c0 + j;
+                const size_t r = static_cast<size_t>(b) * rows + j;
                 const bool active = p < to[b];
                 tok[r] = active ? tokens[static_cast<size_t>(b) * stride + p] : 0;
                 pos[r] = active ? p : -1;
                 seq[r] = b;
             }
-        const size_t bytes = tok.size() * sizeof(int32_t);
+        const size_t bytes = static_cast<size_t>(batch) * rows * sizeof(int32_t);
         SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_token, tok.data(), bytes, cudaMemcpyHostToDevice, ctx->stream));
         SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_pos, pos.data(), bytes, cudaMemcpyHostToDevice, ctx->stream));
         SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_seq, seq.data(), bytes, cudaMemcpyHostToDevice, ctx->stream));
-        SPEC_TRY(forward(ctx, ctx->model[which], batch, chunk, 0, nullptr, nullptr, nullptr));
+        SPEC_TRY(forward(ctx, ctx->model[which], row_meta(ctx), batch, rows, 0, nullptr, nullptr, nullptr));
         SPEC_CUDA_TRY(cudaStreamSynchronize(ctx->stream));  // the host vectors are reused
     }
     return SPEC_OK;
@@ -708,8 +762,9 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     ctx->has_draft = draft_cfg != nullptr;
     ctx->pages_per_seq = (rt.max_len + rt.page_size - 1) / rt.page_size;
     ctx->max_logit_rows = std::max(rt.max_batch * std::max(rt.max_gamma + 1, 2), 64);
-    // The prompt pass takes up to 256 rows at a time (weights streamed once per chunk).
-    ctx->max_rows = std::max(ctx->max_logit_rows, std::min(256, rt.max_batch * rt.max_len));
+    // The prompt pass takes up to 2048 rows at a time: the GEMMs reach their full rate from about 1024 rows on (4096-wide
+    // block, one prompt of 1024 tokens, 256-row chunks 54 ms, one chunk 32 ms), narrow models like more.
+    ctx->max_rows = std::max(ctx->max_logit_rows, std::min(2048, rt.max_batch * rt.max_len));
     if (t5) {  // an encoder pass takes every source row of the batch at once
         ctx->src_pages_per_seq = (rt.max_src_len + rt.page_size - 1) / rt.page_size;
         ctx->max_rows = std::max(ctx->max_rows, rt.max_batch * rt.max_src_len);
@@ -741,11 +796,15 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
 #define SPEC_ALLOC(ptr, count) \
     if ((status = dev_alloc(ctx, &ctx->ptr, (count))) != SPEC_OK) return cleanup(status)
     SPEC_ALLOC(h, R * d);
-    SPEC_ALLOC(a, R * d);
     SPEC_ALLOC(qkv, R * std::max(qkv, 2 * att));
-    SPEC_ALLOC(att, R * att);
-    SPEC_ALLOC(u, R * fin);
-    SPEC_ALLOC(f, R * ff);
+    bool any_fp32 = false;  // (bf16 models hand over partial sums and bf16 terms instead)
+    for (int i = 0; i < (ctx->has_draft ? 2 : 1); ++i) any_fp32 |= !ctx->model[i].bf16();
+    if (any_fp32) {
+        SPEC_ALLOC(a, R * d);
+        SPEC_ALLOC(att, R * att);
+        SPEC_ALLOC(u, R * fin);
+        SPEC_ALLOC(f, R * ff);
+    }
     {
         size_t attn = 0;
         for (int i = 0; i < (ctx->has_draft ? 2 : 1); ++i) {
@@ -776,8 +835,7 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
             for (int s = 0; s < 7; ++s) {
                 if (!m.t5() && (s == 4 || s == 5)) continue;  // cross-attention projections
                 const int most = s == 6 ? ctx->max_logit_rows : ctx->max_rows;  // the head only sees decode rows
-                for (int rows = 1; rows <= most; ++rows)
-                    partial = std::max(partial, gemm_tc_partial_elems(shapes[s][0], shapes[s][1], rows));
+                partial = std::max(partial, gemm_tc_most_partial_elems(shapes[s][0], shapes[s][1], most));
             }
         }
         if (any_bf16) {
@@ -795,11 +853,12 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
                 return cleanup(status);
         }
     }
-    SPEC_ALLOC(row_token, R);
-    SPEC_ALLOC(row_pos, R);
-    SPEC_ALLOC(row_seq, R);
-    SPEC_ALLOC(logit_src, R);
-    SPEC_ALLOC(logit_dst, R);
+    SPEC_ALLOC(row_block, 5 * R + 16 + 4 * B);  // (a prompt chunk's three padded row arrays and up to B + 1 segments fit)
+    ctx->row_token = ctx->row_block;
+    ctx->row_pos = ctx->row_block + R;
+    ctx->row_seq = ctx->row_block + 2 * R;
+    ctx->logit_src = ctx->row_block + 3 * R;
+    ctx->logit_dst = ctx->row_block + 4 * R;
     SPEC_ALLOC(page_table, B * ctx->pages_per_seq);
     if (t5) {
         SPEC_ALLOC(src_page_table, B * ctx->src_pages_per_seq);
@@ -948,10 +1007,10 @@ int begin_session(spec_ctx* ctx, const int32_t* prompt, const int32_t* prompt_le
     // prompt pass: positions 0..prompt_len-2 (the last prompt token is fed by the first iteration)
     SPEC_CUDA_TRY(cudaEventRecord(ctx->ev[0], st));
     if (t5) SPEC_TRY(encode_sources(ctx, source, source_len, source_stride, batch, gamma > 0 ? 2 : 1));
-    std::vector<int> from(batch, 0), to(batch);
+    std::vector<int> to(batch);
     for (int b = 0; b < batch; ++b) to[b] = prompt_len[b] - 1;
-    SPEC_TRY(feed_host_tokens(ctx, 0, prompt, prompt_stride, from, to, batch));
-    if (gamma > 0) SPEC_TRY(feed_host_tokens(ctx, 1, prompt, prompt_stride, from, to, batch));
+    SPEC_TRY(feed_host_tokens(ctx, 0, prompt, prompt_stride, to, batch));
+    if (gamma > 0) SPEC_TRY(feed_host_tokens(ctx, 1, prompt, prompt_stride, to, batch));
     SPEC_CUDA_TRY(cudaEventRecord(ctx->ev[1], st));
     SPEC_TRY(build_graph(ctx, batch, gamma, temperature));
     SPEC_CUDA_TRY(cudaStreamSynchronize(st));  // host_tokens goes out of scope
@@ -1256,10 +1315,10 @@ extern "C" int spec_pass_trace(spec_ctx* ctx, int which, int batch, int rows, un
     if (err == cudaSuccess) err = cudaMemcpyAsync(ctx->row_seq, seq.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st);
     int status = SPEC_OK;
     if (err == cudaSuccess) {
-        status = forward(ctx, m, batch, rows, n, nullptr, nullptr, ctx->target_logits);  // untimed: warms the caches
+        status = forward(ctx, m, row_meta(ctx), batch, rows, n, nullptr, nullptr, ctx->target_logits);  // untimed: warms the caches
         ctx->pass_trace = dev;
         ctx->pass_trace_capacity = capacity;
-        if (status == SPEC_OK) status = forward(ctx, m, batch, rows, n, nullptr, nullptr, ctx->target_logits);
+        if (status == SPEC_OK) status = forward(ctx, m, row_meta(ctx), batch, rows, n, nullptr, nullptr, ctx->target_logits);
         ctx->pass_trace = nullptr;
         ctx->pass_trace_capacity = 0;
     }
@@ -1302,7 +1361,7 @@ extern "C" int spec_time_forward(spec_ctx* ctx, int which, int batch, int rows, 
     SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_seq, seq.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     SPEC_CUDA_TRY(cudaStreamSynchronize(st));
     SPEC_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    const int status = forward(ctx, m, batch, rows, n, nullptr, nullptr, ctx->target_logits);
+    const int status = forward(ctx, m, row_meta(ctx), batch, rows, n, nullptr, nullptr, ctx->target_logits);
     cudaGraph_t g = nullptr;
     const cudaError_t end = cudaStreamEndCapture(st, &g);
     if (status != SPEC_OK) {
@@ -1357,7 +1416,7 @@ extern "C" int spec_forward_logits(spec_ctx* ctx, int which, const int32_t* toke
     SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_token, tok.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_pos, pos.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_seq, seq.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    SPEC_TRY(forward(ctx, m, batch, rows, n, nullptr, nullptr, logits));
+    SPEC_TRY(forward(ctx, m, row_meta(ctx), batch, rows, n, nullptr, nullptr, logits));
     SPEC_CUDA_TRY(cudaStreamSynchronize(st));
     if (const int gave_up = device_gave_up(ctx)) return fail(SPEC_ERR_DEVICE_TIMEOUT, "a kernel gave up on a bounded wait (code %d)", gave_up);
     for (int b = 0; b < batch; ++b) ctx->cached[which][b] += rows;

@@ -464,6 +464,15 @@ size_t gemm_tc_partial_elems(int n_out, int k, int n_rows) {
     return static_cast<size_t>(gemm_tc_plan(n_out, k, n_rows).slots) * n_rows * n_out;
 }
 
+// The most partial sums of any pass of up to `most_rows` rows: up to 128 rows and, above, within 256 rows (the same
+// number of row tiles) the number of sums per element does not depend on the rows.
+size_t gemm_tc_most_partial_elems(int n_out, int k, int most_rows) {
+    size_t most = gemm_tc_partial_elems(n_out, k, std::min(most_rows, 128));
+    for (int rows = 256; rows < most_rows + 256; rows += 256)
+        most = std::max(most, gemm_tc_partial_elems(n_out, k, std::min(rows, most_rows)));
+    return most;
+}
+
 size_t packed_weight_elems(int n_out, int k) {
     return static_cast<size_t>((n_out + kTileM - 1) / kTileM) * ((k + kTileK - 1) / kTileK) * kTileM * kTileK;
 }

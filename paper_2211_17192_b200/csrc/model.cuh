@@ -108,6 +108,7 @@ int launch_gemm_rows(const float* x, const void* w, bool w_bf16, const float* re
 // for the next kernel to add up, launch_gemm_tc adds them up itself.
 PartialPlan gemm_tc_plan(int n_out, int k, int n_rows);
 size_t gemm_tc_partial_elems(int n_out, int k, int n_rows);
+size_t gemm_tc_most_partial_elems(int n_out, int k, int most_rows);
 int launch_split_bf16(const float* x, size_t n, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t stream);
 // `packed`: w is the tile-major copy made by launch_pack_weight (every [128 x 64]
 // tile contiguous, so a CTA's weight stream is one sequential run of HBM).
@@ -174,6 +175,17 @@ size_t attention_partial_elems(int rows, int n_heads, int d_head, int slices);
 // (slices from attention_slices with the same batch, m_rows and max_keys, the capacity of the key set)
 int launch_attention(const Model& m, const AttnSource& src, const RowMeta& rows, int batch, int m_rows, int slices,
                      int max_keys, float* part, float* att, __nv_bfloat16* att_hi, __nv_bfloat16* att_lo, cudaStream_t stream);
+
+// A prompt chunk: the rows of `count` segments one after another, table[i] (device) = (first row, rows, sequence,
+// position of the first row), `longest` the most rows of any.
+struct PromptSegments {
+    const int4* table;
+    int count, longest;
+};
+// Whether the prompt kernel takes a chunk with this many (row, key it sees) pairs.
+bool prompt_attention_serves(const Model& m, long long query_keys);
+int launch_prompt_attention(const Model& m, const AttnSource& src, const PromptSegments& segs, __nv_bfloat16* att_hi,
+                            __nv_bfloat16* att_lo, cudaStream_t stream);
 
 // f = gelu(u)  |  gelu(u[:, :F]) * u[:, F:]  |  silu(u[:, :F]) * u[:, F:], u given in full or as partial sums.
 int launch_ffn_act(const float* u, const float* partial, const PartialPlan& plan, int n_rows, int d_ff, int ffn, float* f,

@@ -54,25 +54,34 @@ __device__ __forceinline__ float fast_exp2(float x) {
 
 // A row of fp32 logits addressed in groups of four elements.  VEC: the vocabulary
 // is a multiple of four and every row starts on a 16-byte boundary, so a group
-// is one unconditional 128-bit load.  Otherwise four guarded scalar loads, with
-// elements past the end of the row reading as `pad`.  Logits below `floor` read
+// is one unconditional 128-bit load.  Logits below `floor` read
 // as -inf: that is top-k standardisation (Section 2.2) with `floor` the row's
 // k-th largest logit, and no change with floor = -inf.
+//
+// Without VEC a row may begin anywhere (a vocabulary that is not a multiple of four): `shift`, 0 to 3, is how many
+// elements before the row its first aligned group starts, group g holds elements 4g - shift .., and elements outside
+// the row read as `pad` (24 x 9 rows of 50003: statistics 30.4 us with four guarded loads per group, 10.9 so).  A caller
+// that pairs two rows element by element passes aligned = false and gets unshifted groups of guarded loads.
+__host__ __device__ __forceinline__ int row_shift(const float* row) { return static_cast<int>((reinterpret_cast<uintptr_t>(row) >> 2) & 3u); }
+
 template <bool VEC, bool CUT = false>
 struct Row {
     const float* base;
     int vocab;
     float floor;  // used only with CUT, so that the usual path pays nothing for it
+    int shift;
 
+    __device__ __forceinline__ int groups() const { return (vocab + shift + 3) >> 2; }
     __device__ __forceinline__ float kept(float v) const { return (!CUT || v >= floor) ? v : -INFINITY; }
     __device__ __forceinline__ float4 raw(int g, float pad) const {
         if (VEC) return __ldg(reinterpret_cast<const float4*>(base) + g);
-        const int j = 4 * g;
+        const int j = 4 * g - shift;
+        if (shift == row_shift(base) && j >= 0 && j + 4 <= vocab) return __ldg(reinterpret_cast<const float4*>(base + j));
         float4 v;
-        v.x = j + 0 < vocab ? __ldg(base + j + 0) : pad;
-        v.y = j + 1 < vocab ? __ldg(base + j + 1) : pad;
-        v.z = j + 2 < vocab ? __ldg(base + j + 2) : pad;
-        v.w = j + 3 < vocab ? __ldg(base + j + 3) : pad;
+        v.x = j + 0 >= 0 && j + 0 < vocab ? __ldg(base + j + 0) : pad;
+        v.y = j + 1 >= 0 && j + 1 < vocab ? __ldg(base + j + 1) : pad;
+        v.z = j + 2 >= 0 && j + 2 < vocab ? __ldg(base + j + 2) : pad;
+        v.w = j + 3 >= 0 && j + 3 < vocab ? __ldg(base + j + 3) : pad;
         return v;
     }
     __device__ __forceinline__ float4 load(int g, float pad) const {
@@ -83,8 +92,9 @@ struct Row {
 };
 
 template <bool VEC, bool CUT = false>
-__device__ __forceinline__ Row<VEC, CUT> make_row(const float* base, int vocab, float floor = -INFINITY) {
+__device__ __forceinline__ Row<VEC, CUT> make_row(const float* base, int vocab, float floor = -INFINITY, bool aligned = true) {
     Row<VEC, CUT> r;
+    r.shift = VEC || !aligned ? 0 : row_shift(base);
     r.base = base;
     r.vocab = vocab;
     r.floor = floor;
@@ -105,6 +115,8 @@ struct PlainWeights {
     __device__ __forceinline__ Raw nothing() const {
         return Raw{make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY)};
     }
+    __device__ __forceinline__ int groups() const { return p.groups(); }
+    __device__ __forceinline__ int shift() const { return p.shift; }
     __device__ __forceinline__ float one(float lp) const { return fast_exp2((lp - max_p) * c2); }
     __device__ __forceinline__ float4 weigh(const Raw& r) const {
         return make_float4(one(r.a.x), one(r.a.y), one(r.a.z), one(r.a.w));
@@ -124,6 +136,8 @@ struct ResidualWeights {
         const float4 z = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         return Raw{z, z};
     }
+    __device__ __forceinline__ int groups() const { return p.groups(); }
+    __device__ __forceinline__ int shift() const { return 0; }
     __device__ __forceinline__ float one(float lp, float lq) const {
         // (both products are rounded before the subtraction: contracted into a multiply-add, one of them would not
         // be, and p = q would leave rounding residue instead of the exact zero that the fallback to p tests for)
@@ -292,7 +306,7 @@ __device__ int locate_in_range(const Weights& w, int r0, int r1, float rem, bool
 template <int WARPS, class Weights>
 __device__ int block_inverse_cdf(const Weights& w, int vocab, float u, CdfScratch<WARPS>& s, float* total_out) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int groups = (vocab + 3) >> 2;
+    const int groups = w.groups();
     const int seg = (groups + WARPS - 1) / WARPS;
     const int g0 = min(groups, warp * seg), g1 = min(groups, g0 + seg);
     const float acc = warp_range_sum<kCdfBatch>(w, g0, g1, lane);
@@ -310,7 +324,7 @@ __device__ int block_inverse_cdf(const Weights& w, int vocab, float u, CdfScratc
     const int r0 = min(groups, hit * seg), r1 = min(groups, r0 + seg);
     const int k = locate_in_range<WARPS>(w, r0, r1, target - before, want_hit, s);
     *total_out = total;
-    return max(0, min(k, vocab - 1));
+    return max(0, min(k - w.shift(), vocab - 1));
 }
 
 // The same draw by a thread-block cluster: CTA `rank` of `nctas` owns a
@@ -324,7 +338,7 @@ __device__ int cluster_inverse_cdf(const Weights& w, int vocab, float u, CdfScra
     const int nctas = static_cast<int>(cluster.num_blocks());
     const int rank = static_cast<int>(cluster.block_rank());
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int groups = (vocab + 3) >> 2;
+    const int groups = w.groups();
     const int slice = (groups + nctas - 1) / nctas;
     const int seg = (slice + WARPS - 1) / WARPS;
     auto seg_begin = [&](int part) {  // part = cta * WARPS + warp
@@ -423,7 +437,7 @@ __device__ int cluster_inverse_cdf(const Weights& w, int vocab, float u, CdfScra
         } else {
             k = locate_in_range<WARPS>(w, seg_begin(hit), seg_end(hit), target - before, want_hit, s);
         }
-        k = max(0, min(k, vocab - 1));
+        k = max(0, min(k - w.shift(), vocab - 1));
     }
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // nobody reads this CTA's totals any more
     return k;
@@ -478,7 +492,7 @@ verify_stats_kernel(const float* __restrict__ target_logits, const float* __rest
         : draft_logits + (static_cast<size_t>(b) * gamma + (row - gamma - 1)) * vocab;
     const float floor = CUT ? __ldcg(floors + static_cast<size_t>(b) * rows + row) : -INFINITY;
     const Row<VEC, CUT> r = make_row<VEC, CUT>(src, vocab, floor);
-    const int groups = (vocab + 3) >> 2;
+    const int groups = r.groups();
     const int per_chunk = (groups + chunks - 1) / chunks;
     const int g0 = chunk * per_chunk;
     const int g1 = min(groups, g0 + per_chunk);
@@ -489,7 +503,7 @@ verify_stats_kernel(const float* __restrict__ target_logits, const float* __rest
     float xlogit = 0.0f;
     if (tid == 0 && !GREEDY && row != gamma) {
         const int x = draft_tokens[static_cast<size_t>(b) * gamma + (row < gamma ? row : row - gamma - 1)];
-        if (x >= 4 * g0 && x < min(vocab, 4 * g1)) xlogit = r.kept(__ldg(src + x));
+        if (x >= 0 && x < vocab && x + r.shift >= 4 * g0 && x + r.shift < 4 * g1) xlogit = r.kept(__ldg(src + x));
     }
 
     // Every thread streams groups g0+tid, g0+tid+T, ... with kUnroll 128-bit
@@ -510,7 +524,7 @@ verify_stats_kernel(const float* __restrict__ target_logits, const float* __rest
         if (GREEDY) {
 #pragma unroll
             for (int i = 0; i < kUnroll; ++i) {
-                const int j = 4 * (base + i * kStatThreads);  // indices grow with i: '>' keeps the lowest on ties
+                const int j = 4 * (base + i * kStatThreads) - r.shift;  // indices grow with i: '>' keeps the lowest on ties
                 if (v[i].x > m) { m = v[i].x; arg = j; }
                 if (v[i].y > m) { m = v[i].y; arg = j + 1; }
                 if (v[i].z > m) { m = v[i].z; arg = j + 2; }
@@ -584,8 +598,6 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
     const float c2 = inv_t * kLog2e;
     const float* tl = target_logits + static_cast<size_t>(b) * (gamma + 1) * vocab;
     const float* ql = GREEDY ? nullptr : draft_logits + static_cast<size_t>(b) * gamma * vocab;
-    const int groups = (vocab + 3) >> 2;
-    const int per_chunk = (groups + chunks - 1) / chunks;
 
     // Inputs that the statistics kernel does not produce can be fetched before
     // waiting for it.
@@ -609,7 +621,10 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
         float M = -FLT_MAX, A = 0.0f, X = 0.0f;
         int best = 0x7fffffff;
         bool bad = false;
-        const int xchunk = (my_x >= 0 && my_x < vocab) ? (my_x >> 2) / per_chunk : -1;
+        // (the chunks of this row, as the statistics kernel cut it)
+        const int shift = VEC || GREEDY ? 0 : row_shift(tid <= gamma ? tl + static_cast<size_t>(tid) * vocab : ql + static_cast<size_t>(tid - gamma - 1) * vocab);
+        const int per_chunk = (((vocab + shift + 3) >> 2) + chunks - 1) / chunks;
+        const int xchunk = (my_x >= 0 && my_x < vocab) ? ((my_x + shift) >> 2) / per_chunk : -1;
         constexpr int kMergeBatch = 8;  // chunk statistics fetched together
         for (int c0 = 0; c0 < chunks; c0 += kMergeBatch) {
             float4 st[kMergeBatch];
@@ -679,8 +694,8 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
         bool plain = n == gamma;
         if (!plain) {
             ResidualWeights<VEC, CUT> rw;
-            rw.p = pw.p;
-            rw.q = make_row<VEC, CUT>(ql + static_cast<size_t>(n) * vocab, vocab, CUT ? __ldcg(fl + gamma + 1 + n) : -INFINITY);
+            rw.p = make_row<VEC, CUT>(pw.p.base, vocab, pw.p.floor, false);
+            rw.q = make_row<VEC, CUT>(ql + static_cast<size_t>(n) * vocab, vocab, CUT ? __ldcg(fl + gamma + 1 + n) : -INFINITY, false);
             rw.max_p = sh.row_max[n];
             rw.max_q = sh.row_max[gamma + 1 + n];
             rw.inv_sum_p = 1.0f / sh.row_aux[n];
@@ -714,14 +729,14 @@ sample_kernel(const float* __restrict__ logits, size_t logit_stride, const float
     const int tid = threadIdx.x;
     const Row<VEC, CUT> r = make_row<VEC, CUT>(logits + static_cast<size_t>(blockIdx.x) * logit_stride, vocab,
                                                CUT ? __ldcg(floors + blockIdx.x) : -INFINITY);
-    const int groups = (vocab + 3) >> 2;
+    const int groups = r.groups();
     float m = -FLT_MAX;
     int arg = 0x7fffffff;
     bool bad = false;  // a NaN or +inf logit
 #pragma unroll 4
     for (int g = tid; g < groups; g += kSampleThreads) {
         const float4 v = r.load(g, -INFINITY);
-        const int j = 4 * g;
+        const int j = 4 * g - r.shift;
         if (v.x > m) { m = v.x; arg = j; }
         if (v.y > m) { m = v.y; arg = j + 1; }
         if (v.z > m) { m = v.z; arg = j + 2; }
@@ -765,14 +780,13 @@ sample_kernel(const float* __restrict__ logits, size_t logit_stride, const float
 // float-to-int conversion for the bin, one 32-bit atomic plus a rare carry for
 // the mass (a 64-bit shared-memory atomic cost 48 us of 180 on 960 rows of 32000),
 // a two-instruction test before a logit is asked whether it is in the chosen bin.
-constexpr int kSelThreads = 256;
-constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelBins = 2048;
-constexpr int kSelPerThread = kSelBins / kSelThreads;
 constexpr int kSelCap = 1024;   // logits ranked against each other at the end
 constexpr int kSelLevels = 40;  // every level shrinks the range; fp32 allows far fewer than this
 
+template <int kSelThreads>
 struct SelShared {
+    static constexpr int kSelWarps = kSelThreads / 32;
     unsigned cnt[kSelBins];
     unsigned mass_lo[kSelBins], mass_hi[kSelBins];  // a bin's mass, low and high word (apart: the low words then spread over all banks)
     float cand[kSelCap];
@@ -790,7 +804,7 @@ struct SelShared {
 // f(v) for every logit of the row, kSelLoads 128-bit loads in flight per thread.
 constexpr int kSelLoads = 8;
 
-template <bool VEC, class F>
+template <int kSelThreads, bool VEC, class F>
 __device__ __forceinline__ void for_each_logit(const Row<VEC>& r, int groups, F f) {
     for (int g0 = threadIdx.x; g0 < groups; g0 += kSelLoads * kSelThreads) {
         float4 v[kSelLoads];
@@ -818,13 +832,14 @@ __device__ __forceinline__ float warp_min(float v) {
 // The floor among the finite logits >= kf: MASS = false, the k-th largest of
 // them; MASS = true, the nucleus of mass top_p with weights exp2((l - max) * c2).
 // Every thread returns the same value; -inf means "keep everything".
-template <bool VEC, bool MASS>
-__device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned k, float top_p, float c2, SelShared& sh) {
+template <int kSelThreads, bool VEC, bool MASS>
+__device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned k, float top_p, float c2, SelShared<kSelThreads>& sh) {
+    constexpr int kSelWarps = kSelThreads / 32, kSelPerThread = kSelBins / kSelThreads;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // 1. range and number of the logits in play
     float lo = INFINITY, hi = -INFINITY;
     unsigned n = 0;
-    for_each_logit(r, groups, [&](float v) {
+    for_each_logit<kSelThreads>(r, groups, [&](float v) {
         const bool in_play = fabsf(v) < INFINITY && v >= kf;
         const float u = in_play ? v : __int_as_float(0x7fc00000);  // (fminf and fmaxf pass over a NaN operand)
         lo = fminf(lo, u);
@@ -865,7 +880,7 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
         }
         if (tid == 0) { sh.n_cand = 0; sh.bin = kSelBins - 1; sh.before_cnt = before_cnt; sh.before_mass = before_mass; }
         __syncthreads();
-        for_each_logit(r, groups, [&](float v) {
+        for_each_logit<kSelThreads>(r, groups, [&](float v) {
             const int b = bin_of(v);
             if (b >= 0) {
                 if (MASS) {
@@ -935,7 +950,7 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
         auto in_the_bin = [&](float v) { return fabsf(v - centre) <= reach && bin_of(v) == bin; };
         if (few) {
             // 3. copy the bin's logits out and rank them against each other
-            for_each_logit(r, groups, [&](float v) {
+            for_each_logit<kSelThreads>(r, groups, [&](float v) {
                 if (in_the_bin(v)) {
                     const unsigned at = atomicAdd(&sh.n_cand, 1u);
                     if (at < kSelCap) { sh.cand[at] = v; if (MASS) sh.cand_mass[at] = fixed_mass(v); }
@@ -965,7 +980,7 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
         }
         // the bin is crowded: its own range is searched next
         float new_lo = INFINITY, new_hi = -INFINITY;
-        for_each_logit(r, groups, [&](float v) {
+        for_each_logit<kSelThreads>(r, groups, [&](float v) {
             const bool here = in_the_bin(v);
             new_lo = fminf(new_lo, here ? v : INFINITY);
             new_hi = fmaxf(new_hi, here ? v : -INFINITY);
@@ -982,20 +997,25 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
     return lo;
 }
 
-// Top-k for k up to half the number of threads, without bins: the k-th largest of the threads' own maxima is a
-// value that at least k logits reach, so the k-th largest logit of the row is among those that reach it - a few
-// more than k as a rule.  One pass for the maxima, one that copies out what reaches the pivot, then the exact
-// ranking of step 3 above.  Returns false, having decided nothing, when fewer than k threads hold a finite logit
+// Top-k for k up to 128, without bins: every warp gives its largest lane maxima, 3 k of them in all; the k-th largest of
+// these is a value that at least k logits reach, so the k-th largest logit of the row is among those that reach it - a
+// few more than k as a rule.  One pass for the maxima, one that copies out what reaches the pivot, then the exact
+// ranking of step 3 above.  Returns false, having decided nothing, when fewer than k lanes hold a finite logit
 // or more than kSelCap logits reach the pivot (heavy ties): the binned selection then does the row.
-template <bool VEC>
-__device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelShared& sh, float* floor) {
+constexpr int kMostTops = 512;
+
+template <int kSelThreads, bool VEC>
+__device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelShared<kSelThreads>& sh, float* floor) {
+    constexpr int kSelWarps = kSelThreads / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // (measured on 960 rows of 32000: k = 40 66 us per call against 82 binned, k = 128 71, k = 200 92: the pivot sinks
     // with k and lets ever more logits through)
-    if (k > static_cast<unsigned>(kSelThreads) / 2) return false;
+    if (k > 128) return false;
+    const int per_warp = min(min(32, kMostTops / kSelWarps), (3 * static_cast<int>(k) + kSelWarps - 1) / kSelWarps);
+    const int n_tops = per_warp * kSelWarps;
     float mine = -INFINITY;
     unsigned n = 0;
-    for_each_logit(r, groups, [&](float v) {
+    for_each_logit<kSelThreads>(r, groups, [&](float v) {
         const bool finite = fabsf(v) < INFINITY;
         mine = fmaxf(mine, finite ? v : -INFINITY);
         n += finite;
@@ -1003,7 +1023,19 @@ __device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelSha
     n = __reduce_add_sync(0xffffffffu, n);
     __syncthreads();  // (the shared arrays may still be read by a previous call)
     if (lane == 0) sh.warp_cnt[warp] = n;
-    sh.cand[tid] = mine;
+    {
+        // (keys: the floats' order as unsigned integers, for the warp-wide integer maximum; 0 marks a lane that is out)
+        const unsigned u = __float_as_uint(mine);
+        unsigned key = u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u), top = 0;
+        float given = -INFINITY;
+        for (int i = 0; i < per_warp; ++i) {
+            top = __reduce_max_sync(0xffffffffu, key);
+            const unsigned who = __ballot_sync(0xffffffffu, key == top);
+            if (lane == __ffs(who) - 1) key = 0;
+            if (lane == i && top != 0) given = __uint_as_float(top ^ ((top >> 31) ? 0x80000000u : 0xffffffffu));
+        }
+        if (lane < per_warp) sh.cand[warp * per_warp + lane] = given;
+    }
     if (tid == 0) sh.n_cand = 0;
     __syncthreads();
     n = 0;
@@ -1013,17 +1045,27 @@ __device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelSha
         *floor = -INFINITY;
         return true;
     }
-    // the k-th largest of the maxima: the largest one that at least k of them reach
-    unsigned reach = 0;
-    for (int j = 0; j < kSelThreads; ++j) reach += sh.cand[j] >= mine;
-    float pivot = warp_max(reach >= k ? mine : -INFINITY);
+    // the k-th largest of the maxima: the largest one that at least k of them reach; `per` threads count for each
+    int per = 1;
+    while (per * 2 * n_tops <= kSelThreads && per < 32) per *= 2;
+    float pivot = -INFINITY;
+    for (int base = 0; base < n_tops; base += kSelThreads / per) {
+        const int i = base + tid / per;
+        const float top = i < n_tops ? sh.cand[i] : INFINITY;
+        unsigned reach = 0;
+#pragma unroll 8
+        for (int j = tid % per; j < n_tops; j += per) reach += sh.cand[j] >= top;
+        for (int o = per / 2; o > 0; o >>= 1) reach += __shfl_xor_sync(0xffffffffu, reach, o);
+        if (i < n_tops && reach >= k) pivot = fmaxf(pivot, top);
+    }
+    pivot = warp_max(pivot);
     if (lane == 0) sh.warp_hi[warp] = pivot;
     __syncthreads();  // (every thread has read the maxima: the list can be reused)
     pivot = -INFINITY;
 #pragma unroll
     for (int w = 0; w < kSelWarps; ++w) pivot = fmaxf(pivot, sh.warp_hi[w]);
     if (!(pivot > -INFINITY)) return false;
-    for_each_logit(r, groups, [&](float v) {
+    for_each_logit<kSelThreads>(r, groups, [&](float v) {
         if (v >= pivot && v < INFINITY) {
             const unsigned at = atomicAdd(&sh.n_cand, 1u);
             if (at < kSelCap) sh.cand[at] = v;
@@ -1055,13 +1097,14 @@ __device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelSha
 // one pass copies them out, then they are ranked against each other as in step 3
 // above.  Returns false, having decided nothing, if more than kSelCap logits are
 // in play (a large tie at the top-k floor).
-template <bool VEC>
-__device__ bool nucleus_of_few(const Row<VEC>& r, int groups, float kf, float top_p, float c2, SelShared& sh, float* floor) {
+template <int kSelThreads, bool VEC>
+__device__ bool nucleus_of_few(const Row<VEC>& r, int groups, float kf, float top_p, float c2, SelShared<kSelThreads>& sh, float* floor) {
+    constexpr int kSelWarps = kSelThreads / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __syncthreads();  // (the shared arrays may still be read by a previous call)
     if (tid == 0) sh.n_cand = 0;
     __syncthreads();
-    for_each_logit(r, groups, [&](float v) {
+    for_each_logit<kSelThreads>(r, groups, [&](float v) {
         if (fabsf(v) < INFINITY && v >= kf) {
             const unsigned at = atomicAdd(&sh.n_cand, 1u);
             if (at < kSelCap) sh.cand[at] = v;
@@ -1115,11 +1158,11 @@ __device__ bool nucleus_of_few(const Row<VEC>& r, int groups, float kf, float to
 // floors[s * (a_rows + b_rows) + r] for sequence s's a_rows rows of `a`, then its
 // b_rows rows of `b`: top-k first (0 < top_k < vocab), then the nucleus (0 < top_p < 1)
 // of what top-k left.
-template <bool VEC>
+template <bool VEC, int kSelThreads>
 __global__ void __launch_bounds__(kSelThreads)
 cut_floor_kernel(const float* __restrict__ a, size_t a_stride, int a_rows, const float* __restrict__ b,
                  size_t b_stride, int b_rows, int vocab, int top_k, float top_p, float c2, float* __restrict__ floors) {
-    __shared__ SelShared sh;
+    __shared__ SelShared<kSelThreads> sh;
     pdl_trigger();
     pdl_wait();
     const int per_seq = a_rows + b_rows;
@@ -1127,15 +1170,15 @@ cut_floor_kernel(const float* __restrict__ a, size_t a_stride, int a_rows, const
     const float* src = row < a_rows ? a + (static_cast<size_t>(seq) * a_rows + row) * a_stride
                                     : b + (static_cast<size_t>(seq) * b_rows + (row - a_rows)) * b_stride;
     const Row<VEC> r = make_row<VEC>(src, vocab);
-    const int groups = (vocab + 3) >> 2;
+    const int groups = r.groups();
     float floor = -INFINITY;
-    if (top_k > 0 && top_k < vocab && !top_k_by_pivot<VEC>(r, groups, static_cast<unsigned>(top_k), sh, &floor))
-        floor = select_floor<VEC, false>(r, groups, -INFINITY, static_cast<unsigned>(top_k), 0.0f, 0.0f, sh);
+    if (top_k > 0 && top_k < vocab && !top_k_by_pivot<kSelThreads, VEC>(r, groups, static_cast<unsigned>(top_k), sh, &floor))
+        floor = select_floor<kSelThreads, VEC, false>(r, groups, -INFINITY, static_cast<unsigned>(top_k), 0.0f, 0.0f, sh);
     if (top_p > 0.0f && top_p < 1.0f) {
         // after a top-k that leaves few logits the nucleus needs no binning
         const bool few = floor > -INFINITY && top_k <= kSelCap;
-        if (!few || !nucleus_of_few<VEC>(r, groups, floor, top_p, c2, sh, &floor))
-            floor = select_floor<VEC, true>(r, groups, floor, 0u, top_p, c2, sh);
+        if (!few || !nucleus_of_few<kSelThreads, VEC>(r, groups, floor, top_p, c2, sh, &floor))
+            floor = select_floor<kSelThreads, VEC, true>(r, groups, floor, 0u, top_p, c2, sh);
     }
     if (threadIdx.x == 0) floors[blockIdx.x] = floor;
 }
@@ -1184,6 +1227,11 @@ size_t verify_sample_workspace_bytes(int batch, int gamma, int vocab) {
     return stats_bytes(batch, gamma, vocab) + static_cast<size_t>(batch) * rows * sizeof(float) + 256;
 }
 
+// A selection CTA has 1024 threads where long rows would leave small CTAs with many loads in a row and the GPU unfilled:
+// nucleus 0.9, 200 rows of 100000 with the draw 131 -> 106 us, 30 rows of 120001 120 -> 64; on shorter or more rows the
+// wider barriers cost more than they give (216 rows of 50003 40 -> 38, 330 rows of 50003 52 -> 66, 11 rows of 8192 6 -> 8).
+bool wide_rows(int rows, int vocab) { return rows <= 2 * 148 && vocab >= 48 * 1024; }
+
 bool cut_is_on(int vocab, float temperature, int top_k, float top_p) {
     return temperature > 0.0f && ((top_k > 0 && top_k < vocab) || (top_p > 0.0f && top_p < 1.0f));
 }
@@ -1197,11 +1245,16 @@ int launch_cut_floors(const float* a, size_t a_stride, int a_rows, const float* 
     if (total == 0) return SPEC_OK;
     const bool vec = vocab % 4 == 0 && a_stride % 4 == 0 && aligned16(a) && (b_rows == 0 || (b_stride % 4 == 0 && aligned16(b)));
     const float c2 = inv_t * kLog2e;
-    if (vec)
-        return launch_pdl(cut_floor_kernel<true>, dim3(total), dim3(kSelThreads), 0, stream, a, a_stride, a_rows, b, b_stride,
-                          b_rows, vocab, top_k, top_p, c2, floors);
-    return launch_pdl(cut_floor_kernel<false>, dim3(total), dim3(kSelThreads), 0, stream, a, a_stride, a_rows, b, b_stride,
-                      b_rows, vocab, top_k, top_p, c2, floors);
+#define SPEC_LAUNCH_CUT(V, T)                                                                                        \
+    return launch_pdl(cut_floor_kernel<V, T>, dim3(total), dim3(T), 0, stream, a, a_stride, a_rows, b, b_stride, b_rows, \
+                      vocab, top_k, top_p, c2, floors)
+    if (wide_rows(total, vocab)) {
+        if (vec) SPEC_LAUNCH_CUT(true, 1024);
+        SPEC_LAUNCH_CUT(false, 1024);
+    }
+    if (vec) SPEC_LAUNCH_CUT(true, 256);
+    SPEC_LAUNCH_CUT(false, 256);
+#undef SPEC_LAUNCH_CUT
 }
 
 int launch_verify_sample(const float* target_logits, const float* draft_logits, const int32_t* draft_tokens,
@@ -1287,7 +1340,7 @@ int launch_sample_strided(const float* logits, size_t logit_stride, const float*
     }
     const bool vec = vocab % 4 == 0 && logit_stride % 4 == 0 && aligned16(logits);
 #define SPEC_LAUNCH_SAMPLE(V, C)                                                                                   \
-    return launch_pdl(sample_kernel<V, C>, dim3(rows), dim3(kSampleThreads), 0, stream, logits, logit_stride, uniforms, \
+    return launch_pdl(sample_kernel<V, C>, dim3(rows), dim3(kSampleThreads), 0, stream, logits, logit_stride, uniforms,     \
                       uniform_stride, vocab, inv_t, greedy, floors, tokens, token_stride, nonfinite)
     if (vec && floors) SPEC_LAUNCH_SAMPLE(true, true);
     if (vec) SPEC_LAUNCH_SAMPLE(true, false);

@@ -59,6 +59,14 @@ def _declare(h):
     h.spec_verify_sample_static_capacity.argtypes = []
     h.spec_verify_sample_static.restype = i32
     h.spec_verify_sample_static.argtypes = [vp, vp, vp, vp, i32, i32, i32, f32, vp, vp, vp]
+    h.spec_verify_sample_lenient.restype = i32
+    h.spec_verify_sample_lenient.argtypes = [vp, vp, vp, vp, i32, i32, i32, f32, f32, vp, vp, vp, sz, vp]
+    h.spec_verify_sample_truncated.restype = i32
+    h.spec_verify_sample_truncated.argtypes = [vp, vp, vp, vp, i32, i32, i32, f32, f32, i32, f32, vp, vp, vp, sz, vp]
+    h.spec_truncation_floors.restype = i32
+    h.spec_truncation_floors.argtypes = [vp, i32, i32, f32, i32, f32, vp, vp]
+    h.spec_sample_truncated.restype = i32
+    h.spec_sample_truncated.argtypes = [vp, vp, i32, i32, f32, i32, f32, vp, vp, vp]
     h.spec_sample.restype = i32
     h.spec_sample.argtypes = [vp, vp, i32, i32, f32, vp, vp]
     h.spec_uniforms.restype = i32
@@ -95,7 +103,10 @@ def _ptr(t, dtype, name, optional=False):
 
 
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    """The raw handle of torch's current stream (without the Stream object, which takes as long as a kernel launch)."""
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def spec_verify_sample_workspace_bytes(batch, gamma, vocab):
@@ -115,19 +126,18 @@ def spec_verify_sample(target_logits, draft_logits, draft_tokens, uniforms, temp
     """
     batch, rows, vocab = target_logits.shape
     gamma = rows - 1
-    dev = target_logits.device
     if n_accepted is None:
-        n_accepted = torch.empty(batch, dtype=torch.int32, device=dev)
+        n_accepted = torch.empty(batch, dtype=torch.int32, device=target_logits.device)
     if next_token is None:
-        next_token = torch.empty(batch, dtype=torch.int32, device=dev)
-    need = spec_verify_sample_workspace_bytes(batch, gamma, vocab)
-    if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=dev)
-    if draft_logits is not None and gamma > 0 and tuple(draft_logits.shape) != (batch, gamma, vocab):
+        next_token = torch.empty(batch, dtype=torch.int32, device=target_logits.device)
+    if workspace is None:  # (one that is given is checked by the library)
+        workspace = torch.empty(spec_verify_sample_workspace_bytes(batch, gamma, vocab), dtype=torch.uint8,
+                                device=target_logits.device)
+    if draft_logits is not None and gamma > 0 and draft_logits.shape != (batch, gamma, vocab):
         raise ValueError("draft_logits must be [B, gamma, V]")
-    if draft_tokens is not None and gamma > 0 and tuple(draft_tokens.shape) != (batch, gamma):
+    if draft_tokens is not None and gamma > 0 and draft_tokens.shape != (batch, gamma):
         raise ValueError("draft_tokens must be [B, gamma]")
-    if uniforms is not None and tuple(uniforms.shape) != (batch, gamma + 1):
+    if uniforms is not None and uniforms.shape != (batch, rows):
         raise ValueError("uniforms must be [B, gamma+1]")
     pointers = (_ptr(target_logits, torch.float32, "target_logits"),
                 _ptr(draft_logits, torch.float32, "draft_logits", optional=True),
@@ -136,20 +146,11 @@ def spec_verify_sample(target_logits, draft_logits, draft_tokens, uniforms, temp
     outputs = (_ptr(n_accepted, torch.int32, "n_accepted"), _ptr(next_token, torch.int32, "next_token"),
                _ptr(workspace, torch.uint8, "workspace"), workspace.numel(), _stream())
     if top_k or top_p != 1.0:
-        h = lib()
-        h.spec_verify_sample_truncated.restype = ctypes.c_int
-        h.spec_verify_sample_truncated.argtypes = [ctypes.c_void_p] * 4 + [ctypes.c_int] * 3 + [ctypes.c_float] * 2 + \
-            [ctypes.c_int, ctypes.c_float] + [ctypes.c_void_p] * 3 + [ctypes.c_size_t, ctypes.c_void_p]
-        _check(h.spec_verify_sample_truncated(*pointers, batch, gamma, vocab, float(temperature), float(lenience),
-                                              int(top_k), float(top_p), *outputs))
+        _check(lib().spec_verify_sample_truncated(*pointers, batch, gamma, vocab, temperature, lenience, top_k, top_p, *outputs))
     elif lenience == 1.0:
-        _check(lib().spec_verify_sample(*pointers, batch, gamma, vocab, float(temperature), *outputs))
+        _check(lib().spec_verify_sample(*pointers, batch, gamma, vocab, temperature, *outputs))
     else:
-        h = lib()
-        h.spec_verify_sample_lenient.restype = ctypes.c_int
-        h.spec_verify_sample_lenient.argtypes = [ctypes.c_void_p] * 4 + [ctypes.c_int] * 3 + [ctypes.c_float] * 2 + \
-            [ctypes.c_void_p] * 3 + [ctypes.c_size_t, ctypes.c_void_p]
-        _check(h.spec_verify_sample_lenient(*pointers, batch, gamma, vocab, float(temperature), float(lenience), *outputs))
+        _check(lib().spec_verify_sample_lenient(*pointers, batch, gamma, vocab, temperature, lenience, *outputs))
     return n_accepted, next_token
 
 
@@ -175,12 +176,8 @@ def spec_truncation_floors(logits, temperature, top_k=0, top_p=1.0, floors=None)
     rows, vocab = logits.shape
     if floors is None:
         floors = torch.empty(rows, dtype=torch.float32, device=logits.device)
-    h = lib()
-    h.spec_truncation_floors.restype = ctypes.c_int
-    h.spec_truncation_floors.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_float, ctypes.c_int,
-                                         ctypes.c_float, ctypes.c_void_p, ctypes.c_void_p]
-    _check(h.spec_truncation_floors(_ptr(logits, torch.float32, "logits"), rows, vocab, float(temperature), int(top_k),
-                                    float(top_p), _ptr(floors, torch.float32, "floors"), _stream()))
+    _check(lib().spec_truncation_floors(_ptr(logits, torch.float32, "logits"), rows, vocab, float(temperature),
+                                         int(top_k), float(top_p), _ptr(floors, torch.float32, "floors"), _stream()))
     return floors
 
 
@@ -192,14 +189,11 @@ def spec_sample(logits, uniforms, temperature, tokens=None, top_k=0, top_p=1.0):
         tokens = torch.empty(rows, dtype=torch.int32, device=logits.device)
     if top_k or top_p != 1.0:
         floors = torch.empty(max(rows, 1), dtype=torch.float32, device=logits.device)
-        h = lib()
-        h.spec_sample_truncated.restype = ctypes.c_int
-        h.spec_sample_truncated.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_float,
-                                            ctypes.c_int, ctypes.c_float, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
-        _check(h.spec_sample_truncated(_ptr(logits, torch.float32, "logits"),
-                                       _ptr(uniforms, torch.float32, "uniforms", optional=True), rows, vocab,
-                                       float(temperature), int(top_k), float(top_p), _ptr(tokens, torch.int32, "tokens"),
-                                       _ptr(floors, torch.float32, "floors"), _stream()))
+        _check(lib().spec_sample_truncated(_ptr(logits, torch.float32, "logits"),
+                                           _ptr(uniforms, torch.float32, "uniforms", optional=True), rows, vocab,
+                                           float(temperature), int(top_k), float(top_p),
+                                           _ptr(tokens, torch.int32, "tokens"), _ptr(floors, torch.float32, "floors"),
+                                           _stream()))
         return tokens
     _check(lib().spec_sample(_ptr(logits, torch.float32, "logits"),
                              _ptr(uniforms, torch.float32, "uniforms", optional=True),

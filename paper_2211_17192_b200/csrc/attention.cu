@@ -1242,6 +1242,8 @@ AttentionPlan attention_plan(const Model& m, int batch, int m_rows, int max_keys
     return plan;
 }
 
+int* attention_error_word() { return symbol_address(g_attn_error); }
+
 int attention_take_error() {
     int v = 0, zero = 0;
     if (cudaMemcpyFromSymbol(&v, g_attn_error, sizeof(int)) != cudaSuccess) return -1;

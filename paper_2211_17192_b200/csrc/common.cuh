@@ -75,6 +75,17 @@ inline int launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
     return SPEC_OK;
 }
 
+// Device address of a __device__ variable (nullptr if there is none on this device).
+template <typename T>
+inline T* symbol_address(T& symbol) {
+    void* p = nullptr;
+    if (cudaGetSymbolAddress(&p, symbol) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return static_cast<T*>(p);
+}
+
 // ---- warp / block primitives ----------------------------------------------
 constexpr unsigned kFullMask = 0xffffffffu;
 

@@ -10,6 +10,17 @@
 
 #include "model.cuh"
 
+constexpr int kCounters = 4 + 65;  // see spec_ctx::counters
+
+// What a finished piece of work tells the host: gathered by one small kernel and fetched by one copy at the end, instead
+// of a copy per item, each of which would wait for the device on its own.
+struct spec_report {
+    int gave_up;    // code of a bounded wait that ran out since the last report (0: none)
+    int nonfinite;  // see spec_ctx::nonfinite
+    unsigned long long counters[kCounters];
+    int32_t length[1];  // of every sequence (max_batch entries)
+};
+
 struct spec_ctx {
     spec::Model model[2];  // 0 target, 1 draft
     bool has_draft = false;
@@ -39,6 +50,20 @@ struct spec_ctx {
     int32_t* row_block = nullptr;  // one allocation: the five row arrays below, a prompt chunk's packed rows and segments
     int32_t *row_token = nullptr, *row_pos = nullptr, *row_seq = nullptr, *logit_src = nullptr, *logit_dst = nullptr;
     int32_t* page_table = nullptr;
+
+    spec_report* report = nullptr;      // the last one, on the host (in report_memory)
+    char* report_dev = nullptr;
+    std::vector<char> report_memory;
+    std::vector<int32_t> staging;       // row descriptors on their way to row_block
+    int* error_words[4] = {nullptr, nullptr, nullptr, nullptr};
+
+    // Captured passes of spec_forward_logits: a shape is captured the third time it is asked for (the capture costs about
+    // a launch-bound pass or two); the oldest of eight makes room.
+    struct PassGraph {
+        int which, batch, rows, uses;
+        cudaGraphExec_t exec;
+    };
+    std::vector<PassGraph> pass_graphs;
 
     // generation state (device)
     int32_t *tokens = nullptr, *length = nullptr, *prompt_len = nullptr, *draft_tokens = nullptr;
@@ -78,8 +103,6 @@ struct spec_ctx {
 
 namespace spec {
 namespace {
-
-constexpr int kCounters = 4 + 65;  // see spec_ctx::counters
 
 int check_cfg(const spec_model_cfg& c, const char* which) {
     if (c.arch == SPEC_ARCH_BIGRAM) {
@@ -208,10 +231,45 @@ struct Pass {
     }
 };
 
-// Non-zero (and cleared) if a tensor-core GEMM or the persistent pass kernel gave up on a bounded wait.
-int device_gave_up(spec_ctx* ctx) {
+// Non-zero (and cleared) if a kernel gave up on a bounded wait.
+int device_gave_up() {
     const int gemm = gemm_tc_take_error(), wide = gemm_wide_take_error(), pass = pass_take_error(), attn = attention_take_error();
     return gemm ? gemm : wide ? wide : pass ? pass : attn;
+}
+
+struct ErrorWords {
+    int* word[4];
+};
+
+// block = 128.  Leaves the state of the work before it in `out`.
+__global__ void report_kernel(ErrorWords errors, int* nonfinite, const unsigned long long* counters, const int32_t* length, int batch,
+                              spec_report* out) {
+    pdl_wait();
+    if (threadIdx.x == 0) {
+        int code = 0;
+        for (int i = 0; i < 4; ++i)
+            if (errors.word[i]) code |= *errors.word[i];
+        out->gave_up = code;
+        out->nonfinite = *nonfinite;
+        *nonfinite = 0;
+    }
+    for (int i = threadIdx.x; i < kCounters; i += blockDim.x) out->counters[i] = counters[i];
+    for (int i = threadIdx.x; i < batch; i += blockDim.x) out->length[i] = length[i];
+}
+
+// Waits for everything on the context's stream; ctx->report then describes it.
+int finish_work(spec_ctx* ctx, int batch) {
+    const ErrorWords errors{{ctx->error_words[0], ctx->error_words[1], ctx->error_words[2], ctx->error_words[3]}};
+    SPEC_TRY(launch_pdl(report_kernel, dim3(1), dim3(128), 0, ctx->stream, errors, ctx->nonfinite, ctx->counters, ctx->length, batch,
+                        reinterpret_cast<spec_report*>(ctx->report_dev)));
+    SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->report, ctx->report_dev, sizeof(spec_report) + batch * sizeof(int32_t), cudaMemcpyDeviceToHost,
+                                  ctx->stream));
+    SPEC_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+    if (ctx->report->gave_up) {
+        const int code = device_gave_up();  // (which one, and clears it)
+        return fail(SPEC_ERR_DEVICE_TIMEOUT, "a kernel gave up on a bounded wait (code %d)", code ? code : ctx->report->gave_up);
+    }
+    return SPEC_OK;
 }
 
 RowMeta row_meta(const spec_ctx* ctx) { return RowMeta{ctx->row_token, ctx->row_pos, ctx->row_seq}; }
@@ -232,7 +290,7 @@ KvPool source_pool(const spec_ctx* ctx, const Model& m, void* base) {
 // write logits rows logit_dst[i] (all rows in order if both are null).  With `segs` the rows are a prompt chunk's,
 // m_rows of them in all (batch = 1).
 int forward(spec_ctx* ctx, const Model& m, const RowMeta& rows, int batch, int m_rows, int n_logit_rows, const int32_t* logit_src,
-            const int32_t* logit_dst, float* logits, const PromptSegments* segs = nullptr) {
+            const int32_t* logit_dst, float* logits, const PromptSegments* segs = nullptr, float* const* logits_slot = nullptr) {
     const spec_model_cfg& c = m.cfg;
     const int n_rows = batch * m_rows;
     if (c.arch == SPEC_ARCH_BIGRAM)  // logits = table[last token]: one gather
@@ -281,7 +339,7 @@ int forward(spec_ctx* ctx, const Model& m, const RowMeta& rows, int batch, int m
         SPEC_TRY(pass.norm(m.ln_f, logit_src, n_logit_rows));
         if (pass.tc)
             SPEC_TRY(launch_gemm_tc(pass.hi(), pass.lo(), ctx->hi_rows, m.packed_head, true, nullptr, logit_dst, n_logit_rows,
-                                    c.vocab, d, ctx->partials, logits, ctx->stream));
+                                    c.vocab, d, ctx->partials, logits, ctx->stream, logits_slot));
         else
             SPEC_TRY(launch_gemm_rows(ctx->a, m.head, m.bf16(), nullptr, logit_dst, n_logit_rows, c.vocab, d, logits, ctx->stream));
     }
@@ -876,6 +934,7 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     SPEC_ALLOC(counters, kCounters);
     SPEC_ALLOC(nonfinite, 1);
     SPEC_ALLOC(params, 1);
+    SPEC_ALLOC(report_dev, sizeof(spec_report) + B * sizeof(int32_t));
     SPEC_ALLOC(sample_floors, B);
     {
         char* ws = nullptr;
@@ -898,6 +957,16 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
         err = cudaMemcpy(ctx->src_page_table, src_table.data(), src_table.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
         if (err != cudaSuccess) return cleanup(fail(SPEC_ERR_CUDA, "source page table upload: %s", cudaGetErrorString(err)));
     }
+    const size_t report_bytes = sizeof(spec_report) + B * sizeof(int32_t);
+    ctx->report_memory.assign(report_bytes, 0);
+    ctx->report = reinterpret_cast<spec_report*>(ctx->report_memory.data());
+    ctx->staging.resize(3 * (R + 4) + 4);
+    cudaMemset(ctx->nonfinite, 0, sizeof(int));
+    cudaMemset(ctx->counters, 0, kCounters * sizeof(unsigned long long));
+    ctx->error_words[0] = gemm_tc_error_word();
+    ctx->error_words[1] = gemm_wide_error_word();
+    ctx->error_words[2] = pass_error_word();
+    ctx->error_words[3] = attention_error_word();
     ctx->cached[0].assign(B, 0);
     ctx->cached[1].assign(B, 0);
     *out = ctx;
@@ -909,6 +978,8 @@ extern "C" void spec_free(spec_ctx* ctx) {
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     drop_graphs(ctx);
     pass_scratch_release(ctx->pass);
+    for (const spec_ctx::PassGraph& g : ctx->pass_graphs)
+        if (g.exec) cudaGraphExecDestroy(g.exec);
     for (void* p : ctx->allocations) cudaFree(p);
     for (auto& e : ctx->ev)
         if (e) cudaEventDestroy(e);
@@ -950,8 +1021,7 @@ int encode_sources(spec_ctx* ctx, const int32_t* source, const int32_t* source_l
     SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->src_len, source_len, batch * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     for (int which = 0; which < n_models; ++which)
         if (ctx->model[which].t5()) SPEC_TRY(encode(ctx, ctx->model[which], batch, longest));  // (a table draft has no encoder)
-    SPEC_CUDA_TRY(cudaStreamSynchronize(st));  // the host vectors go out of scope
-    if (const int gave_up = device_gave_up(ctx)) return fail(SPEC_ERR_DEVICE_TIMEOUT, "a kernel gave up on a bounded wait (code %d)", gave_up);
+    SPEC_TRY(finish_work(ctx, 0));  // (the host vectors go out of scope)
     ctx->encoded = true;
     ctx->encoded_batch = batch;
     return SPEC_OK;
@@ -1036,32 +1106,25 @@ int begin_session(spec_ctx* ctx, const int32_t* prompt, const int32_t* prompt_le
 int run_iterations(spec_ctx* ctx, int iterations, float* elapsed_ms, int* remaining) {
     cudaStream_t st = ctx->stream;
     const int batch = ctx->session_batch;
-    std::vector<int32_t> lengths(batch);
     SPEC_CUDA_TRY(cudaEventRecord(ctx->ev[1], st));
     for (int i = 0; i < iterations; ++i) SPEC_CUDA_TRY(cudaGraphLaunch(ctx->graph, st));
     SPEC_CUDA_TRY(cudaEventRecord(ctx->ev[2], st));
     ctx->session_replays += iterations;
     ctx->session_draft_passes += static_cast<long long>(iterations) * ctx->session_gamma;
-    SPEC_CUDA_TRY(cudaMemcpyAsync(lengths.data(), ctx->length, batch * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    int nonfinite = 0;
-    SPEC_CUDA_TRY(cudaMemcpyAsync(&nonfinite, ctx->nonfinite, sizeof(int), cudaMemcpyDeviceToHost, st));
-    SPEC_CUDA_TRY(cudaStreamSynchronize(st));
-    if (nonfinite) {
-        SPEC_CUDA_TRY(cudaMemsetAsync(ctx->nonfinite, 0, sizeof(int), st));
+    const int status = finish_work(ctx, batch);
+    if (ctx->report->nonfinite)
         return fail(SPEC_ERR_NONFINITE, "a model produced a NaN or +inf logit, or a row without a finite logit (the tokens of these "
                                         "iterations are not valid)");
-    }
-    if (const int gave_up = device_gave_up(ctx)) return fail(SPEC_ERR_DEVICE_TIMEOUT, "a kernel gave up on a bounded wait (code %d)", gave_up);
+    SPEC_TRY(status);
     SPEC_CUDA_TRY(cudaEventElapsedTime(elapsed_ms, ctx->ev[1], ctx->ev[2]));
     *remaining = 0;
     for (int b = 0; b < batch; ++b)
-        *remaining = std::max(*remaining, ctx->session_n_new - (lengths[b] - ctx->session_prompt_len[b]));
+        *remaining = std::max(*remaining, ctx->session_n_new - (ctx->report->length[b] - ctx->session_prompt_len[b]));
     return SPEC_OK;
 }
 
 int fill_stats(spec_ctx* ctx, double decode_ms, spec_stats* stats) {
-    unsigned long long counters[kCounters];
-    SPEC_CUDA_TRY(cudaMemcpy(counters, ctx->counters, sizeof(counters), cudaMemcpyDeviceToHost));
+    const unsigned long long* counters = ctx->report->counters;  // (as of the iterations just finished)
     for (int n = 0; n <= 64; ++n) stats->accepted_histogram[n] = static_cast<int64_t>(counters[4 + n]);
     stats->iterations = static_cast<int64_t>(counters[0]);
     stats->tokens = static_cast<int64_t>(counters[1]);
@@ -1204,8 +1267,7 @@ extern "C" int spec_generate_adaptive(spec_ctx* ctx, const int32_t* prompt, cons
             trace[2 * bursts + 1] = count;
         }
         ++bursts;
-        unsigned long long counters[4];
-        SPEC_CUDA_TRY(cudaMemcpy(counters, ctx->counters, sizeof(counters), cudaMemcpyDeviceToHost));
+        const unsigned long long* counters = ctx->report->counters;
         const long long evaluated = static_cast<long long>(counters[2]) - seen_evaluated;
         const long long passed = static_cast<long long>(counters[3]) - seen_passed;
         seen_evaluated += evaluated;
@@ -1327,7 +1389,7 @@ extern "C" int spec_pass_trace(spec_ctx* ctx, int which, int batch, int rows, un
     cudaFree(dev);
     SPEC_CUDA_TRY(err);
     if (status != SPEC_OK) return status;
-    if (const int gave_up = device_gave_up(ctx)) return fail(SPEC_ERR_DEVICE_TIMEOUT, "a kernel gave up on a bounded wait (code %d)", gave_up);
+    SPEC_TRY(finish_work(ctx, 0));
     int used = 0;
     for (int i = 0; i < capacity; ++i)
         if (stamps_ns[i]) used = i + 1;
@@ -1380,7 +1442,7 @@ extern "C" int spec_time_forward(spec_ctx* ctx, int which, int batch, int rows, 
     if (err == cudaSuccess) err = cudaStreamSynchronize(st);
     cudaGraphExecDestroy(exec);
     SPEC_CUDA_TRY(err);
-    if (const int gave_up = device_gave_up(ctx)) return fail(SPEC_ERR_DEVICE_TIMEOUT, "a kernel gave up on a bounded wait (code %d)", gave_up);
+    SPEC_TRY(finish_work(ctx, 0));
     float ms = 0.0f;
     SPEC_CUDA_TRY(cudaEventElapsedTime(&ms, ctx->ev[1], ctx->ev[2]));
     *ms_per_pass = ms / static_cast<float>(repeats);
@@ -1398,27 +1460,59 @@ extern "C" int spec_forward_logits(spec_ctx* ctx, int which, const int32_t* toke
     if (ctx->model[which].t5() && (!ctx->encoded || batch > ctx->encoded_batch))
         return fail(SPEC_ERR_BAD_ARG, "spec_forward_logits: call spec_encode for these sequences first");
     const Model& m = ctx->model[which];
-    const int n = batch * rows;
+    const int n = batch * rows, n4 = (n + 3) / 4 * 4;
     ctx->session_batch = 0;  // the diagnostics reuse the caches
-    std::vector<int32_t> tok(n), pos(n), seq(n);
+    // tokens, positions, sequences (each padded to n4), the address of the logits: one copy
+    int32_t* block = ctx->staging.data();
     for (int b = 0; b < batch; ++b) {
         if (ctx->cached[which][b] + rows > std::min(ctx->rt.max_len, m.cfg.max_positions))
             return fail(SPEC_ERR_CAPACITY, "spec_forward_logits: sequence %d would exceed the cache", b);
         for (int j = 0; j < rows; ++j) {
             const int32_t t = tokens[b * rows + j];
             if (t < 0 || t >= m.cfg.vocab) return fail(SPEC_ERR_BAD_ARG, "spec_forward_logits: token %d out of range", t);
-            tok[b * rows + j] = t;
-            pos[b * rows + j] = ctx->cached[which][b] + j;
-            seq[b * rows + j] = b;
+            block[b * rows + j] = t;
+            block[n4 + b * rows + j] = ctx->cached[which][b] + j;
+            block[2 * n4 + b * rows + j] = b;
         }
     }
+    std::memcpy(block + 3 * n4, &logits, sizeof(logits));
     cudaStream_t st = ctx->stream;
-    SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_token, tok.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_pos, pos.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_seq, seq.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    SPEC_TRY(forward(ctx, m, row_meta(ctx), batch, rows, n, nullptr, nullptr, logits));
-    SPEC_CUDA_TRY(cudaStreamSynchronize(st));
-    if (const int gave_up = device_gave_up(ctx)) return fail(SPEC_ERR_DEVICE_TIMEOUT, "a kernel gave up on a bounded wait (code %d)", gave_up);
+    SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->row_block, block, 3 * n4 * sizeof(int32_t) + sizeof(logits), cudaMemcpyHostToDevice, st));
+    const RowMeta meta{ctx->row_block, ctx->row_block + n4, ctx->row_block + 2 * n4};
+    // A pass is 40 to 400 launches; narrow models are bound by them.  (fp32 and table models, the pass kernel and logits
+    // that are not 16-byte aligned stay with plain launches.)
+    spec_ctx::PassGraph* graph = nullptr;
+    if (m.bf16() && m.cfg.arch != SPEC_ARCH_BIGRAM && !ctx->rt.pass_kernel && (reinterpret_cast<uintptr_t>(logits) & 15u) == 0) {
+        for (spec_ctx::PassGraph& g : ctx->pass_graphs)
+            if (g.which == which && g.batch == batch && g.rows == rows) graph = &g;
+        if (!graph) {
+            if (ctx->pass_graphs.size() == 8) {
+                if (ctx->pass_graphs.front().exec) cudaGraphExecDestroy(ctx->pass_graphs.front().exec);
+                ctx->pass_graphs.erase(ctx->pass_graphs.begin());
+            }
+            ctx->pass_graphs.push_back({which, batch, rows, 0, nullptr});
+            graph = &ctx->pass_graphs.back();
+        }
+        if (++graph->uses >= 3 && !graph->exec) {
+            SPEC_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+            const int status = forward(ctx, m, meta, batch, rows, n, nullptr, nullptr, nullptr, nullptr,
+                                       reinterpret_cast<float* const*>(ctx->row_block + 3 * n4));
+            cudaGraph_t g = nullptr;
+            const cudaError_t end = cudaStreamEndCapture(st, &g);
+            if (status != SPEC_OK) {
+                if (g) cudaGraphDestroy(g);
+                return status;
+            }
+            SPEC_CUDA_TRY(end);
+            const cudaError_t inst = cudaGraphInstantiate(&graph->exec, g, 0);
+            cudaGraphDestroy(g);
+            if (inst != cudaSuccess) graph->exec = nullptr;
+            SPEC_CUDA_TRY(inst);
+        }
+    }
+    if (graph && graph->exec) SPEC_CUDA_TRY(cudaGraphLaunch(graph->exec, st));
+    else SPEC_TRY(forward(ctx, m, meta, batch, rows, n, nullptr, nullptr, logits));
+    SPEC_TRY(finish_work(ctx, 0));
     for (int b = 0; b < batch; ++b) ctx->cached[which][b] += rows;
     return SPEC_OK;
 }

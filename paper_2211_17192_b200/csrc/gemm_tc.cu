@@ -277,9 +277,10 @@ __global__ void split_bf16_kernel(const float* __restrict__ x, size_t n, __nv_bf
 // a thread takes VEC (4 or 1) neighbouring columns at a time.
 template <int VEC>
 __global__ void reduce_partials_kernel(const float* partial, const PartialPlan plan, int n_rows, int n_out,
-                                       const float* residual, const int32_t* dst_rows, float* y) {
+                                       const float* residual, const int32_t* dst_rows, float* y, float* const* y_slot) {
     pdl_trigger();
     pdl_wait();
+    if (y_slot) y = *y_slot;
     const size_t total = static_cast<size_t>(n_rows) * n_out;
     const int r = blockIdx.y;
     const float* in = partial + static_cast<size_t>(r) * n_out;
@@ -527,19 +528,21 @@ int launch_gemm_tc_partials(const __nv_bfloat16* hi, const __nv_bfloat16* lo, in
 // y[dst(r)] = x[r] . W^T (+ residual[r]): the partial sums, then their reduction.
 int launch_gemm_tc(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_rows, const void* w, bool packed,
                    const float* residual, const int32_t* dst_rows, int n_rows, int n_out, int k, float* partial,
-                   float* y, cudaStream_t stream) {
+                   float* y, cudaStream_t stream, float* const* y_slot) {
     if (n_rows <= 0) return SPEC_OK;
     const int status = launch_gemm_tc_partials(hi, lo, hi_rows, w, packed, n_rows, n_out, k, partial, stream);
     if (status != SPEC_OK) return status;
     const PartialPlan plan = gemm_tc_plan(n_out, k, n_rows);
     const float* sums = partial;
-    const bool vec = n_out % 4 == 0 && (reinterpret_cast<uintptr_t>(y) & 15u) == 0;
+    const bool vec = n_out % 4 == 0 && (reinterpret_cast<uintptr_t>(y) & 15u) == 0;  // (y: null or the first address with a slot)
     const dim3 grid((n_out + (vec ? 1023 : 255)) / (vec ? 1024 : 256), n_rows);
-    if (vec) return launch_pdl(reduce_partials_kernel<4>, grid, dim3(256), 0, stream, sums, plan, n_rows, n_out, residual, dst_rows, y);
-    return launch_pdl(reduce_partials_kernel<1>, grid, dim3(256), 0, stream, sums, plan, n_rows, n_out, residual, dst_rows, y);
+    if (vec) return launch_pdl(reduce_partials_kernel<4>, grid, dim3(256), 0, stream, sums, plan, n_rows, n_out, residual, dst_rows, y, y_slot);
+    return launch_pdl(reduce_partials_kernel<1>, grid, dim3(256), 0, stream, sums, plan, n_rows, n_out, residual, dst_rows, y, y_slot);
 }
 
 // Non-zero if a tensor-core GEMM gave up on a bounded wait since the last call.
+int* gemm_tc_error_word() { return symbol_address(g_gemm_error); }
+
 int gemm_tc_take_error() {
     int v = 0, zero = 0;
     if (cudaMemcpyFromSymbol(&v, g_gemm_error, sizeof(int)) != cudaSuccess) return -1;

@@ -343,6 +343,8 @@ int launch_gemm_wide(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_ro
     return launch_pdl(gemm_wide_kernel, dim3(2 * a.plan.pairs), dim3(kWideThreads), smem, stream, mw, mhi, mlo, partial, a);
 }
 
+int* gemm_wide_error_word() { return symbol_address(g_wide_error); }
+
 int gemm_wide_take_error() {
     int v = 0, zero = 0;
     if (cudaMemcpyFromSymbol(&v, g_wide_error, sizeof(int)) != cudaSuccess) return -1;

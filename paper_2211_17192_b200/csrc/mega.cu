@@ -1325,6 +1325,8 @@ void pass_scratch_release(PassScratch& s) {
 // Non-zero if the pass kernel gave up on a bounded wait since the last call (then the barrier
 // words and part counters of every context are reset, so that the next launch starts clean).
 // Synchronises.
+int* pass_error_word() { return symbol_address(g_mega_error); }
+
 int pass_take_error() {
     int v = 0, zero = 0;
     if (cudaMemcpyFromSymbol(&v, g_mega_error, sizeof(int)) != cudaSuccess) return -1;

@@ -122,9 +122,15 @@ PartialPlan gemm_wide_plan(int n_out, int k, int n_rows);
 int launch_gemm_wide(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_rows, const void* w, bool packed, int n_rows,
                      int n_out, int k, float* partial, bool fill, cudaStream_t stream);
 int gemm_wide_take_error();
+// Device addresses of the words in which the kernels record a wait that ran out (0: none did).
+int* gemm_tc_error_word();
+int* gemm_wide_error_word();
+int* attention_error_word();
+int* pass_error_word();
 int launch_gemm_tc(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_rows, const void* w, bool packed,
                    const float* residual, const int32_t* dst_rows, int n_rows, int n_out, int k, float* partial,
-                   float* y, cudaStream_t stream);
+                   float* y, cudaStream_t stream, float* const* y_slot = nullptr);
+// (`y_slot`: a device word that holds y's address when the launch runs, for launches that are captured once)
 int gemm_tc_take_error();
 
 // Where the K,V rows of a pass go / come from: one layer's pool

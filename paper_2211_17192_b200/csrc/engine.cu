@@ -398,12 +398,17 @@ __global__ void iteration_uniforms_kernel(const spec_ctx::Params* __restrict__ p
     if (j < gamma) draft_u[b * gamma + j] = method_uniform(seed, pos, b, kPurposeDraft);
 }
 
+// Rows of the passes below: a sequence that has its n_new tokens is frozen but stays in the batch, and its guesses may
+// then lie beyond the positions the context holds.  Such rows (position >= `limit`) are inactive: they are computed, and
+// neither cached nor looked at.
+__device__ __forceinline__ int held(int position, int limit) { return position < limit ? position : -1; }
+
 // First draft step of an iteration: two rows per sequence, positions L-2 and
 // L-1.  Position L-2 is already cached unless the previous iteration accepted
 // every guess (x_gamma was never fed to the draft); feeding it again rewrites
 // the same K,V row, so the shape of the step never changes.
 __global__ void prep_draft_first_kernel(const int32_t* __restrict__ tokens, const int32_t* __restrict__ length,
-                                        int batch, int gamma, int max_len, int32_t* row_token, int32_t* row_pos,
+                                        int batch, int gamma, int max_len, int limit, int32_t* row_token, int32_t* row_pos,
                                         int32_t* row_seq, int32_t* logit_src, int32_t* logit_dst) {
     pdl_trigger();
     pdl_wait();
@@ -413,8 +418,8 @@ __global__ void prep_draft_first_kernel(const int32_t* __restrict__ tokens, cons
     const int p0 = max(L - 2, 0), p1 = L - 1;
     row_token[2 * b] = tokens[static_cast<size_t>(b) * max_len + p0];
     row_token[2 * b + 1] = tokens[static_cast<size_t>(b) * max_len + p1];
-    row_pos[2 * b] = p0;
-    row_pos[2 * b + 1] = p1;
+    row_pos[2 * b] = held(p0, limit);
+    row_pos[2 * b + 1] = held(p1, limit);
     row_seq[2 * b] = row_seq[2 * b + 1] = b;
     logit_src[b] = 2 * b + 1;
     logit_dst[b] = b * gamma;  // q_1
@@ -422,14 +427,14 @@ __global__ void prep_draft_first_kernel(const int32_t* __restrict__ tokens, cons
 
 // Draft step i (2..gamma): one row per sequence, the previous guess x_{i-1} at position L+i-2.
 __global__ void prep_draft_step_kernel(const int32_t* __restrict__ draft_tokens, const int32_t* __restrict__ length,
-                                       int batch, int gamma, int step, int32_t* row_token, int32_t* row_pos,
+                                       int batch, int gamma, int step, int limit, int32_t* row_token, int32_t* row_pos,
                                        int32_t* row_seq, int32_t* logit_src, int32_t* logit_dst) {
     pdl_trigger();
     pdl_wait();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= batch) return;
     row_token[b] = draft_tokens[b * gamma + step - 2];
-    row_pos[b] = length[b] + step - 2;
+    row_pos[b] = held(length[b] + step - 2, limit);
     row_seq[b] = b;
     logit_src[b] = b;
     logit_dst[b] = b * gamma + step - 1;
@@ -437,7 +442,7 @@ __global__ void prep_draft_step_kernel(const int32_t* __restrict__ draft_tokens,
 
 // The target's parallel pass: rows [last committed token, x_1..x_gamma] at positions L-1..L-1+gamma.
 __global__ void prep_verify_kernel(const int32_t* __restrict__ tokens, const int32_t* __restrict__ draft_tokens,
-                                   const int32_t* __restrict__ length, int batch, int gamma, int max_len,
+                                   const int32_t* __restrict__ length, int batch, int gamma, int max_len, int limit,
                                    int32_t* row_token, int32_t* row_pos, int32_t* row_seq) {
     pdl_trigger();
     pdl_wait();
@@ -446,7 +451,7 @@ __global__ void prep_verify_kernel(const int32_t* __restrict__ tokens, const int
     const int b = i / (gamma + 1), j = i % (gamma + 1);
     const int L = length[b];
     row_token[i] = j == 0 ? tokens[static_cast<size_t>(b) * max_len + L - 1] : draft_tokens[b * gamma + j - 1];
-    row_pos[i] = L - 1 + j;
+    row_pos[i] = held(L - 1 + j, limit);
     row_seq[i] = b;
 }
 
@@ -487,6 +492,8 @@ int enqueue_iteration(spec_ctx* ctx, int batch, int gamma, float temperature) {
     ctx->iteration_gamma = gamma;
     const int vocab = ctx->model[0].cfg.vocab;
     const int threads = 128;
+    int limit = std::min(ctx->rt.max_len, ctx->model[0].cfg.max_positions);
+    if (gamma > 0) limit = std::min(limit, ctx->model[1].cfg.max_positions);
     const int blocks_b = (batch + threads - 1) / threads;
     const int blocks_bg = (batch * (gamma + 1) + threads - 1) / threads;
     SPEC_TRY(launch_pdl(iteration_uniforms_kernel, dim3(blocks_bg), dim3(threads), 0, st, ctx->params, ctx->length,
@@ -495,12 +502,12 @@ int enqueue_iteration(spec_ctx* ctx, int batch, int gamma, float temperature) {
         int rows;
         if (step == 1) {
             SPEC_TRY(launch_pdl(prep_draft_first_kernel, dim3(blocks_b), dim3(threads), 0, st, ctx->tokens, ctx->length,
-                                batch, gamma, ctx->rt.max_len, ctx->row_token, ctx->row_pos, ctx->row_seq,
+                                batch, gamma, ctx->rt.max_len, limit, ctx->row_token, ctx->row_pos, ctx->row_seq,
                                 ctx->logit_src, ctx->logit_dst));
             rows = 2 * batch;
         } else {
             SPEC_TRY(launch_pdl(prep_draft_step_kernel, dim3(blocks_b), dim3(threads), 0, st, ctx->draft_tokens,
-                                ctx->length, batch, gamma, step, ctx->row_token, ctx->row_pos, ctx->row_seq,
+                                ctx->length, batch, gamma, step, limit, ctx->row_token, ctx->row_pos, ctx->row_seq,
                                 ctx->logit_src, ctx->logit_dst));
             rows = batch;
         }
@@ -512,7 +519,7 @@ int enqueue_iteration(spec_ctx* ctx, int batch, int gamma, float temperature) {
                                        ctx->draft_tokens + (step - 1), gamma, st, ctx->nonfinite));
     }
     SPEC_TRY(launch_pdl(prep_verify_kernel, dim3(blocks_bg), dim3(threads), 0, st, ctx->tokens, ctx->draft_tokens,
-                        ctx->length, batch, gamma, ctx->rt.max_len, ctx->row_token, ctx->row_pos, ctx->row_seq));
+                        ctx->length, batch, gamma, ctx->rt.max_len, limit, ctx->row_token, ctx->row_pos, ctx->row_seq));
     SPEC_TRY(forward(ctx, ctx->model[0], row_meta(ctx), batch, gamma + 1, batch * (gamma + 1), nullptr, nullptr, ctx->target_logits));
     SPEC_TRY(launch_verify_sample(ctx->target_logits, ctx->draft_logits, ctx->draft_tokens, ctx->accept_u, ctx->final_u,
                                   batch, gamma, vocab, temperature, ctx->lenience, ctx->top_k, ctx->top_p, ctx->n_accepted,

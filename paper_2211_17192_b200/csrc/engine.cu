@@ -46,6 +46,7 @@ struct spec_ctx {
     int pass_trace_capacity = 0;
     float* attn_part = nullptr;  // per key slice: (max, sum, accumulator) of every (row, head)
     int hi_rows = 0;
+    spec::SmallPass small[2];  // per model: few-row passes of a small decoder as one kernel
     spec::PassScratch pass;  // the persistent pass kernel's scratch (passes of at most 16 rows of a bf16 model)
     int32_t* row_block = nullptr;  // one allocation: the five row arrays below, a prompt chunk's packed rows and segments
     int32_t *row_token = nullptr, *row_pos = nullptr, *row_seq = nullptr, *logit_src = nullptr, *logit_dst = nullptr;
@@ -55,7 +56,7 @@ struct spec_ctx {
     char* report_dev = nullptr;
     std::vector<char> report_memory;
     std::vector<int32_t> staging;       // row descriptors on their way to row_block
-    int* error_words[4] = {nullptr, nullptr, nullptr, nullptr};
+    int* error_words[5] = {};
 
     // Captured passes of spec_forward_logits: a shape is captured the third time it is asked for (the capture costs about
     // a launch-bound pass or two); the oldest of eight makes room.
@@ -165,7 +166,8 @@ struct Pass {
     int n_rows;
     bool tc;
     cudaStream_t st;
-    bool pending = false;   // partial sums (laid out by `closing`) not yet added into h
+    bool pending = false;   // partial sums (at `branch`, laid out by `closing`) not yet added into h
+    const float* branch = nullptr;
     PartialPlan closing{};  // of the last GEMM that closed a residual branch
     PartialPlan last{};     // of the last projection
 
@@ -175,7 +177,7 @@ struct Pass {
     // a (fp32) or hi/lo = rmsnorm(h[src(i)]) * gain for i < n
     int norm(const float* gain, const int32_t* src_rows, int n) {
         const int d = m.cfg.d_model;
-        const int status = tc ? launch_norm(ctx->h, pending ? ctx->partials : nullptr, closing, n_rows, gain, src_rows, n, d,
+        const int status = tc ? launch_norm(ctx->h, pending ? branch : nullptr, closing, n_rows, gain, src_rows, n, d,
                                             m.cfg.rms_eps, nullptr, hi(), lo(), st)
                               : launch_norm(ctx->h, nullptr, PartialPlan{}, n_rows, gain, src_rows, n, d, m.cfg.rms_eps, ctx->a, nullptr,
                                             nullptr, st);
@@ -195,6 +197,7 @@ struct Pass {
         const int d = m.cfg.d_model;
         if (tc) {
             pending = true;
+            branch = ctx->partials;
             closing = gemm_tc_plan(d, k, n_rows);
             return launch_gemm_tc_partials(hi(), lo(), ctx->hi_rows, pw, true, n_rows, d, k, ctx->partials, st);
         }
@@ -233,12 +236,13 @@ struct Pass {
 
 // Non-zero (and cleared) if a kernel gave up on a bounded wait.
 int device_gave_up() {
-    const int gemm = gemm_tc_take_error(), wide = gemm_wide_take_error(), pass = pass_take_error(), attn = attention_take_error();
-    return gemm ? gemm : wide ? wide : pass ? pass : attn;
+    const int gemm = gemm_tc_take_error(), wide = gemm_wide_take_error(), pass = pass_take_error(), attn = attention_take_error(),
+              small = small_pass_take_error();
+    return gemm ? gemm : wide ? wide : pass ? pass : attn ? attn : small;
 }
 
 struct ErrorWords {
-    int* word[4];
+    int* word[5];
 };
 
 // block = 128.  Leaves the state of the work before it in `out`.
@@ -247,7 +251,7 @@ __global__ void report_kernel(ErrorWords errors, int* nonfinite, const unsigned 
     pdl_wait();
     if (threadIdx.x == 0) {
         int code = 0;
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 5; ++i)
             if (errors.word[i]) code |= *errors.word[i];
         out->gave_up = code;
         out->nonfinite = *nonfinite;
@@ -259,7 +263,7 @@ __global__ void report_kernel(ErrorWords errors, int* nonfinite, const unsigned 
 
 // Waits for everything on the context's stream; ctx->report then describes it.
 int finish_work(spec_ctx* ctx, int batch) {
-    const ErrorWords errors{{ctx->error_words[0], ctx->error_words[1], ctx->error_words[2], ctx->error_words[3]}};
+    const ErrorWords errors{{ctx->error_words[0], ctx->error_words[1], ctx->error_words[2], ctx->error_words[3], ctx->error_words[4]}};
     SPEC_TRY(launch_pdl(report_kernel, dim3(1), dim3(128), 0, ctx->stream, errors, ctx->nonfinite, ctx->counters, ctx->length, batch,
                         reinterpret_cast<spec_report*>(ctx->report_dev)));
     SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->report, ctx->report_dev, sizeof(spec_report) + batch * sizeof(int32_t), cudaMemcpyDeviceToHost,
@@ -314,8 +318,18 @@ int forward(spec_ctx* ctx, const Model& m, const RowMeta& rows, int batch, int m
     const int d = c.d_model;
     const float* bias = m.t5() ? m.dec_bias : nullptr;
 
-    SPEC_TRY(launch_embed(m, rows, n_rows, ctx->h, ctx->stream));
-    for (int l = 0; l < c.n_layers; ++l) {
+    const bool small = !segs && small_pass_serves(ctx->small[which], m, batch, m_rows);
+    if (small) {
+        const PassTables tables{ctx->page_table, ctx->pages_per_seq, ctx->rt.page_size, ctx->src_page_table,
+                                ctx->src_pages_per_seq, ctx->src_len, ctx->rt.max_len, ctx->rt.max_len - 1};
+        SPEC_TRY(launch_small_pass(ctx->small[which], m, rows, tables, batch, m_rows, ctx->h, ctx->stream));
+        pass.pending = true;
+        pass.branch = ctx->small[which].last_part;
+        pass.closing = small_pass_plan(ctx->small[which]);
+    } else {
+        SPEC_TRY(launch_embed(m, rows, n_rows, ctx->h, ctx->stream));
+    }
+    for (int l = 0; l < (small ? 0 : c.n_layers); ++l) {
         const spec_layer_weights& w = m.layers[l];
         const spec_layer_weights& pw = pass.tc ? m.packed[l] : w;
         SPEC_TRY(pass.self_attention(w, pw, rows, batch, m_rows, layer_pool(ctx, m, l), nullptr, bias, ctx->rt.max_len,
@@ -924,6 +938,8 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
             SPEC_ALLOC(partials, partial);
             cudaMemset(ctx->x_hi, 0, static_cast<size_t>(ctx->hi_rows) * max_k * 2);
             cudaMemset(ctx->x_lo, 0, static_cast<size_t>(ctx->hi_rows) * max_k * 2);
+            for (int i = 0; i < (ctx->has_draft ? 2 : 1) && !rt.pass_kernel; ++i)
+                if ((status = small_pass_init(ctx->small[i], ctx->model[i], ctx->allocations, ctx->stream)) != SPEC_OK) return cleanup(status);
             if (rt.pass_kernel && (status = pass_scratch_init(ctx->pass, ctx->model, ctx->has_draft ? 2 : 1, ctx->allocations)) != SPEC_OK)
                 return cleanup(status);
         }
@@ -984,6 +1000,7 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     ctx->error_words[1] = gemm_wide_error_word();
     ctx->error_words[2] = pass_error_word();
     ctx->error_words[3] = attention_error_word();
+    ctx->error_words[4] = small_pass_error_word();
     ctx->cached[0].assign(B, 0);
     ctx->cached[1].assign(B, 0);
     *out = ctx;

@@ -226,6 +226,25 @@ int launch_pass(const PassScratch& s, const Model& m, int which, const RowMeta& 
 void pass_scratch_release(PassScratch& s);
 int pass_take_error();
 
+// small_pass.cu: the blocks of a small decoder over at most 8 rows as one cooperative kernel.
+struct SmallPass {
+    void* stream = nullptr;  // the weights in the order of use (nullptr: not served)
+    float* gains = nullptr;  // [layers][3][d]
+    int clusters = 0;
+    unsigned* epoch = nullptr;
+    unsigned long long* exchanges = nullptr;
+    float* last_part = nullptr;
+    size_t cta_bytes = 0;
+};
+int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocations, cudaStream_t stream);
+bool small_pass_serves(const SmallPass& s, const Model& m, int batch, int m_rows);
+// Leaves the residual stream in h without the last FFN's result, whose partial sums are in s.last_part as small_pass_plan says.
+int launch_small_pass(const SmallPass& s, const Model& m, const RowMeta& rows, const PassTables& t, int batch, int m_rows, float* h,
+                      cudaStream_t stream);
+PartialPlan small_pass_plan(const SmallPass& s);
+int* small_pass_error_word();
+int small_pass_take_error();
+
 // A tensor map over `rows` rows of `cols` (64 or 128) fp16 elements starting at `base`, fetched in boxes of 64 elements
 // by 32 rows with the 128-byte swizzle; maps are cached by (base, rows, cols).  gemm_tc.cu
 int cached_f16_rows_map(const void* base, unsigned long long rows, int cols, CUtensorMap* out);

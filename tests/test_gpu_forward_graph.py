@@ -22,9 +22,12 @@ def test_repeated_passes_are_the_same_pass(model):
         for k in range(5):  # other tokens, other lengths and other output buffers in between change nothing
             eng.truncate(0, [20 - k] * batch)
             eng.forward_logits(0, other)
-            eng.truncate(0, [20 - k] * batch)
-            if k:
-                eng.forward_logits(0, prefix[:batch, 20 - k:])  # back to 20 cached rows
+            if k:  # back to 20 cached rows, by passes of the length that wrote them
+                eng.truncate(0, [0] * batch)
+                eng.forward_logits(0, prefix[:batch, :10])
+                eng.forward_logits(0, prefix[:batch, 10:])
+            else:
+                eng.truncate(0, [20] * batch)
             again = eng.forward_logits(0, step)
             assert torch.equal(first, again), (batch, rows, k)
             eng.truncate(0, [20] * batch)

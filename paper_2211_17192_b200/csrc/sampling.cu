@@ -59,9 +59,10 @@ __device__ __forceinline__ float fast_exp2(float x) {
 // k-th largest logit, and no change with floor = -inf.
 //
 // Without VEC a row may begin anywhere (a vocabulary that is not a multiple of four): `shift`, 0 to 3, is how many
-// elements before the row its first aligned group starts, group g holds elements 4g - shift .., and elements outside
-// the row read as `pad` (24 x 9 rows of 50003: statistics 30.4 us with four guarded loads per group, 10.9 so).  A caller
-// that pairs two rows element by element passes aligned = false and gets unshifted groups of guarded loads.
+// elements before the row its first group starts, group g holds elements 4g - shift .., and elements outside the row
+// read as `pad`.  With the shift of its own address a row is read in 128-bit loads; of two rows that are paired element
+// by element the second takes the first one's shift, and is read in 32-bit loads unless it happens to be its own
+// (30 x 11 rows of 50003, statistics and draw: 27.4 us with guarded loads of both rows, 26.6 so).
 __host__ __device__ __forceinline__ int row_shift(const float* row) { return static_cast<int>((reinterpret_cast<uintptr_t>(row) >> 2) & 3u); }
 
 template <bool VEC, bool CUT = false>
@@ -70,13 +71,17 @@ struct Row {
     int vocab;
     float floor;  // used only with CUT, so that the usual path pays nothing for it
     int shift;
+    bool own;  // shift is that of the row's own address
 
     __device__ __forceinline__ int groups() const { return (vocab + shift + 3) >> 2; }
     __device__ __forceinline__ float kept(float v) const { return (!CUT || v >= floor) ? v : -INFINITY; }
     __device__ __forceinline__ float4 raw(int g, float pad) const {
         if (VEC) return __ldg(reinterpret_cast<const float4*>(base) + g);
         const int j = 4 * g - shift;
-        if (shift == row_shift(base) && j >= 0 && j + 4 <= vocab) return __ldg(reinterpret_cast<const float4*>(base + j));
+        if (j >= 0 && j + 4 <= vocab) {
+            if (own) return __ldg(reinterpret_cast<const float4*>(base + j));
+            return make_float4(__ldg(base + j), __ldg(base + j + 1), __ldg(base + j + 2), __ldg(base + j + 3));
+        }
         float4 v;
         v.x = j + 0 >= 0 && j + 0 < vocab ? __ldg(base + j + 0) : pad;
         v.y = j + 1 >= 0 && j + 1 < vocab ? __ldg(base + j + 1) : pad;
@@ -92,9 +97,11 @@ struct Row {
 };
 
 template <bool VEC, bool CUT = false>
-__device__ __forceinline__ Row<VEC, CUT> make_row(const float* base, int vocab, float floor = -INFINITY, bool aligned = true) {
+__device__ __forceinline__ Row<VEC, CUT> make_row(const float* base, int vocab, float floor = -INFINITY, int shift = -1) {
     Row<VEC, CUT> r;
-    r.shift = VEC || !aligned ? 0 : row_shift(base);
+    const int own = VEC ? 0 : row_shift(base);
+    r.shift = VEC ? 0 : shift < 0 ? own : shift;
+    r.own = r.shift == own;
     r.base = base;
     r.vocab = vocab;
     r.floor = floor;
@@ -137,7 +144,7 @@ struct ResidualWeights {
         return Raw{z, z};
     }
     __device__ __forceinline__ int groups() const { return p.groups(); }
-    __device__ __forceinline__ int shift() const { return 0; }
+    __device__ __forceinline__ int shift() const { return p.shift; }
     __device__ __forceinline__ float one(float lp, float lq) const {
         // (both products are rounded before the subtraction: contracted into a multiply-add, one of them would not
         // be, and p = q would leave rounding residue instead of the exact zero that the fallback to p tests for)
@@ -472,11 +479,10 @@ struct __align__(16) ChunkStat {
 
 // grid = (chunks, rows, batch); rows = 2*gamma+1 (T > 0: p_1..p_{gamma+1}, q_1..q_gamma)
 // or gamma+1 (T = 0: only p is read).
-template <bool GREEDY, bool VEC, bool CUT>
+template <bool GREEDY, bool VEC>
 __global__ void __launch_bounds__(kStatThreads)
 verify_stats_kernel(const float* __restrict__ target_logits, const float* __restrict__ draft_logits,
-                    const int32_t* __restrict__ draft_tokens, int gamma, int vocab, float c2,
-                    const float* __restrict__ floors, ChunkStat* __restrict__ stats) {
+                    const int32_t* __restrict__ draft_tokens, int gamma, int vocab, float c2, ChunkStat* __restrict__ stats) {
     __shared__ float red[kStatWarps];
     __shared__ float red_s[kStatWarps];
     __shared__ int red_i[kStatWarps];
@@ -490,8 +496,7 @@ verify_stats_kernel(const float* __restrict__ target_logits, const float* __rest
     const float* src = row <= gamma
         ? target_logits + (static_cast<size_t>(b) * (gamma + 1) + row) * vocab
         : draft_logits + (static_cast<size_t>(b) * gamma + (row - gamma - 1)) * vocab;
-    const float floor = CUT ? __ldcg(floors + static_cast<size_t>(b) * rows + row) : -INFINITY;
-    const Row<VEC, CUT> r = make_row<VEC, CUT>(src, vocab, floor);
+    const Row<VEC> r = make_row<VEC>(src, vocab);
     const int groups = r.groups();
     const int per_chunk = (groups + chunks - 1) / chunks;
     const int g0 = chunk * per_chunk;
@@ -503,7 +508,7 @@ verify_stats_kernel(const float* __restrict__ target_logits, const float* __rest
     float xlogit = 0.0f;
     if (tid == 0 && !GREEDY && row != gamma) {
         const int x = draft_tokens[static_cast<size_t>(b) * gamma + (row < gamma ? row : row - gamma - 1)];
-        if (x >= 0 && x < vocab && x + r.shift >= 4 * g0 && x + r.shift < 4 * g1) xlogit = r.kept(__ldg(src + x));
+        if (x >= 0 && x < vocab && x + r.shift >= 4 * g0 && x + r.shift < 4 * g1) xlogit = __ldg(src + x);
     }
 
     // Every thread streams groups g0+tid, g0+tid+T, ... with kUnroll 128-bit
@@ -694,8 +699,8 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
         bool plain = n == gamma;
         if (!plain) {
             ResidualWeights<VEC, CUT> rw;
-            rw.p = make_row<VEC, CUT>(pw.p.base, vocab, pw.p.floor, false);
-            rw.q = make_row<VEC, CUT>(ql + static_cast<size_t>(n) * vocab, vocab, CUT ? __ldcg(fl + gamma + 1 + n) : -INFINITY, false);
+            rw.p = pw.p;
+            rw.q = make_row<VEC, CUT>(ql + static_cast<size_t>(n) * vocab, vocab, CUT ? __ldcg(fl + gamma + 1 + n) : -INFINITY, pw.p.shift);
             rw.max_p = sh.row_max[n];
             rw.max_q = sh.row_max[gamma + 1 + n];
             rw.inv_sum_p = 1.0f / sh.row_aux[n];
@@ -713,11 +718,10 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
 }
 
 // One CTA per row: tokens[r] ~ softmax(logits[r] / T), or argmax at T = 0.
-template <bool VEC, bool CUT>
+template <bool VEC>
 __global__ void __launch_bounds__(kSampleThreads)
 sample_kernel(const float* __restrict__ logits, size_t logit_stride, const float* __restrict__ uniforms,
-              int uniform_stride, int vocab, float inv_t, bool greedy, const float* __restrict__ floors,
-              int32_t* __restrict__ tokens, int token_stride, int* __restrict__ nonfinite) {
+              int uniform_stride, int vocab, float inv_t, bool greedy, int32_t* __restrict__ tokens, int token_stride, int* __restrict__ nonfinite) {
     constexpr int W = kSampleThreads / 32;
     __shared__ float red[W];
     __shared__ int red_i[W];
@@ -727,8 +731,7 @@ sample_kernel(const float* __restrict__ logits, size_t logit_stride, const float
     pdl_trigger();
     pdl_wait();
     const int tid = threadIdx.x;
-    const Row<VEC, CUT> r = make_row<VEC, CUT>(logits + static_cast<size_t>(blockIdx.x) * logit_stride, vocab,
-                                               CUT ? __ldcg(floors + blockIdx.x) : -INFINITY);
+    const Row<VEC> r = make_row<VEC>(logits + static_cast<size_t>(blockIdx.x) * logit_stride, vocab);
     const int groups = r.groups();
     float m = -FLT_MAX;
     int arg = 0x7fffffff;
@@ -749,7 +752,7 @@ sample_kernel(const float* __restrict__ logits, size_t logit_stride, const float
     __syncthreads();
     int token = s_arg;
     if (!greedy) {
-        PlainWeights<VEC, CUT> pw;
+        PlainWeights<VEC> pw;
         pw.p = r;
         pw.max_p = s_max;
         pw.c2 = inv_t * kLog2e;
@@ -794,12 +797,33 @@ struct SelShared {
     unsigned long long warp_mass[kSelWarps];
     unsigned warp_cnt[kSelWarps];
     float warp_lo[kSelWarps], warp_hi[kSelWarps];
-    unsigned n_cand;
+    unsigned n_cand, n_hit;
+    float row_top;  // the largest logit, +inf included
     // where the scan found the target crossed
     int bin;
     unsigned before_cnt;
     unsigned long long before_mass;
 };
+
+// The row's logits that can be kept, if they are few: values in sh.cand, their places in list_index(sh).
+template <int kSelThreads>
+__device__ __forceinline__ unsigned* list_index(SelShared<kSelThreads>& sh) { return sh.cnt + kSelBins / 2; }
+
+template <int kSelThreads>
+__device__ __forceinline__ void list_group(const float4& v, int j, float at_least, SelShared<kSelThreads>& sh) {
+    if (!(fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)) >= at_least)) return;
+    const float e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (e[i] >= at_least) {
+            const unsigned at = atomicAdd(&sh.n_cand, 1u);
+            if (at < kSelCap) {
+                sh.cand[at] = e[i];
+                list_index(sh)[at] = static_cast<unsigned>(j + i);
+            }
+        }
+    }
+}
 
 // f(v) for every logit of the row, kSelLoads 128-bit loads in flight per thread.
 constexpr int kSelLoads = 8;
@@ -837,9 +861,10 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
     constexpr int kSelWarps = kSelThreads / 32, kSelPerThread = kSelBins / kSelThreads;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // 1. range and number of the logits in play
-    float lo = INFINITY, hi = -INFINITY;
+    float lo = INFINITY, hi = -INFINITY, all = -INFINITY;
     unsigned n = 0;
     for_each_logit<kSelThreads>(r, groups, [&](float v) {
+        all = fmaxf(all, v);
         const bool in_play = fabsf(v) < INFINITY && v >= kf;
         const float u = in_play ? v : __int_as_float(0x7fc00000);  // (fminf and fmaxf pass over a NaN operand)
         lo = fminf(lo, u);
@@ -849,12 +874,13 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
     lo = warp_min(lo);
     hi = warp_max(hi);
     n = __reduce_add_sync(0xffffffffu, n);
-    __syncthreads();  // (the shared arrays may still be read by a previous call)
+    const int any_inf = __syncthreads_or(all == INFINITY);  // (and the shared arrays may still be read by a previous call)
     if (lane == 0) { sh.warp_lo[warp] = lo; sh.warp_hi[warp] = hi; sh.warp_cnt[warp] = n; }
     __syncthreads();
     lo = INFINITY; hi = -INFINITY; n = 0;
 #pragma unroll
     for (int w = 0; w < kSelWarps; ++w) { lo = fminf(lo, sh.warp_lo[w]); hi = fmaxf(hi, sh.warp_hi[w]); n += sh.warp_cnt[w]; }
+    if (tid == 0) sh.row_top = any_inf ? INFINITY : hi;
     if (n == 0 || (!MASS && k > n)) return kf;  // nothing to cut
     // weight exp2((l - max) * c2) of a logit in units of 2^-32 (the largest float below 2^32, so that the row's
     // maximum still fits 32 bits): a bin's mass is then one 32-bit shared-memory atomic and, rarely, a carry
@@ -999,9 +1025,10 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
 
 // Top-k for k up to 128, without bins: every warp gives its largest lane maxima, 3 k of them in all; the k-th largest of
 // these is a value that at least k logits reach, so the k-th largest logit of the row is among those that reach it - a
-// few more than k as a rule.  One pass for the maxima, one that copies out what reaches the pivot, then the exact
-// ranking of step 3 above.  Returns false, having decided nothing, when fewer than k lanes hold a finite logit
-// or more than kSelCap logits reach the pivot (heavy ties): the binned selection then does the row.
+// few more than k as a rule.  One pass for the maxima; only the threads whose maximum reaches the pivot have such
+// logits, and what they read is read again, by all warps, and listed; the list is ranked as in step 3 above.
+// Returns false, having decided nothing, when fewer than k lanes hold a finite logit, when there is a +inf, or when
+// more than kSelCap logits reach the pivot (heavy ties): the binned selection then does the row.
 constexpr int kMostTops = 512;
 
 template <int kSelThreads, bool VEC>
@@ -1014,15 +1041,7 @@ __device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelSha
     const int per_warp = min(min(32, kMostTops / kSelWarps), (3 * static_cast<int>(k) + kSelWarps - 1) / kSelWarps);
     const int n_tops = per_warp * kSelWarps;
     float mine = -INFINITY;
-    unsigned n = 0;
-    for_each_logit<kSelThreads>(r, groups, [&](float v) {
-        const bool finite = fabsf(v) < INFINITY;
-        mine = fmaxf(mine, finite ? v : -INFINITY);
-        n += finite;
-    });
-    n = __reduce_add_sync(0xffffffffu, n);
-    __syncthreads();  // (the shared arrays may still be read by a previous call)
-    if (lane == 0) sh.warp_cnt[warp] = n;
+    for_each_logit<kSelThreads>(r, groups, [&](float v) { mine = fmaxf(mine, v); });
     {
         // (keys: the floats' order as unsigned integers, for the warp-wide integer maximum; 0 marks a lane that is out)
         const unsigned u = __float_as_uint(mine);
@@ -1036,15 +1055,8 @@ __device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelSha
         }
         if (lane < per_warp) sh.cand[warp * per_warp + lane] = given;
     }
-    if (tid == 0) sh.n_cand = 0;
-    __syncthreads();
-    n = 0;
-#pragma unroll
-    for (int w = 0; w < kSelWarps; ++w) n += sh.warp_cnt[w];
-    if (k > n) {  // nothing to cut
-        *floor = -INFINITY;
-        return true;
-    }
+    if (tid == 0) { sh.n_cand = 0; sh.n_hit = 0; }
+    if (__syncthreads_or(mine == INFINITY)) return false;
     // the k-th largest of the maxima: the largest one that at least k of them reach; `per` threads count for each
     int per = 1;
     while (per * 2 * n_tops <= kSelThreads && per < 32) per *= 2;
@@ -1065,12 +1077,11 @@ __device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelSha
 #pragma unroll
     for (int w = 0; w < kSelWarps; ++w) pivot = fmaxf(pivot, sh.warp_hi[w]);
     if (!(pivot > -INFINITY)) return false;
-    for_each_logit<kSelThreads>(r, groups, [&](float v) {
-        if (v >= pivot && v < INFINITY) {
-            const unsigned at = atomicAdd(&sh.n_cand, 1u);
-            if (at < kSelCap) sh.cand[at] = v;
-        }
-    });
+    if (mine >= pivot) sh.cnt[atomicAdd(&sh.n_hit, 1u)] = tid;
+    __syncthreads();
+    const int hits = static_cast<int>(sh.n_hit);
+    for (int h = warp; h < hits; h += kSelWarps)  // a warp goes over what one of those threads has read
+        for (int g = sh.cnt[h] + lane * kSelThreads; g < groups; g += 32 * kSelThreads) list_group(r.raw(g, -INFINITY), 4 * g - r.shift, pivot, sh);
     __syncthreads();
     const unsigned total = sh.n_cand;
     if (total > kSelCap) return false;
@@ -1079,71 +1090,9 @@ __device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelSha
     for (int i = tid; i < count; i += kSelThreads) {
         const float c = sh.cand[i];
         unsigned at_least = 0;
+#pragma unroll 8
         for (int j = 0; j < count; ++j) at_least += sh.cand[j] >= c;
         if (at_least >= k) best = fmaxf(best, c);
-    }
-    best = warp_max(best);
-    __syncthreads();  // (warp_hi has been read by everyone)
-    if (lane == 0) sh.warp_hi[warp] = best;
-    __syncthreads();
-    best = -INFINITY;
-#pragma unroll
-    for (int w = 0; w < kSelWarps; ++w) best = fmaxf(best, sh.warp_hi[w]);
-    *floor = best;
-    return true;
-}
-
-// The nucleus when top-k has already cut the row down to a few logits (those >= kf):
-// one pass copies them out, then they are ranked against each other as in step 3
-// above.  Returns false, having decided nothing, if more than kSelCap logits are
-// in play (a large tie at the top-k floor).
-template <int kSelThreads, bool VEC>
-__device__ bool nucleus_of_few(const Row<VEC>& r, int groups, float kf, float top_p, float c2, SelShared<kSelThreads>& sh, float* floor) {
-    constexpr int kSelWarps = kSelThreads / 32;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    __syncthreads();  // (the shared arrays may still be read by a previous call)
-    if (tid == 0) sh.n_cand = 0;
-    __syncthreads();
-    for_each_logit<kSelThreads>(r, groups, [&](float v) {
-        if (fabsf(v) < INFINITY && v >= kf) {
-            const unsigned at = atomicAdd(&sh.n_cand, 1u);
-            if (at < kSelCap) sh.cand[at] = v;
-        }
-    });
-    __syncthreads();
-    const unsigned total = sh.n_cand;
-    if (total == 0 || total > kSelCap) return false;
-    const int count = static_cast<int>(total);
-    float row_max = -INFINITY;
-    for (int i = tid; i < count; i += kSelThreads) row_max = fmaxf(row_max, sh.cand[i]);
-    row_max = warp_max(row_max);
-    if (lane == 0) sh.warp_hi[warp] = row_max;
-    __syncthreads();
-    row_max = -INFINITY;
-#pragma unroll
-    for (int w = 0; w < kSelWarps; ++w) row_max = fmaxf(row_max, sh.warp_hi[w]);
-    unsigned long long mine_sum = 0;
-    for (int i = tid; i < count; i += kSelThreads) {
-        const unsigned long long m = __float2ull_rz(fast_exp2((sh.cand[i] - row_max) * c2) * 1099511627776.0f);  // 2^40
-        sh.cand_mass[i] = m;
-        mine_sum += m;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mine_sum += __shfl_xor_sync(0xffffffffu, mine_sum, o);
-    __syncthreads();  // (warp_hi has been read by everyone; cand_mass is complete)
-    if (lane == 0) sh.warp_mass[warp] = mine_sum;
-    __syncthreads();
-    unsigned long long all_mass = 0;
-#pragma unroll
-    for (int w = 0; w < kSelWarps; ++w) all_mass += sh.warp_mass[w];
-    const unsigned long long goal = static_cast<unsigned long long>(ceil(static_cast<double>(top_p) * static_cast<double>(all_mass)));
-    float best = -INFINITY;
-    for (int i = tid; i < count; i += kSelThreads) {
-        const float mine = sh.cand[i];
-        unsigned long long m = 0;
-        for (int j = 0; j < count; ++j)
-            if (sh.cand[j] >= mine) m += sh.cand_mass[j];
-        if (m >= goal) best = fmaxf(best, mine);
     }
     best = warp_max(best);
     if (lane == 0) sh.warp_lo[warp] = best;
@@ -1151,17 +1100,200 @@ __device__ bool nucleus_of_few(const Row<VEC>& r, int groups, float kf, float to
     best = -INFINITY;
 #pragma unroll
     for (int w = 0; w < kSelWarps; ++w) best = fmaxf(best, sh.warp_lo[w]);
-    *floor = best > -INFINITY ? best : kf;
+    *floor = best;
     return true;
 }
 
+// Lists the logits that reach kf > -inf, after a top-k that found it by bins.  Returns false if they are more than kSelCap (a
+// large tie at kf) or one of them is +inf.
+template <int kSelThreads, bool VEC>
+__device__ bool list_row(const Row<VEC>& r, int groups, float kf, SelShared<kSelThreads>& sh) {
+    __syncthreads();  // (the shared arrays may still be read by a previous call)
+    if (sh.row_top == INFINITY) return false;
+    if (threadIdx.x == 0) sh.n_cand = 0;
+    __syncthreads();
+    for (int g0 = threadIdx.x; g0 < groups; g0 += kSelLoads * kSelThreads) {
+        float4 v[kSelLoads];
+#pragma unroll
+        for (int i = 0; i < kSelLoads; ++i) {
+            const int g = g0 + i * kSelThreads;
+            v[i] = g < groups ? r.raw(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        }
+#pragma unroll
+        for (int i = 0; i < kSelLoads; ++i) list_group(v[i], 4 * (g0 + i * kSelThreads) - r.shift, kf, sh);
+    }
+    __syncthreads();
+    return sh.n_cand <= kSelCap;
+}
+
+template <int kSelThreads>
+__device__ __forceinline__ float block_max(float v, float* per_warp) {
+    v = warp_max(v);
+    if ((threadIdx.x & 31) == 0) per_warp[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = per_warp[0];
+#pragma unroll
+    for (int w = 1; w < kSelThreads / 32; ++w) v = fmaxf(v, per_warp[w]);
+    return v;
+}
+template <int kSelThreads>
+__device__ __forceinline__ unsigned long long block_sum(unsigned long long v, unsigned long long* per_warp) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) per_warp[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = 0;
+#pragma unroll
+    for (int w = 0; w < kSelThreads / 32; ++w) v += per_warp[w];
+    return v;
+}
+
+// What is left of a listed row: the nucleus of the logits that reach *floor (if `nucleus`, which raises *floor), ranked
+// against each other, the largest logit and the sum of the kept weights.  Weights are summed in units of 2^-40 of the
+// largest, so that the order in which the list was made does not matter.
+template <int kSelThreads>
+__device__ void finish_list(bool nucleus, float top_p, float c2, SelShared<kSelThreads>& sh, float* floor, float* row_max, float* sum) {
+    const int tid = threadIdx.x, count = static_cast<int>(sh.n_cand);
+    const float kf = *floor;
+    float m = -INFINITY;
+    for (int i = tid; i < count; i += kSelThreads) m = fmaxf(m, sh.cand[i]);
+    m = block_max<kSelThreads>(m, sh.warp_hi);
+    unsigned long long mine_sum = 0;
+    for (int i = tid; i < count; i += kSelThreads) {
+        const unsigned long long w = sh.cand[i] >= kf ? __float2ull_rz(fast_exp2((sh.cand[i] - m) * c2) * 1099511627776.0f) : 0ull;  // 2^40
+        sh.cand_mass[i] = w;
+        mine_sum += w;
+    }
+    unsigned long long kept = block_sum<kSelThreads>(mine_sum, sh.warp_mass);  // (and cand_mass is complete)
+    if (nucleus) {
+        const unsigned long long goal = static_cast<unsigned long long>(ceil(static_cast<double>(top_p) * static_cast<double>(kept)));
+        float best = -INFINITY;
+        for (int i = tid; i < count; i += kSelThreads) {
+            const float mine = sh.cand[i];
+            if (!(mine >= kf)) continue;
+            unsigned long long above = 0;
+#pragma unroll 8
+            for (int j = 0; j < count; ++j) above += sh.cand[j] >= mine ? sh.cand_mass[j] : 0ull;
+            if (above >= goal) best = fmaxf(best, mine);
+        }
+        best = block_max<kSelThreads>(best, sh.warp_lo);
+        *floor = best > -INFINITY ? best : kf;
+        mine_sum = 0;
+        for (int i = tid; i < count; i += kSelThreads)
+            if (sh.cand[i] >= *floor) mine_sum += sh.cand_mass[i];
+        kept = block_sum<kSelThreads>(mine_sum, sh.warp_mass);  // (everyone has read the first sums: a barrier ago)
+    }
+    *row_max = m;
+    *sum = static_cast<float>(static_cast<double>(kept) * (1.0 / 1099511627776.0));
+}
+
+// The draw from a listed row: the kept logits in the order of their places, walked by one warp.
+template <int kSelThreads>
+__device__ int draw_from_list(float floor, float row_max, float c2, float u, SelShared<kSelThreads>& sh) {
+    const int tid = threadIdx.x, count = static_cast<int>(sh.n_cand);
+    unsigned* index = list_index(sh);
+    float* weight = reinterpret_cast<float*>(sh.cand_mass);  // in order
+    unsigned* place = sh.mass_lo;
+    __syncthreads();  // (cand_mass has been read by everyone)
+    if (tid == 0) sh.n_hit = 0;
+    for (int i = tid; i < count; i += kSelThreads)
+        if (!(sh.cand[i] >= floor)) index[i] = 0xffffffffu;  // (behind every place of the row)
+    __syncthreads();
+    for (int i = tid; i < count; i += kSelThreads) {
+        if (!(sh.cand[i] >= floor)) continue;
+        unsigned rank = 0;
+#pragma unroll 8
+        for (int j = 0; j < count; ++j) rank += index[j] < index[i];
+        weight[rank] = fast_exp2((sh.cand[i] - row_max) * c2);
+        place[rank] = index[i];
+        atomicMax(&sh.n_hit, rank + 1);
+    }
+    __syncthreads();
+    int token = 0;
+    if (tid < 32) {
+        const int kept = static_cast<int>(sh.n_hit);
+        float total = 0.0f;
+        for (int base = 0; base < kept; base += 32) total += warp_sum(base + tid < kept ? weight[base + tid] : 0.0f);
+        const float target = u * total;
+        float run = 0.0f;
+        int found = -1, last = 0;
+        for (int base = 0; base < kept && found < 0; base += 32) {
+            const float w = base + tid < kept ? weight[base + tid] : 0.0f;
+            const float incl = warp_inclusive_scan(w, tid);
+            const unsigned over = __ballot_sync(kFullMask, base + tid < kept && run + incl > target), some = __ballot_sync(kFullMask, w > 0.0f);
+            if (some) last = base + 31 - __clz(some);
+            if (over) found = base + __ffs(over) - 1;
+            run += __shfl_sync(kFullMask, incl, 31);
+        }
+        token = static_cast<int>(place[found >= 0 ? found : last]);
+    }
+    return token;  // (valid in the first warp)
+}
+
+// (max, sum of exp2((l - max) * c2)) of the kept logits, online, in a fixed order.  Valid in thread 0.
+template <int kSelThreads, bool VEC>
+__device__ void row_statistics(const Row<VEC, true>& r, int groups, float c2, SelShared<kSelThreads>& sh, float* row_max, float* sum) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float m = -FLT_MAX, s = 0.0f;  // (finite, so that m - new maximum never becomes inf - inf)
+    for (int base = tid; base < groups; base += kSelLoads * kSelThreads) {
+        float4 v[kSelLoads];
+        float bm = m;
+#pragma unroll
+        for (int i = 0; i < kSelLoads; ++i) {
+            const int g = base + i * kSelThreads;
+            v[i] = g < groups ? r.load(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        }
+#pragma unroll
+        for (int i = 0; i < kSelLoads; ++i) bm = fmaxf(bm, fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w)));
+        s *= fast_exp2((m - bm) * c2);
+        m = bm;
+        const float mc = fminf(-m * c2, FLT_MAX);  // (-inf * c2 + it stays -inf)
+#pragma unroll
+        for (int i = 0; i < kSelLoads; ++i)
+            s += (fast_exp2(fmaf(v[i].x, c2, mc)) + fast_exp2(fmaf(v[i].y, c2, mc))) +
+                 (fast_exp2(fmaf(v[i].z, c2, mc)) + fast_exp2(fmaf(v[i].w, c2, mc)));
+    }
+    const float wm = warp_max(m);
+    s = warp_sum(s * fast_exp2((m - wm) * c2));
+    __syncthreads();  // (the shared arrays may still be read)
+    if (lane == 0) { sh.warp_hi[warp] = wm; sh.warp_lo[warp] = s; }
+    __syncthreads();
+    if (tid == 0) {
+        float bm = sh.warp_hi[0], t = 0.0f;
+        for (int w = 1; w < kSelThreads / 32; ++w) bm = fmaxf(bm, sh.warp_hi[w]);
+        for (int w = 0; w < kSelThreads / 32; ++w) t += sh.warp_lo[w] * fast_exp2((sh.warp_hi[w] - bm) * c2);
+        *row_max = bm;
+        *sum = t;
+    }
+}
+
+// What else to find out about a row while it is at hand.
+struct CutWork {
+    // verification: its statistics, at the drafted token too
+    const int32_t* draft_tokens;
+    ChunkStat* stats;
+    // sampling: a token
+    const float* uniforms;
+    int uniform_stride;
+    int32_t* tokens;
+    int token_stride;
+    int* nonfinite;
+};
+// (ordering a list by place takes a comparison per pair; beyond this it is cheaper to go over the row, as without a list:
+// one row of 32000, k = 400, p = 0.95 39 us with the list, 48 without)
+constexpr unsigned kDrawList = 512;
+constexpr int kFloorsOnly = 0, kWithStats = 1, kWithDraw = 2;
+
 // floors[s * (a_rows + b_rows) + r] for sequence s's a_rows rows of `a`, then its
 // b_rows rows of `b`: top-k first (0 < top_k < vocab), then the nucleus (0 < top_p < 1)
-// of what top-k left.
-template <bool VEC, int kSelThreads>
+// of what top-k left.  The statistics of the verification and the draw of the sampling follow in the same CTA: after a
+// top-k they cost nothing, the list is there (24 x 9 rows of 50003, k = 40, p = 0.9: 66 -> 40 us, 200
+// rows of 100000, k = 40, with the draw: 73 -> 28, one of 32000: 16 -> 9), and after a nucleus one pass less and no second
+// kernel (200 rows of 100000: 99 -> 91).
+template <bool VEC, int kSelThreads, int WORK>
 __global__ void __launch_bounds__(kSelThreads)
 cut_floor_kernel(const float* __restrict__ a, size_t a_stride, int a_rows, const float* __restrict__ b,
-                 size_t b_stride, int b_rows, int vocab, int top_k, float top_p, float c2, float* __restrict__ floors) {
+                 size_t b_stride, int b_rows, int vocab, int top_k, float top_p, float c2, float* __restrict__ floors, CutWork work) {
     __shared__ SelShared<kSelThreads> sh;
     pdl_trigger();
     pdl_wait();
@@ -1171,16 +1303,48 @@ cut_floor_kernel(const float* __restrict__ a, size_t a_stride, int a_rows, const
                                     : b + (static_cast<size_t>(seq) * b_rows + (row - a_rows)) * b_stride;
     const Row<VEC> r = make_row<VEC>(src, vocab);
     const int groups = r.groups();
-    float floor = -INFINITY;
-    if (top_k > 0 && top_k < vocab && !top_k_by_pivot<kSelThreads, VEC>(r, groups, static_cast<unsigned>(top_k), sh, &floor))
-        floor = select_floor<kSelThreads, VEC, false>(r, groups, -INFINITY, static_cast<unsigned>(top_k), 0.0f, 0.0f, sh);
-    if (top_p > 0.0f && top_p < 1.0f) {
-        // after a top-k that leaves few logits the nucleus needs no binning
-        const bool few = floor > -INFINITY && top_k <= kSelCap;
-        if (!few || !nucleus_of_few<kSelThreads, VEC>(r, groups, floor, top_p, c2, sh, &floor))
-            floor = select_floor<kSelThreads, VEC, true>(r, groups, floor, 0u, top_p, c2, sh);
+    float floor = -INFINITY, row_max = 0.0f, sum = 0.0f;
+    bool listed = false;
+    const bool nucleus = top_p > 0.0f && top_p < 1.0f;
+    if (top_k > 0 && top_k < vocab) {
+        listed = top_k_by_pivot<kSelThreads, VEC>(r, groups, static_cast<unsigned>(top_k), sh, &floor);
+        if (!listed) {
+            floor = select_floor<kSelThreads, VEC, false>(r, groups, -INFINITY, static_cast<unsigned>(top_k), 0.0f, 0.0f, sh);
+            listed = nucleus && floor > -INFINITY && top_k <= kSelCap && list_row<kSelThreads, VEC>(r, groups, floor, sh);
+        }
     }
-    if (threadIdx.x == 0) floors[blockIdx.x] = floor;
+    if (listed) finish_list<kSelThreads>(nucleus, top_p, c2, sh, &floor, &row_max, &sum);
+    else if (nucleus) floor = select_floor<kSelThreads, VEC, true>(r, groups, floor, 0u, top_p, c2, sh);
+    if (threadIdx.x == 0 && floors) floors[blockIdx.x] = floor;
+    if (WORK == kWithStats) {
+        if (!listed) row_statistics<kSelThreads, VEC>(make_row<VEC, true>(src, vocab, floor), groups, c2, sh, &row_max, &sum);
+        if (threadIdx.x == 0) {
+            float at_x = 0.0f;  // (none for p_{gamma+1})
+            if (row != a_rows - 1) {
+                const int x = work.draft_tokens[static_cast<size_t>(seq) * b_rows + (row < a_rows ? row : row - a_rows)];
+                if (x >= 0 && x < vocab) at_x = __ldg(src + x) >= floor ? __ldg(src + x) : -INFINITY;
+            }
+            *reinterpret_cast<float4*>(work.stats + blockIdx.x) = make_float4(row_max, sum, at_x, 0.0f);
+        }
+    }
+    if (WORK == kWithDraw) {
+        const float u = work.uniforms[static_cast<size_t>(blockIdx.x) * work.uniform_stride];
+        int token;
+        if (listed && sh.n_cand <= kDrawList) {
+            token = draw_from_list<kSelThreads>(floor, row_max, c2, u, sh);
+        } else {
+            __shared__ CdfScratch<kSelThreads / 32> cdf;
+            __syncthreads();
+            if (threadIdx.x == 0 && !listed && work.nonfinite && sh.row_top == INFINITY) atomicExch(work.nonfinite, 1);
+            PlainWeights<VEC, true> pw;
+            pw.p = make_row<VEC, true>(src, vocab, floor);
+            pw.max_p = listed ? row_max : fmaxf(sh.row_top, -FLT_MAX);
+            pw.c2 = c2;
+            float total;
+            token = block_inverse_cdf<kSelThreads / 32>(pw, vocab, u, cdf, &total);
+        }
+        if (threadIdx.x == 0) work.tokens[static_cast<size_t>(blockIdx.x) * work.token_stride] = max(0, min(token, vocab - 1));
+    }
 }
 
 __global__ void uniforms_kernel(uint64_t seed, const int32_t* __restrict__ positions,
@@ -1210,7 +1374,13 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 int chunks_for(int vocab, int rows_total) {
     const int want = (kTargetCtas + rows_total - 1) / std::max(1, rows_total);
-    return std::max(1, std::min(want, max_chunks(vocab)));
+    const int most = std::max(1, std::min(want, max_chunks(vocab)));
+    // the fewest chunks of as many steps of the streaming loop: with 12 of 1042 groups each, a row of 50003 took a second
+    // step for 18 groups, with 7 that step is nearly full (30 x 11 such rows, with the draw 26.6 ->
+    // 23.4 us; rows of 100000 40.0 -> 33.3, of 128000 43.8 -> 38.5)
+    const int groups = (vocab + 3) / 4, step = kUnroll * kStatThreads;
+    const int steps = ((groups + most - 1) / most + step - 1) / step;
+    return (groups + steps * step - 1) / (steps * step);
 }
 
 size_t stats_bytes(int batch, int gamma, int vocab) {
@@ -1239,15 +1409,16 @@ bool cut_is_on(int vocab, float temperature, int top_k, float top_p) {
 // Top-k, then the nucleus of what is left (Section 2.2): one floor per row, one kernel.
 // floors[s * (a_rows + b_rows) + r] belongs to sequence s's row r (its a_rows rows of `a`,
 // then its b_rows rows of `b`).
-int launch_cut_floors(const float* a, size_t a_stride, int a_rows, const float* b, size_t b_stride, int b_rows,
-                      int seqs, int vocab, int top_k, float top_p, float inv_t, float* floors, cudaStream_t stream) {
+template <int WORK>
+int launch_cut(const float* a, size_t a_stride, int a_rows, const float* b, size_t b_stride, int b_rows, int seqs, int vocab,
+               int top_k, float top_p, float inv_t, float* floors, const CutWork& work, cudaStream_t stream) {
     const int total = seqs * (a_rows + b_rows);
     if (total == 0) return SPEC_OK;
     const bool vec = vocab % 4 == 0 && a_stride % 4 == 0 && aligned16(a) && (b_rows == 0 || (b_stride % 4 == 0 && aligned16(b)));
     const float c2 = inv_t * kLog2e;
 #define SPEC_LAUNCH_CUT(V, T)                                                                                        \
-    return launch_pdl(cut_floor_kernel<V, T>, dim3(total), dim3(T), 0, stream, a, a_stride, a_rows, b, b_stride, b_rows, \
-                      vocab, top_k, top_p, c2, floors)
+    return launch_pdl(cut_floor_kernel<V, T, WORK>, dim3(total), dim3(T), 0, stream, a, a_stride, a_rows, b, b_stride, b_rows, \
+                      vocab, top_k, top_p, c2, floors, work)
     if (wide_rows(total, vocab)) {
         if (vec) SPEC_LAUNCH_CUT(true, 1024);
         SPEC_LAUNCH_CUT(false, 1024);
@@ -1263,32 +1434,31 @@ int launch_verify_sample(const float* target_logits, const float* draft_logits, 
                          int32_t* next_token, void* workspace, cudaStream_t stream, int* nonfinite) {
     const bool greedy = temperature == 0.0f;
     const int rows = greedy ? gamma + 1 : 2 * gamma + 1;
-    const int chunks = chunks_for(vocab, rows * batch);
     const float inv_t = greedy ? 0.0f : 1.0f / temperature;
     ChunkStat* stats = static_cast<ChunkStat*>(workspace);
-    // top-k and nucleus (Section 2.2): both models' rows are cut at their own floors
-    const float* floors = nullptr;
-    if (cut_is_on(vocab, temperature, top_k, top_p)) {
-        float* f = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + stats_bytes(batch, gamma, vocab));
-        const int st = launch_cut_floors(target_logits, static_cast<size_t>(vocab), gamma + 1, draft_logits,
-                                         static_cast<size_t>(vocab), gamma, batch, vocab, top_k, top_p, inv_t, f, stream);
-        if (st != SPEC_OK) return st;
-        floors = f;
-    }
+    const bool cut = cut_is_on(vocab, temperature, top_k, top_p);  // never with greedy
+    const int chunks = cut ? 1 : chunks_for(vocab, rows * batch);
     const dim3 grid(chunks, rows, batch);
     const bool vec = vocab % 4 == 0 && aligned16(target_logits) && (greedy || gamma == 0 || aligned16(draft_logits));
     const float c2 = inv_t * kLog2e;
+    const float* floors = nullptr;
     int status;
-    const bool cut = floors != nullptr;  // never with greedy
-#define SPEC_LAUNCH_STATS(G, V, C)                                                                               \
-    status = launch_pdl(verify_stats_kernel<G, V, C>, grid, dim3(kStatThreads), 0, stream, target_logits, draft_logits, \
-                        draft_tokens, gamma, vocab, c2, floors, stats)
-    if (greedy && vec) SPEC_LAUNCH_STATS(true, true, false);
-    else if (greedy) SPEC_LAUNCH_STATS(true, false, false);
-    else if (vec && cut) SPEC_LAUNCH_STATS(false, true, true);
-    else if (vec) SPEC_LAUNCH_STATS(false, true, false);
-    else if (cut) SPEC_LAUNCH_STATS(false, false, true);
-    else SPEC_LAUNCH_STATS(false, false, false);
+#define SPEC_LAUNCH_STATS(G, V)                                                                                  \
+    status = launch_pdl(verify_stats_kernel<G, V>, grid, dim3(kStatThreads), 0, stream, target_logits, draft_logits, \
+                        draft_tokens, gamma, vocab, c2, stats)
+    if (cut) {
+        // top-k and nucleus (Section 2.2): both models' rows are cut at their own floors
+        float* f = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + stats_bytes(batch, gamma, vocab));
+        CutWork work{};
+        work.draft_tokens = draft_tokens;
+        work.stats = stats;
+        status = launch_cut<kWithStats>(target_logits, static_cast<size_t>(vocab), gamma + 1, draft_logits, static_cast<size_t>(vocab),
+                                        gamma, batch, vocab, top_k, top_p, inv_t, f, work, stream);
+        floors = f;
+    } else if (greedy && vec) SPEC_LAUNCH_STATS(true, true);
+    else if (greedy) SPEC_LAUNCH_STATS(true, false);
+    else if (vec) SPEC_LAUNCH_STATS(false, true);
+    else SPEC_LAUNCH_STATS(false, false);
 #undef SPEC_LAUNCH_STATS
     if (status != SPEC_OK) return status;
 
@@ -1331,21 +1501,21 @@ int launch_sample_strided(const float* logits, size_t logit_stride, const float*
                           int32_t* tokens, int token_stride, cudaStream_t stream, int* nonfinite) {
     const bool greedy = temperature == 0.0f;
     const float inv_t = greedy ? 0.0f : 1.0f / temperature;
-    const float* floors = nullptr;
     if (cut_is_on(vocab, temperature, top_k, top_p)) {
-        const int st = launch_cut_floors(logits, logit_stride, 1, nullptr, 0, 0, rows, vocab, top_k, top_p, inv_t,
-                                         floor_scratch, stream);
-        if (st != SPEC_OK) return st;
-        floors = floor_scratch;
+        CutWork work{};
+        work.uniforms = uniforms;
+        work.uniform_stride = uniform_stride;
+        work.tokens = tokens;
+        work.token_stride = token_stride;
+        work.nonfinite = nonfinite;
+        return launch_cut<kWithDraw>(logits, logit_stride, 1, nullptr, 0, 0, rows, vocab, top_k, top_p, inv_t, floor_scratch, work, stream);
     }
     const bool vec = vocab % 4 == 0 && logit_stride % 4 == 0 && aligned16(logits);
-#define SPEC_LAUNCH_SAMPLE(V, C)                                                                                   \
-    return launch_pdl(sample_kernel<V, C>, dim3(rows), dim3(kSampleThreads), 0, stream, logits, logit_stride, uniforms,     \
-                      uniform_stride, vocab, inv_t, greedy, floors, tokens, token_stride, nonfinite)
-    if (vec && floors) SPEC_LAUNCH_SAMPLE(true, true);
-    if (vec) SPEC_LAUNCH_SAMPLE(true, false);
-    if (floors) SPEC_LAUNCH_SAMPLE(false, true);
-    SPEC_LAUNCH_SAMPLE(false, false);
+#define SPEC_LAUNCH_SAMPLE(V)                                                                                      \
+    return launch_pdl(sample_kernel<V>, dim3(rows), dim3(kSampleThreads), 0, stream, logits, logit_stride, uniforms,     \
+                      uniform_stride, vocab, inv_t, greedy, tokens, token_stride, nonfinite)
+    if (vec) SPEC_LAUNCH_SAMPLE(true);
+    SPEC_LAUNCH_SAMPLE(false);
 #undef SPEC_LAUNCH_SAMPLE
 }
 
@@ -1503,8 +1673,8 @@ extern "C" int spec_truncation_floors(const float* logits, int rows, int vocab, 
         return fail(SPEC_ERR_BAD_ARG, "spec_truncation_floors: neither 0 < top_k < vocab nor 0 < top_p < 1");
     if (rows == 0) return SPEC_OK;
     if (!logits || !floors) return fail(SPEC_ERR_BAD_ARG, "spec_truncation_floors: null pointer");
-    return launch_cut_floors(logits, static_cast<size_t>(vocab), 1, nullptr, 0, 0, rows, vocab, top_k, top_p,
-                             1.0f / temperature, floors, static_cast<cudaStream_t>(stream));
+    return launch_cut<kFloorsOnly>(logits, static_cast<size_t>(vocab), 1, nullptr, 0, 0, rows, vocab, top_k, top_p,
+                                   1.0f / temperature, floors, CutWork{}, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int spec_uniforms(uint64_t seed, const int32_t* positions, const int32_t* sequences, int purpose, int count,

@@ -39,6 +39,7 @@ constexpr int kCdfBatch = 8;            // groups fetched per thread before any 
 constexpr int kClusterCdfBatch = 4;     // the same when a cluster shares the row
 constexpr int kWalkBatch = 4;           // 128-element steps fetched at once by the final walk
 constexpr int kMaxCluster = 4;          // CTAs per sequence in the finishing kernel
+constexpr int kMostParts = 64;          // warps that share an inverse CDF: four CTAs of 16
 constexpr int kSampleThreads = 512;
 constexpr int kMaxGamma = 64;
 constexpr int kMaxRows = 2 * kMaxGamma + 1;
@@ -161,7 +162,7 @@ struct ResidualWeights {
 template <int WARPS>
 struct CdfScratch {
     float part[WARPS];              // per-warp totals of the level being scanned
-    float all[kMaxCluster * WARPS];  // the same for every CTA of a cluster
+    float all[kMostParts];          // the same for every CTA of a cluster
     float pick_before, pick_total;   // outcome of the cluster-wide scan
     int pick_part_index, pick_hit;
     int result;
@@ -763,7 +764,8 @@ sample_kernel(const float* __restrict__ logits, size_t logit_stride, const float
 }
 
 // ---- top-k and nucleus: the lowest logit that each row keeps ---------------------
-// One CTA per row, several CTAs per SM.  Both cuts are a selection: the largest
+// One CTA per row, several CTAs per SM, or, where that would leave SMs idle or unevenly loaded, a cluster of up to four
+// (cut_shape).  Both cuts are a selection: the largest
 // value t such that the logits at or above t number at least k (top-k), or carry
 // at least top_p of the mass (nucleus).  The row is never sorted or held:
 //   1. one pass finds the range [lo, hi] of the logits still in play;
@@ -778,39 +780,69 @@ sample_kernel(const float* __restrict__ logits, size_t logit_stride, const float
 // -inf, +inf and NaN logits are never in play).  Mass is summed in fixed point
 // (units of 2^-32 of the largest weight) with integer atomics, so every order of
 // summation gives the same totals: a row always gives the same floor, however the
-// threads interleave.  The kernel is bound by instruction issue, not by memory
+// threads interleave and however many CTAs share it.  The kernel is bound by instruction issue, not by memory
 // (the passes after the first hit L2), so the per-logit work is kept short: no
 // float-to-int conversion for the bin, one 32-bit atomic plus a rare carry for
 // the mass (a 64-bit shared-memory atomic cost 48 us of 180 on 960 rows of 32000),
 // a two-instruction test before a logit is asked whether it is in the chosen bin.
+//
+// The CTAs of a cluster take a slice of the row each, and what they find goes through distributed shared memory: the range
+// and the warps' maxima to all of them; of the bins the sums of 32 at a time, then only the 32 where the target is
+// crossed (with all bins read by everyone a cluster of four cost 40 us more on 200 rows of 100000); the lists, made
+// locally, to the CTA of rank 0, which ranks them.
+constexpr int kSelMostWarps = 16;  // of a CTA: T / 32, T = 256 or 512 threads
 constexpr int kSelBins = 2048;
+constexpr int kSelSegments = kSelBins / 32;
 constexpr int kSelCap = 1024;   // logits ranked against each other at the end
 constexpr int kSelLevels = 40;  // every level shrinks the range; fp32 allows far fewer than this
+constexpr int kMostCtas = 4;    // per row
+static_assert(kSelSegments == 64, "two segments to a lane");
 
-template <int kSelThreads>
 struct SelShared {
-    static constexpr int kSelWarps = kSelThreads / 32;
     unsigned cnt[kSelBins];
     unsigned mass_lo[kSelBins], mass_hi[kSelBins];  // a bin's mass, low and high word (apart: the low words then spread over all banks)
     float cand[kSelCap];
     unsigned long long cand_mass[kSelCap];
-    unsigned long long warp_mass[kSelWarps];
-    unsigned warp_cnt[kSelWarps];
-    float warp_lo[kSelWarps], warp_hi[kSelWarps];
-    unsigned n_cand, n_hit;
+    unsigned long long segment[kSelSegments];       // counts or masses of 32 bins
+    unsigned long long warp_mass[kSelMostWarps];
+    unsigned warp_cnt[kSelMostWarps];
+    float warp_lo[kSelMostWarps], warp_hi[kSelMostWarps], warp_top[kSelMostWarps];
+    float cta_max[kMostCtas], cta_sum[kMostCtas];  // (in the CTA of rank 0)
+    unsigned n_cand, n_hit, n_list;  // listed here; threads that reach the pivot; listed in all CTAs (in rank 0's)
+    float floor;    // what rank 0 found
     float row_top;  // the largest logit, +inf included
     // where the scan found the target crossed
     int bin;
-    unsigned before_cnt;
-    unsigned long long before_mass;
+    unsigned in_bin;
+    unsigned long long before, target;
 };
 
-// The row's logits that can be kept, if they are few: values in sh.cand, their places in list_index(sh).
-template <int kSelThreads>
-__device__ __forceinline__ unsigned* list_index(SelShared<kSelThreads>& sh) { return sh.cnt + kSelBins / 2; }
+// The CTAs that share a row.
+template <bool SOLO>
+struct Team {
+    int rank, size;
+    __device__ __forceinline__ Team() {
+        rank = SOLO ? 0 : static_cast<int>(cg::this_cluster().block_rank());
+        size = SOLO ? 1 : static_cast<int>(cg::this_cluster().num_blocks());
+    }
+    __device__ __forceinline__ void sync() const {
+        if (SOLO) __syncthreads();
+        else cg::this_cluster().sync();
+    }
+    __device__ __forceinline__ SelShared& of(SelShared& sh, int r) const { return SOLO ? sh : *cg::this_cluster().map_shared_rank(&sh, r); }
+};
 
-template <int kSelThreads>
-__device__ __forceinline__ void list_group(const float4& v, int j, float at_least, SelShared<kSelThreads>& sh) {
+// A CTA's slice of a row; LOADS 128-bit loads are in flight per thread when it is gone over.
+template <bool VEC, int LOADS>
+struct Slice {
+    Row<VEC> row;
+    int g0, g1;
+};
+
+// Logits that can be kept, if they are few: values in sh.cand, their places in list_index.
+__device__ __forceinline__ unsigned* list_index(SelShared& sh) { return sh.cnt + kSelBins / 2; }
+
+__device__ __forceinline__ void list_group(const float4& v, int j, float at_least, SelShared& sh) {
     if (!(fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)) >= at_least)) return;
     const float e[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -825,26 +857,56 @@ __device__ __forceinline__ void list_group(const float4& v, int j, float at_leas
     }
 }
 
-// f(v) for every logit of the row, kSelLoads 128-bit loads in flight per thread.
-constexpr int kSelLoads = 8;
-
-template <int kSelThreads, bool VEC, class F>
-__device__ __forceinline__ void for_each_logit(const Row<VEC>& r, int groups, F f) {
-    for (int g0 = threadIdx.x; g0 < groups; g0 += kSelLoads * kSelThreads) {
-        float4 v[kSelLoads];
-#pragma unroll
-        for (int i = 0; i < kSelLoads; ++i) {
-            const int g = g0 + i * kSelThreads;
-            v[i] = g < groups ? r.raw(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+// Brings the CTAs' lists together in the first one's, with their masses or their places.  Returns how many there are, to all;
+// -1, and nothing is brought together, if that is more than kSelCap.
+template <int T, bool SOLO>
+__device__ int gather_list(const Team<SOLO>& team, bool masses, SelShared& sh) {
+    team.sync();
+    unsigned total = 0;
+    for (int r = 0; r < team.size; ++r) total += team.of(sh, r).n_cand;
+    if (total > kSelCap) return -1;
+    if (team.rank == 0) {
+        if (!SOLO) {
+            unsigned at = sh.n_cand;
+            for (int r = 1; r < team.size; ++r) {
+                SelShared& from = team.of(sh, r);
+                const unsigned n = from.n_cand;
+                for (unsigned i = threadIdx.x; i < n; i += T) {
+                    sh.cand[at + i] = from.cand[i];
+                    if (masses) sh.cand_mass[at + i] = from.cand_mass[i];
+                    else list_index(sh)[at + i] = list_index(from)[i];
+                }
+                at += n;
+            }
         }
-#pragma unroll
-        for (int i = 0; i < kSelLoads; ++i) {
-            f(v[i].x);
-            f(v[i].y);
-            f(v[i].z);
-            f(v[i].w);
-        }
+        if (threadIdx.x == 0) sh.n_list = total;
+        __syncthreads();
     }
+    return static_cast<int>(total);
+}
+
+// f(four logits, their group) over the slice.
+template <int T, bool VEC, int LOADS, class F>
+__device__ __forceinline__ void for_each_group(const Slice<VEC, LOADS>& s, F f) {
+    for (int base = s.g0 + threadIdx.x; base < s.g1; base += LOADS * T) {
+        float4 v[LOADS];
+#pragma unroll
+        for (int i = 0; i < LOADS; ++i) {
+            const int g = base + i * T;
+            v[i] = g < s.g1 ? s.row.raw(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        }
+#pragma unroll
+        for (int i = 0; i < LOADS; ++i) f(v[i], base + i * T);
+    }
+}
+template <int T, bool VEC, int LOADS, class F>
+__device__ __forceinline__ void for_each_logit(const Slice<VEC, LOADS>& s, F f) {
+    for_each_group<T>(s, [&](const float4& v, int) {
+        f(v.x);
+        f(v.y);
+        f(v.z);
+        f(v.w);
+    });
 }
 
 __device__ __forceinline__ float warp_min(float v) {
@@ -855,15 +917,14 @@ __device__ __forceinline__ float warp_min(float v) {
 
 // The floor among the finite logits >= kf: MASS = false, the k-th largest of
 // them; MASS = true, the nucleus of mass top_p with weights exp2((l - max) * c2).
-// Every thread returns the same value; -inf means "keep everything".
-template <int kSelThreads, bool VEC, bool MASS>
-__device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned k, float top_p, float c2, SelShared<kSelThreads>& sh) {
-    constexpr int kSelWarps = kSelThreads / 32, kSelPerThread = kSelBins / kSelThreads;
+// Every thread of the team returns the same value; -inf means "keep everything".
+template <int T, bool MASS, bool VEC, int LOADS, bool SOLO>
+__device__ float select_floor(const Slice<VEC, LOADS>& s, const Team<SOLO>& team, float kf, unsigned k, float top_p, float c2, SelShared& sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // 1. range and number of the logits in play
     float lo = INFINITY, hi = -INFINITY, all = -INFINITY;
     unsigned n = 0;
-    for_each_logit<kSelThreads>(r, groups, [&](float v) {
+    for_each_logit<T>(s, [&](float v) {
         all = fmaxf(all, v);
         const bool in_play = fabsf(v) < INFINITY && v >= kf;
         const float u = in_play ? v : __int_as_float(0x7fc00000);  // (fminf and fmaxf pass over a NaN operand)
@@ -871,24 +932,38 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
         hi = fmaxf(hi, u);
         n += in_play;
     });
-    lo = warp_min(lo);
-    hi = warp_max(hi);
-    n = __reduce_add_sync(0xffffffffu, n);
-    const int any_inf = __syncthreads_or(all == INFINITY);  // (and the shared arrays may still be read by a previous call)
-    if (lane == 0) { sh.warp_lo[warp] = lo; sh.warp_hi[warp] = hi; sh.warp_cnt[warp] = n; }
-    __syncthreads();
-    lo = INFINITY; hi = -INFINITY; n = 0;
-#pragma unroll
-    for (int w = 0; w < kSelWarps; ++w) { lo = fminf(lo, sh.warp_lo[w]); hi = fmaxf(hi, sh.warp_hi[w]); n += sh.warp_cnt[w]; }
-    if (tid == 0) sh.row_top = any_inf ? INFINITY : hi;
+    // what the warps of the whole team found
+    auto of_all = [&](float& least, float& most, float& top, unsigned& count) {
+        least = warp_min(least);
+        most = warp_max(most);
+        top = warp_max(top);
+        count = __reduce_add_sync(0xffffffffu, count);
+        if (lane == 0) { sh.warp_lo[warp] = least; sh.warp_hi[warp] = most; sh.warp_top[warp] = top; sh.warp_cnt[warp] = count; }
+        team.sync();
+        least = INFINITY; most = top = -INFINITY; count = 0;
+        for (int i = lane; i < team.size * (T / 32); i += 32) {
+            const SelShared& from = team.of(sh, i / (T / 32));
+            const int w = i % (T / 32);
+            least = fminf(least, from.warp_lo[w]);
+            most = fmaxf(most, from.warp_hi[w]);
+            top = fmaxf(top, from.warp_top[w]);
+            count += from.warp_cnt[w];
+        }
+        least = warp_min(least);
+        most = warp_max(most);
+        top = warp_max(top);
+        count = __reduce_add_sync(0xffffffffu, count);
+    };
+    team.sync();  // (the shared arrays may still be read by a previous call)
+    of_all(lo, hi, all, n);
+    if (tid == 0) sh.row_top = all;
     if (n == 0 || (!MASS && k > n)) return kf;  // nothing to cut
     // weight exp2((l - max) * c2) of a logit in units of 2^-32 (the largest float below 2^32, so that the row's
     // maximum still fits 32 bits): a bin's mass is then one 32-bit shared-memory atomic and, rarely, a carry
     const float mc = fminf(-hi * c2, FLT_MAX);
     auto fixed_mass = [&](float v) { return __float2uint_rz(fast_exp2(fmaf(v, c2, mc)) * 4294967040.0f); };
 
-    unsigned before_cnt = 0;
-    unsigned long long before_mass = 0, goal = 0;
+    unsigned long long before = 0, target = k;  // counts, or masses
     for (int level = 0; level < kSelLevels; ++level) {
         if (lo == hi) return hi;  // everything left is one value: it stays whole
         const float top = hi, bottom = lo;
@@ -901,12 +976,12 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
             return (v >= bottom && v <= top) ? b : -1;
         };
         // 2. counts (and masses) per bin
-        for (int i = tid; i < kSelBins; i += kSelThreads) {
+        for (int i = tid; i < kSelBins; i += T) {
             if (MASS) { sh.mass_lo[i] = 0; sh.mass_hi[i] = 0; } else { sh.cnt[i] = 0; }
         }
-        if (tid == 0) { sh.n_cand = 0; sh.bin = kSelBins - 1; sh.before_cnt = before_cnt; sh.before_mass = before_mass; }
+        if (tid == 0) { sh.n_cand = sh.in_bin = 0; sh.bin = kSelBins - 1; sh.before = before; }
         __syncthreads();
-        for_each_logit<kSelThreads>(r, groups, [&](float v) {
+        for_each_logit<T>(s, [&](float v) {
             const int b = bin_of(v);
             if (b >= 0) {
                 if (MASS) {
@@ -919,56 +994,64 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
             }
         });
         __syncthreads();
-        // scan over the bins from the top: thread t owns bins t*P .. t*P+P-1
-        unsigned my_cnt = 0;
-        unsigned long long my_mass = 0;
+        {
+            unsigned long long sum = 0;
 #pragma unroll
-        for (int i = 0; i < kSelPerThread; ++i) {
-            const int b = tid * kSelPerThread + i;
-            if (MASS) my_mass += (static_cast<unsigned long long>(sh.mass_hi[b]) << 32) | sh.mass_lo[b];
-            else my_cnt += sh.cnt[b];
-        }
-        unsigned inc_cnt = my_cnt;
-        unsigned long long inc_mass = my_mass;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned c = __shfl_up_sync(0xffffffffu, inc_cnt, d);
-            const unsigned long long m = __shfl_up_sync(0xffffffffu, inc_mass, d);
-            if (lane >= d) { inc_cnt += c; inc_mass += m; }
-        }
-        if (lane == 31) { sh.warp_cnt[warp] = inc_cnt; sh.warp_mass[warp] = inc_mass; }
-        __syncthreads();
-        unsigned ex_cnt = before_cnt + inc_cnt - my_cnt;
-        unsigned long long ex_mass = before_mass + inc_mass - my_mass, all_mass = 0;
-#pragma unroll
-        for (int w = 0; w < kSelWarps; ++w) {
-            if (w < warp) { ex_cnt += sh.warp_cnt[w]; ex_mass += sh.warp_mass[w]; }
-            all_mass += sh.warp_mass[w];
-        }
-        if (MASS && level == 0)  // the first level sees every logit in play: top_p of their mass is the target
-            goal = static_cast<unsigned long long>(ceil(static_cast<double>(top_p) * static_cast<double>(all_mass)));
-        // the one thread whose bins contain the crossing records it
-        if (MASS ? ex_mass < goal : ex_cnt < k) {
-            unsigned run_cnt = ex_cnt;
-            unsigned long long run_mass = ex_mass;
-#pragma unroll
-            for (int i = 0; i < kSelPerThread; ++i) {
-                const int b = tid * kSelPerThread + i;
-                const unsigned c = MASS ? 0u : sh.cnt[b];
-                const unsigned long long m = MASS ? (static_cast<unsigned long long>(sh.mass_hi[b]) << 32) | sh.mass_lo[b] : 0ull;
-                const bool was_below = MASS ? run_mass < goal : run_cnt < k;
-                const bool reaches = MASS ? run_mass + m >= goal : run_cnt + c >= k;
-                if (was_below && reaches) { sh.bin = b; sh.before_cnt = run_cnt; sh.before_mass = run_mass; }
-                run_cnt += c;
-                run_mass += m;
+            for (int i = 0; i < (kSelBins / T); ++i) {
+                const int b = tid * (kSelBins / T) + i;
+                sum += MASS ? (static_cast<unsigned long long>(sh.mass_hi[b]) << 32) | sh.mass_lo[b] : sh.cnt[b];
             }
+            constexpr int kThreads = 32 * T / kSelBins;  // to a segment
+#pragma unroll
+            for (int d = 1; d < kThreads; d *= 2) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+            if (lane % kThreads == 0) sh.segment[tid / kThreads] = sum;
+        }
+        team.sync();
+        if (warp == 0) {  // scan from the top: over the segments of all CTAs, then over the bins of one of them
+            auto scan = [&](unsigned long long v) {
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const unsigned long long o = __shfl_up_sync(0xffffffffu, v, d);
+                    if (lane >= d) v += o;
+                }
+                return v;
+            };
+            unsigned long long a = 0, b = 0;
+            for (int r = 0; r < team.size; ++r) {
+                const unsigned long long* from = team.of(sh, r).segment + 2 * lane;
+                a += from[0];
+                b += from[1];
+            }
+            const unsigned long long upto = scan(a + b), all_of_it = __shfl_sync(0xffffffffu, upto, 31);
+            if (MASS && level == 0)  // the first level sees every logit in play: top_p of their mass is the target
+                target = static_cast<unsigned long long>(ceil(static_cast<double>(top_p) * static_cast<double>(all_of_it)));
+            const unsigned long long above = before + upto - (a + b);
+            const unsigned who = __ballot_sync(0xffffffffu, above < target && above + a + b >= target);
+            if (who) {
+                const int at = __ffs(who) - 1;
+                const bool second = __shfl_sync(0xffffffffu, above + a < target ? 1 : 0, at) != 0;
+                const unsigned long long over = __shfl_sync(0xffffffffu, second ? above + a : above, at);
+                const int bin = 32 * (2 * at + (second ? 1 : 0)) + lane;
+                unsigned long long mine = 0;
+                for (int r = 0; r < team.size; ++r) {
+                    const SelShared& from = team.of(sh, r);
+                    mine += MASS ? (static_cast<unsigned long long>(from.mass_hi[bin]) << 32) | from.mass_lo[bin] : from.cnt[bin];
+                }
+                const unsigned long long ex = over + scan(mine) - mine;
+                if (ex < target && ex + mine >= target) {
+                    sh.bin = bin;
+                    sh.before = ex;
+                    sh.in_bin = static_cast<unsigned>(mine);
+                }
+            }
+            if (lane == 0) sh.target = target;
         }
         __syncthreads();
         const int bin = sh.bin;
-        before_cnt = sh.before_cnt;
-        before_mass = sh.before_mass;
+        before = sh.before;
+        target = sh.target;
         // top-k knows how many logits the bin holds; the nucleus keeps no counts and finds out by copying them
-        const bool few = MASS || sh.cnt[bin] <= kSelCap;
+        const bool few = MASS || sh.in_bin <= kSelCap;
         // a cheap test that no logit of the bin fails (its centre, half its width and the roundings of bin_of, with
         // room to spare); the few that pass are then asked for their bin
         const float centre = top - (static_cast<float>(bin) + 0.5f) / scale;
@@ -976,49 +1059,52 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
         auto in_the_bin = [&](float v) { return fabsf(v - centre) <= reach && bin_of(v) == bin; };
         if (few) {
             // 3. copy the bin's logits out and rank them against each other
-            for_each_logit<kSelThreads>(r, groups, [&](float v) {
+            for_each_logit<T>(s, [&](float v) {
                 if (in_the_bin(v)) {
                     const unsigned at = atomicAdd(&sh.n_cand, 1u);
                     if (at < kSelCap) { sh.cand[at] = v; if (MASS) sh.cand_mass[at] = fixed_mass(v); }
                 }
             });
-            __syncthreads();
-            if (sh.n_cand <= kSelCap) {  // (always so for top-k)
-                const int count = static_cast<int>(min(sh.n_cand, static_cast<unsigned>(kSelCap)));
-                float best = -INFINITY;
-                for (int i = tid; i < count; i += kSelThreads) {
-                    const float mine = sh.cand[i];
-                    unsigned c = 0;
-                    unsigned long long m = 0;
-                    for (int j = 0; j < count; ++j)
-                        if (sh.cand[j] >= mine) { ++c; if (MASS) m += sh.cand_mass[j]; }
-                    const bool enough = MASS ? before_mass + m >= goal : before_cnt + c >= k;
-                    if (enough) best = fmaxf(best, mine);
-                }
-                best = warp_max(best);
-                if (lane == 0) sh.warp_hi[warp] = best;
-                __syncthreads();
-                best = -INFINITY;
+            const int count = gather_list<T>(team, MASS, sh);
+            if (count >= 0) {  // (always so for top-k)
+                if (team.rank == 0) {
+                    float best = -INFINITY;
+                    for (int i = tid; i < count; i += T) {
+                        const float mine = sh.cand[i];
+                        unsigned long long m = before;
+#pragma unroll 8
+                        for (int j = 0; j < count; ++j) {
+                            const unsigned long long w = MASS ? sh.cand_mass[j] : 1ull;
+                            m += sh.cand[j] >= mine ? w : 0ull;
+                        }
+                        if (m >= target) best = fmaxf(best, mine);
+                    }
+                    best = warp_max(best);
+                    if (lane == 0) sh.warp_hi[warp] = best;
+                    __syncthreads();
+                    best = -INFINITY;
 #pragma unroll
-                for (int w = 0; w < kSelWarps; ++w) best = fmaxf(best, sh.warp_hi[w]);
-                return best > -INFINITY ? best : bottom;
+                    for (int w = 0; w < (T / 32); ++w) best = fmaxf(best, sh.warp_hi[w]);
+                    best = best > -INFINITY ? best : bottom;
+                    if (SOLO) return best;
+                    if (tid < team.size) team.of(sh, tid).floor = best;
+                }
+                team.sync();
+                return sh.floor;
             }
         }
         // the bin is crowded: its own range is searched next
-        float new_lo = INFINITY, new_hi = -INFINITY;
-        for_each_logit<kSelThreads>(r, groups, [&](float v) {
+        float new_lo = INFINITY, new_hi = -INFINITY, unused = -INFINITY;
+        unsigned none = 0;
+        for_each_logit<T>(s, [&](float v) {
             const bool here = in_the_bin(v);
             new_lo = fminf(new_lo, here ? v : INFINITY);
             new_hi = fmaxf(new_hi, here ? v : -INFINITY);
         });
-        new_lo = warp_min(new_lo);
-        new_hi = warp_max(new_hi);
-        if (lane == 0) { sh.warp_lo[warp] = new_lo; sh.warp_hi[warp] = new_hi; }
-        __syncthreads();
-        lo = INFINITY; hi = -INFINITY;
-#pragma unroll
-        for (int w = 0; w < kSelWarps; ++w) { lo = fminf(lo, sh.warp_lo[w]); hi = fmaxf(hi, sh.warp_hi[w]); }
-        __syncthreads();
+        team.sync();  // (everyone has read the others' counts and bins)
+        of_all(new_lo, new_hi, unused, none);
+        lo = new_lo;
+        hi = new_hi;
     }
     return lo;
 }
@@ -1026,22 +1112,24 @@ __device__ float select_floor(const Row<VEC>& r, int groups, float kf, unsigned 
 // Top-k for k up to 128, without bins: every warp gives its largest lane maxima, 3 k of them in all; the k-th largest of
 // these is a value that at least k logits reach, so the k-th largest logit of the row is among those that reach it - a
 // few more than k as a rule.  One pass for the maxima; only the threads whose maximum reaches the pivot have such
-// logits, and what they read is read again, by all warps, and listed; the list is ranked as in step 3 above.
-// Returns false, having decided nothing, when fewer than k lanes hold a finite logit, when there is a +inf, or when
-// more than kSelCap logits reach the pivot (heavy ties): the binned selection then does the row.
+// logits, and what they read is read again, by all warps, and listed.
+// Returns how many are listed, or -1, having decided nothing, when fewer than k lanes hold a finite logit, when there is a
+// +inf, or when more than kSelCap logits reach the pivot (heavy ties): the binned selection then does the row.
 constexpr int kMostTops = 512;
 
-template <int kSelThreads, bool VEC>
-__device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelShared<kSelThreads>& sh, float* floor) {
-    constexpr int kSelWarps = kSelThreads / 32;
+template <int T, bool VEC, int LOADS, bool SOLO>
+__device__ int top_k_list(const Slice<VEC, LOADS>& s, const Team<SOLO>& team, unsigned k, SelShared& sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // (measured on 960 rows of 32000: k = 40 66 us per call against 82 binned, k = 128 71, k = 200 92: the pivot sinks
     // with k and lets ever more logits through)
-    if (k > 128) return false;
-    const int per_warp = min(min(32, kMostTops / kSelWarps), (3 * static_cast<int>(k) + kSelWarps - 1) / kSelWarps);
-    const int n_tops = per_warp * kSelWarps;
+    if (k > 128) return -1;
+    float* own = reinterpret_cast<float*>(sh.cand_mass);  // this CTA's maxima, then everyone's
+    float* tops = own + kMostTops;
+    const int warps = (T / 32) * team.size;
+    const int per_warp = min(min(32, kMostTops / warps), (3 * static_cast<int>(k) + warps - 1) / warps);
+    const int n_tops = per_warp * warps, per_cta = per_warp * (T / 32);
     float mine = -INFINITY;
-    for_each_logit<kSelThreads>(r, groups, [&](float v) { mine = fmaxf(mine, v); });
+    for_each_logit<T>(s, [&](float v) { mine = fmaxf(mine, v); });
     {
         // (keys: the floats' order as unsigned integers, for the warp-wide integer maximum; 0 marks a lane that is out)
         const unsigned u = __float_as_uint(mine);
@@ -1053,41 +1141,54 @@ __device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelSha
             if (lane == __ffs(who) - 1) key = 0;
             if (lane == i && top != 0) given = __uint_as_float(top ^ ((top >> 31) ? 0x80000000u : 0xffffffffu));
         }
-        if (lane < per_warp) sh.cand[warp * per_warp + lane] = given;
+        if (lane < per_warp) own[warp * per_warp + lane] = given;
     }
     if (tid == 0) { sh.n_cand = 0; sh.n_hit = 0; }
-    if (__syncthreads_or(mine == INFINITY)) return false;
+    team.sync();
+    for (int i = tid; i < n_tops; i += T) tops[i] = reinterpret_cast<const float*>(team.of(sh, i / per_cta).cand_mass)[i % per_cta];
+    __syncthreads();
     // the k-th largest of the maxima: the largest one that at least k of them reach; `per` threads count for each
     int per = 1;
-    while (per * 2 * n_tops <= kSelThreads && per < 32) per *= 2;
-    float pivot = -INFINITY;
-    for (int base = 0; base < n_tops; base += kSelThreads / per) {
+    while (per * 2 * n_tops <= T && per < 32) per *= 2;
+    float pivot = -INFINITY, most = -INFINITY;
+    for (int base = 0; base < n_tops; base += T / per) {
         const int i = base + tid / per;
-        const float top = i < n_tops ? sh.cand[i] : INFINITY;
+        const float top = i < n_tops ? tops[i] : INFINITY;
         unsigned reach = 0;
 #pragma unroll 8
-        for (int j = tid % per; j < n_tops; j += per) reach += sh.cand[j] >= top;
+        for (int j = tid % per; j < n_tops; j += per) reach += tops[j] >= top;
         for (int o = per / 2; o > 0; o >>= 1) reach += __shfl_xor_sync(0xffffffffu, reach, o);
-        if (i < n_tops && reach >= k) pivot = fmaxf(pivot, top);
+        if (i < n_tops) {
+            most = fmaxf(most, top);
+            if (reach >= k) pivot = fmaxf(pivot, top);
+        }
     }
     pivot = warp_max(pivot);
-    if (lane == 0) sh.warp_hi[warp] = pivot;
-    __syncthreads();  // (every thread has read the maxima: the list can be reused)
-    pivot = -INFINITY;
+    most = warp_max(most);
+    if (lane == 0) { sh.warp_hi[warp] = pivot; sh.warp_top[warp] = most; }
+    __syncthreads();
+    pivot = most = -INFINITY;
 #pragma unroll
-    for (int w = 0; w < kSelWarps; ++w) pivot = fmaxf(pivot, sh.warp_hi[w]);
-    if (!(pivot > -INFINITY)) return false;
+    for (int w = 0; w < (T / 32); ++w) {
+        pivot = fmaxf(pivot, sh.warp_hi[w]);
+        most = fmaxf(most, sh.warp_top[w]);
+    }
+    if (!(pivot > -INFINITY) || most == INFINITY) return -1;
     if (mine >= pivot) sh.cnt[atomicAdd(&sh.n_hit, 1u)] = tid;
     __syncthreads();
     const int hits = static_cast<int>(sh.n_hit);
-    for (int h = warp; h < hits; h += kSelWarps)  // a warp goes over what one of those threads has read
-        for (int g = sh.cnt[h] + lane * kSelThreads; g < groups; g += 32 * kSelThreads) list_group(r.raw(g, -INFINITY), 4 * g - r.shift, pivot, sh);
-    __syncthreads();
-    const unsigned total = sh.n_cand;
-    if (total > kSelCap) return false;
-    const int count = static_cast<int>(total);
+    for (int h = warp; h < hits; h += (T / 32))  // a warp goes over what one of those threads has read
+        for (int g = s.g0 + sh.cnt[h] + lane * T; g < s.g1; g += 32 * T)
+            list_group(s.row.raw(g, -INFINITY), 4 * g - s.row.shift, pivot, sh);
+    return gather_list<T>(team, false, sh);
+}
+
+// The k-th largest of the listed logits.  In the first CTA.
+template <int T>
+__device__ float top_k_of_list(unsigned k, SelShared& sh) {
+    const int tid = threadIdx.x, count = static_cast<int>(sh.n_list);
     float best = -INFINITY;
-    for (int i = tid; i < count; i += kSelThreads) {
+    for (int i = tid; i < count; i += T) {
         const float c = sh.cand[i];
         unsigned at_least = 0;
 #pragma unroll 8
@@ -1095,48 +1196,37 @@ __device__ bool top_k_by_pivot(const Row<VEC>& r, int groups, unsigned k, SelSha
         if (at_least >= k) best = fmaxf(best, c);
     }
     best = warp_max(best);
-    if (lane == 0) sh.warp_lo[warp] = best;
+    if ((tid & 31) == 0) sh.warp_lo[tid >> 5] = best;
     __syncthreads();
     best = -INFINITY;
 #pragma unroll
-    for (int w = 0; w < kSelWarps; ++w) best = fmaxf(best, sh.warp_lo[w]);
-    *floor = best;
-    return true;
+    for (int w = 0; w < (T / 32); ++w) best = fmaxf(best, sh.warp_lo[w]);
+    return best;
 }
 
-// Lists the logits that reach kf > -inf, after a top-k that found it by bins.  Returns false if they are more than kSelCap (a
-// large tie at kf) or one of them is +inf.
-template <int kSelThreads, bool VEC>
-__device__ bool list_row(const Row<VEC>& r, int groups, float kf, SelShared<kSelThreads>& sh) {
-    __syncthreads();  // (the shared arrays may still be read by a previous call)
-    if (sh.row_top == INFINITY) return false;
+// Lists the logits that reach kf > -inf, after a top-k that found it by bins.  Returns how many, or -1 if they are more than
+// kSelCap (a large tie at kf) or one of them is +inf.
+template <int T, bool VEC, int LOADS, bool SOLO>
+__device__ int list_row(const Slice<VEC, LOADS>& s, const Team<SOLO>& team, float kf, SelShared& sh) {
+    team.sync();  // (the shared arrays may still be read by a previous call)
+    if (sh.row_top == INFINITY) return -1;
     if (threadIdx.x == 0) sh.n_cand = 0;
     __syncthreads();
-    for (int g0 = threadIdx.x; g0 < groups; g0 += kSelLoads * kSelThreads) {
-        float4 v[kSelLoads];
-#pragma unroll
-        for (int i = 0; i < kSelLoads; ++i) {
-            const int g = g0 + i * kSelThreads;
-            v[i] = g < groups ? r.raw(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-        }
-#pragma unroll
-        for (int i = 0; i < kSelLoads; ++i) list_group(v[i], 4 * (g0 + i * kSelThreads) - r.shift, kf, sh);
-    }
-    __syncthreads();
-    return sh.n_cand <= kSelCap;
+    for_each_group<T>(s, [&](const float4& v, int g) { list_group(v, 4 * g - s.row.shift, kf, sh); });
+    return gather_list<T>(team, false, sh);
 }
 
-template <int kSelThreads>
+template <int T>
 __device__ __forceinline__ float block_max(float v, float* per_warp) {
     v = warp_max(v);
     if ((threadIdx.x & 31) == 0) per_warp[threadIdx.x >> 5] = v;
     __syncthreads();
     v = per_warp[0];
 #pragma unroll
-    for (int w = 1; w < kSelThreads / 32; ++w) v = fmaxf(v, per_warp[w]);
+    for (int w = 1; w < (T / 32); ++w) v = fmaxf(v, per_warp[w]);
     return v;
 }
-template <int kSelThreads>
+template <int T>
 __device__ __forceinline__ unsigned long long block_sum(unsigned long long v, unsigned long long* per_warp) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -1144,31 +1234,31 @@ __device__ __forceinline__ unsigned long long block_sum(unsigned long long v, un
     __syncthreads();
     v = 0;
 #pragma unroll
-    for (int w = 0; w < kSelThreads / 32; ++w) v += per_warp[w];
+    for (int w = 0; w < (T / 32); ++w) v += per_warp[w];
     return v;
 }
 
 // What is left of a listed row: the nucleus of the logits that reach *floor (if `nucleus`, which raises *floor), ranked
 // against each other, the largest logit and the sum of the kept weights.  Weights are summed in units of 2^-40 of the
-// largest, so that the order in which the list was made does not matter.
-template <int kSelThreads>
-__device__ void finish_list(bool nucleus, float top_p, float c2, SelShared<kSelThreads>& sh, float* floor, float* row_max, float* sum) {
-    const int tid = threadIdx.x, count = static_cast<int>(sh.n_cand);
+// largest, so that the order in which the list was made does not matter.  In the first CTA.
+template <int T>
+__device__ void finish_list(bool nucleus, float top_p, float c2, SelShared& sh, float* floor, float* row_max, float* sum) {
+    const int tid = threadIdx.x, count = static_cast<int>(sh.n_list);
     const float kf = *floor;
     float m = -INFINITY;
-    for (int i = tid; i < count; i += kSelThreads) m = fmaxf(m, sh.cand[i]);
-    m = block_max<kSelThreads>(m, sh.warp_hi);
+    for (int i = tid; i < count; i += T) m = fmaxf(m, sh.cand[i]);
+    m = block_max<T>(m, sh.warp_hi);
     unsigned long long mine_sum = 0;
-    for (int i = tid; i < count; i += kSelThreads) {
+    for (int i = tid; i < count; i += T) {
         const unsigned long long w = sh.cand[i] >= kf ? __float2ull_rz(fast_exp2((sh.cand[i] - m) * c2) * 1099511627776.0f) : 0ull;  // 2^40
         sh.cand_mass[i] = w;
         mine_sum += w;
     }
-    unsigned long long kept = block_sum<kSelThreads>(mine_sum, sh.warp_mass);  // (and cand_mass is complete)
+    unsigned long long kept = block_sum<T>(mine_sum, sh.warp_mass);  // (and cand_mass is complete)
     if (nucleus) {
         const unsigned long long goal = static_cast<unsigned long long>(ceil(static_cast<double>(top_p) * static_cast<double>(kept)));
         float best = -INFINITY;
-        for (int i = tid; i < count; i += kSelThreads) {
+        for (int i = tid; i < count; i += T) {
             const float mine = sh.cand[i];
             if (!(mine >= kf)) continue;
             unsigned long long above = 0;
@@ -1176,30 +1266,30 @@ __device__ void finish_list(bool nucleus, float top_p, float c2, SelShared<kSelT
             for (int j = 0; j < count; ++j) above += sh.cand[j] >= mine ? sh.cand_mass[j] : 0ull;
             if (above >= goal) best = fmaxf(best, mine);
         }
-        best = block_max<kSelThreads>(best, sh.warp_lo);
+        best = block_max<T>(best, sh.warp_lo);
         *floor = best > -INFINITY ? best : kf;
         mine_sum = 0;
-        for (int i = tid; i < count; i += kSelThreads)
+        for (int i = tid; i < count; i += T)
             if (sh.cand[i] >= *floor) mine_sum += sh.cand_mass[i];
-        kept = block_sum<kSelThreads>(mine_sum, sh.warp_mass);  // (everyone has read the first sums: a barrier ago)
+        kept = block_sum<T>(mine_sum, sh.warp_mass);  // (everyone has read the first sums: a barrier ago)
     }
     *row_max = m;
     *sum = static_cast<float>(static_cast<double>(kept) * (1.0 / 1099511627776.0));
 }
 
-// The draw from a listed row: the kept logits in the order of their places, walked by one warp.
-template <int kSelThreads>
-__device__ int draw_from_list(float floor, float row_max, float c2, float u, SelShared<kSelThreads>& sh) {
-    const int tid = threadIdx.x, count = static_cast<int>(sh.n_cand);
+// The draw from a listed row: the kept logits in the order of their places, walked by one warp.  In the first CTA.
+template <int T>
+__device__ int draw_from_list(float floor, float row_max, float c2, float u, SelShared& sh) {
+    const int tid = threadIdx.x, count = static_cast<int>(sh.n_list);
     unsigned* index = list_index(sh);
     float* weight = reinterpret_cast<float*>(sh.cand_mass);  // in order
     unsigned* place = sh.mass_lo;
     __syncthreads();  // (cand_mass has been read by everyone)
     if (tid == 0) sh.n_hit = 0;
-    for (int i = tid; i < count; i += kSelThreads)
+    for (int i = tid; i < count; i += T)
         if (!(sh.cand[i] >= floor)) index[i] = 0xffffffffu;  // (behind every place of the row)
     __syncthreads();
-    for (int i = tid; i < count; i += kSelThreads) {
+    for (int i = tid; i < count; i += T) {
         if (!(sh.cand[i] >= floor)) continue;
         unsigned rank = 0;
 #pragma unroll 8
@@ -1230,40 +1320,56 @@ __device__ int draw_from_list(float floor, float row_max, float c2, float u, Sel
     return token;  // (valid in the first warp)
 }
 
-// (max, sum of exp2((l - max) * c2)) of the kept logits, online, in a fixed order.  Valid in thread 0.
-template <int kSelThreads, bool VEC>
-__device__ void row_statistics(const Row<VEC, true>& r, int groups, float c2, SelShared<kSelThreads>& sh, float* row_max, float* sum) {
+// (max, sum of exp2((l - max) * c2)) of the kept logits, online, in a fixed order.  Valid in thread 0 of the first CTA.
+template <int T, bool VEC, int LOADS, bool SOLO>
+__device__ void row_statistics(const Slice<VEC, LOADS>& s, const Team<SOLO>& team, float floor, float c2, SelShared& sh, float* row_max, float* sum) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float m = -FLT_MAX, s = 0.0f;  // (finite, so that m - new maximum never becomes inf - inf)
-    for (int base = tid; base < groups; base += kSelLoads * kSelThreads) {
-        float4 v[kSelLoads];
+    Row<VEC, true> r;
+    r.base = s.row.base;
+    r.vocab = s.row.vocab;
+    r.floor = floor;
+    r.shift = s.row.shift;
+    r.own = s.row.own;
+    float m = -FLT_MAX, t = 0.0f;  // (finite, so that m - new maximum never becomes inf - inf)
+    for (int base = s.g0 + tid; base < s.g1; base += LOADS * T) {
+        float4 v[LOADS];
         float bm = m;
 #pragma unroll
-        for (int i = 0; i < kSelLoads; ++i) {
-            const int g = base + i * kSelThreads;
-            v[i] = g < groups ? r.load(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        for (int i = 0; i < LOADS; ++i) {
+            const int g = base + i * T;
+            v[i] = g < s.g1 ? r.load(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         }
 #pragma unroll
-        for (int i = 0; i < kSelLoads; ++i) bm = fmaxf(bm, fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w)));
-        s *= fast_exp2((m - bm) * c2);
+        for (int i = 0; i < LOADS; ++i) bm = fmaxf(bm, fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w)));
+        t *= fast_exp2((m - bm) * c2);
         m = bm;
         const float mc = fminf(-m * c2, FLT_MAX);  // (-inf * c2 + it stays -inf)
 #pragma unroll
-        for (int i = 0; i < kSelLoads; ++i)
-            s += (fast_exp2(fmaf(v[i].x, c2, mc)) + fast_exp2(fmaf(v[i].y, c2, mc))) +
+        for (int i = 0; i < LOADS; ++i)
+            t += (fast_exp2(fmaf(v[i].x, c2, mc)) + fast_exp2(fmaf(v[i].y, c2, mc))) +
                  (fast_exp2(fmaf(v[i].z, c2, mc)) + fast_exp2(fmaf(v[i].w, c2, mc)));
     }
     const float wm = warp_max(m);
-    s = warp_sum(s * fast_exp2((m - wm) * c2));
-    __syncthreads();  // (the shared arrays may still be read)
-    if (lane == 0) { sh.warp_hi[warp] = wm; sh.warp_lo[warp] = s; }
+    t = warp_sum(t * fast_exp2((m - wm) * c2));
+    team.sync();  // (the shared arrays may still be read)
+    if (lane == 0) { sh.warp_hi[warp] = wm; sh.warp_lo[warp] = t; }
     __syncthreads();
-    if (tid == 0) {
-        float bm = sh.warp_hi[0], t = 0.0f;
-        for (int w = 1; w < kSelThreads / 32; ++w) bm = fmaxf(bm, sh.warp_hi[w]);
-        for (int w = 0; w < kSelThreads / 32; ++w) t += sh.warp_lo[w] * fast_exp2((sh.warp_hi[w] - bm) * c2);
+    auto merge = [&](const float* max, const float* part, int count) {
+        float bm = max[0], all = 0.0f;
+        for (int w = 1; w < count; ++w) bm = fmaxf(bm, max[w]);
+        for (int w = 0; w < count; ++w) all += part[w] * fast_exp2((max[w] - bm) * c2);
         *row_max = bm;
-        *sum = t;
+        *sum = all;
+    };
+    if (tid == 0) {
+        merge(sh.warp_hi, sh.warp_lo, (T / 32));
+        SelShared& first = team.of(sh, 0);
+        first.cta_max[team.rank] = *row_max;
+        first.cta_sum[team.rank] = *sum;
+    }
+    if (!SOLO) {
+        team.sync();
+        if (tid == 0 && team.rank == 0) merge(sh.cta_max, sh.cta_sum, team.size);
     }
 }
 
@@ -1281,70 +1387,91 @@ struct CutWork {
 };
 // (ordering a list by place takes a comparison per pair; beyond this it is cheaper to go over the row, as without a list:
 // one row of 32000, k = 400, p = 0.95 39 us with the list, 48 without)
-constexpr unsigned kDrawList = 512;
+constexpr int kDrawList = 512;
 constexpr int kFloorsOnly = 0, kWithStats = 1, kWithDraw = 2;
 
 // floors[s * (a_rows + b_rows) + r] for sequence s's a_rows rows of `a`, then its
 // b_rows rows of `b`: top-k first (0 < top_k < vocab), then the nucleus (0 < top_p < 1)
-// of what top-k left.  The statistics of the verification and the draw of the sampling follow in the same CTA: after a
-// top-k they cost nothing, the list is there (24 x 9 rows of 50003, k = 40, p = 0.9: 66 -> 40 us, 200
-// rows of 100000, k = 40, with the draw: 73 -> 28, one of 32000: 16 -> 9), and after a nucleus one pass less and no second
-// kernel (200 rows of 100000: 99 -> 91).
-template <bool VEC, int kSelThreads, int WORK>
-__global__ void __launch_bounds__(kSelThreads)
+// of what top-k left.  The statistics of the verification and the draw of the sampling follow in the same CTAs: after a
+// top-k they cost nothing, the list is there (24 x 9 rows of 50003, k = 40, p = 0.9: 66 us with kernels of their own, 40 so
+// with 1024 threads to a row, 32 with 512; 200 rows of 100000, k = 40, with the draw: 73, 28 and 22; one of 32000: 16, 9 and
+// 8), and after a nucleus one pass less and no second kernel (200 rows of 100000: 99, 91 and 70).
+template <int T, int LOADS, bool VEC, bool SOLO, int WORK>
+__global__ void __launch_bounds__(T, T == 256 ? 5 : LOADS == 8 ? 2 : 3)
 cut_floor_kernel(const float* __restrict__ a, size_t a_stride, int a_rows, const float* __restrict__ b,
                  size_t b_stride, int b_rows, int vocab, int top_k, float top_p, float c2, float* __restrict__ floors, CutWork work) {
-    __shared__ SelShared<kSelThreads> sh;
+    __shared__ SelShared sh;
     pdl_trigger();
     pdl_wait();
+    const Team<SOLO> team;
+    const int at = blockIdx.x / team.size;
     const int per_seq = a_rows + b_rows;
-    const int seq = blockIdx.x / per_seq, row = blockIdx.x % per_seq;
+    const int seq = at / per_seq, row = at % per_seq;
     const float* src = row < a_rows ? a + (static_cast<size_t>(seq) * a_rows + row) * a_stride
                                     : b + (static_cast<size_t>(seq) * b_rows + (row - a_rows)) * b_stride;
-    const Row<VEC> r = make_row<VEC>(src, vocab);
-    const int groups = r.groups();
+    Slice<VEC, LOADS> s;
+    s.row = make_row<VEC>(src, vocab);
+    const int groups = s.row.groups(), each = (groups + team.size - 1) / team.size;
+    s.g0 = min(groups, team.rank * each);
+    s.g1 = min(groups, s.g0 + each);
+    const bool first = team.rank == 0;
     float floor = -INFINITY, row_max = 0.0f, sum = 0.0f;
-    bool listed = false;
+    int listed = -1;  // logits listed (the same in all CTAs; floor, row_max and sum of a listed row are the first one's)
     const bool nucleus = top_p > 0.0f && top_p < 1.0f;
     if (top_k > 0 && top_k < vocab) {
-        listed = top_k_by_pivot<kSelThreads, VEC>(r, groups, static_cast<unsigned>(top_k), sh, &floor);
-        if (!listed) {
-            floor = select_floor<kSelThreads, VEC, false>(r, groups, -INFINITY, static_cast<unsigned>(top_k), 0.0f, 0.0f, sh);
-            listed = nucleus && floor > -INFINITY && top_k <= kSelCap && list_row<kSelThreads, VEC>(r, groups, floor, sh);
+        listed = top_k_list<T>(s, team, static_cast<unsigned>(top_k), sh);
+        if (listed >= 0) {
+            if (first) floor = top_k_of_list<T>(static_cast<unsigned>(top_k), sh);
+        } else {
+            floor = select_floor<T, false>(s, team, -INFINITY, static_cast<unsigned>(top_k), 0.0f, 0.0f, sh);
+            if (nucleus && floor > -INFINITY && top_k <= kSelCap) listed = list_row<T>(s, team, floor, sh);
         }
     }
-    if (listed) finish_list<kSelThreads>(nucleus, top_p, c2, sh, &floor, &row_max, &sum);
-    else if (nucleus) floor = select_floor<kSelThreads, VEC, true>(r, groups, floor, 0u, top_p, c2, sh);
-    if (threadIdx.x == 0 && floors) floors[blockIdx.x] = floor;
+    if (listed >= 0) {
+        if (first) finish_list<T>(nucleus, top_p, c2, sh, &floor, &row_max, &sum);
+    } else if (nucleus) {
+        floor = select_floor<T, true>(s, team, floor, 0u, top_p, c2, sh);
+    }
+    if (threadIdx.x == 0 && first && floors) floors[at] = floor;
     if (WORK == kWithStats) {
-        if (!listed) row_statistics<kSelThreads, VEC>(make_row<VEC, true>(src, vocab, floor), groups, c2, sh, &row_max, &sum);
-        if (threadIdx.x == 0) {
+        if (listed < 0) row_statistics<T>(s, team, floor, c2, sh, &row_max, &sum);
+        if (threadIdx.x == 0 && first) {
             float at_x = 0.0f;  // (none for p_{gamma+1})
             if (row != a_rows - 1) {
                 const int x = work.draft_tokens[static_cast<size_t>(seq) * b_rows + (row < a_rows ? row : row - a_rows)];
                 if (x >= 0 && x < vocab) at_x = __ldg(src + x) >= floor ? __ldg(src + x) : -INFINITY;
             }
-            *reinterpret_cast<float4*>(work.stats + blockIdx.x) = make_float4(row_max, sum, at_x, 0.0f);
+            *reinterpret_cast<float4*>(work.stats + at) = make_float4(row_max, sum, at_x, 0.0f);
         }
     }
     if (WORK == kWithDraw) {
-        const float u = work.uniforms[static_cast<size_t>(blockIdx.x) * work.uniform_stride];
-        int token;
-        if (listed && sh.n_cand <= kDrawList) {
-            token = draw_from_list<kSelThreads>(floor, row_max, c2, u, sh);
+        __shared__ CdfScratch<T / 32> cdf;
+        const float u = work.uniforms[static_cast<size_t>(at) * work.uniform_stride];
+        int token = -1;
+        if (listed >= 0 && listed <= kDrawList) {
+            if (first) token = draw_from_list<T>(floor, row_max, c2, u, sh);
         } else {
-            __shared__ CdfScratch<kSelThreads / 32> cdf;
+            if (listed >= 0) {  // the others need what the first one found
+                if (first && threadIdx.x < team.size) {
+                    team.of(sh, threadIdx.x).floor = floor;
+                    team.of(sh, threadIdx.x).row_top = row_max;
+                }
+                team.sync();
+                floor = sh.floor;
+            }
             __syncthreads();
-            if (threadIdx.x == 0 && !listed && work.nonfinite && sh.row_top == INFINITY) atomicExch(work.nonfinite, 1);
+            if (threadIdx.x == 0 && first && work.nonfinite && sh.row_top == INFINITY) atomicExch(work.nonfinite, 1);
             PlainWeights<VEC, true> pw;
             pw.p = make_row<VEC, true>(src, vocab, floor);
-            pw.max_p = listed ? row_max : fmaxf(sh.row_top, -FLT_MAX);
+            pw.max_p = fmaxf(sh.row_top, -FLT_MAX);
             pw.c2 = c2;
             float total;
-            token = block_inverse_cdf<kSelThreads / 32>(pw, vocab, u, cdf, &total);
+            token = SOLO ? block_inverse_cdf<T / 32>(pw, vocab, u, cdf, &total) : cluster_inverse_cdf<T / 32>(pw, vocab, u, cdf, &total);
         }
-        if (threadIdx.x == 0) work.tokens[static_cast<size_t>(blockIdx.x) * work.token_stride] = max(0, min(token, vocab - 1));
+        // (of a cluster one CTA has drawn, and the others have -1)
+        if (threadIdx.x == 0 && (SOLO || token >= 0)) work.tokens[static_cast<size_t>(at) * work.token_stride] = max(0, min(token, vocab - 1));
     }
+    if (!SOLO) team.sync();  // nobody leaves while another may still look here
 }
 
 __global__ void uniforms_kernel(uint64_t seed, const int32_t* __restrict__ positions,
@@ -1397,10 +1524,25 @@ size_t verify_sample_workspace_bytes(int batch, int gamma, int vocab) {
     return stats_bytes(batch, gamma, vocab) + static_cast<size_t>(batch) * rows * sizeof(float) + 256;
 }
 
-// A selection CTA has 1024 threads where long rows would leave small CTAs with many loads in a row and the GPU unfilled:
-// nucleus 0.9, 200 rows of 100000 with the draw 131 -> 106 us, 30 rows of 120001 120 -> 64; on shorter or more rows the
-// wider barriers cost more than they give (216 rows of 50003 40 -> 38, 330 rows of 50003 52 -> 66, 11 rows of 8192 6 -> 8).
-bool wide_rows(int rows, int vocab) { return rows <= 2 * 148 && vocab >= 48 * 1024; }
+// How the rows of a cut are shared out.
+struct CutShape {
+    int threads, loads, ctas;  // of a CTA; in flight per thread; CTAs per row
+};
+// Both ways measured (us per call, with what follows the cut):
+// - 512 threads with eight loads each, two rows to an SM, while that is one wave (200 x 100000, p = 0.9: 70, with 1024 threads
+//   90, with 256 103; 216 x 32000: 31, with four loads and three rows to an SM 37); with more rows four loads (330 x
+//   50003: 98, 74), and with many short ones 256 threads (960 x 32000 88, 512 threads 98; 960 x 8192 32, 50; but 960 x
+//   50003 157, 223).  A short row that is binned is all barriers: 256 threads (64 x 8192: 10, 12; 64 x 16000: 15, 14).
+// - a cluster pays where few rows are long and binned (4 x 512 threads against 512: 16 x 50003 26, 37; 16 x 128000 29, 53;
+//   64 x 100000 32, 50; 2 x 512: 128 x 100000 51, 66), not on more rows (200 x 100000 with two: 87, 70), shorter ones (16 x
+//   32000: 19, 18) or a list, whose passes are few (16 x 100000, k = 50: 13, 13).
+CutShape cut_shape(int rows, int vocab, int top_k) {
+    const bool binned = top_k <= 0 || top_k > 128 || top_k >= vocab, long_row = vocab >= 48 * 1024;
+    if (rows > 4 * 148 && !long_row) return CutShape{256, 4, 1};
+    if (binned && vocab < 12 * 1024) return CutShape{256, 4, 1};
+    if (rows > 2 * 148) return CutShape{512, 4, 1};
+    return CutShape{512, 8, binned && long_row ? (rows <= 74 ? 4 : rows <= 148 ? 2 : 1) : 1};
+}
 
 bool cut_is_on(int vocab, float temperature, int top_k, float top_p) {
     return temperature > 0.0f && ((top_k > 0 && top_k < vocab) || (top_p > 0.0f && top_p < 1.0f));
@@ -1416,16 +1558,39 @@ int launch_cut(const float* a, size_t a_stride, int a_rows, const float* b, size
     if (total == 0) return SPEC_OK;
     const bool vec = vocab % 4 == 0 && a_stride % 4 == 0 && aligned16(a) && (b_rows == 0 || (b_stride % 4 == 0 && aligned16(b)));
     const float c2 = inv_t * kLog2e;
-#define SPEC_LAUNCH_CUT(V, T)                                                                                        \
-    return launch_pdl(cut_floor_kernel<V, T, WORK>, dim3(total), dim3(T), 0, stream, a, a_stride, a_rows, b, b_stride, b_rows, \
-                      vocab, top_k, top_p, c2, floors, work)
-    if (wide_rows(total, vocab)) {
-        if (vec) SPEC_LAUNCH_CUT(true, 1024);
-        SPEC_LAUNCH_CUT(false, 1024);
+    const CutShape shape = cut_shape(total, vocab, top_k);
+    const int ctas = shape.ctas;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(total * ctas);
+    cfg.blockDim = dim3(shape.threads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (pdl_enabled()) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
     }
-    if (vec) SPEC_LAUNCH_CUT(true, 256);
-    SPEC_LAUNCH_CUT(false, 256);
+    if (ctas > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = ctas;
+        attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+#define SPEC_LAUNCH_CUT(T, L, S)                                                                                              \
+    do {                                                                                                                      \
+        if (vec) SPEC_CUDA_TRY(cudaLaunchKernelEx(&cfg, cut_floor_kernel<T, L, true, S, WORK>, a, a_stride, a_rows, b, b_stride,   \
+                                                  b_rows, vocab, top_k, top_p, c2, floors, work));                            \
+        else SPEC_CUDA_TRY(cudaLaunchKernelEx(&cfg, cut_floor_kernel<T, L, false, S, WORK>, a, a_stride, a_rows, b, b_stride, \
+                                              b_rows, vocab, top_k, top_p, c2, floors, work));                                \
+    } while (0)
+    if (ctas > 1) SPEC_LAUNCH_CUT(512, 8, false);
+    else if (shape.threads == 256) SPEC_LAUNCH_CUT(256, 4, true);
+    else if (shape.loads == 4) SPEC_LAUNCH_CUT(512, 4, true);
+    else SPEC_LAUNCH_CUT(512, 8, true);
 #undef SPEC_LAUNCH_CUT
+    return SPEC_OK;
 }
 
 int launch_verify_sample(const float* target_logits, const float* draft_logits, const int32_t* draft_tokens,

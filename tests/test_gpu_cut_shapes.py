@@ -1,0 +1,46 @@
+"""A row's cut is the same however the rows are shared out: alone, where a cluster of thread blocks takes it, among few, among
+as many as fit on the GPU at once and among more (the number of rows at which the launch changes, and one more)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2211_17192_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("top_k,top_p", [(0, 0.9), (40, 1.0), (50, 0.95), (129, 0.9), (300, 1.0)])
+@pytest.mark.parametrize("vocab", [4099, 12288, 49152, 50003])
+def test_floors_and_draws_do_not_depend_on_the_number_of_rows(vocab, top_k, top_p):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(vocab + top_k)
+    few = torch.randn(5, vocab, device="cuda", generator=gen) * torch.tensor([0.5, 1.0, 2.0, 4.0, 8.0], device="cuda")[:, None]
+    few[1, ::3] = 0.25  # heavy ties, where the cut may fall
+    few[2, 7] = -torch.inf
+    u = torch.rand(5, device="cuda", generator=gen)
+    floors = torch.cat([binding.spec_truncation_floors(few[i:i + 1].contiguous(), 0.8, top_k=top_k, top_p=top_p) for i in range(5)])
+    tokens = torch.cat([binding.spec_sample(few[i:i + 1].contiguous(), u[i:i + 1].contiguous(), 0.8, top_k=top_k, top_p=top_p) for i in range(5)])
+    # by hand, in double precision: what a floor keeps is at least k logits, or at least top_p of the mass of what top-k keeps
+    for i in range(5):
+        row = np.sort(few[i].double().cpu().numpy())[::-1]
+        kept = row >= float(floors[i])
+        allowed = row >= row[top_k - 1] if top_k else np.ones_like(kept)
+        mass = np.where(allowed, np.exp((row - row[0]) / 0.8), 0.0)
+        if top_p < 1.0:
+            # (masses are summed in units of 2^-32 of the largest, rounded down, and a weight is good to 2^-21)
+            slack = vocab * 2.0 ** -31 + mass.sum() * 2.0 ** -20
+            assert mass[kept].sum() >= top_p * mass.sum() - slack
+            # and no less would do
+            assert mass[row > float(floors[i])].sum() < top_p * mass.sum() + slack
+        else:
+            assert float(floors[i]) == row[top_k - 1]
+        assert float(few[i, int(tokens[i])]) >= float(floors[i])
+    for rows in (5, 74, 75, 148, 149, 296, 297, 592, 593):
+        many = few.repeat((rows + 4) // 5, 1)[:rows].contiguous()
+        us = u.repeat((rows + 4) // 5)[:rows].contiguous()
+        got = binding.spec_truncation_floors(many, 0.8, top_k=top_k, top_p=top_p)
+        assert torch.equal(got, floors.repeat((rows + 4) // 5)[:rows]), rows
+        drawn = binding.spec_sample(many, us, 0.8, top_k=top_k, top_p=top_p)
+        # (weights are added in another order: 2^-20 of their sum at most, so a uniform number next to a step may fall on
+        # the other side; of five, none is)
+        assert torch.equal(drawn, tokens.repeat((rows + 4) // 5)[:rows]), rows

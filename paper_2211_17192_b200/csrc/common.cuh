@@ -86,6 +86,14 @@ inline T* symbol_address(T& symbol) {
     return static_cast<T*>(p);
 }
 
+// ---- activations ------------------------------------------------------------
+__device__ __forceinline__ float gelu_tanh(float x) {
+    const float k = 0.7978845608028654f;  // sqrt(2 / pi)
+    return 0.5f * x * (1.0f + tanhf(k * (x + 0.044715f * x * x * x)));
+}
+
+__device__ __forceinline__ float silu(float x) { return x / (1.0f + expf(-x)); }
+
 // ---- warp / block primitives ----------------------------------------------
 constexpr unsigned kFullMask = 0xffffffffu;
 

@@ -37,7 +37,7 @@ struct spec_ctx {
     int encoded_batch = 0;
 
     // activations (sized for the wider model)
-    float *h = nullptr, *a = nullptr, *qkv = nullptr, *att = nullptr, *u = nullptr, *f = nullptr;
+    float *h = nullptr, *a = nullptr, *qkv = nullptr, *att = nullptr, *f = nullptr;
     float *target_logits = nullptr, *draft_logits = nullptr;
     // tensor-core GEMM path: bf16 hi/lo copies of the GEMM input, split-K partial sums
     __nv_bfloat16 *x_hi = nullptr, *x_lo = nullptr;
@@ -170,6 +170,7 @@ struct Pass {
     const float* branch = nullptr;
     PartialPlan closing{};  // of the last GEMM that closed a residual branch
     PartialPlan last{};     // of the last projection
+    RowNorm normed{};       // fp32 path: the norm that the next projection applies itself
 
     __nv_bfloat16* hi() const { return ctx->x_hi; }
     __nv_bfloat16* lo() const { return ctx->x_lo; }
@@ -177,6 +178,12 @@ struct Pass {
     // a (fp32) or hi/lo = rmsnorm(h[src(i)]) * gain for i < n
     int norm(const float* gain, const int32_t* src_rows, int n) {
         const int d = m.cfg.d_model;
+        normed = RowNorm{};
+        // (on many rows of a wide model the squares and gains would be half as much work again as the products)
+        if (!tc && !m.bf16() && (n <= 8 || (n <= kMostNormedRows && d <= 512))) {
+            normed = RowNorm{gain, src_rows, m.cfg.rms_eps};
+            return SPEC_OK;
+        }
         const int status = tc ? launch_norm(ctx->h, pending ? branch : nullptr, closing, n_rows, gain, src_rows, n, d,
                                             m.cfg.rms_eps, nullptr, hi(), lo(), st)
                               : launch_norm(ctx->h, nullptr, PartialPlan{}, n_rows, gain, src_rows, n, d, m.cfg.rms_eps, ctx->a, nullptr,
@@ -184,13 +191,14 @@ struct Pass {
         pending = false;
         return status;
     }
-    // y = x . W^T for a consumer that is not the residual stream: partial sums (tc) or `y` (fp32 path, input `x`)
-    int proj(const void* w, const void* pw, int n_out, int k, const float* x, float* y) {
+    // y = rmsnorm(h) . W^T for a consumer that is not the residual stream: partial sums (tc) or `y` (fp32 path; with ffn >= 0
+    // the FFN's function of it)
+    int proj(const void* w, const void* pw, int n_out, int k, float* y, int ffn = -1) {
         if (tc) {
             last = gemm_tc_plan(n_out, k, n_rows);
             return launch_gemm_tc_partials(hi(), lo(), ctx->hi_rows, pw, true, n_rows, n_out, k, ctx->partials, st);
         }
-        return launch_gemm_rows(x, w, m.bf16(), nullptr, nullptr, n_rows, n_out, k, y, st);
+        return launch_gemm_rows(normed.gain ? ctx->h : ctx->a, w, m.bf16(), nullptr, nullptr, n_rows, n_out, k, y, st, normed, ffn);
     }
     // h += x . W^T
     int residual(const void* w, const void* pw, int k, const float* x) {
@@ -208,9 +216,12 @@ struct Pass {
     int ffn(const spec_layer_weights& w, const spec_layer_weights& pw) {
         const spec_model_cfg& c = m.cfg;
         SPEC_TRY(norm(w.ln2, nullptr, n_rows));
-        SPEC_TRY(proj(w.w_in, pw.w_in, m.ffn_in_dim(), c.d_model, ctx->a, ctx->u));
-        SPEC_TRY(launch_ffn_act(tc ? nullptr : ctx->u, partials(), last, n_rows, c.d_ff, c.ffn, tc ? nullptr : ctx->f,
-                                tc ? hi() : nullptr, tc ? lo() : nullptr, st));
+        if (tc) {
+            SPEC_TRY(proj(w.w_in, pw.w_in, m.ffn_in_dim(), c.d_model, nullptr));
+            SPEC_TRY(launch_ffn_act(ctx->partials, last, n_rows, c.d_ff, c.ffn, hi(), lo(), st));
+        } else {
+            SPEC_TRY(proj(w.w_in, pw.w_in, c.d_ff, c.d_model, ctx->f, c.ffn));
+        }
         return residual(w.w_out, pw.w_out, c.d_ff, ctx->f);
     }
     // h += Wo . attention(projection of rmsnorm(h) * gain) over `pool`
@@ -219,7 +230,7 @@ struct Pass {
                        int max_keys, const PromptSegments* segs = nullptr) {
         const spec_model_cfg& c = m.cfg;
         SPEC_TRY(norm(w.ln1, nullptr, n_rows));
-        SPEC_TRY(proj(w.wqkv, pw.wqkv, m.qkv_dim(), c.d_model, ctx->a, ctx->qkv));
+        SPEC_TRY(proj(w.wqkv, pw.wqkv, m.qkv_dim(), c.d_model, ctx->qkv));
         SPEC_TRY(launch_qkv(c.n_heads, c.n_kv_heads, c.d_head, c.arch == SPEC_ARCH_LLAMA ? m.rope_table : nullptr, pool, rows,
                             n_rows, ctx->qkv, partials(), last, st));
         const AttnSource src{ctx->qkv, m.qkv_dim(), pool, kv_len, bias, bias_span, bias_zero};
@@ -336,7 +347,7 @@ int forward(spec_ctx* ctx, const Model& m, const RowMeta& rows, int batch, int m
                                      ctx->rt.max_len - 1, ctx->rt.max_len, segs));
         if (m.t5()) {  // cross-attention over the source's K,V (every row sees every source position)
             SPEC_TRY(pass.norm(w.lnx, nullptr, n_rows));
-            SPEC_TRY(pass.proj(w.wq_x, pw.wq_x, m.q_dim(), d, ctx->a, ctx->qkv));
+            SPEC_TRY(pass.proj(w.wq_x, pw.wq_x, m.q_dim(), d, ctx->qkv));
             if (pass.tc)  // the partial sums become the query rows
                 SPEC_TRY(launch_qkv(c.n_heads, 0, c.d_head, nullptr, KvPool{}, rows, n_rows, ctx->qkv, ctx->partials,
                                     pass.last, ctx->stream));
@@ -355,7 +366,8 @@ int forward(spec_ctx* ctx, const Model& m, const RowMeta& rows, int batch, int m
             SPEC_TRY(launch_gemm_tc(pass.hi(), pass.lo(), ctx->hi_rows, m.packed_head, true, nullptr, logit_dst, n_logit_rows,
                                     c.vocab, d, ctx->partials, logits, ctx->stream, logits_slot));
         else
-            SPEC_TRY(launch_gemm_rows(ctx->a, m.head, m.bf16(), nullptr, logit_dst, n_logit_rows, c.vocab, d, logits, ctx->stream));
+            SPEC_TRY(launch_gemm_rows(pass.normed.gain ? ctx->h : ctx->a, m.head, m.bf16(), nullptr, logit_dst, n_logit_rows, c.vocab, d,
+                                      logits, ctx->stream, pass.normed));
     }
     return SPEC_OK;
 }
@@ -381,7 +393,7 @@ int encode(spec_ctx* ctx, const Model& m, int batch, int m_rows) {
     for (int l = 0; l < c.n_layers; ++l) {
         const spec_layer_weights& w = m.layers[l];
         const spec_layer_weights& pw = pass.tc ? m.packed[l] : w;
-        SPEC_TRY(pass.proj(w.wkv_x, pw.wkv_x, 2 * m.kv_dim(), c.d_model, ctx->a, ctx->qkv));
+        SPEC_TRY(pass.proj(w.wkv_x, pw.wkv_x, 2 * m.kv_dim(), c.d_model, ctx->qkv));
         const KvPool pool = source_pool(ctx, m, static_cast<char*>(m.cross_kv) + static_cast<size_t>(l) * m.cross_stride);
         SPEC_TRY(launch_qkv(0, c.n_kv_heads, c.d_head, nullptr, pool, rows, n_rows, ctx->qkv, pass.partials(),
                             pass.last, ctx->stream));
@@ -871,13 +883,12 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     if (status == SPEC_OK && draft_cfg) status = init_model(ctx, 1, *draft_cfg, *draft_weights);
     if (status != SPEC_OK) return cleanup(status);
 
-    size_t d = 0, qkv = 0, att = 0, fin = 0, ff = 0;
+    size_t d = 0, qkv = 0, att = 0, ff = 0;
     for (int i = 0; i < (ctx->has_draft ? 2 : 1); ++i) {
         const Model& m = ctx->model[i];
         d = std::max<size_t>(d, m.cfg.d_model);
         qkv = std::max<size_t>(qkv, m.qkv_dim());
         att = std::max<size_t>(att, m.q_dim());
-        fin = std::max<size_t>(fin, m.ffn_in_dim());
         ff = std::max<size_t>(ff, m.cfg.d_ff);
     }
     const size_t R = ctx->max_rows, B = rt.max_batch, G = rt.max_gamma, V = target_cfg->vocab;
@@ -891,7 +902,6 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     if (any_fp32) {
         SPEC_ALLOC(a, R * d);
         SPEC_ALLOC(att, R * att);
-        SPEC_ALLOC(u, R * fin);
         SPEC_ALLOC(f, R * ff);
     }
     {

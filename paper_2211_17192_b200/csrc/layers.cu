@@ -287,18 +287,10 @@ __global__ void copy_logits_kernel(const int32_t* tokens, int max_len, const int
         out[v] = v == guess ? 0.0f : -INFINITY;
 }
 
-__device__ __forceinline__ float gelu_tanh(float x) {
-    const float k = 0.7978845608028654f;  // sqrt(2 / pi)
-    return 0.5f * x * (1.0f + tanhf(k * (x + 0.044715f * x * x * x)));
-}
-
-__device__ __forceinline__ float silu(float x) { return x / (1.0f + expf(-x)); }
-
-// f = gelu(u)  |  gelu(gate) * up  |  silu(gate) * up, with u either given in
-// full or as the partial sums of the FFN-in GEMM.  grid = (ceil(d_ff / 4 / block), rows): four columns per thread.
+// f = gelu(u)  |  gelu(gate) * up  |  silu(gate) * up, with u the partial sums of the FFN-in GEMM, as two bf16 terms.
+// grid = (ceil(d_ff / 4 / block), rows): four columns per thread.
 template <int FFN>
-__global__ void ffn_act_kernel(const float* u, const float* partial, const PartialPlan plan, int n_rows,
-                               int d_ff, float* f, __nv_bfloat16* f_hi,
+__global__ void ffn_act_kernel(const float* partial, const PartialPlan plan, int n_rows, int d_ff, __nv_bfloat16* f_hi,
                                __nv_bfloat16* f_lo) {
     pdl_trigger();
     pdl_wait();
@@ -309,36 +301,29 @@ __global__ void ffn_act_kernel(const float* u, const float* partial, const Parti
     const size_t stride = static_cast<size_t>(n_rows) * width;
     const size_t at = static_cast<size_t>(r) * width + c;
     float4 g = make_float4(0.f, 0.f, 0.f, 0.f), up = g;
-    if (!partial) {
-        g = *reinterpret_cast<const float4*>(u + at);
-        if (kGated) up = *reinterpret_cast<const float4*>(u + at + d_ff);
+    const int n_gate = partial_count(plan, r, c), n_up = kGated ? partial_count(plan, r, c + d_ff) : n_gate;
+    if (kGated && n_gate == n_up) {
+        const size_t where[2] = {at, at + d_ff};
+        float4 both[2] = {g, g};
+        sum_partials<2, 4>(partial, n_gate, stride, where, both);
+        g = both[0];
+        up = both[1];
     } else {
-        const int n_gate = partial_count(plan, r, c), n_up = kGated ? partial_count(plan, r, c + d_ff) : n_gate;
-        if (kGated && n_gate == n_up) {
-            const size_t where[2] = {at, at + d_ff};
-            float4 both[2] = {g, g};
-            sum_partials<2, 4>(partial, n_gate, stride, where, both);
-            g = both[0];
-            up = both[1];
-        } else {
-            const size_t where[1] = {at};
-            float4 one[1] = {g};
-            sum_partials<1, 8>(partial, n_gate, stride, where, one);
-            g = one[0];
-            if (kGated) {
-                const size_t where_up[1] = {at + d_ff};
-                sum_partials<1, 8>(partial, n_up, stride, where_up, one);
-                up = one[0];
-            }
+        const size_t where[1] = {at};
+        float4 one[1] = {g};
+        sum_partials<1, 8>(partial, n_gate, stride, where, one);
+        g = one[0];
+        if (kGated) {
+            const size_t where_up[1] = {at + d_ff};
+            sum_partials<1, 8>(partial, n_up, stride, where_up, one);
+            up = one[0];
         }
     }
     float4 y;
     if (FFN == SPEC_FFN_GELU) y = make_float4(gelu_tanh(g.x), gelu_tanh(g.y), gelu_tanh(g.z), gelu_tanh(g.w));
     else if (FFN == SPEC_FFN_SWIGLU) y = make_float4(silu(g.x) * up.x, silu(g.y) * up.y, silu(g.z) * up.z, silu(g.w) * up.w);
     else y = make_float4(gelu_tanh(g.x) * up.x, gelu_tanh(g.y) * up.y, gelu_tanh(g.z) * up.z, gelu_tanh(g.w) * up.w);
-    const size_t i = static_cast<size_t>(r) * d_ff + c;
-    if (f) *reinterpret_cast<float4*>(f + i) = y;
-    if (f_hi) store_split4(f_hi, f_lo, i, y);
+    store_split4(f_hi, f_lo, static_cast<size_t>(r) * d_ff + c, y);
 }
 
 }  // namespace
@@ -402,12 +387,12 @@ int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, cons
                       pool.pages_per_seq, pool.page_size);
 }
 
-int launch_ffn_act(const float* u, const float* partial, const PartialPlan& plan, int n_rows, int d_ff, int ffn, float* f,
-                   __nv_bfloat16* f_hi, __nv_bfloat16* f_lo, cudaStream_t stream) {
+int launch_ffn_act(const float* partial, const PartialPlan& plan, int n_rows, int d_ff, int ffn, __nv_bfloat16* f_hi,
+                   __nv_bfloat16* f_lo, cudaStream_t stream) {
     const int threads = n_rows <= 16 ? 64 : 256;
     const dim3 grid((d_ff / 4 + threads - 1) / threads, n_rows);
 #define SPEC_LAUNCH_ACT(F) \
-    return launch_pdl(ffn_act_kernel<F>, grid, dim3(threads), 0, stream, u, partial, plan, n_rows, d_ff, f, f_hi, f_lo)
+    return launch_pdl(ffn_act_kernel<F>, grid, dim3(threads), 0, stream, partial, plan, n_rows, d_ff, f_hi, f_lo)
     if (ffn == SPEC_FFN_GELU) SPEC_LAUNCH_ACT(SPEC_FFN_GELU);
     if (ffn == SPEC_FFN_SWIGLU) SPEC_LAUNCH_ACT(SPEC_FFN_SWIGLU);
     SPEC_LAUNCH_ACT(SPEC_FFN_GATED_GELU);

@@ -100,8 +100,16 @@ int launch_norm(float* h, const float* partial, const PartialPlan& plan, int row
 
 // y[dst(r)] = x[r] . W^T (+ residual[r]) on the FMA pipes;  W is [n_out, k] row-major in fp32 or bf16.
 // dst(r) = dst_rows ? dst_rows[r] : r.  y and residual may alias.
+// With norm.gain, fp32 weights and at most kMostNormedRows rows, rmsnorm(x[src(r)]) * gain stands for x[r]; with ffn >= 0 (and
+// fp32 weights) W is the FFN's first matrix and y[r], n_out wide, what its function makes of the product.
+constexpr int kMostNormedRows = 64;
+struct RowNorm {
+    const float* gain = nullptr;
+    const int32_t* src_rows = nullptr;
+    float eps = 0.0f;
+};
 int launch_gemm_rows(const float* x, const void* w, bool w_bf16, const float* residual, const int32_t* dst_rows,
-                     int n_rows, int n_out, int k, float* y, cudaStream_t stream);
+                     int n_rows, int n_out, int k, float* y, cudaStream_t stream, const RowNorm& norm = RowNorm{}, int ffn = -1);
 
 // Tensor-core path for bf16 weights (gemm_tc.cu): x arrives as two bf16 terms;
 // launch_gemm_tc_partials leaves the split-K partial sums [splits][n_rows][n_out]
@@ -193,9 +201,9 @@ bool prompt_attention_serves(const Model& m, long long query_keys);
 int launch_prompt_attention(const Model& m, const AttnSource& src, const PromptSegments& segs, __nv_bfloat16* att_hi,
                             __nv_bfloat16* att_lo, cudaStream_t stream);
 
-// f = gelu(u)  |  gelu(u[:, :F]) * u[:, F:]  |  silu(u[:, :F]) * u[:, F:], u given in full or as partial sums.
-int launch_ffn_act(const float* u, const float* partial, const PartialPlan& plan, int n_rows, int d_ff, int ffn, float* f,
-                   __nv_bfloat16* f_hi, __nv_bfloat16* f_lo, cudaStream_t stream);
+// f = gelu(u)  |  gelu(u[:, :F]) * u[:, F:]  |  silu(u[:, :F]) * u[:, F:], u the partial sums, f two bf16 terms.
+int launch_ffn_act(const float* partial, const PartialPlan& plan, int n_rows, int d_ff, int ffn, __nv_bfloat16* f_hi,
+                   __nv_bfloat16* f_lo, cudaStream_t stream);
 
 // mega.cu: one forward pass over at most 16 rows as one persistent cooperative kernel
 // (bf16 decoder-only models).

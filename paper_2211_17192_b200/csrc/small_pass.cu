@@ -196,11 +196,6 @@ __device__ __forceinline__ float exp2_fast(float x) {
     return y;
 }
 __device__ __forceinline__ float clamp_half(float x) { return __half2float(__float2half_rn(fminf(fmaxf(x, -65504.0f), 65504.0f))); }
-__device__ __forceinline__ float small_gelu(float x) {
-    const float k = 0.7978845608028654f;  // sqrt(2 / pi)
-    return 0.5f * x * (1.0f + tanhf(k * (x + 0.044715f * x * x * x)));
-}
-
 // One CTA's view of the pass.  KI = d / 256: k-steps per warp.
 template <int KI, int R>
 struct Pass {
@@ -784,9 +779,9 @@ struct Pass {
                 float y = summed(u * per, v) * scale;
                 if (a.gated) {
                     const float up = summed(u * per + 1, v) * scale;
-                    y = (a.ffn == SPEC_FFN_SWIGLU ? y / (1.0f + expf(-y)) : small_gelu(y)) * up;
+                    y = (a.ffn == SPEC_FFN_SWIGLU ? silu(y) : gelu_tanh(y)) * up;
                 } else {
-                    y = small_gelu(y);
+                    y = gelu_tanh(y);
                 }
                 const __nv_bfloat16 hi = __float2bfloat16_rn(y);
                 ah[(u * kRows + row) * 16 + f] = hi;

@@ -16,7 +16,7 @@
 // rows' buffers leave room for, refilled after every barrier that follows a read, which so runs ahead across every wait.
 // The rows (at most 8) are the N side, as two bf16 terms.  With K cut over 16 warps the B fragments of a whole phase sit in
 // registers.  The factor per row of the norms is applied to the projections' sums, not to their inputs: a projection
-// starts when the residual stream is there.  The first keys of a warp load while the projection runs.
+// starts when the residual stream is there.  The first keys of a warp load while the projection's sums are made.
 //
 // What is left is the length of the chain of such steps, a third of it waiting for another SM, and instruction issue: the
 // code runs once per block, straight through.  So every loop that is not a handful of instructions stays a loop, and what
@@ -26,8 +26,8 @@
 // Every wait is bounded.  A wait that runs out is recorded and the kernel goes on with whatever is there (nobody leaves:
 // the others count on it); further waits then give up at once.
 //
-// Measured, a whole pass with its head, chain of kernels against this: 160M shape, one row at context 1024 351 -> 203 us,
-// four sequences at 777 397 -> 268, eight at 500 411 -> 340; 97M shape, six rows at 200 348 -> 248, eight sequences at 500
+// Measured, a whole pass with its head, chain of kernels against this: 160M shape, one row at context 1024 351 -> 199 us,
+// four sequences at 777 397 -> 267, eight at 500 411 -> 340; 97M shape, six rows at 200 348 -> 245, eight sequences at 500
 // 393 -> 324; 6M shape 56 -> 29; decoder of the small T5 shape, one row 257 -> 121, eight sequences 272 -> 193.  More rows
 // would need a second column tile per fragment and twice the shared memory: the chain takes them.
 #include <algorithm>
@@ -472,16 +472,16 @@ struct Pass {
         ++epoch;
         uint32_t bh[KI][2], bl[KI][2];
         weighted(bh, bl);
-        if (key < n_keys) {  // (back by the time that the scores need them)
-            kr = key_rows(pool, page, n_keys, key);
-            load_k(x.k, kr);
-        }
         const int n_tiles = cross ? group * 4 : qkv_tiles(group);
         const int tiles = tiles_of(n_tiles, rank);
         const int width = (group + 2) * kDh;
         await_bytes(kBarQ, a.rows * n_tiles * 16 * 4);
         project(0, tiles, bh, bl);
-        if (key < n_keys) load_v(x.v, kr);
+        if (key < n_keys) {  // (back by the time that the scores need them; asked for earlier they only cost registers)
+            kr = key_rows(pool, page, n_keys, key);
+            load_k(x.k, kr);
+            load_v(x.v, kr);
+        }
         sync_consumers();
         refill();
         // Rotary positions, the scale of the scores (in base-2 units), the rounding of cached rows, and off to the cluster.

@@ -15,6 +15,8 @@
 //      the warp whose segment holds the target walks it without another trip to
 //      memory.  It is chained with programmatic dependent launch, so its launch
 //      latency and prologue overlap the tail of the first kernel.
+// With few logits, where launches are what a call costs, one kernel does both (one_kernel); with a cut the selection kernel
+// leaves the statistics (cut_floor_kernel).
 #include <algorithm>
 #include <cfloat>
 #include <mutex>
@@ -39,7 +41,7 @@ constexpr int kCdfBatch = 8;            // groups fetched per thread before any 
 constexpr int kClusterCdfBatch = 4;     // the same when a cluster shares the row
 constexpr int kWalkBatch = 4;           // 128-element steps fetched at once by the final walk
 constexpr int kMaxCluster = 4;          // CTAs per sequence in the finishing kernel
-constexpr int kMostParts = 64;          // warps that share an inverse CDF: four CTAs of 16
+constexpr int kMostParts = 128;         // warps that share an inverse CDF: eight CTAs of 16
 constexpr int kSampleThreads = 512;
 constexpr int kMaxGamma = 64;
 constexpr int kMaxRows = 2 * kMaxGamma + 1;
@@ -478,40 +480,17 @@ struct __align__(16) ChunkStat {
     float bad;     // T = 0: non-zero if the chunk holds a NaN or +inf logit (T > 0: the sums show it)
 };
 
-// grid = (chunks, rows, batch); rows = 2*gamma+1 (T > 0: p_1..p_{gamma+1}, q_1..q_gamma)
-// or gamma+1 (T = 0: only p is read).
-template <bool GREEDY, bool VEC>
-__global__ void __launch_bounds__(kStatThreads)
-verify_stats_kernel(const float* __restrict__ target_logits, const float* __restrict__ draft_logits,
-                    const int32_t* __restrict__ draft_tokens, int gamma, int vocab, float c2, ChunkStat* __restrict__ stats) {
-    __shared__ float red[kStatWarps];
-    __shared__ float red_s[kStatWarps];
-    __shared__ int red_i[kStatWarps];
-    pdl_trigger();  // the finishing kernel's CTAs may take their places as this grid drains
-    pdl_wait();
+template <int W>
+struct StatShared {
+    float max[W], sum[W];
+    int index[W];
+};
+
+// The statistics of groups [g0, g1) of a row by a CTA of T threads; valid in thread 0, the logit at the drafted token left out.
+template <int T, bool GREEDY, bool VEC>
+__device__ __forceinline__ float4 chunk_statistics(const Row<VEC>& r, int g0, int g1, float c2, StatShared<T / 32>& sh) {
+    constexpr int W = T / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int chunk = blockIdx.x, chunks = gridDim.x;
-    const int row = blockIdx.y, rows = gridDim.y;
-    const int b = blockIdx.z;
-
-    const float* src = row <= gamma
-        ? target_logits + (static_cast<size_t>(b) * (gamma + 1) + row) * vocab
-        : draft_logits + (static_cast<size_t>(b) * gamma + (row - gamma - 1)) * vocab;
-    const Row<VEC> r = make_row<VEC>(src, vocab);
-    const int groups = r.groups();
-    const int per_chunk = (groups + chunks - 1) / chunks;
-    const int g0 = chunk * per_chunk;
-    const int g1 = min(groups, g0 + per_chunk);
-
-    // The drafted token this row is tested at (none for p_{gamma+1}): thread 0
-    // fetches the row's logit there if it lies in this chunk, so the accept test
-    // needs no further trip to memory.
-    float xlogit = 0.0f;
-    if (tid == 0 && !GREEDY && row != gamma) {
-        const int x = draft_tokens[static_cast<size_t>(b) * gamma + (row < gamma ? row : row - gamma - 1)];
-        if (x >= 0 && x < vocab && x + r.shift >= 4 * g0 && x + r.shift < 4 * g1) xlogit = __ldg(src + x);
-    }
-
     // Every thread streams groups g0+tid, g0+tid+T, ... with kUnroll 128-bit
     // loads in flight and keeps a running (max, sum exp) pair that is rescaled
     // when the maximum moves; one block-wide merge at the end.
@@ -520,17 +499,17 @@ verify_stats_kernel(const float* __restrict__ target_logits, const float* __rest
     float s = 0.0f;
     int arg = 0x7fffffff;
     bool bad = false;  // T = 0 only: a NaN or +inf logit (the comparisons below would pass over a NaN in silence)
-    for (int base = g0 + tid; base < g1; base += kUnroll * kStatThreads) {
+    for (int base = g0 + tid; base < g1; base += kUnroll * T) {
         float4 v[kUnroll];
 #pragma unroll
         for (int i = 0; i < kUnroll; ++i) {
-            const int g = base + i * kStatThreads;
+            const int g = base + i * T;
             v[i] = g < g1 ? r.load(g, kPad) : make_float4(kPad, kPad, kPad, kPad);
         }
         if (GREEDY) {
 #pragma unroll
             for (int i = 0; i < kUnroll; ++i) {
-                const int j = 4 * (base + i * kStatThreads) - r.shift;  // indices grow with i: '>' keeps the lowest on ties
+                const int j = 4 * (base + i * T) - r.shift;  // indices grow with i: '>' keeps the lowest on ties
                 if (v[i].x > m) { m = v[i].x; arg = j; }
                 if (v[i].y > m) { m = v[i].y; arg = j + 1; }
                 if (v[i].z > m) { m = v[i].z; arg = j + 2; }
@@ -553,25 +532,60 @@ verify_stats_kernel(const float* __restrict__ target_logits, const float* __rest
                      (fast_exp2(fmaf(v[i].z, c2, mc)) + fast_exp2(fmaf(v[i].w, c2, mc)));
         }
     }
-    ChunkStat* out = stats + (static_cast<size_t>(b) * rows + row) * chunks + chunk;
     if (GREEDY) {
         const int any_bad = __syncthreads_or(bad ? 1 : 0);
-        block_argmax<kStatWarps>(m, arg, red, red_i);
-        if (tid == 0) *reinterpret_cast<float4*>(out) = make_float4(m, __int_as_float(arg), 0.0f, any_bad ? 1.0f : 0.0f);
+        block_argmax<W>(m, arg, sh.max, sh.index);
+        return make_float4(m, __int_as_float(arg), 0.0f, any_bad ? 1.0f : 0.0f);
     } else {
         const float wm = warp_max(m);
         s = warp_sum(s * fast_exp2((m - wm) * c2));
-        if (lane == 0) { red[warp] = wm; red_s[warp] = s; }
+        if (lane == 0) { sh.max[warp] = wm; sh.sum[warp] = s; }
         __syncthreads();
+        float bm = sh.max[0], t = 0.0f;
         if (tid == 0) {
-            float bm = red[0];
 #pragma unroll
-            for (int i = 1; i < kStatWarps; ++i) bm = fmaxf(bm, red[i]);
-            float t = 0.0f;
+            for (int i = 1; i < W; ++i) bm = fmaxf(bm, sh.max[i]);
 #pragma unroll
-            for (int i = 0; i < kStatWarps; ++i) t += red_s[i] * fast_exp2((red[i] - bm) * c2);
-            *reinterpret_cast<float4*>(out) = make_float4(bm, t, xlogit, 0.0f);
+            for (int i = 0; i < W; ++i) t += sh.sum[i] * fast_exp2((sh.max[i] - bm) * c2);
         }
+        return make_float4(bm, t, 0.0f, 0.0f);
+    }
+}
+
+// The logits of row `row` of a sequence: p_1..p_{gamma+1}, q_1..q_gamma.
+__device__ __forceinline__ const float* verify_row(const float* target_logits, const float* draft_logits, int b, int row, int gamma, int vocab) {
+    return row <= gamma ? target_logits + (static_cast<size_t>(b) * (gamma + 1) + row) * vocab
+                        : draft_logits + (static_cast<size_t>(b) * gamma + (row - gamma - 1)) * vocab;
+}
+// Its logit at the drafted token (none for p_{gamma+1}) if that lies in groups [g0, g1): the accept test then needs no further
+// trip to memory.
+template <bool VEC>
+__device__ __forceinline__ float verify_logit(const Row<VEC>& r, const int32_t* draft_tokens, int b, int row, int gamma, int g0, int g1) {
+    if (row == gamma) return 0.0f;
+    const int x = draft_tokens[static_cast<size_t>(b) * gamma + (row < gamma ? row : row - gamma - 1)];
+    return x >= 0 && x < r.vocab && x + r.shift >= 4 * g0 && x + r.shift < 4 * g1 ? __ldg(r.base + x) : 0.0f;
+}
+
+// grid = (chunks, rows, batch); rows = 2*gamma+1 (T > 0: p_1..p_{gamma+1}, q_1..q_gamma)
+// or gamma+1 (T = 0: only p is read).
+template <bool GREEDY, bool VEC>
+__global__ void __launch_bounds__(kStatThreads)
+verify_stats_kernel(const float* __restrict__ target_logits, const float* __restrict__ draft_logits,
+                    const int32_t* __restrict__ draft_tokens, int gamma, int vocab, float c2, ChunkStat* __restrict__ stats) {
+    __shared__ StatShared<kStatWarps> sh;
+    pdl_trigger();  // the finishing kernel's CTAs may take their places as this grid drains
+    pdl_wait();
+    const int chunk = blockIdx.x, chunks = gridDim.x, row = blockIdx.y, rows = gridDim.y, b = blockIdx.z;
+    const Row<VEC> r = make_row<VEC>(verify_row(target_logits, draft_logits, b, row, gamma, vocab), vocab);
+    const int groups = r.groups();
+    const int per_chunk = (groups + chunks - 1) / chunks;
+    const int g0 = chunk * per_chunk, g1 = min(groups, g0 + per_chunk);
+    float xlogit = 0.0f;
+    if (threadIdx.x == 0 && !GREEDY) xlogit = verify_logit(r, draft_tokens, b, row, gamma, g0, g1);
+    float4 found = chunk_statistics<kStatThreads, GREEDY, VEC>(r, g0, g1, c2, sh);
+    if (threadIdx.x == 0) {
+        if (!GREEDY) found.z = xlogit;
+        *reinterpret_cast<float4*>(stats + (static_cast<size_t>(b) * rows + row) * chunks + chunk) = found;
     }
 }
 
@@ -589,11 +603,12 @@ struct FinishShared {
 // after the statistics: merge, accept tests, adjusted distribution, draw.  The
 // cheap decision part is repeated in every CTA of the cluster; the pass over
 // row n+1 is split between them.
-template <bool GREEDY, bool VEC, bool CUT>
+// ALONE: the statistics too, a row at a time to each CTA (one_kernel).
+template <bool GREEDY, bool VEC, bool CUT, bool ALONE>
 __global__ void __launch_bounds__(kFinishThreads, 2)
 verify_finish_kernel(const float* __restrict__ target_logits, const float* __restrict__ draft_logits,
                      const int32_t* __restrict__ draft_tokens, const float* __restrict__ uniforms, int gamma,
-                     int vocab, float inv_t, int chunks, int cluster_size, const ChunkStat* __restrict__ stats,
+                     int vocab, float inv_t, int chunks, int cluster_size, ChunkStat* stats,
                      const float* __restrict__ final_uniforms, float lenience, const float* __restrict__ floors,
                      int32_t* __restrict__ n_accepted, int32_t* __restrict__ next_token, int* __restrict__ nonfinite) {
     __shared__ FinishShared sh;
@@ -607,6 +622,19 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
 
     // Inputs that the statistics kernel does not produce can be fetched before
     // waiting for it.
+    if (ALONE) {
+        pdl_trigger();
+        __shared__ StatShared<kFinishThreads / 32> stat;
+        for (int row = rank; row < rows; row += cluster_size) {
+            const Row<VEC> r = make_row<VEC>(verify_row(target_logits, draft_logits, b, row, gamma, vocab), vocab);
+            float4 found = chunk_statistics<kFinishThreads, GREEDY, VEC>(r, 0, r.groups(), c2, stat);
+            if (tid == 0) {
+                if (!GREEDY) found.z = verify_logit(r, draft_tokens, b, row, gamma, 0, r.groups());
+                *reinterpret_cast<float4*>(stats + static_cast<size_t>(b) * rows + row) = found;
+            }
+            __syncthreads();  // (`stat` is used again)
+        }
+    }
     float my_uniform = 0.5f;
     if (!GREEDY && tid <= gamma) my_uniform = __ldg(uniforms + static_cast<size_t>(b) * (gamma + 1) + tid);
     int my_x = -1;
@@ -618,8 +646,12 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
     // The generation loop keys the final draw by the position it decides, which depends on n: it passes one
     // candidate uniform per possible n; all of them are fetched now.
     if (!GREEDY && final_uniforms && tid <= gamma) sh.u_cand[tid] = __ldg(final_uniforms + static_cast<size_t>(b) * (gamma + 1) + tid);
-    pdl_trigger();
-    pdl_wait();
+    if (ALONE) {
+        cg::this_cluster().sync();  // (every CTA sees the others' statistics)
+    } else {
+        pdl_trigger();
+        pdl_wait();
+    }
 
     // merge the chunk statistics of row `tid` (eight loads in flight at a time)
     if (tid < rows) {
@@ -1497,6 +1529,16 @@ int finish_cluster_size(int vocab) {
     return c;
 }
 
+// One kernel for statistics and decision, where a call is bound by its launches and not by the GPU: a lone decision of
+// 4 x 8192 logits takes the host 10.5 us instead of 12.3, at 7.9 us of the GPU instead of 6.5 (a cluster of eight SMs reads all
+// rows, and nothing of it overlaps the call before).  The line is where the GPU's time meets the host's: 7 rows of 32000
+// 9.6, 11 rows of 32000 11.7, 17 of 32000 13.7, 7 of 50003 11.9 (two kernels: 12.3 of the host); at T = 0, 4 x 128000
+// 8.7, 9 x 128000 14.1.  The generation loop replays a graph, to which only the GPU's time matters: never there.
+constexpr int kMostAlone = 8;  // CTAs to a sequence
+bool one_kernel(int batch, int rows, int vocab, bool greedy) {
+    return batch <= 8 && static_cast<long long>((rows + kMostAlone - 1) / kMostAlone) * vocab <= (greedy ? 128 * 1024 : 32 * 1024);
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 int chunks_for(int vocab, int rows_total) {
@@ -1602,12 +1644,13 @@ int launch_verify_sample(const float* target_logits, const float* draft_logits, 
     const float inv_t = greedy ? 0.0f : 1.0f / temperature;
     ChunkStat* stats = static_cast<ChunkStat*>(workspace);
     const bool cut = cut_is_on(vocab, temperature, top_k, top_p);  // never with greedy
-    const int chunks = cut ? 1 : chunks_for(vocab, rows * batch);
+    const bool alone = !cut && !final_uniforms && one_kernel(batch, rows, vocab, greedy);
+    const int chunks = cut || alone ? 1 : chunks_for(vocab, rows * batch);
     const dim3 grid(chunks, rows, batch);
     const bool vec = vocab % 4 == 0 && aligned16(target_logits) && (greedy || gamma == 0 || aligned16(draft_logits));
     const float c2 = inv_t * kLog2e;
     const float* floors = nullptr;
-    int status;
+    int status = SPEC_OK;
 #define SPEC_LAUNCH_STATS(G, V)                                                                                  \
     status = launch_pdl(verify_stats_kernel<G, V>, grid, dim3(kStatThreads), 0, stream, target_logits, draft_logits, \
                         draft_tokens, gamma, vocab, c2, stats)
@@ -1620,6 +1663,7 @@ int launch_verify_sample(const float* target_logits, const float* draft_logits, 
         status = launch_cut<kWithStats>(target_logits, static_cast<size_t>(vocab), gamma + 1, draft_logits, static_cast<size_t>(vocab),
                                         gamma, batch, vocab, top_k, top_p, inv_t, f, work, stream);
         floors = f;
+    } else if (alone) {
     } else if (greedy && vec) SPEC_LAUNCH_STATS(true, true);
     else if (greedy) SPEC_LAUNCH_STATS(true, false);
     else if (vec) SPEC_LAUNCH_STATS(false, true);
@@ -1628,7 +1672,7 @@ int launch_verify_sample(const float* target_logits, const float* draft_logits, 
     if (status != SPEC_OK) return status;
 
     // One cluster per sequence; more CTAs per cluster for longer rows.
-    const int cluster_size = greedy ? 1 : finish_cluster_size(vocab);
+    const int cluster_size = alone ? std::min(kMostAlone, rows) : greedy ? 1 : finish_cluster_size(vocab);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(batch * cluster_size);
     cfg.blockDim = dim3(kFinishThreads);
@@ -1642,18 +1686,21 @@ int launch_verify_sample(const float* target_logits, const float* draft_logits, 
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl_enabled() ? 2 : 1;
-    const ChunkStat* stats_in = stats;
-#define SPEC_LAUNCH_FINISH(G, V, C)                                                                                  \
-    SPEC_CUDA_TRY(cudaLaunchKernelEx(&cfg, verify_finish_kernel<G, V, C>, target_logits, draft_logits, draft_tokens, \
-                                     uniforms, gamma, vocab, inv_t, chunks, cluster_size, stats_in,                 \
-                                     final_uniforms, lenience, floors, n_accepted, next_token, nonfinite))
-    if (greedy && vec) SPEC_LAUNCH_FINISH(true, true, false);
-    else if (greedy) SPEC_LAUNCH_FINISH(true, false, false);
-    else if (vec && cut) SPEC_LAUNCH_FINISH(false, true, true);
-    else if (vec) SPEC_LAUNCH_FINISH(false, true, false);
-    else if (cut) SPEC_LAUNCH_FINISH(false, false, true);
-    else SPEC_LAUNCH_FINISH(false, false, false);
+    cfg.numAttrs = pdl_enabled() && !alone ? 2 : 1;  // (the logits are read through the non-coherent path, right after the start)
+#define SPEC_LAUNCH_FINISH(G, V, C, A)                                                                                  \
+    SPEC_CUDA_TRY(cudaLaunchKernelEx(&cfg, verify_finish_kernel<G, V, C, A>, target_logits, draft_logits, draft_tokens, \
+                                     uniforms, gamma, vocab, inv_t, chunks, cluster_size, stats, final_uniforms,       \
+                                     lenience, floors, n_accepted, next_token, nonfinite))
+    if (alone && greedy && vec) SPEC_LAUNCH_FINISH(true, true, false, true);
+    else if (alone && greedy) SPEC_LAUNCH_FINISH(true, false, false, true);
+    else if (alone && vec) SPEC_LAUNCH_FINISH(false, true, false, true);
+    else if (alone) SPEC_LAUNCH_FINISH(false, false, false, true);
+    else if (greedy && vec) SPEC_LAUNCH_FINISH(true, true, false, false);
+    else if (greedy) SPEC_LAUNCH_FINISH(true, false, false, false);
+    else if (vec && cut) SPEC_LAUNCH_FINISH(false, true, true, false);
+    else if (vec) SPEC_LAUNCH_FINISH(false, true, false, false);
+    else if (cut) SPEC_LAUNCH_FINISH(false, false, true, false);
+    else SPEC_LAUNCH_FINISH(false, false, false, false);
 #undef SPEC_LAUNCH_FINISH
     return SPEC_OK;
 }

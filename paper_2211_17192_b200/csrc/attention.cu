@@ -104,10 +104,10 @@ __device__ __forceinline__ void cluster_merge_write(const float* fin, int n_q, i
 // grid is launched as clusters over the slice dimension and writes `out` itself.
 template <typename KV, int DH, bool FUSED>
 __global__ void __launch_bounds__(32 * kMaxAttnWarps)
-attention_kernel(const float* __restrict__ qkv, int q_stride, const int32_t* __restrict__ pos,
-                 const int32_t* __restrict__ seq, int m_rows, int n_heads, int n_kv_heads, int ks,
-                 const KV* __restrict__ kv_layer, const int32_t* __restrict__ page_table, int pages_per_seq,
-                 int page_size, const int32_t* __restrict__ kv_len, const float* __restrict__ bias, int bias_span,
+attention_kernel(const float* qkv, int q_stride, const int32_t* pos,
+                 const int32_t* seq, int m_rows, int n_heads, int n_kv_heads, int ks,
+                 const KV* kv_layer, const int32_t* __restrict__ page_table, int pages_per_seq,
+                 int page_size, const int32_t* kv_len, const float* __restrict__ bias, int bias_span,
                  int bias_zero, float scale, float* __restrict__ part, const AttnOut out) {
     __shared__ float share[kMaxAttnWarps][DH + 2];  // states of the warps that share a query (ks > 1)
     pdl_trigger();
@@ -222,10 +222,10 @@ struct MmaSmem {
 // grid = (slices, n_kv_heads * m_blocks, batch), block = 32 * kMmaWarps.
 template <typename KV, int DH, bool FUSED, bool IN_TURN>
 __global__ void __launch_bounds__(32 * kMmaWarps)
-attention_mma_kernel(const float* __restrict__ qkv, int q_stride, const int32_t* __restrict__ pos,
-                     const int32_t* __restrict__ seq, int m_rows, int n_heads, int n_kv_heads, int m_blocks,
-                     const KV* __restrict__ kv_layer, const int32_t* __restrict__ page_table, int pages_per_seq,
-                     int page_size, const int32_t* __restrict__ kv_len, const float* __restrict__ bias, int bias_span,
+attention_mma_kernel(const float* qkv, int q_stride, const int32_t* pos,
+                     const int32_t* seq, int m_rows, int n_heads, int n_kv_heads, int m_blocks,
+                     const KV* kv_layer, const int32_t* __restrict__ page_table, int pages_per_seq,
+                     int page_size, const int32_t* kv_len, const float* __restrict__ bias, int bias_span,
                      int bias_zero, float scale, float* __restrict__ part, const AttnOut out) {
     using S = MmaSmem<DH, IN_TURN>;
     extern __shared__ __align__(16) float smem_f[];
@@ -564,10 +564,10 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 // exponential is one ex2.approx; the running maximum goes back to natural units when the state is stored.
 template <int DH, int MB, bool FUSED>
 __global__ void __launch_bounds__(32 * kF16Warps)
-attention_f16_kernel(const float* __restrict__ qkv, int q_stride, const int32_t* __restrict__ pos,
-                     const int32_t* __restrict__ seq, int m_rows, int n_heads, int n_kv_heads, int q_blocks,
+attention_f16_kernel(const float* qkv, int q_stride, const int32_t* pos,
+                     const int32_t* seq, int m_rows, int n_heads, int n_kv_heads, int q_blocks,
                      const __grid_constant__ CUtensorMap kv_map, const int32_t* __restrict__ page_table, int pages_per_seq,
-                     int page_size, const int32_t* __restrict__ kv_len, const float* __restrict__ bias, int bias_span,
+                     int page_size, const int32_t* kv_len, const float* __restrict__ bias, int bias_span,
                      int bias_zero, float scale, float* __restrict__ part, const AttnOut out) {
     using S = F16Smem<DH, MB>;
     constexpr int KP = kF16Warps / MB;        // key parts of a tile
@@ -1087,7 +1087,7 @@ attention_prompt_kernel(const float* qkv, int q_stride, const int4* segs, int n_
 
 // grid = rows * n_heads, block = DH: merge the key slices of one (row, head).
 template <int DH>
-__global__ void attention_combine_kernel(const float* __restrict__ part, int slices, float* __restrict__ att,
+__global__ void attention_combine_kernel(const float* part, int slices, float* __restrict__ att,
                                          __nv_bfloat16* __restrict__ att_hi, __nv_bfloat16* __restrict__ att_lo) {
     __shared__ float w_sh[64];  // weight of every slice, then their normaliser at [slices]
     pdl_trigger();

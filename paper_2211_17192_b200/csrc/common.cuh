@@ -42,6 +42,13 @@ inline int fail(int status, const char* fmt, ...) {
 // grid has completed and its writes are visible; because every kernel waits,
 // completion is transitive along the stream.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A load through a const __restrict__ pointer, or by __ldg, may be moved in front of pdl_wait(), where what the kernel before
+// writes is not there yet.  A pointer that has come through here after the wait holds it back.
+template <typename T>
+__device__ __forceinline__ T* after_wait(T* p) {
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // SPEC_NO_PDL=1 in the environment launches every kernel fully serialised (for debugging; the one

@@ -408,10 +408,10 @@ int encode(spec_ctx* ctx, const Model& m, int batch, int m_rows) {
 //   draft_u[b, i]  draw of x_{i+1} at position L+i           (purpose 0)
 //   accept_u[b, i] accept test of x_{i+1} at position L+i     (purpose 1)
 //   final_u[b, n]  final draw t at position L+n, n = 0..gamma (purpose 2)
-__global__ void iteration_uniforms_kernel(const spec_ctx::Params* __restrict__ params,
-                                          const int32_t* __restrict__ length, int batch, int gamma,
-                                          float* __restrict__ draft_u, float* __restrict__ accept_u,
-                                          float* __restrict__ final_u) {
+__global__ void iteration_uniforms_kernel(const spec_ctx::Params* params,
+                                          const int32_t* length, int batch, int gamma,
+                                          float* draft_u, float* accept_u,
+                                          float* final_u) {
     pdl_trigger();
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -433,7 +433,7 @@ __device__ __forceinline__ int held(int position, int limit) { return position <
 // L-1.  Position L-2 is already cached unless the previous iteration accepted
 // every guess (x_gamma was never fed to the draft); feeding it again rewrites
 // the same K,V row, so the shape of the step never changes.
-__global__ void prep_draft_first_kernel(const int32_t* __restrict__ tokens, const int32_t* __restrict__ length,
+__global__ void prep_draft_first_kernel(const int32_t* tokens, const int32_t* length,
                                         int batch, int gamma, int max_len, int limit, int32_t* row_token, int32_t* row_pos,
                                         int32_t* row_seq, int32_t* logit_src, int32_t* logit_dst) {
     pdl_trigger();
@@ -452,7 +452,7 @@ __global__ void prep_draft_first_kernel(const int32_t* __restrict__ tokens, cons
 }
 
 // Draft step i (2..gamma): one row per sequence, the previous guess x_{i-1} at position L+i-2.
-__global__ void prep_draft_step_kernel(const int32_t* __restrict__ draft_tokens, const int32_t* __restrict__ length,
+__global__ void prep_draft_step_kernel(const int32_t* draft_tokens, const int32_t* length,
                                        int batch, int gamma, int step, int limit, int32_t* row_token, int32_t* row_pos,
                                        int32_t* row_seq, int32_t* logit_src, int32_t* logit_dst) {
     pdl_trigger();
@@ -467,8 +467,8 @@ __global__ void prep_draft_step_kernel(const int32_t* __restrict__ draft_tokens,
 }
 
 // The target's parallel pass: rows [last committed token, x_1..x_gamma] at positions L-1..L-1+gamma.
-__global__ void prep_verify_kernel(const int32_t* __restrict__ tokens, const int32_t* __restrict__ draft_tokens,
-                                   const int32_t* __restrict__ length, int batch, int gamma, int max_len, int limit,
+__global__ void prep_verify_kernel(const int32_t* tokens, const int32_t* draft_tokens,
+                                   const int32_t* length, int batch, int gamma, int max_len, int limit,
                                    int32_t* row_token, int32_t* row_pos, int32_t* row_seq) {
     pdl_trigger();
     pdl_wait();
@@ -485,9 +485,9 @@ __global__ void prep_verify_kernel(const int32_t* __restrict__ tokens, const int
 // movement: both caches are valid up to position L_new - 2 by construction and
 // whatever lies beyond is overwritten by the next iteration.  A sequence that
 // already has its n_new tokens is frozen.
-__global__ void commit_kernel(const spec_ctx::Params* __restrict__ params, const int32_t* __restrict__ draft_tokens,
-                              const int32_t* __restrict__ n_accepted, const int32_t* __restrict__ next_token,
-                              const float* __restrict__ accept_u, const int32_t* __restrict__ prompt_len, int batch,
+__global__ void commit_kernel(const spec_ctx::Params* params, const int32_t* draft_tokens,
+                              const int32_t* n_accepted, const int32_t* next_token,
+                              const float* accept_u, const int32_t* prompt_len, int batch,
                               int gamma, int max_len, int32_t* tokens, int32_t* length, unsigned long long* counters) {
     pdl_trigger();
     pdl_wait();

@@ -570,11 +570,14 @@ __device__ __forceinline__ float verify_logit(const Row<VEC>& r, const int32_t* 
 // or gamma+1 (T = 0: only p is read).
 template <bool GREEDY, bool VEC>
 __global__ void __launch_bounds__(kStatThreads)
-verify_stats_kernel(const float* __restrict__ target_logits, const float* __restrict__ draft_logits,
-                    const int32_t* __restrict__ draft_tokens, int gamma, int vocab, float c2, ChunkStat* __restrict__ stats) {
+verify_stats_kernel(const float* target_logits, const float* draft_logits, const int32_t* draft_tokens, int gamma, int vocab,
+                    float c2, ChunkStat* stats) {
     __shared__ StatShared<kStatWarps> sh;
-    pdl_trigger();  // the finishing kernel's CTAs may take their places as this grid drains
     pdl_wait();
+    pdl_trigger();  // after the wait: the finishing kernel, which may take its places as this grid drains, fetches inputs at once
+    target_logits = after_wait(target_logits);
+    draft_logits = after_wait(draft_logits);
+    draft_tokens = after_wait(draft_tokens);
     const int chunk = blockIdx.x, chunks = gridDim.x, row = blockIdx.y, rows = gridDim.y, b = blockIdx.z;
     const Row<VEC> r = make_row<VEC>(verify_row(target_logits, draft_logits, b, row, gamma, vocab), vocab);
     const int groups = r.groups();
@@ -609,7 +612,7 @@ __global__ void __launch_bounds__(kFinishThreads, 2)
 verify_finish_kernel(const float* __restrict__ target_logits, const float* __restrict__ draft_logits,
                      const int32_t* __restrict__ draft_tokens, const float* __restrict__ uniforms, int gamma,
                      int vocab, float inv_t, int chunks, int cluster_size, ChunkStat* stats,
-                     const float* __restrict__ final_uniforms, float lenience, const float* __restrict__ floors,
+                     const float* __restrict__ final_uniforms, float lenience, const float* floors,
                      int32_t* __restrict__ n_accepted, int32_t* __restrict__ next_token, int* __restrict__ nonfinite) {
     __shared__ FinishShared sh;
     const int tid = threadIdx.x;
@@ -620,8 +623,8 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
     const float* tl = target_logits + static_cast<size_t>(b) * (gamma + 1) * vocab;
     const float* ql = GREEDY ? nullptr : draft_logits + static_cast<size_t>(b) * gamma * vocab;
 
-    // Inputs that the statistics kernel does not produce can be fetched before
-    // waiting for it.
+    // Inputs that the kernel before does not produce can be fetched before waiting for it: it lets this one start when its
+    // own wait is over, and so what came before it is complete.
     if (ALONE) {
         pdl_trigger();
         __shared__ StatShared<kFinishThreads / 32> stat;
@@ -651,6 +654,7 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
     } else {
         pdl_trigger();
         pdl_wait();
+        floors = after_wait(floors);
     }
 
     // merge the chunk statistics of row `tid` (eight loads in flight at a time)
@@ -753,8 +757,8 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
 // One CTA per row: tokens[r] ~ softmax(logits[r] / T), or argmax at T = 0.
 template <bool VEC>
 __global__ void __launch_bounds__(kSampleThreads)
-sample_kernel(const float* __restrict__ logits, size_t logit_stride, const float* __restrict__ uniforms,
-              int uniform_stride, int vocab, float inv_t, bool greedy, int32_t* __restrict__ tokens, int token_stride, int* __restrict__ nonfinite) {
+sample_kernel(const float* logits, size_t logit_stride, const float* uniforms, int uniform_stride, int vocab, float inv_t, bool greedy,
+              int32_t* tokens, int token_stride, int* nonfinite) {
     constexpr int W = kSampleThreads / 32;
     __shared__ float red[W];
     __shared__ int red_i[W];
@@ -763,6 +767,8 @@ sample_kernel(const float* __restrict__ logits, size_t logit_stride, const float
     __shared__ int s_arg;
     pdl_trigger();
     pdl_wait();
+    logits = after_wait(logits);
+    uniforms = after_wait(uniforms);
     const int tid = threadIdx.x;
     const Row<VEC> r = make_row<VEC>(logits + static_cast<size_t>(blockIdx.x) * logit_stride, vocab);
     const int groups = r.groups();
@@ -1430,11 +1436,13 @@ constexpr int kFloorsOnly = 0, kWithStats = 1, kWithDraw = 2;
 // 8), and after a nucleus one pass less and no second kernel (200 rows of 100000: 99, 91 and 70).
 template <int T, int LOADS, bool VEC, bool SOLO, int WORK>
 __global__ void __launch_bounds__(T, T == 256 ? 5 : LOADS == 8 ? 2 : 3)
-cut_floor_kernel(const float* __restrict__ a, size_t a_stride, int a_rows, const float* __restrict__ b,
-                 size_t b_stride, int b_rows, int vocab, int top_k, float top_p, float c2, float* __restrict__ floors, CutWork work) {
+cut_floor_kernel(const float* a, size_t a_stride, int a_rows, const float* b, size_t b_stride, int b_rows, int vocab, int top_k,
+                 float top_p, float c2, float* floors, CutWork work) {
     __shared__ SelShared sh;
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();  // after the wait: the finishing kernel fetches inputs at once
+    a = after_wait(a);
+    b = after_wait(b);
     const Team<SOLO> team;
     const int at = blockIdx.x / team.size;
     const int per_seq = a_rows + b_rows;

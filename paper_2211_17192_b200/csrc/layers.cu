@@ -83,21 +83,29 @@ __global__ void embed_kernel(const void* tok_emb, const void* pos_emb, bool bf16
 // RMSNorm(h[src(r)]) * gain.  If `partial` is given, h[r] += sum of the partial
 // results first (the residual add of the GEMM that produced them) and the new h
 // is stored.  A thread holds up to PER float4 of the row in registers.
+// With CTAS > 1 a cluster of that many CTAs shares a row (d at most 4 * THREADS * CTAS, PER = 1, grid = rows * CTAS): a
+// row of 4096 with its eight partial sums is 147 KB, a microsecond of what one SM takes in, and nothing else runs
+// meanwhile.  The CTAs give one another their warps' sums of squares through distributed shared memory.
 constexpr int kNormMaxWidth = 4 * 1024 * 4;
+constexpr int kNormCtas = 8;  // of a cluster that shares a row
+constexpr int kNormClusterRows = 128;  // at most (launch_norm has both sides)
 
-template <int THREADS, int PER>
+template <int THREADS, int PER, int CTAS = 1>
 __global__ void __launch_bounds__(THREADS)
 norm_kernel(float* h, const float* partial, const PartialPlan plan, int n_rows, const float* gain,
             const int32_t* src_rows, int d, float eps, float* out,
             __nv_bfloat16* out_hi, __nv_bfloat16* out_lo) {
-    __shared__ float red[THREADS / 32];
-    const int r = blockIdx.x;
+    static_assert(CTAS == 1 || (PER == 1 && CTAS * THREADS / 32 == 32), "a lane per warp of the cluster");
+    __shared__ float red[CTAS * THREADS / 32];
+    const int r = blockIdx.x / CTAS;
     const int groups = d / 4;
+    const int first = CTAS > 1 ? blockIdx.x % CTAS * THREADS + threadIdx.x : threadIdx.x;
+    if constexpr (CTAS > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // (its peers are there)
     // the gains are constants: fetched while the kernel before this one is still finishing
     float4 gg[PER];
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        const int g = threadIdx.x + j * THREADS;
+        const int g = first + j * THREADS;
         gg[j] = g < groups ? *reinterpret_cast<const float4*>(gain + 4 * g) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     pdl_wait();
@@ -111,7 +119,7 @@ norm_kernel(float* h, const float* partial, const PartialPlan plan, int n_rows, 
     float4 v[PER];
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        const int g = threadIdx.x + j * THREADS;
+        const int g = first + j * THREADS;
         v[j] = g < groups ? *reinterpret_cast<const float4*>(h + src + 4 * g) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     if (partial) {
@@ -119,7 +127,7 @@ norm_kernel(float* h, const float* partial, const PartialPlan plan, int n_rows, 
         int splits[PER], most = 0;
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
-            const int g = threadIdx.x + j * THREADS;
+            const int g = first + j * THREADS;
             splits[j] = g < groups ? partial_count(plan, src_row, 4 * g) : 0;
             most = max(most, splits[j]);
         }
@@ -130,7 +138,7 @@ norm_kernel(float* h, const float* partial, const PartialPlan plan, int n_rows, 
 #pragma unroll
                 for (int j = 0; j < PER; ++j)
                     p[k][j] = s0 + k < splits[j] ? *reinterpret_cast<const float4*>(partial + static_cast<size_t>(s0 + k) * stride + src +
-                                                                                    4 * (threadIdx.x + j * THREADS))
+                                                                                    4 * (first + j * THREADS))
                                                  : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int k = 0; k < kBatch; ++k)
@@ -140,7 +148,7 @@ norm_kernel(float* h, const float* partial, const PartialPlan plan, int n_rows, 
         }
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
-            const int g = threadIdx.x + j * THREADS;
+            const int g = first + j * THREADS;
             if (g < groups) *reinterpret_cast<float4*>(h + src + 4 * g) = v[j];
         }
     }
@@ -148,16 +156,31 @@ norm_kernel(float* h, const float* partial, const PartialPlan plan, int n_rows, 
 #pragma unroll
     for (int j = 0; j < PER; ++j) ss += (v[j].x * v[j].x + v[j].y * v[j].y) + (v[j].z * v[j].z + v[j].w * v[j].w);
     ss = warp_sum(ss);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-    __syncthreads();
     float total = 0.0f;
+    if constexpr (CTAS > 1) {
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        const int lane = threadIdx.x & 31;
+        if (lane < CTAS) {
+            const uint32_t here = static_cast<uint32_t>(__cvta_generic_to_shared(&red[first >> 5]));
+            asm volatile("{\n\t.reg .b32 there;\n\tmapa.shared::cluster.u32 there, %0, %1;\n\tst.shared::cluster.f32 [there], %2;\n\t}"
+                         ::"r"(here), "r"(lane), "f"(ss)
+                         : "memory");
+        }
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        total = warp_sum(red[lane]);
+    } else {
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+        __syncthreads();
 #pragma unroll
-    for (int i = 0; i < THREADS / 32; ++i) total += red[i];
+        for (int i = 0; i < THREADS / 32; ++i) total += red[i];
+    }
     const float scale = rsqrtf(total / static_cast<float>(d) + eps);
     const size_t dst = static_cast<size_t>(r) * d;
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        const int g = threadIdx.x + j * THREADS;
+        const int g = first + j * THREADS;
         if (g < groups) {
             const float4 y = make_float4(v[j].x * scale * gg[j].x, v[j].y * scale * gg[j].y, v[j].z * scale * gg[j].z,
                                          v[j].w * scale * gg[j].w);
@@ -358,8 +381,15 @@ int launch_norm(float* h, const float* partial, const PartialPlan& plan, int row
     return launch_pdl(norm_kernel<T, P>, dim3(n_rows), dim3(T), 0, stream, h, partial, plan, rows_total, gain, src_rows, d, \
                       eps, out, out_hi, out_lo)
     // a thread per 128-bit group of the row (fewer warps to reduce over where the row is narrow); with more rows than
-    // SMs, small CTAs with several groups per thread, so that the CTAs of an SM wait for memory side by side
+    // SMs, small CTAs with several groups per thread, so that the CTAs of an SM wait for memory side by side.
+    // Wide rows that leave SMs idle go to a cluster each.  Whole pass of the 7B shape at 500 cached tokens, a CTA of 1024
+    // threads per row against a cluster, ms: 1 row 2.779 / 2.761, 3 rows 2.865 / 2.839, 7 rows 2.937 / 2.915, 16 rows
+    // 3.111 / 3.123 (the runs of one side differ by as much), 32 rows 3.196 / 3.152, 64 rows 3.748 / 3.734, 126 rows
+    // 5.232 / 5.216; beyond, a CTA per row is enough for the GPU.
     const int groups = d / 4;
+    if (groups > 512 && groups <= 128 * kNormCtas && n_rows <= kNormClusterRows)
+        return launch_cluster(norm_kernel<128, 1, kNormCtas>, kNormCtas, dim3(n_rows * kNormCtas), dim3(128), 0, stream, h, partial,
+                              plan, rows_total, gain, src_rows, d, eps, out, out_hi, out_lo);
     if (groups <= 128) SPEC_LAUNCH_NORM(128, 1);
     if (groups <= 256) SPEC_LAUNCH_NORM(256, 1);
     if (groups <= 1024 && n_rows > 148) SPEC_LAUNCH_NORM(256, 4);

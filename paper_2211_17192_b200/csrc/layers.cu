@@ -278,7 +278,8 @@ __global__ void table_logits_kernel(const void* table, bool bf16, int vocab, con
 // tokens of the sequence up to the row's position, or the last token again if there is
 // none.  Positions below length[seq] read the committed tokens, later ones this
 // iteration's guesses.  grid = (chunks, rows): every CTA repeats the search (a few
-// thousand token compares) and writes its share of the row.
+// thousand token compares) and writes its share of the row.  An inactive row (position < 0) has no
+// last token; its guess, which nobody looks at, is token 0.
 __global__ void copy_logits_kernel(const int32_t* tokens, int max_len, const int32_t* length,
                                    const int32_t* draft_tokens, int gamma, const int32_t* row_pos,
                                    const int32_t* row_seq, const int32_t* src_rows,
@@ -304,7 +305,7 @@ __global__ void copy_logits_kernel(const int32_t* tokens, int max_len, const int
     if ((threadIdx.x & 31) == 0) best[threadIdx.x >> 5] = found;
     __syncthreads();
     for (int w = 0; w < static_cast<int>(blockDim.x) / 32; ++w) found = max(found, best[w]);
-    const int guess = min(max(at(found >= 0 ? found + 1 : last), 0), vocab - 1);
+    const int guess = last < 0 ? 0 : min(max(at(found >= 0 ? found + 1 : last), 0), vocab - 1);
     float* out = logits + static_cast<size_t>(dst_rows ? dst_rows[i] : i) * vocab;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < vocab; v += gridDim.x * blockDim.x)
         out[v] = v == guess ? 0.0f : -INFINITY;

@@ -419,6 +419,32 @@ def test_copy_from_context_draft_matches_the_oracle(ngram):
         eng.close()
 
 
+@pytest.mark.parametrize("gamma", [3, 4])
+def test_copy_draft_of_a_frozen_sequence_at_the_end_of_the_context(gamma):
+    """A sequence that ends with every guess accepted, in a context that holds exactly what a generation may ask for: from the
+    third draft step on its rows lie beyond the context.  Stepped further, it keeps its tokens, as in a roomy context."""
+    tcfg = workloads.model_config("tiny_target")
+    tw = workloads.make_weights(tcfg, 1)
+    dcfg = workloads.model_config("copy_8k")
+    prompts = [workloads.make_repetitive_prompt(15, 26, tcfg["vocab"], 7), workloads.make_repetitive_prompt(16, 21, tcfg["vocab"], 4)]
+    n_new = 4 * (gamma + 1) + 1  # one token more than four iterations emit: the fifth ends gamma tokens beyond
+    runs = []
+    for room in (0, 40):
+        eng = binding.Engine(tcfg, tw, dcfg, {}, max_batch=2, max_len=26 + n_new + gamma + 1 + room, page_size=32, max_gamma=gamma)
+        try:
+            eng.set_lenience(1e-30)  # (accepts every guess)
+            eng.begin(prompts, n_new, gamma, 0.0, 0)
+            left, st = eng.step(5)
+            assert left <= 0 and st["tests_passed"] == st["tests_evaluated"] == 2 * 5 * gamma
+            ended = eng.read_tokens()
+            eng.step(3)
+            assert np.array_equal(eng.read_tokens(), ended)
+            runs.append(ended)
+        finally:
+            eng.close()
+    assert np.array_equal(runs[0], runs[1])
+
+
 def test_adaptive_gamma_generation(tiny):
     """Section 3.5's varying gamma: the library picks gamma burst by burst.  The trace it reports,
     replayed by the oracle (and by the phased entry points), gives the same tokens; at T = 0 the

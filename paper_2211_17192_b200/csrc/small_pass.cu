@@ -887,7 +887,8 @@ small_pass_kernel(const __grid_constant__ SmallArgs a) {
 #pragma unroll 1
         for (int i = tid; i < a.rows * 32; i += kThreads)
             reinterpret_cast<float2*>(sm + S::kRope)[i] = a.rope[static_cast<size_t>(max(a.pos[i >> 5], 0)) * 32 + (i & 31)];
-    // (the last CTA to need the epoch has read it long before the first CTA ends and advances it)
+    // (CTA 0 advances the epoch at its end.  By then every CTA has read it: from two blocks on, CTA 0 has gathered an FFN's sums
+    // of its peer in every cluster, each of which needed something of every CTA of that cluster.  shape_fits has the rest)
     sync_consumers();
 #pragma unroll 1
     for (int l = 0; l < a.n_layers; ++l) {
@@ -1017,6 +1018,9 @@ Variant pick(int ki, int rows) { return ki == 1 ? pick<1>(rows) : ki == 2 ? pick
 
 bool shape_fits(const Model& m) {
     const spec_model_cfg& c = m.cfg;
+    // In a model of one block nothing makes CTA 0 wait for the clusters without a head: one that starts late would read the
+    // epoch of the next pass and poll for exchanges that never come.
+    if (c.n_layers < 2) return false;
     if (!m.bf16() || (c.arch != SPEC_ARCH_GPT && c.arch != SPEC_ARCH_LLAMA && c.arch != SPEC_ARCH_T5)) return false;
     const int group = c.n_heads / c.n_kv_heads;
     return c.d_head == kDh && c.d_model % 256 == 0 && c.d_model <= kMaxD && c.n_kv_heads <= kClusters && group <= 4 && c.d_ff % 16 == 0 &&

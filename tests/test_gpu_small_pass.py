@@ -3,6 +3,7 @@ of one to four query heads per KV head, FFNs of fewer columns than thread blocks
 sequences, and contexts around the edges of sixteen keys, of a page and of what one step of all warps covers."""
 import numpy as np
 import pytest
+import torch
 
 from oracle.decoder import Decoder
 from oracle.encdec import START_TOKEN, EncoderDecoder
@@ -70,3 +71,28 @@ def test_few_rows_with_cross_attention():
                 assert err <= LOGIT_TOL * max(1.0, np.abs(want[b]).max()), (batch, rows, at, b, err)
             at += rows
     eng.close()
+
+
+def test_a_decoder_of_one_block():
+    """Only a few clusters of thread blocks would have a head, and nothing in one block makes the pass wait for the others: such a
+    model is left to the chain of kernels.  Passes back to back, each right after the last."""
+    cfg = workloads.scaled_config(workloads.model_config("llama_test_target"), d_model=256, n_heads=4, n_kv_heads=1, n_layers=1,
+                                  tied=False, vocab=512, max_positions=512)
+    w = workloads.make_weights(cfg, 7)
+    tokens = workloads.make_prompt(50, 320, cfg["vocab"])
+    want = Decoder(cfg, w).forward_full(tokens)
+    eng = binding.Engine(cfg, w, max_batch=1, max_len=330, page_size=32, max_gamma=7)
+    got = [eng.forward_logits(0, tokens[None, i:i + 1])[0] for i in range(320)]
+    eng.close()
+    assert np.abs(torch.cat(got).cpu().numpy() - want).max() <= LOGIT_TOL
+    # drawn by generation too, whose passes follow one another without the host in between
+    draft = workloads.scaled_config(cfg, n_heads=2, n_kv_heads=2)
+    eng = binding.Engine(cfg, w, draft, workloads.make_weights(draft, 8), max_batch=1, max_len=330, page_size=32, max_gamma=3)
+    greedy, _ = eng.generate([tokens[:20]], 200, 0, 0.0, 1)
+    guessed, _ = eng.generate([tokens[:20]], 200, 3, 0.0, 1)
+    eng.close()
+    full = Decoder(cfg, w).forward_full(np.concatenate([tokens[:20], greedy[0]]))[19:-1]
+    for stream in (greedy[0], guessed[0]):
+        n = next((i for i in range(200) if stream[i] != greedy[0][i]), 199)
+        gap = full[:n + 1].max(axis=1) - full[np.arange(n + 1), stream[:n + 1]]
+        assert (gap <= 2 * LOGIT_TOL).all()

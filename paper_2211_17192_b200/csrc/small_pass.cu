@@ -1081,6 +1081,10 @@ int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocation
     const size_t gain_bytes = static_cast<size_t>(c.n_layers) * 3 * c.d_model * sizeof(float), epoch_bytes = 256;
     const size_t ll_bytes = static_cast<size_t>(4) * kClusters * kRows * c.d_model * sizeof(unsigned long long);
     const size_t part_bytes = static_cast<size_t>(kClusters) * kRows * c.d_model * sizeof(float);
+    // (the packing kernel's pointers pass through the partial sums' memory, which nothing uses yet; 1820 blocks of the narrowest
+    // model fit)
+    std::vector<PackLayer> pack(c.n_layers);
+    if (pack.size() * sizeof(PackLayer) > part_bytes) return SPEC_OK;
     char* base = nullptr;
     int status = alloc(reinterpret_cast<void**>(&base), gain_bytes + epoch_bytes + ll_bytes + part_bytes + s.cta_bytes * ctas);
     if (status != SPEC_OK) return status;
@@ -1089,14 +1093,11 @@ int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocation
     s.exchanges = reinterpret_cast<unsigned long long*>(base + gain_bytes + epoch_bytes);
     s.last_part = reinterpret_cast<float*>(base + gain_bytes + epoch_bytes + ll_bytes);
     s.stream = base + gain_bytes + epoch_bytes + ll_bytes + part_bytes;
-    std::vector<PackLayer> pack(c.n_layers);
     auto b = [](const void* p) { return static_cast<const __nv_bfloat16*>(p); };
     for (int l = 0; l < c.n_layers; ++l) {
         const spec_layer_weights& w = m.layers[l];
         pack[l] = PackLayer{b(w.wqkv), b(w.wo), b(w.w_in), b(w.w_out), b(w.wq_x), b(w.wo_x), w.ln1, w.lnx, w.ln2};
     }
-    // (the packing kernel's pointers pass through the partial sums' memory, which nothing uses yet)
-    if (pack.size() * sizeof(PackLayer) > part_bytes) return SPEC_OK;
     SPEC_CUDA_TRY(cudaMemcpyAsync(s.last_part, pack.data(), pack.size() * sizeof(PackLayer), cudaMemcpyHostToDevice, stream));
     // (no epoch is 0: the pairs start as nobody's)
     SPEC_CUDA_TRY(cudaMemsetAsync(s.epoch, 0, epoch_bytes + ll_bytes, stream));

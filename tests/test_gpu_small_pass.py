@@ -96,3 +96,25 @@ def test_a_decoder_of_one_block():
         n = next((i for i in range(200) if stream[i] != greedy[0][i]), 199)
         gap = full[:n + 1].max(axis=1) - full[np.arange(n + 1), stream[:n + 1]]
         assert (gap <= 2 * LOGIT_TOL).all()
+
+
+def test_more_blocks_than_the_packing_takes():
+    """The pointers of at most 1820 blocks of the narrowest model fit the memory in which they reach the packing kernel: a deeper
+    model's passes are the chain's, not a kernel's on weights that were never packed."""
+    layers = 1821
+    cfg = workloads.scaled_config(workloads.model_config("llama_test_target"), d_model=256, n_heads=1, n_kv_heads=1, d_ff=16,
+                                  n_layers=layers, tied=False, vocab=64, max_positions=64)
+    drawn = workloads.make_weights(workloads.scaled_config(cfg, n_layers=2), 13)
+    # (two blocks' weights in turn, on the device once)
+    matrices = ("wqkv", "wo", "w_in", "w_out")
+    cuda = {k: torch.from_numpy(np.ascontiguousarray(v)).cuda().to(torch.bfloat16 if k.split(".")[-1] in matrices + ("tok_emb", "head")
+                                                                     else torch.float32) for k, v in drawn.items()}
+    repeat = lambda w: {k: v for k, v in w.items() if "." not in k} | {
+        f"l{l}.{n}": w[f"l{l % 2}.{n}"] for l in range(layers) for n in ("ln1", "ln2") + matrices}
+    tokens = workloads.make_prompt(51, 3, cfg["vocab"])
+    want = Decoder(cfg, repeat(drawn)).forward_full(tokens)
+    eng = binding.Engine(cfg, repeat(cuda), max_batch=1, max_len=32, page_size=32, max_gamma=3)
+    got = torch.cat([eng.forward_logits(0, tokens[None, i:i + 1])[0] for i in range(3)]).cpu().numpy()
+    eng.close()
+    # (fp16 keys and values, 2^-11 of each, block after block: the errors add up like the blocks' outputs do)
+    assert np.abs(got - want).max() <= LOGIT_TOL * np.abs(want).max()

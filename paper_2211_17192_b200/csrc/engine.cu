@@ -948,8 +948,6 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
             SPEC_ALLOC(partials, partial);
             cudaMemset(ctx->x_hi, 0, static_cast<size_t>(ctx->hi_rows) * max_k * 2);
             cudaMemset(ctx->x_lo, 0, static_cast<size_t>(ctx->hi_rows) * max_k * 2);
-            for (int i = 0; i < (ctx->has_draft ? 2 : 1) && !rt.pass_kernel; ++i)
-                if ((status = small_pass_init(ctx->small[i], ctx->model[i], ctx->allocations, ctx->stream)) != SPEC_OK) return cleanup(status);
             if (rt.pass_kernel && (status = pass_scratch_init(ctx->pass, ctx->model, ctx->has_draft ? 2 : 1, ctx->allocations)) != SPEC_OK)
                 return cleanup(status);
         }
@@ -1013,6 +1011,9 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     ctx->error_words[4] = small_pass_error_word();
     ctx->cached[0].assign(B, 0);
     ctx->cached[1].assign(B, 0);
+    // (last: everything that a context cannot do without has its memory)
+    for (int i = 0; i < (ctx->has_draft ? 2 : 1) && !rt.pass_kernel; ++i)
+        if ((status = small_pass_init(ctx->small[i], ctx->model[i], ctx->allocations, ctx->stream)) != SPEC_OK) return cleanup(status);
     *out = ctx;
     return SPEC_OK;
 }

@@ -234,6 +234,17 @@ int launch_pass(const PassScratch& s, const Model& m, int which, const RowMeta& 
 void pass_scratch_release(PassScratch& s);
 int pass_take_error();
 
+// Whether `bytes` of device memory can be taken for something that only makes a context faster: 512 MB more stay free, for
+// the graphs that the context will capture and for what the caller allocates next.
+inline bool memory_to_spare(size_t bytes) {
+    size_t free = 0, total = 0;
+    if (cudaMemGetInfo(&free, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return free >= bytes + (static_cast<size_t>(512) << 20);
+}
+
 // small_pass.cu: the blocks of a small decoder over at most 8 rows as one cooperative kernel.
 struct SmallPass {
     void* stream = nullptr;  // the weights in the order of use (nullptr: not served)

@@ -1068,15 +1068,6 @@ int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocation
         most = std::max(most, n);
     }
     s.cta_bytes = most * c.n_layers * ki * kChunk;
-    auto alloc = [&](void** p, size_t bytes) {
-        const cudaError_t err = cudaMalloc(p, bytes);
-        if (err != cudaSuccess) {
-            cudaGetLastError();
-            return fail(SPEC_ERR_OOM, "cudaMalloc of %zu bytes failed: %s", bytes, cudaGetErrorString(err));
-        }
-        allocations.push_back(*p);
-        return static_cast<int>(SPEC_OK);
-    };
     // one allocation: gains, the epoch, exchange buffers, the last partial sums, the stream
     const size_t gain_bytes = static_cast<size_t>(c.n_layers) * 3 * c.d_model * sizeof(float), epoch_bytes = 256;
     const size_t ll_bytes = static_cast<size_t>(4) * kClusters * kRows * c.d_model * sizeof(unsigned long long);
@@ -1086,8 +1077,13 @@ int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocation
     std::vector<PackLayer> pack(c.n_layers);
     if (pack.size() * sizeof(PackLayer) > part_bytes) return SPEC_OK;
     char* base = nullptr;
-    int status = alloc(reinterpret_cast<void**>(&base), gain_bytes + epoch_bytes + ll_bytes + part_bytes + s.cta_bytes * ctas);
-    if (status != SPEC_OK) return status;
+    const size_t bytes = gain_bytes + epoch_bytes + ll_bytes + part_bytes + s.cta_bytes * ctas;
+    // a third copy of the weights, for speed alone: without room for it the chain of kernels serves the model
+    if (!memory_to_spare(bytes) || cudaMalloc(reinterpret_cast<void**>(&base), bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return SPEC_OK;
+    }
+    allocations.push_back(base);
     s.gains = reinterpret_cast<float*>(base);
     s.epoch = reinterpret_cast<unsigned*>(base + gain_bytes);
     s.exchanges = reinterpret_cast<unsigned long long*>(base + gain_bytes + epoch_bytes);

@@ -864,12 +864,17 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     ctx->pages_per_seq = (rt.max_len + rt.page_size - 1) / rt.page_size;
     ctx->max_logit_rows = std::max(rt.max_batch * std::max(rt.max_gamma + 1, 2), 64);
     // The prompt pass takes up to 2048 rows at a time: the GEMMs reach their full rate from about 1024 rows on (4096-wide
-    // block, one prompt of 1024 tokens, 256-row chunks 54 ms, one chunk 32 ms), narrow models like more.
-    ctx->max_rows = std::max(ctx->max_logit_rows, std::min(2048, rt.max_batch * rt.max_len));
+    // block, one prompt of 1024 tokens, 256-row chunks 54 ms, one chunk 32 ms), narrow models like more.  Where memory is short
+    // (the partial sums of 2048 rows of the 7B shape are 0.4 GB), 256.
+    int src_rows = 0;
     if (t5) {  // an encoder pass takes every source row of the batch at once
         ctx->src_pages_per_seq = (rt.max_src_len + rt.page_size - 1) / rt.page_size;
-        ctx->max_rows = std::max(ctx->max_rows, rt.max_batch * rt.max_src_len);
+        src_rows = rt.max_batch * rt.max_src_len;
     }
+    auto pass_rows = [&](int chunk) {
+        return std::max({ctx->max_logit_rows, src_rows, static_cast<int>(std::min<long long>(chunk, static_cast<long long>(rt.max_batch) * rt.max_len))});
+    };
+    ctx->max_rows = pass_rows(2048);
     auto cleanup = [&](int status) {
         spec_free(ctx);
         return status;
@@ -891,73 +896,24 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
         att = std::max<size_t>(att, m.q_dim());
         ff = std::max<size_t>(ff, m.cfg.d_ff);
     }
-    const size_t R = ctx->max_rows, B = rt.max_batch, G = rt.max_gamma, V = target_cfg->vocab;
+    const size_t B = rt.max_batch, G = rt.max_gamma, V = target_cfg->vocab;
     const size_t RL = ctx->max_logit_rows;
+    const int n_models = ctx->has_draft ? 2 : 1;
+    bool any_fp32 = false, any_bf16 = false;  // (bf16 models hand over partial sums and bf16 terms; a table or a copy draft neither)
+    for (int i = 0; i < n_models; ++i) {
+        const Model& m = ctx->model[i];
+        any_fp32 |= !m.bf16();
+        any_bf16 |= m.bf16() && m.cfg.arch != SPEC_ARCH_BIGRAM && m.cfg.arch != SPEC_ARCH_COPY;
+    }
 #define SPEC_ALLOC(ptr, count) \
     if ((status = dev_alloc(ctx, &ctx->ptr, (count))) != SPEC_OK) return cleanup(status)
-    SPEC_ALLOC(h, R * d);
-    SPEC_ALLOC(qkv, R * std::max(qkv, 2 * att));
-    bool any_fp32 = false;  // (bf16 models hand over partial sums and bf16 terms instead)
-    for (int i = 0; i < (ctx->has_draft ? 2 : 1); ++i) any_fp32 |= !ctx->model[i].bf16();
-    if (any_fp32) {
-        SPEC_ALLOC(a, R * d);
-        SPEC_ALLOC(att, R * att);
-        SPEC_ALLOC(f, R * ff);
-    }
-    {
-        size_t attn = 0;
-        for (int i = 0; i < (ctx->has_draft ? 2 : 1); ++i) {
-            const Model& m = ctx->model[i];
-            for (int b = 1; b <= rt.max_batch; ++b)
-                for (int mr = 1; b * mr <= ctx->max_rows; ++mr)
-                    for (int keys : {rt.max_len, rt.max_src_len})
-                        if (keys > 0)
-                            attn = std::max(attn, attention_partial_elems(b * mr, m.cfg.n_heads, m.cfg.d_head,
-                                                                          attention_slices(m, b, mr, keys)));
-        }
-        SPEC_ALLOC(attn_part, attn);
-    }
     SPEC_ALLOC(target_logits, RL * V);
     SPEC_ALLOC(draft_logits, std::max<size_t>(B * G, 1) * V);
-    {
-        // Tensor-core path (any bf16 model): inputs as two bf16 terms, split-K partial sums.
-        size_t max_k = 0, partial = 0;
-        bool any_bf16 = false;
-        for (int i = 0; i < (ctx->has_draft ? 2 : 1); ++i) {
-            const Model& m = ctx->model[i];
-            if (!m.bf16() || m.cfg.arch == SPEC_ARCH_BIGRAM || m.cfg.arch == SPEC_ARCH_COPY) continue;
-            any_bf16 = true;
-            max_k = std::max<size_t>({max_k, static_cast<size_t>(m.cfg.d_model), static_cast<size_t>(m.q_dim()), static_cast<size_t>(m.cfg.d_ff)});
-            const int shapes[7][2] = {{m.qkv_dim(), m.cfg.d_model}, {m.cfg.d_model, m.q_dim()}, {m.ffn_in_dim(), m.cfg.d_model},
-                                      {m.cfg.d_model, m.cfg.d_ff}, {m.q_dim(), m.cfg.d_model}, {2 * m.kv_dim(), m.cfg.d_model},
-                                      {m.cfg.vocab, m.cfg.d_model}};
-            for (int s = 0; s < 7; ++s) {
-                if (!m.t5() && (s == 4 || s == 5)) continue;  // cross-attention projections
-                const int most = s == 6 ? ctx->max_logit_rows : ctx->max_rows;  // the head only sees decode rows
-                partial = std::max(partial, gemm_tc_most_partial_elems(shapes[s][0], shapes[s][1], most));
-            }
-        }
-        if (any_bf16) {
-            for (int i = 0; i < (ctx->has_draft ? 2 : 1); ++i)
-                if (ctx->model[i].bf16() && ctx->model[i].cfg.arch != SPEC_ARCH_BIGRAM &&
-                    (status = pack_model(ctx, ctx->model[i])) != SPEC_OK)
-                    return cleanup(status);
-            ctx->hi_rows = (ctx->max_rows + 255) / 256 * 256;  // whole token tiles of the widest GEMM variant
-            SPEC_ALLOC(x_hi, static_cast<size_t>(ctx->hi_rows) * max_k);
-            SPEC_ALLOC(x_lo, static_cast<size_t>(ctx->hi_rows) * max_k);
-            SPEC_ALLOC(partials, partial);
-            cudaMemset(ctx->x_hi, 0, static_cast<size_t>(ctx->hi_rows) * max_k * 2);
-            cudaMemset(ctx->x_lo, 0, static_cast<size_t>(ctx->hi_rows) * max_k * 2);
-            if (rt.pass_kernel && (status = pass_scratch_init(ctx->pass, ctx->model, ctx->has_draft ? 2 : 1, ctx->allocations)) != SPEC_OK)
-                return cleanup(status);
-        }
-    }
-    SPEC_ALLOC(row_block, 5 * R + 16 + 4 * B);  // (a prompt chunk's three padded row arrays and up to B + 1 segments fit)
-    ctx->row_token = ctx->row_block;
-    ctx->row_pos = ctx->row_block + R;
-    ctx->row_seq = ctx->row_block + 2 * R;
-    ctx->logit_src = ctx->row_block + 3 * R;
-    ctx->logit_dst = ctx->row_block + 4 * R;
+    for (int i = 0; i < n_models; ++i)
+        if (ctx->model[i].bf16() && ctx->model[i].cfg.arch != SPEC_ARCH_BIGRAM && (status = pack_model(ctx, ctx->model[i])) != SPEC_OK)
+            return cleanup(status);
+    if (any_bf16 && rt.pass_kernel && (status = pass_scratch_init(ctx->pass, ctx->model, n_models, ctx->allocations)) != SPEC_OK)
+        return cleanup(status);
     SPEC_ALLOC(page_table, B * ctx->pages_per_seq);
     if (t5) {
         SPEC_ALLOC(src_page_table, B * ctx->src_pages_per_seq);
@@ -984,6 +940,69 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
         ctx->sampler_ws = ws;
     }
 #undef SPEC_ALLOC
+    // the arrays that hold the rows of a pass
+    auto alloc_rows = [&]() -> int {
+        const size_t R = ctx->max_rows;
+        SPEC_TRY(dev_alloc(ctx, &ctx->h, R * d));
+        SPEC_TRY(dev_alloc(ctx, &ctx->qkv, R * std::max(qkv, 2 * att)));
+        if (any_fp32) {
+            SPEC_TRY(dev_alloc(ctx, &ctx->a, R * d));
+            SPEC_TRY(dev_alloc(ctx, &ctx->att, R * att));
+            SPEC_TRY(dev_alloc(ctx, &ctx->f, R * ff));
+        }
+        size_t attn = 0;
+        for (int i = 0; i < n_models; ++i) {
+            const Model& m = ctx->model[i];
+            for (int b = 1; b <= rt.max_batch; ++b)
+                for (int mr = 1; b * mr <= ctx->max_rows; ++mr)
+                    for (int keys : {rt.max_len, rt.max_src_len})
+                        if (keys > 0)
+                            attn = std::max(attn, attention_partial_elems(b * mr, m.cfg.n_heads, m.cfg.d_head,
+                                                                          attention_slices(m, b, mr, keys)));
+        }
+        SPEC_TRY(dev_alloc(ctx, &ctx->attn_part, attn));
+        if (any_bf16) {  // tensor-core path: inputs as two bf16 terms, split-K partial sums
+            size_t max_k = 0, partial = 0;
+            for (int i = 0; i < n_models; ++i) {
+                const Model& m = ctx->model[i];
+                if (!m.bf16() || m.cfg.arch == SPEC_ARCH_BIGRAM || m.cfg.arch == SPEC_ARCH_COPY) continue;
+                max_k = std::max<size_t>({max_k, static_cast<size_t>(m.cfg.d_model), static_cast<size_t>(m.q_dim()), static_cast<size_t>(m.cfg.d_ff)});
+                const int shapes[7][2] = {{m.qkv_dim(), m.cfg.d_model}, {m.cfg.d_model, m.q_dim()}, {m.ffn_in_dim(), m.cfg.d_model},
+                                          {m.cfg.d_model, m.cfg.d_ff}, {m.q_dim(), m.cfg.d_model}, {2 * m.kv_dim(), m.cfg.d_model},
+                                          {m.cfg.vocab, m.cfg.d_model}};
+                for (int s = 0; s < 7; ++s) {
+                    if (!m.t5() && (s == 4 || s == 5)) continue;  // cross-attention projections
+                    const int most = s == 6 ? ctx->max_logit_rows : ctx->max_rows;  // the head only sees decode rows
+                    partial = std::max(partial, gemm_tc_most_partial_elems(shapes[s][0], shapes[s][1], most));
+                }
+            }
+            ctx->hi_rows = (ctx->max_rows + 255) / 256 * 256;  // whole token tiles of the widest GEMM variant
+            const size_t terms = static_cast<size_t>(ctx->hi_rows) * max_k;
+            SPEC_TRY(dev_alloc(ctx, &ctx->x_hi, terms));
+            SPEC_TRY(dev_alloc(ctx, &ctx->x_lo, terms));
+            SPEC_TRY(dev_alloc(ctx, &ctx->partials, partial));
+            SPEC_CUDA_TRY(cudaMemsetAsync(ctx->x_hi, 0, terms * sizeof(__nv_bfloat16), ctx->stream));
+            SPEC_CUDA_TRY(cudaMemsetAsync(ctx->x_lo, 0, terms * sizeof(__nv_bfloat16), ctx->stream));
+        }
+        SPEC_TRY(dev_alloc(ctx, &ctx->row_block, 5 * R + 16 + 4 * B));  // (a prompt chunk's three padded row arrays and up to B + 1 segments fit)
+        ctx->row_token = ctx->row_block;
+        ctx->row_pos = ctx->row_block + R;
+        ctx->row_seq = ctx->row_block + 2 * R;
+        ctx->logit_src = ctx->row_block + 3 * R;
+        ctx->logit_dst = ctx->row_block + 4 * R;
+        ctx->staging.resize(3 * (R + 4) + 4);
+        return SPEC_OK;
+    };
+    const size_t before_rows = ctx->allocations.size();
+    status = alloc_rows();
+    if (ctx->max_rows > pass_rows(256) && (status == SPEC_ERR_OOM || (status == SPEC_OK && !memory_to_spare(0)))) {
+        cudaStreamSynchronize(ctx->stream);
+        for (size_t i = before_rows; i < ctx->allocations.size(); ++i) cudaFree(ctx->allocations[i]);
+        ctx->allocations.resize(before_rows);
+        ctx->max_rows = pass_rows(256);
+        status = alloc_rows();
+    }
+    if (status != SPEC_OK) return cleanup(status);
     // Page j of sequence b is pool page j * max_batch + b: consecutive pages of a
     // sequence are not adjacent in memory, so every access goes through the table.
     std::vector<int32_t> table(B * ctx->pages_per_seq);
@@ -1001,7 +1020,6 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     const size_t report_bytes = sizeof(spec_report) + B * sizeof(int32_t);
     ctx->report_memory.assign(report_bytes, 0);
     ctx->report = reinterpret_cast<spec_report*>(ctx->report_memory.data());
-    ctx->staging.resize(3 * (R + 4) + 4);
     cudaMemset(ctx->nonfinite, 0, sizeof(int));
     cudaMemset(ctx->counters, 0, kCounters * sizeof(unsigned long long));
     ctx->error_words[0] = gemm_tc_error_word();
@@ -1012,7 +1030,7 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     ctx->cached[0].assign(B, 0);
     ctx->cached[1].assign(B, 0);
     // (last: everything that a context cannot do without has its memory)
-    for (int i = 0; i < (ctx->has_draft ? 2 : 1) && !rt.pass_kernel; ++i)
+    for (int i = 0; i < n_models && !rt.pass_kernel; ++i)
         if ((status = small_pass_init(ctx->small[i], ctx->model[i], ctx->allocations, ctx->stream)) != SPEC_OK) return cleanup(status);
     *out = ctx;
     return SPEC_OK;

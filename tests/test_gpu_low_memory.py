@@ -73,3 +73,23 @@ def test_a_context_without_room_for_the_packed_copy(fixture):
         assert np.array_equal(same, tokens)
     finally:
         fixture.release()
+
+
+def test_a_context_without_room_for_long_prompt_chunks(fixture):
+    """Prompts go in chunks of 2048 rows, or of 256 where the partial sums of more would not leave room enough."""
+    _, tokens, most = fixture.run()
+    try:
+        fixture.leave(most + 256 * MB)
+        _, same, least = fixture.run()
+        assert np.array_equal(same, tokens)
+        # a context that packs no second copy takes less than this by what 1792 rows of partial sums need
+        cfg = fixture.cfg
+        rows = 1792 * 2 * cfg["d_ff"] * 4
+        packed = 2 * sum(t.numel() for n, t in fixture.weights.items() if n.split(".")[-1] in ("wqkv", "wo", "w_in", "w_out"))
+        assert least < most - packed - rows
+        # and fits where it always has
+        fixture.leave(least + 16 * MB)
+        _, same, _ = fixture.run()
+        assert np.array_equal(same, tokens)
+    finally:
+        fixture.release()

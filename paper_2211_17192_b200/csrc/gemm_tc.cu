@@ -273,8 +273,9 @@ __global__ void split_bf16_kernel(const float* __restrict__ x, size_t n, __nv_bf
     }
 }
 
-// y[dst(r)][n] = sum_s partial[s][r][n] (+ residual[r][n]), splits added in index order.  grid = (column blocks, rows);
-// a thread takes VEC (4 or 1) neighbouring columns at a time.
+// y[dst(r)][n] = sum_s partial[s][r][n] (+ residual[r][n]), splits added in index order.  grid = (column blocks, rows, rows
+// beyond the kMostGridY that y holds); a thread takes VEC (4 or 1) neighbouring columns at a time.
+constexpr int kMostGridY = 65535;
 template <int VEC>
 __global__ void reduce_partials_kernel(const float* partial, const PartialPlan plan, int n_rows, int n_out,
                                        const float* residual, const int32_t* dst_rows, float* y, float* const* y_slot) {
@@ -282,7 +283,8 @@ __global__ void reduce_partials_kernel(const float* partial, const PartialPlan p
     pdl_wait();
     if (y_slot) y = *y_slot;
     const size_t total = static_cast<size_t>(n_rows) * n_out;
-    const int r = blockIdx.y;
+    const int r = blockIdx.z * kMostGridY + blockIdx.y;
+    if (r >= n_rows) return;
     const float* in = partial + static_cast<size_t>(r) * n_out;
     float* out = y + static_cast<size_t>(dst_rows ? dst_rows[r] : r) * n_out;
     for (int n = VEC * (blockIdx.x * blockDim.x + threadIdx.x); n < n_out; n += VEC * gridDim.x * blockDim.x) {
@@ -535,7 +537,7 @@ int launch_gemm_tc(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_rows
     const PartialPlan plan = gemm_tc_plan(n_out, k, n_rows);
     const float* sums = partial;
     const bool vec = n_out % 4 == 0 && (reinterpret_cast<uintptr_t>(y) & 15u) == 0;  // (y: null or the first address with a slot)
-    const dim3 grid((n_out + (vec ? 1023 : 255)) / (vec ? 1024 : 256), n_rows);
+    const dim3 grid((n_out + (vec ? 1023 : 255)) / (vec ? 1024 : 256), std::min(n_rows, kMostGridY), (n_rows + kMostGridY - 1) / kMostGridY);
     if (vec) return launch_pdl(reduce_partials_kernel<4>, grid, dim3(256), 0, stream, sums, plan, n_rows, n_out, residual, dst_rows, y, y_slot);
     return launch_pdl(reduce_partials_kernel<1>, grid, dim3(256), 0, stream, sums, plan, n_rows, n_out, residual, dst_rows, y, y_slot);
 }

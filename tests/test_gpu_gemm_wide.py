@@ -36,3 +36,15 @@ def test_many_rows_against_fp64(rows, n_out, k):
         # (2^-17 + 2^-24 sqrt(k)) * sum |x w|, far below the bound
         bound = 2.0 ** -16 * (x.double().abs() @ w[c:c + 8192].double().abs().T)
         assert bool(((y[:, c:c + 8192].double() - ref).abs() <= bound + 1e-30).all())
+
+
+@pytest.mark.parametrize("n_out", [8, 5])  # columns by fours, and one by one
+@pytest.mark.parametrize("rows", [65535, 65536, 131073])
+def test_more_rows_than_a_grid_has_along_y(rows, n_out):
+    gen = torch.Generator(device="cuda").manual_seed(rows + n_out)
+    x = torch.randn((rows, 64), device="cuda", generator=gen)
+    w = (torch.randn((n_out, 64), device="cuda", generator=gen) * 0.05).to(torch.bfloat16)
+    ref = x.double() @ w.double().T
+    bound = 2.0 ** -16 * (x.double().abs() @ w.double().abs().T)  # (as above)
+    for y in (binding.spec_linear(x, w, "tensor"), binding.spec_linear(x, binding.spec_pack_weight(w), "tensor_packed", n_out=n_out)):
+        assert bool(((y.double() - ref).abs() <= bound + 1e-30).all())

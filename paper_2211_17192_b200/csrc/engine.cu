@@ -272,7 +272,7 @@ __global__ void report_kernel(ErrorWords errors, int* nonfinite, const unsigned 
     for (int i = threadIdx.x; i < batch; i += blockDim.x) out->length[i] = length[i];
 }
 
-// Waits for everything on the context's stream; ctx->report then describes it.
+// Waits for everything on the context's stream; if it returns SPEC_OK, ctx->report describes it.
 int finish_work(spec_ctx* ctx, int batch) {
     const ErrorWords errors{{ctx->error_words[0], ctx->error_words[1], ctx->error_words[2], ctx->error_words[3], ctx->error_words[4]}};
     SPEC_TRY(launch_pdl(report_kernel, dim3(1), dim3(128), 0, ctx->stream, errors, ctx->nonfinite, ctx->counters, ctx->length, batch,
@@ -1174,11 +1174,10 @@ int run_iterations(spec_ctx* ctx, int iterations, float* elapsed_ms, int* remain
     SPEC_CUDA_TRY(cudaEventRecord(ctx->ev[2], st));
     ctx->session_replays += iterations;
     ctx->session_draft_passes += static_cast<long long>(iterations) * ctx->session_gamma;
-    const int status = finish_work(ctx, batch);
+    SPEC_TRY(finish_work(ctx, batch));  // (without a report there is nothing to read from it; after a wait that ran out, logits mean nothing)
     if (ctx->report->nonfinite)
         return fail(SPEC_ERR_NONFINITE, "a model produced a NaN or +inf logit, or a row without a finite logit (the tokens of these "
                                         "iterations are not valid)");
-    SPEC_TRY(status);
     SPEC_CUDA_TRY(cudaEventElapsedTime(elapsed_ms, ctx->ev[1], ctx->ev[2]));
     *remaining = 0;
     for (int b = 0; b < batch; ++b)

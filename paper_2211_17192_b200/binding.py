@@ -146,7 +146,7 @@ def spec_verify_sample(target_logits, draft_logits, draft_tokens, uniforms, temp
     outputs = (_ptr(n_accepted, torch.int32, "n_accepted"), _ptr(next_token, torch.int32, "next_token"),
                _ptr(workspace, torch.uint8, "workspace"), workspace.numel(), _stream())
     if top_k or top_p != 1.0:
-        _check(lib().spec_verify_sample_truncated(*pointers, batch, gamma, vocab, temperature, lenience, top_k, top_p, *outputs))
+        _check(lib().spec_verify_sample_truncated(*pointers, batch, gamma, vocab, temperature, lenience, int(top_k), top_p, *outputs))
     elif lenience == 1.0:
         _check(lib().spec_verify_sample(*pointers, batch, gamma, vocab, temperature, *outputs))
     else:

@@ -32,3 +32,15 @@ def test_any_alignment_against_the_oracle(vocab, temperature, top_k, top_p):
         for r in range(rows.shape[0]):
             token, margin = oracle_sampling.sample_token(rows[r], us.reshape(-1)[r], temperature, top_k, top_p)[:2]
             assert tokens[r] == token or margin < 1e-5 or top_p < 1.0 and oracle_sampling.nucleus_floor(rows[r], temperature, top_k, top_p)[1] < 5e-5
+
+
+def test_numbers_of_any_kind_as_options():
+    vocab, batch, gamma = 300, 2, 2
+    tl, ql = workloads.make_sampler_logits(1, batch, gamma, vocab, 1.0)
+    us = workloads.make_uniform_grid(2, (batch, gamma + 1))
+    xs = ql.argmax(axis=2).astype(np.int32)
+    t, q, x, u = to_dev(tl), to_dev(ql), to_dev(xs), to_dev(us)
+    want = binding.spec_verify_sample(t, q, x, u, 0.75, lenience=0.5, top_k=40, top_p=0.875)
+    for kind in (np.float32, np.float64, torch.tensor):
+        got = binding.spec_verify_sample(t, q, x, u, kind(0.75), lenience=kind(0.5), top_k=kind(40.0), top_p=kind(0.875))
+        assert all(torch.equal(a, b) for a, b in zip(got, want))

@@ -1020,8 +1020,10 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     const size_t report_bytes = sizeof(spec_report) + B * sizeof(int32_t);
     ctx->report_memory.assign(report_bytes, 0);
     ctx->report = reinterpret_cast<spec_report*>(ctx->report_memory.data());
-    cudaMemset(ctx->nonfinite, 0, sizeof(int));
-    cudaMemset(ctx->counters, 0, kCounters * sizeof(unsigned long long));
+    // (on the context's stream: nothing orders it after the default stream)
+    err = cudaMemsetAsync(ctx->nonfinite, 0, sizeof(int), ctx->stream);
+    if (err == cudaSuccess) err = cudaMemsetAsync(ctx->counters, 0, kCounters * sizeof(unsigned long long), ctx->stream);
+    if (err != cudaSuccess) return cleanup(fail(SPEC_ERR_CUDA, "counters: %s", cudaGetErrorString(err)));
     ctx->error_words[0] = gemm_tc_error_word();
     ctx->error_words[1] = gemm_wide_error_word();
     ctx->error_words[2] = pass_error_word();

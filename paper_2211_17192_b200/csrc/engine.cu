@@ -61,8 +61,9 @@ struct spec_ctx {
     // Captured passes of spec_forward_logits: a shape is captured the third time it is asked for (the capture costs about
     // a launch-bound pass or two); the oldest of eight makes room.
     struct PassGraph {
-        int which, batch, rows, uses;
+        int which, batch, rows, uses;  // (uses before there is a graph)
         cudaGraphExec_t exec;
+        bool refused;  // it could not be captured: plain launches for good
     };
     std::vector<PassGraph> pass_graphs;
 
@@ -1554,28 +1555,33 @@ extern "C" int spec_forward_logits(spec_ctx* ctx, int which, const int32_t* toke
                 if (ctx->pass_graphs.front().exec) cudaGraphExecDestroy(ctx->pass_graphs.front().exec);
                 ctx->pass_graphs.erase(ctx->pass_graphs.begin());
             }
-            ctx->pass_graphs.push_back({which, batch, rows, 0, nullptr});
+            ctx->pass_graphs.push_back({which, batch, rows, 0, nullptr, false});
             graph = &ctx->pass_graphs.back();
         }
-        if (++graph->uses >= 3 && !graph->exec) {
-            SPEC_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            const int status = forward(ctx, m, meta, batch, rows, n, nullptr, nullptr, nullptr, nullptr,
-                                       reinterpret_cast<float* const*>(ctx->row_block + 3 * n4));
+        if (!graph->exec && !graph->refused && ++graph->uses >= 3) {
+            // (a graph takes memory of its own, and without it the pass is the same, so a failure here is none of the call)
             cudaGraph_t g = nullptr;
-            const cudaError_t end = cudaStreamEndCapture(st, &g);
-            if (status != SPEC_OK) {
-                if (g) cudaGraphDestroy(g);
-                return status;
+            bool captured = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+            if (captured) {
+                captured = forward(ctx, m, meta, batch, rows, n, nullptr, nullptr, nullptr, nullptr,
+                                   reinterpret_cast<float* const*>(ctx->row_block + 3 * n4)) == SPEC_OK;
+                captured = cudaStreamEndCapture(st, &g) == cudaSuccess && captured;
             }
-            SPEC_CUDA_TRY(end);
-            const cudaError_t inst = cudaGraphInstantiate(&graph->exec, g, 0);
-            cudaGraphDestroy(g);
-            if (inst != cudaSuccess) graph->exec = nullptr;
-            SPEC_CUDA_TRY(inst);
+            if (!captured || cudaGraphInstantiate(&graph->exec, g, 0) != cudaSuccess) {
+                graph->exec = nullptr;
+                graph->refused = true;
+                cudaGetLastError();
+            }
+            if (g) cudaGraphDestroy(g);
         }
     }
-    if (graph && graph->exec) SPEC_CUDA_TRY(cudaGraphLaunch(graph->exec, st));
-    else SPEC_TRY(forward(ctx, m, meta, batch, rows, n, nullptr, nullptr, logits));
+    if (graph && graph->exec && cudaGraphLaunch(graph->exec, st) != cudaSuccess) {
+        cudaGetLastError();
+        cudaGraphExecDestroy(graph->exec);
+        graph->exec = nullptr;
+        graph->refused = true;
+    }
+    if (!graph || !graph->exec) SPEC_TRY(forward(ctx, m, meta, batch, rows, n, nullptr, nullptr, logits));
     SPEC_TRY(finish_work(ctx, 0));
     for (int b = 0; b < batch; ++b) ctx->cached[which][b] += rows;
     return SPEC_OK;

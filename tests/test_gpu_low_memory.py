@@ -93,3 +93,39 @@ def test_a_context_without_room_for_long_prompt_chunks(fixture):
         assert np.array_equal(same, tokens)
     finally:
         fixture.release()
+
+
+def test_repeated_passes_with_no_memory_left(fixture):
+    """From the third pass of a shape on a context replays a captured one, if there is memory for it."""
+    cfg = fixture.cfg
+    eng = binding.Engine(cfg, fixture.weights, max_batch=2, max_len=96, max_gamma=15)
+    outs = [torch.empty(2, rows, cfg["vocab"], device="cuda") for rows in (3, 1)]
+    steps = [np.ascontiguousarray(fixture.tokens[:, 16:16 + rows]) for rows in (3, 1)]
+    blocks = []
+
+    def passes():
+        for out, step in zip(outs, steps):
+            eng.truncate(0, [16, 16])
+            out.fill_(-1.0)
+            torch.cuda.synchronize()
+            binding._check(binding.lib().spec_forward_logits(eng._ctx, 0, step.ctypes.data, 2, step.shape[1], out.data_ptr()))
+
+    try:
+        eng.forward_logits(0, fixture.tokens[:, :16])
+        passes()
+        want = [out.cpu() for out in outs]
+        passes()
+        fixture.leave(8 * MB)
+        for size in (2 * MB, MB // 2):
+            try:
+                while True:
+                    blocks.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            except torch.OutOfMemoryError:
+                pass
+        for _ in range(4):
+            passes()
+            assert all(torch.equal(out.cpu(), w) for out, w in zip(outs, want))
+    finally:
+        blocks.clear()
+        fixture.release()
+        eng.close()

@@ -877,32 +877,37 @@ attention_f16_kernel(const float* qkv, int q_stride, const int32_t* pos,
 // attention_f16_kernel above; there is one key slice, so nothing is merged and the output is written here.  Bound by the
 // mma.sync chains of eight warps per SM.  Against the decode kernels on prompt chunks of 256 rows padded to the longest
 // sequence (7B shape): 16 prompts of 500 .. 1000 tokens 112 -> 22 ms of attention, one of 1024 tokens 19 -> 2 ms.
+//
+// TERMS: fp16 terms of a query.  One, where the decode kernels of the same batch work with one (attention_f16_kernel); two,
+// where they are the tf32 kernel, whose error against 64 bits one term would exceed (its probabilities are relative to the
+// maximum of a warp's own keys, so more of them are exact).  Probabilities are scaled by 2^10, so that small ones keep their
+// bits.
 constexpr int kPromptWarps = 8;
 constexpr int kPromptQueries = 16 * kPromptWarps;
 constexpr int kPromptStages = 3;
 
-template <int DH>
+template <int DH, int TERMS>
 struct PromptSmem {
-    static constexpr int kQ = kPromptQueries * DH;
+    static constexpr int kQ = kPromptQueries * DH;  // (of each term)
     static constexpr int kTile = kF16TileKeys * DH;
     static constexpr int kStage = 2 * kTile;  // K, then V
-    static constexpr size_t kBytes = static_cast<size_t>(kQ + kPromptStages * kStage) * sizeof(__half);
+    static constexpr size_t kBytes = static_cast<size_t>(TERMS * kQ + kPromptStages * kStage) * sizeof(__half);
 };
 
 // grid = (query blocks of the longest segment, n_kv_heads, segments), block = 32 * kPromptWarps.
 // segs[i] = (first row, rows, sequence, position of the first row).
-template <int DH>
+template <int DH, int TERMS>
 __global__ void __launch_bounds__(32 * kPromptWarps, DH == 64 ? 2 : 1)
 attention_prompt_kernel(const float* qkv, int q_stride, const int4* segs, int n_heads, int n_kv_heads,
                         const __grid_constant__ CUtensorMap kv_map, const int32_t* __restrict__ page_table, int pages_per_seq,
                         int page_size, float scale, const AttnOut out) {
-    using S = PromptSmem<DH>;
+    using S = PromptSmem<DH, TERMS>;
     constexpr int NB = kF16TileKeys / 8;
     constexpr float kLog2e = 1.4426950408889634f;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t landed[kPromptStages];
     __half* Qs = reinterpret_cast<__half*>(smem_raw);
-    __half* stages = Qs + S::kQ;
+    __half* stages = Qs + TERMS * S::kQ;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
 #pragma unroll
@@ -960,8 +965,15 @@ attention_prompt_kernel(const float* qkv, int q_stride, const int4* segs, int n_
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (q < queries)
             v = *reinterpret_cast<const float4*>(qkv + static_cast<size_t>(row0 + q / group) * q_stride + (kv_head * group + q % group) * DH + e);
-        *reinterpret_cast<uint2*>(Qs + f16_at<DH>(qi, e & ~7) + (e & 7)) =
-            make_uint2(pack_half2(v.x * q_scale, v.y * q_scale), pack_half2(v.z * q_scale, v.w * q_scale));
+        v = make_float4(v.x * q_scale, v.y * q_scale, v.z * q_scale, v.w * q_scale);
+        __half* to = Qs + f16_at<DH>(qi, e & ~7) + (e & 7);
+        const __half2 xy = __floats2half2_rn(v.x, v.y), zw = __floats2half2_rn(v.z, v.w);
+        *reinterpret_cast<__half2*>(to) = xy;
+        *reinterpret_cast<__half2*>(to + 2) = zw;
+        if (TERMS == 2) {
+            *reinterpret_cast<uint2*>(to + S::kQ) = make_uint2(pack_half2(v.x - __low2float(xy), v.y - __high2float(xy)),
+                                                               pack_half2(v.z - __low2float(zw), v.w - __high2float(zw)));
+        }
     }
     const int g = lane >> 2, t = lane & 3;
     const int q_lo = q0 + warp * 16 + g, q_hi = q_lo + 8;
@@ -1003,12 +1015,22 @@ attention_prompt_kernel(const float* qkv, int q_stride, const int4* segs, int n_
             for (int j = 0; j < 4; ++j) s[nb][j] = 0.0f;
 #pragma unroll
         for (int kp = 0; kp < DH / 32; ++kp) {
+            uint32_t low[2][4];  // (fetched again with every tile: registers hold the high terms only)
+            if (TERMS == 2) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    ldsm_x4(low[h], Qs + S::kQ + f16_at<DH>(warp * 16 + (lane & 7) + 8 * ((lane >> 3) & 1), (2 * kp + h) * 16 + 8 * (lane >> 4)));
+            }
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb) {
                 uint32_t kf[4];
                 ldsm_x4(kf, Kt + nb * 8 * 64 + (kp >> 1) * (kF16TileKeys * 64) + ((kp & 1) ? (k_lane ^ 32) : k_lane));
                 mma_f16(s[nb], qf[2 * kp], kf[0], kf[1]);
                 mma_f16(s[nb], qf[2 * kp + 1], kf[2], kf[3]);
+                if (TERMS == 2) {
+                    mma_f16(s[nb], low[0], kf[0], kf[1]);
+                    mma_f16(s[nb], low[1], kf[2], kf[3]);
+                }
             }
         }
         if (k0 + kF16TileKeys > all_see) {  // (warp-uniform)
@@ -1042,11 +1064,12 @@ attention_prompt_kernel(const float* qkv, int q_stride, const int4* segs, int n_
             m_lo = tmax_lo;
             m_hi = tmax_hi;
         }
+        const float base_lo = m_lo - 10.0f, base_hi = m_hi - 10.0f;  // (the sums carry the 2^10 too)
         uint32_t pa[NB / 2][4];
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb) {
-            const float p0 = exp2_approx(s[nb][0] - m_lo), p1 = exp2_approx(s[nb][1] - m_lo);
-            const float p2 = exp2_approx(s[nb][2] - m_hi), p3 = exp2_approx(s[nb][3] - m_hi);
+            const float p0 = exp2_approx(s[nb][0] - base_lo), p1 = exp2_approx(s[nb][1] - base_lo);
+            const float p2 = exp2_approx(s[nb][2] - base_hi), p3 = exp2_approx(s[nb][3] - base_hi);
             l_lo += p0 + p1;
             l_hi += p2 + p3;
             pa[nb / 2][(nb & 1) * 2] = pack_half2(p0, p1);
@@ -1365,7 +1388,7 @@ int launch_attention_variant(const Model& m, const AttnSource& src, const RowMet
                       static_cast<const float*>(part), slices, out.att, out.hi, out.lo);
 }
 
-template <int DH>
+template <int DH, int TERMS>
 int launch_prompt_variant(const Model& m, const AttnSource& src, const PromptSegments& segs, const AttnOut& out, cudaStream_t stream) {
     const int group = m.cfg.n_heads / m.cfg.n_kv_heads;
     CUtensorMap kv_map;
@@ -1374,18 +1397,18 @@ int launch_prompt_variant(const Model& m, const AttnSource& src, const PromptSeg
     if (status != SPEC_OK) return status;
     static std::atomic<unsigned long long> configured{0};
     if (first_use_on_this_device(configured))
-        SPEC_CUDA_TRY(cudaFuncSetAttribute(attention_prompt_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           static_cast<int>(PromptSmem<DH>::kBytes)));
+        SPEC_CUDA_TRY(cudaFuncSetAttribute(attention_prompt_kernel<DH, TERMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           static_cast<int>(PromptSmem<DH, TERMS>::kBytes)));
     const dim3 grid((group * segs.longest + kPromptQueries - 1) / kPromptQueries, m.cfg.n_kv_heads, segs.count);
-    return launch_pdl(attention_prompt_kernel<DH>, grid, dim3(32 * kPromptWarps), PromptSmem<DH>::kBytes, stream, src.q, src.q_stride,
+    return launch_pdl(attention_prompt_kernel<DH, TERMS>, grid, dim3(32 * kPromptWarps), PromptSmem<DH, TERMS>::kBytes, stream, src.q, src.q_stride,
                       segs.table, m.cfg.n_heads, m.cfg.n_kv_heads, kv_map, src.pool.page_table, src.pool.pages_per_seq,
                       src.pool.page_size, 1.0f / sqrtf(static_cast<float>(DH)), out);
 }
 
 }  // namespace
 
-// The precision of the f16 products is that of the tensor-core kernels that decode passes of bf16 models take (11
-// significant bits), from the same amount of work on; smaller prompts keep the decode kernels' fp32 products.
+// From the amount of work on at which decode passes of bf16 models take a tensor-core kernel; smaller prompts keep the decode
+// kernels' fp32 products.
 bool prompt_attention_serves(const Model& m, long long query_keys) {
     return m.bf16() && !m.t5() && m.kv_dtype == SPEC_DTYPE_FP16 && query_keys * m.cfg.n_heads >= 65536;
 }
@@ -1393,7 +1416,10 @@ bool prompt_attention_serves(const Model& m, long long query_keys) {
 int launch_prompt_attention(const Model& m, const AttnSource& src, const PromptSegments& segs, __nv_bfloat16* att_hi,
                             __nv_bfloat16* att_lo, cudaStream_t stream) {
     const AttnOut out{nullptr, att_hi, att_lo};
-    return m.cfg.d_head == 64 ? launch_prompt_variant<64>(m, src, segs, out, stream) : launch_prompt_variant<128>(m, src, segs, out, stream);
+    // (the line is attention_uses_f16's)
+    if (segs.batch * m.cfg.n_kv_heads >= kF16MinPairs)
+        return m.cfg.d_head == 64 ? launch_prompt_variant<64, 1>(m, src, segs, out, stream) : launch_prompt_variant<128, 1>(m, src, segs, out, stream);
+    return m.cfg.d_head == 64 ? launch_prompt_variant<64, 2>(m, src, segs, out, stream) : launch_prompt_variant<128, 2>(m, src, segs, out, stream);
 }
 
 int launch_attention(const Model& m, const AttnSource& src, const RowMeta& rows, int batch, int m_rows, int slices,

@@ -608,7 +608,7 @@ int feed_packed(spec_ctx* ctx, int which, const int32_t* tokens, int stride, con
     for (int done = 0; done < total;) {
         const int n = std::min(chunk, total - done), n4 = (n + 3) / 4 * 4;
         block.assign(static_cast<size_t>(3) * n4, 0);  // tokens, positions, sequences; then the segments
-        PromptSegments segs{reinterpret_cast<const int4*>(ctx->row_block + 3 * n4), 0, 0};
+        PromptSegments segs{reinterpret_cast<const int4*>(ctx->row_block + 3 * n4), 0, 0, batch};
         for (int r = 0; r < n; ++b, p = 0) {
             const int take = std::min(n - r, to[b] - p);
             if (take > 0) {

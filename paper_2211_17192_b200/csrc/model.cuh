@@ -191,10 +191,10 @@ int launch_attention(const Model& m, const AttnSource& src, const RowMeta& rows,
                      int max_keys, float* part, float* att, __nv_bfloat16* att_hi, __nv_bfloat16* att_lo, cudaStream_t stream);
 
 // A prompt chunk: the rows of `count` segments one after another, table[i] (device) = (first row, rows, sequence,
-// position of the first row), `longest` the most rows of any.
+// position of the first row), `longest` the most rows of any.  `batch`: sequences of the whole prompt pass.
 struct PromptSegments {
     const int4* table;
-    int count, longest;
+    int count, longest, batch;
 };
 // Whether the prompt kernel takes a chunk with this many (row, key it sees) pairs.
 bool prompt_attention_serves(const Model& m, long long query_keys);

@@ -607,15 +607,25 @@ int spec_linear(const float* x, const void* w, int w_dtype, int rows, int n_out,
                 float* y, void* workspace, size_t workspace_bytes, void* stream);
 int spec_device_error(void);
 
-/* Failure-path drill (no counterpart in the paper).  Every wait inside the library's kernels on
- * a barrier or a flag is bounded: when it runs out the kernel records a code, frees the tensor
- * memory it holds and returns, and the next synchronising call of the library reports
- * SPEC_ERR_DEVICE_TIMEOUT instead of hanging the GPU.  This call exercises that path without
- * breaking anything: it launches the tensor-core GEMM kernel on one tile with its producer
- * switched off (nothing is requested from memory, so nothing is in flight when the CTA gives
- * up) and a limit of 4096 polls, waits for it, and returns SPEC_ERR_DEVICE_TIMEOUT if the kernel
- * reported the expired wait as it should (SPEC_ERR_CUDA if it did not).  The device error flag
- * is clear afterwards and the context stays usable.  Synchronises `stream`. */
+/* Failure-path drills (no counterpart in the paper).  Every wait inside the library's kernels on
+ * a barrier or a flag is bounded: when it runs out the kernel records a code, waits (with a limit)
+ * for what it has in flight, frees the tensor memory it holds and returns, and the next
+ * synchronising call of the library reports SPEC_ERR_DEVICE_TIMEOUT instead of hanging the GPU.
+ * The codes are per device, not per context: whichever context synchronises next reports a time-out
+ * of another's kernel on the same device.  These calls exercise the path without breaking anything.
+ *
+ * spec_timeout_drill launches the two tensor-core GEMM kernels (one CTA, and a CTA pair) on one
+ * tile each with their producers switched off (nothing is requested from memory, so nothing is in
+ * flight when the CTAs give up) and a limit of 4096 polls, waits for them, and returns
+ * SPEC_ERR_DEVICE_TIMEOUT if both reported the expired wait as they should (SPEC_ERR_CUDA if not).
+ * The device error flags are clear afterwards and the context stays usable.  Synchronises `stream`.
+ *
+ * spec_timeout_drill_pass does the same for the kernel that runs few-row passes of a small bf16 model
+ * (which: 0 target, 1 draft) as one grid: a row at the cached length of sequence 0, of which no CTA
+ * publishes its share, with a limit of 64 tries per wait.  The cached length stays as it is; a
+ * generation in progress ends.  Errors: SPEC_ERR_DEVICE_TIMEOUT as intended, SPEC_ERR_BAD_CONFIG if
+ * the model's one-row passes are a chain of kernels. */
+int spec_timeout_drill_pass(spec_ctx* ctx, int which);
 int spec_timeout_drill(void* stream);
 
 #ifdef __cplusplus

@@ -540,9 +540,9 @@ __device__ __forceinline__ float exp2_approx(float x) {
 __device__ int g_attn_error;  // set when the bounded wait for a tile of the f16 kernel ran out (0 = none)
 
 // Waits, with a limit, for the phase of the given parity; false when the limit ran out.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, uint32_t limit = 1u << 22) {
     const uint32_t addr = static_cast<uint32_t>(__cvta_generic_to_shared(bar));
-    for (uint32_t spin = 0; spin < (1u << 22); ++spin) {
+    for (uint32_t spin = 0; spin < limit; ++spin) {
         uint32_t done;
         asm volatile(
             "{\n\t"
@@ -556,6 +556,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
         if (done) return true;
     }
     return false;
+}
+
+// Waits, with a limit, until no copy into the stages is in flight, after a wait that ran out.  (A barrier is past one of the
+// two parities at any time.)
+template <int STAGES>
+__device__ __forceinline__ void drain_stages(uint64_t (&landed)[STAGES]) {
+    for (int st = 0; st < STAGES; ++st)
+        for (int parity = 0; parity < 2; ++parity) mbar_wait_bounded(&landed[st], parity, 1u << 14);
 }
 
 // grid = (slices, n_kv_heads * q_blocks, batch), block = 128; q_blocks = ceil(queries / 64).  kv_map: the layer's pool
@@ -697,12 +705,17 @@ attention_f16_kernel(const float* qkv, int q_stride, const int32_t* pos,
     const int all_see = min(__reduce_min_sync(kFullMask, min(keys_lo, keys_hi)), seq_keys);
     const int any_sees = min(__reduce_max_sync(kFullMask, max(p_lo < 0 ? 0 : keys_lo, p_hi < 0 ? 0 : keys_hi)), seq_keys);
 
+    bool ok = true;
     for (int i = 0; i < my_tiles; ++i) {
         // tile i has landed (a wait that runs out is recorded and the pass goes on with what the stage holds: no
-        // thread leaves the loop alone, and the host sees the error)
-        if (!mbar_wait_bounded(&landed[i % S::kStages], (i / S::kStages) & 1)) atomicCAS(&g_attn_error, 0, 1);
-        __syncthreads();                     // everybody is done with tile i - 1, whose stage
-        issue(i + S::kStages - 1, pg_next);  // takes the tile that is kStages - 1 ahead
+        // thread leaves the loop alone, and the host sees the error; the waits that follow give up at once, and nothing
+        // more is asked for: a barrier whose bytes are still on their way must not be armed again)
+        if (!mbar_wait_bounded(&landed[i % S::kStages], (i / S::kStages) & 1, ok ? 1u << 22 : 1u)) {
+            atomicCAS(&g_attn_error, 0, 1);
+            ok = false;
+        }
+        __syncthreads();                             // everybody is done with tile i - 1, whose stage
+        if (ok) issue(i + S::kStages - 1, pg_next);  // takes the tile that is kStages - 1 ahead
         fetch_pages(i + S::kStages, pg_next);
         if (i == 0) {  // (the first barrier also covered the staged queries)
 #pragma unroll
@@ -804,6 +817,7 @@ attention_f16_kernel(const float* qkv, int q_stride, const int32_t* pos,
         }
     }
     // (every tile that was asked for has been waited for: nothing is in flight)
+    if (tid == 0 && !ok) drain_stages(landed);
 
     // park this warp's state in stage 0: [warp][query of the block][max (base-2 units), sum, O[DH]]
     __syncthreads();
@@ -994,11 +1008,15 @@ attention_prompt_kernel(const float* qkv, int q_stride, const int4* segs, int n_
 #pragma unroll
     for (int j = 0; j < 4; ++j) v_chunk[j] = ((((j << 1) | (lane >> 4)) ^ l7) & 7) << 3;
 
+    bool ok = true;
     for (int i = 0; i < tiles; ++i) {
-        // (a wait that runs out is recorded and the pass goes on: no thread leaves the loop alone)
-        if (!mbar_wait_bounded(&landed[i % kPromptStages], (i / kPromptStages) & 1)) atomicCAS(&g_attn_error, 0, 2);
+        // (a wait that runs out: as in attention_f16_kernel)
+        if (!mbar_wait_bounded(&landed[i % kPromptStages], (i / kPromptStages) & 1, ok ? 1u << 22 : 1u)) {
+            atomicCAS(&g_attn_error, 0, 2);
+            ok = false;
+        }
         __syncthreads();
-        issue(i + kPromptStages - 1);
+        if (ok) issue(i + kPromptStages - 1);
         if (i == 0) {
 #pragma unroll
             for (int ks = 0; ks < DH / 16; ++ks)
@@ -1087,6 +1105,7 @@ attention_prompt_kernel(const float* qkv, int q_stride, const int4* segs, int n_
         }
     }
     // (every tile that was asked for has been waited for: nothing is in flight)
+    if (tid == 0 && !ok) drain_stages(landed);
     l_lo += __shfl_xor_sync(kFullMask, l_lo, 1);
     l_lo += __shfl_xor_sync(kFullMask, l_lo, 2);
     l_hi += __shfl_xor_sync(kFullMask, l_hi, 1);

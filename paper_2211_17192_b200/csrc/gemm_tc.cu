@@ -640,14 +640,19 @@ extern "C" int spec_timeout_drill(void* stream) {
     if (status == SPEC_OK) status = cached_bf16_map(base, 16, 64, 16, true, &mx);
     if (status != SPEC_OK) return status;
     SPEC_CUDA_TRY(cudaStreamSynchronize(st));
-    gemm_tc_take_error();  // (whatever was pending is not this drill's)
-    // one CTA, one k-block, nothing requested: the MMA issuer's wait and the epilogue's wait run out after 4096 polls
+    // (whatever was pending is not this drill's)
+    gemm_tc_take_error();
+    gemm_wide_take_error();
+    // one CTA, one k-block, nothing requested: the MMA issuer's wait and the epilogue's wait run out after 4096 polls; then the
+    // same with a CTA pair
     status = launch_tc<16>(mw, mx, mx, reinterpret_cast<float*>(base), 128, 1, 1, 1, 0, st, 4096);
+    if (status == SPEC_OK) status = launch_gemm_wide_drill(base, 4096, st);
     if (status != SPEC_OK) return status;
     SPEC_CUDA_TRY(cudaStreamSynchronize(st));
-    const int code = gemm_tc_take_error();
-    if (code > 0) return fail(SPEC_ERR_DEVICE_TIMEOUT, "drill: the kernel gave up on a bounded wait (code %d), freed its tensor memory and returned", code);
-    return fail(SPEC_ERR_CUDA, "drill: the kernel did not report the wait that should have run out");
+    const int code = gemm_tc_take_error(), wide = gemm_wide_take_error();
+    if (code > 0 && wide > 0)
+        return fail(SPEC_ERR_DEVICE_TIMEOUT, "drill: the kernels gave up on a bounded wait (codes %d, %d), freed their tensor memory and returned", code, wide);
+    return fail(SPEC_ERR_CUDA, "drill: a kernel did not report the wait that should have run out (codes %d, %d)", code, wide);
 }
 
 extern "C" int spec_device_error(void) {

@@ -42,6 +42,8 @@ struct WideArgs {
     PartialPlan plan;
     int n_out, n_rows, stages, packed, fill, stream_once;
     int subs, sub_rows;  // a tile's rows are `subs` accumulators of sub_rows rows each
+    uint32_t limit;      // of every wait
+    int drill;           // spec_timeout_drill: the producers ask for nothing and arm no barrier
 };
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -156,7 +158,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
 
     if (warp == 0) {
         // ---- producer: this CTA's weight tile and its half (hi or lo) of the activation tile per stage ----
-        const bool leader = elect_one();
+        const bool leader = elect_one() && !a.drill;
         uint64_t policy_w, policy_x;
         if (a.stream_once) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy_w));
         else asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy_w));
@@ -187,7 +189,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         for (WideWork w(a, pair); ok && w.next(p, tile, k0, k1);)
             for (int kb = k0; kb < k1; ++kb) {
                 if (it >= ahead) {
-                    if (!mbar_wait_warp(&empty_bar[s], (use - 1) & 1)) { ok = false; break; }
+                    if (!mbar_wait_warp(&empty_bar[s], (use - 1) & 1, a.limit)) { ok = false; break; }
                     load_w(s, tile, kb);
                 }
                 load_x(s, tile, kb);
@@ -210,11 +212,11 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
             int buf = 0, turn = 0;  // accumulator buffer, and how often the buffers have gone round
             int tile, k0, k1;
             for (WideWork w(a, pair); ok && w.next(p, tile, k0, k1);) {
-                if (turn > 0 && !mbar_wait_warp(&acc_empty[buf], (turn - 1) & 1)) { ok = false; break; }
+                if (turn > 0 && !mbar_wait_warp(&acc_empty[buf], (turn - 1) & 1, a.limit)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t acc = tmem + buf * 256;
                 for (int kb = k0; kb < k1; ++kb) {
-                    if (!mbar_wait_warp(&full_bar[s], use & 1)) { ok = false; break; }
+                    if (!mbar_wait_warp(&full_bar[s], use & 1, a.limit)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t a_desc = smem_desc_sw128(base + s * stage_bytes);
                     const uint64_t b_desc = smem_desc_sw128(base + s * stage_bytes + kWeightBytes);
@@ -244,7 +246,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         int buf = 0, turn = 0;
         int tile, k0, k1;
         for (WideWork w(a, pair); w.next(p, tile, k0, k1);) {
-            if (!mbar_wait_warp(&acc_full[buf], turn & 1)) { ok = false; break; }
+            if (!mbar_wait_warp(&acc_full[buf], turn & 1, a.limit)) { ok = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int feature = ((tile / p.token_tiles) * 2 + static_cast<int>(rank)) * kTileM + quarter * 32 + lane;
             const int slot = partial_slot(p, tile, k0);
@@ -327,6 +329,7 @@ int launch_gemm_wide(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_ro
     a.stream_once = a.plan.token_tiles == 1 ? 1 : 0;
     a.subs = wide_subs(n_rows);
     a.sub_rows = a.plan.tok_tile / a.subs;
+    a.limit = kSpinLimit;
     const int stage_bytes = kWeightBytes + a.plan.tok_tile * kTileK * 2;
     a.stages = std::min(kMaxStages, kSmemBudget / stage_bytes);
     const int smem = a.stages * stage_bytes + 1024 + 512;
@@ -341,6 +344,24 @@ int launch_gemm_wide(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_ro
     if (first_use_on_this_device(configured))
         SPEC_CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     return launch_pdl(gemm_wide_kernel, dim3(2 * a.plan.pairs), dim3(kWideThreads), smem, stream, mw, mhi, mlo, partial, a);
+}
+
+// One pair of CTAs, one tile of one k-block, nothing requested, waits of `limit` polls; `base`: 16 KB that are never read.
+int launch_gemm_wide_drill(void* base, uint32_t limit, cudaStream_t stream) {
+    WideArgs a{};
+    a.plan = gemm_wide_plan(kTileM, kTileK, 16);
+    a.n_out = kTileM;
+    a.n_rows = a.sub_rows = 16;
+    a.subs = 1;
+    a.stages = 2;
+    a.limit = limit;
+    a.drill = 1;
+    CUtensorMap mw, mx;
+    int status = cached_bf16_map(base, kTileM, kTileK, kTileM, true, &mw);
+    if (status == SPEC_OK) status = cached_bf16_map(base, 16, kTileK, 16, true, &mx);
+    if (status != SPEC_OK) return status;
+    const int smem = a.stages * (kWeightBytes + a.sub_rows * kTileK * 2) + 1024 + 512;
+    return launch_pdl(gemm_wide_kernel, dim3(2 * a.plan.pairs), dim3(kWideThreads), smem, stream, mw, mx, mx, static_cast<float*>(base), a);
 }
 
 int* gemm_wide_error_word() { return symbol_address(g_wide_error); }

@@ -130,6 +130,7 @@ PartialPlan gemm_wide_plan(int n_out, int k, int n_rows);
 int launch_gemm_wide(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_rows, const void* w, bool packed, int n_rows,
                      int n_out, int k, float* partial, bool fill, cudaStream_t stream);
 int gemm_wide_take_error();
+int launch_gemm_wide_drill(void* base, uint32_t limit, cudaStream_t stream);
 // Device addresses of the words in which the kernels record a wait that ran out (0: none did).
 int* gemm_tc_error_word();
 int* gemm_wide_error_word();
@@ -259,7 +260,8 @@ int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocation
 bool small_pass_serves(const SmallPass& s, const Model& m, int batch, int m_rows);
 // Leaves the residual stream in h without the last FFN's result, whose partial sums are in s.last_part as small_pass_plan says.
 int launch_small_pass(const SmallPass& s, const Model& m, const RowMeta& rows, const PassTables& t, int batch, int m_rows, float* h,
-                      cudaStream_t stream);
+                      cudaStream_t stream, bool drill = false);
+// (`drill`: no CTA publishes its share of an exchange, and every wait gives up after 64 tries)
 PartialPlan small_pass_plan(const SmallPass& s);
 int* small_pass_error_word();
 int small_pass_take_error();

@@ -24,7 +24,8 @@
 // were two thirds slower).
 //
 // Every wait is bounded.  A wait that runs out is recorded and the kernel goes on with whatever is there (nobody leaves:
-// the others count on it); further waits then give up at once.
+// the others count on it); further waits then give up at once, nothing more is asked for - a barrier whose bytes are still
+// on their way must not be armed again -, and at the end the copies that are still in flight are waited for, with a limit.
 //
 // Measured, a whole pass with its head, chain of kernels against this: 160M shape, one row at context 1024 351 -> 199 us,
 // four sequences at 777 397 -> 267, eight at 500 411 -> 340; 97M shape, six rows at 200 348 -> 245, eight sequences at 500
@@ -53,6 +54,7 @@ constexpr int kMaxKi = kMaxD / 256;
 constexpr int kDh = 64;
 constexpr int kStateLen = 68;     // an attention state: max, sum, two of padding, 64 values
 constexpr uint32_t kSpin = 1u << 20;  // tries of a bounded wait: about a second
+constexpr uint32_t kDrain = 1u << 14;  // and of the last ones of a pass that gave up
 constexpr float kLog2e = 1.4426950408889634f;
 
 __device__ int g_small_error;  // first bounded wait that expired (0 = none)
@@ -78,6 +80,8 @@ struct SmallArgs {
     unsigned* epoch;                      // exchanges of all passes so far
     float* last_part;                     // [clusters][rows][d]: the last FFN's partial sums
     float* h_out;
+    uint32_t limit;                       // of every wait, in tries
+    int mute;                             // spec_timeout_drill_pass: nothing is published
 };
 
 // ---- what a CTA streams, phase by phase (the packing kernel and the pass agree on it through these) ----
@@ -215,7 +219,7 @@ struct Pass {
     __device__ __forceinline__ void expect(bool ok) { limit = ok ? limit : 1; }  // (the waits that follow give up at once; nobody leaves)
     // Asks for as many stages as the ring has room for, a lane each.  Called where a barrier has just followed the last reads.
     __device__ __forceinline__ void refill() {
-        if (warp == kWarps - 1) {
+        if (warp == kWarps - 1 && !__any_sync(kFullMask, limit == 1)) {
             int* asked = reinterpret_cast<int*>(sm + S::kMeta) + 24;  // stages so far, and in all
             const int from = asked[0], n = min(taken + kStages, asked[1]) - from;
             __syncwarp();
@@ -245,7 +249,7 @@ struct Pass {
     }
     // `bytes` will be sent to this CTA on barrier `which`; one thread says so.
     __device__ __forceinline__ void await_bytes(int which, int bytes) {
-        if (tid == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bars + which)), "r"(bytes) : "memory");
+        if (tid == 0 && limit != 1) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bars + which)), "r"(bytes) : "memory");
     }
     __device__ __forceinline__ void arrived(int which) {
         expect(bar_wait(bars + which, (turns >> which) & 1, limit));
@@ -262,7 +266,6 @@ struct Pass {
     __device__ __forceinline__ float gather(const unsigned long long* at, int count, unsigned when, float v) {
         const int stride = a.rows * kD;
         unsigned long long w[kClusters];
-#pragma unroll 1
 #pragma unroll 1
         for (uint32_t spin = 0;; ++spin) {
             bool all = true;
@@ -291,7 +294,7 @@ struct Pass {
     // The gain of the norm that follows comes with it.
     __device__ __forceinline__ void collect(int n, bool ffn_first, const float* gain) {
         await_bytes(kBarH, ((n ? a.rows : 0) + 1) * kD * 4);
-        if (tid == 0) {
+        if (tid == 0 && limit != 1) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(sm + S::kGain)),
                          "l"(gain), "r"(kD * 4), "r"(smem_u32(bars + kBarH))
@@ -742,7 +745,7 @@ struct Pass {
             float s = 0.0f;
 #pragma unroll 1
             for (int k = 0; k < ks; ++k) s += red()[(k * kWo + (f >> 4)) * 128 + (f & 15) * 8 + row];
-            publish(exchange(epoch) + (cluster * a.rows + row) * kD + rank * kDs + f, s, epoch);
+            if (!a.mute) publish(exchange(epoch) + (cluster * a.rows + row) * kD + rank * kDs + f, s, epoch);
         }
     }
 
@@ -824,7 +827,7 @@ struct Pass {
             for (int c = 1; c < kC; ++c) s += fred[(c * kDs + f) * R + row];
             const int at = (cluster * a.rows + row) * kD + rank * kDs + f;
             if (plain) plain[at] = s;
-            else publish(exchange(epoch) + at, s, epoch);
+            else if (!a.mute) publish(exchange(epoch) + at, s, epoch);
         }
     }
 };
@@ -860,7 +863,7 @@ small_pass_kernel(const __grid_constant__ SmallArgs a) {
         asked[1] = stages * a.n_layers;
     }
     __syncthreads();
-    P p{a, sm, bars, bars + 4, tid, lane, warp, rank, cluster, kSpin, 0, 0, 0, 0, *a.epoch};
+    P p{a, sm, bars, bars + 4, tid, lane, warp, rank, cluster, a.limit, 0, 0, 0, 0, *a.epoch};
     p.refill();
     // the embedding, every CTA for itself; the rows' positions, sequences and rotations
 #pragma unroll 1
@@ -914,7 +917,12 @@ small_pass_kernel(const __grid_constant__ SmallArgs a) {
         for (int i = tid; i < a.rows * kD; i += kThreads) a.h_out[i] = p.h(p.cur)[i];
         if (tid == 0) *a.epoch = p.epoch;
     }
-    if (p.limit == 1) atomicCAS(&g_small_error, 0, 1);
+    if (p.limit == 1) {
+        atomicCAS(&g_small_error, 0, 1);
+        // the copies that this thread or warp asked for: a barrier is past one of the two parities at any time
+        if (tid == 0) bar_wait(bars + P::kBarH, 0, kDrain), bar_wait(bars + P::kBarH, 1, kDrain);
+        if (warp == kWarps - 1 && lane < S::kStages) bar_wait(&p.full[lane], 0, kDrain), bar_wait(&p.full[lane], 1, kDrain);
+    }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __syncthreads();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");  // nobody leaves while a peer may still write here
@@ -1110,7 +1118,7 @@ bool small_pass_serves(const SmallPass& s, const Model& m, int batch, int m_rows
 }
 
 int launch_small_pass(const SmallPass& s, const Model& m, const RowMeta& rows, const PassTables& t, int batch, int m_rows, float* h,
-                      cudaStream_t stream) {
+                      cudaStream_t stream, bool drill) {
     const spec_model_cfg& c = m.cfg;
     const int group = c.n_heads / c.n_kv_heads;
     SmallArgs a{};
@@ -1161,6 +1169,8 @@ int launch_small_pass(const SmallPass& s, const Model& m, const RowMeta& rows, c
     a.epoch = s.epoch;
     a.last_part = s.last_part;
     a.h_out = h;
+    a.limit = drill ? 64 : kSpin;
+    a.mute = drill ? 1 : 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kC * s.clusters);
     cfg.blockDim = dim3(kThreads);

@@ -65,7 +65,38 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_leaves_the_library_usable(
     assert binding.spec_device_error() == 0
 
 
-def test_greedy_guess_off_the_drafts_argmax():
+@pytest.mark.parametrize("base", ["llama_test_target", "t5_test_target"])
+def test_a_one_kernel_pass_whose_exchange_never_comes(base):
+    """No CTA of the pass publishes its share: all of them give up and go on, the next call reports it, and the pass after it is
+    what it was before."""
+    cfg = workloads.scaled_config(workloads.model_config(base), n_layers=3)
+    eng = binding.Engine(cfg, workloads.make_weights(cfg, 4), max_batch=1, max_len=64, page_size=32, max_gamma=7,
+                         max_src_len=40 if cfg["arch"] == "t5" else 0)
+    h = binding.lib()
+    h.spec_timeout_drill_pass.restype = ctypes.c_int
+    h.spec_timeout_drill_pass.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    try:
+        if cfg["arch"] == "t5":
+            eng.encode([workloads.make_prompt(5, 40, cfg["vocab"])])
+        tokens = workloads.make_prompt(3, 12, cfg["vocab"])[None]
+        eng.forward_logits(0, tokens[:, :8])
+        want = [eng.forward_logits(0, tokens[:, i:i + 1]) for i in range(8, 12)]
+        for _ in range(3):
+            eng.truncate(0, [8])
+            assert h.spec_timeout_drill_pass(eng._ctx, 0) == -6, h.spec_last_error().decode()
+            assert b"gave up on a bounded wait" in h.spec_last_error()
+            assert binding.spec_device_error() == 0
+            for i in range(8, 12):
+                assert torch.equal(eng.forward_logits(0, tokens[:, i:i + 1]), want[i - 8])
+    finally:
+        eng.close()
+    chain = workloads.scaled_config(cfg, n_layers=1)
+    eng = binding.Engine(chain, workloads.make_weights(chain, 4), max_batch=1, max_len=64, page_size=32, max_src_len=40 if cfg["arch"] == "t5" else 0)
+    assert h.spec_timeout_drill_pass(eng._ctx, 0) == -2
+    eng.close()
+
+
+
     """T = 0 with a drafted token that is not the draft's own maximum (x ~ q cannot produce it,
     so Algorithm 1's test decides nothing): library and oracle accept it iff it is the
     target's maximum."""

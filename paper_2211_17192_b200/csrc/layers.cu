@@ -3,7 +3,11 @@
 // in a fixed order, adds the residual) and prepares the input of the GEMM after
 // it (fp32, and/or split into two bf16 terms for the tensor-core path), so that
 // a block is nine launches: norm, qkv GEMM, rope + KV append, attention,
-// out-projection GEMM, norm, FFN-in GEMM, activation, FFN-out GEMM.
+// out-projection GEMM, norm, FFN-in GEMM, activation, FFN-out GEMM; ten where
+// attention's key slices are merged by a kernel of their own (long contexts).
+// fp32 models have the norms and the activation inside their GEMMs
+// (gemm_rows.cu), few rows of a small bf16 model all of it in one kernel
+// (small_pass.cu).
 #include <cmath>
 
 #include "attn_unit.cuh"

@@ -1,7 +1,7 @@
 // Speculative sampling (Section 2.3 / Algorithm 1, accept-adjust-draw part),
 // plain standardised sampling (Section 2.2) and the method's uniforms.
 //
-// spec_verify_sample is two kernels on one stream:
+// spec_verify_sample is two kernels on one stream (few logits: one; with a cut: another first one; see below):
 //   1. verify_stats_kernel streams every logit of p_1..p_{gamma+1} and
 //      q_1..q_gamma exactly once from HBM.  A CTA reduces one chunk of one row
 //      to (max, sum exp) with an online rescale, and also picks up the row's
@@ -1155,17 +1155,17 @@ __device__ float select_floor(const Slice<VEC, LOADS>& s, const Team<SOLO>& team
 // +inf, or when more than kSelCap logits reach the pivot (heavy ties): the binned selection then does the row.
 constexpr int kMostTops = 512;
 
-template <int T, bool VEC, int LOADS, bool SOLO>
-__device__ int top_k_list(const Slice<VEC, LOADS>& s, const Team<SOLO>& team, unsigned k, SelShared& sh) {
+// One CTA to a row: a list has few passes, which a cluster does not pay for (cut_shape).
+template <int T, bool VEC, int LOADS>
+__device__ int top_k_list(const Slice<VEC, LOADS>& s, unsigned k, SelShared& sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // (measured on 960 rows of 32000: k = 40 66 us per call against 82 binned, k = 128 71, k = 200 92: the pivot sinks
     // with k and lets ever more logits through)
     if (k > 128) return -1;
-    float* own = reinterpret_cast<float*>(sh.cand_mass);  // this CTA's maxima, then everyone's
-    float* tops = own + kMostTops;
-    const int warps = (T / 32) * team.size;
-    const int per_warp = min(min(32, kMostTops / warps), (3 * static_cast<int>(k) + warps - 1) / warps);
-    const int n_tops = per_warp * warps, per_cta = per_warp * (T / 32);
+    float* tops = reinterpret_cast<float*>(sh.cand_mass);
+    constexpr int kWarps = T / 32;
+    const int per_warp = min(min(32, kMostTops / kWarps), (3 * static_cast<int>(k) + kWarps - 1) / kWarps);
+    const int n_tops = per_warp * kWarps;
     float mine = -INFINITY;
     for_each_logit<T>(s, [&](float v) { mine = fmaxf(mine, v); });
     {
@@ -1179,11 +1179,9 @@ __device__ int top_k_list(const Slice<VEC, LOADS>& s, const Team<SOLO>& team, un
             if (lane == __ffs(who) - 1) key = 0;
             if (lane == i && top != 0) given = __uint_as_float(top ^ ((top >> 31) ? 0x80000000u : 0xffffffffu));
         }
-        if (lane < per_warp) own[warp * per_warp + lane] = given;
+        if (lane < per_warp) tops[warp * per_warp + lane] = given;
     }
     if (tid == 0) { sh.n_cand = 0; sh.n_hit = 0; }
-    team.sync();
-    for (int i = tid; i < n_tops; i += T) tops[i] = reinterpret_cast<const float*>(team.of(sh, i / per_cta).cand_mass)[i % per_cta];
     __syncthreads();
     // the k-th largest of the maxima: the largest one that at least k of them reach; `per` threads count for each
     int per = 1;
@@ -1218,7 +1216,7 @@ __device__ int top_k_list(const Slice<VEC, LOADS>& s, const Team<SOLO>& team, un
     for (int h = warp; h < hits; h += (T / 32))  // a warp goes over what one of those threads has read
         for (int g = s.g0 + sh.cnt[h] + lane * T; g < s.g1; g += 32 * T)
             list_group(s.row.raw(g, -INFINITY), 4 * g - s.row.shift, pivot, sh);
-    return gather_list<T>(team, false, sh);
+    return gather_list<T>(Team<true>(), false, sh);
 }
 
 // The k-th largest of the listed logits.  In the first CTA.
@@ -1459,7 +1457,7 @@ cut_floor_kernel(const float* a, size_t a_stride, int a_rows, const float* b, si
     int listed = -1;  // logits listed (the same in all CTAs; floor, row_max and sum of a listed row are the first one's)
     const bool nucleus = top_p > 0.0f && top_p < 1.0f;
     if (top_k > 0 && top_k < vocab) {
-        listed = top_k_list<T>(s, team, static_cast<unsigned>(top_k), sh);
+        if constexpr (SOLO) listed = top_k_list<T>(s, static_cast<unsigned>(top_k), sh);
         if (listed >= 0) {
             if (first) floor = top_k_of_list<T>(static_cast<unsigned>(top_k), sh);
         } else {

@@ -1348,10 +1348,8 @@ int launch_attention_variant(const Model& m, const AttnSource& src, const RowMet
 #define SPEC_LAUNCH_F16(MB, F, CLUSTER)                                                                                 \
     do {                                                                                                                \
         static std::atomic<unsigned long long> configured{0};                                                           \
-        if (first_use_on_this_device(configured))                                                                       \
-            SPEC_CUDA_TRY(cudaFuncSetAttribute(attention_f16_kernel<DH, MB, F>,                                         \
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,                             \
-                                               static_cast<int>(F16Smem<DH, MB>::kBytes)));                             \
+        status = allow_shared_memory(configured, attention_f16_kernel<DH, MB, F>, static_cast<int>(F16Smem<DH, MB>::kBytes));  \
+        if (status != SPEC_OK) return status;                                                                            \
         status = launch_attn(attention_f16_kernel<DH, MB, F>, grid, dim3(32 * kF16Warps), F16Smem<DH, MB>::kBytes,      \
                              CLUSTER, stream, src.q, src.q_stride, rows.pos, rows.seq, m_rows, m.cfg.n_heads,           \
                              m.cfg.n_kv_heads, q_blocks, kv_map, src.pool.page_table, src.pool.pages_per_seq,           \
@@ -1375,10 +1373,8 @@ int launch_attention_variant(const Model& m, const AttnSource& src, const RowMet
 #define SPEC_LAUNCH_MMA(F, T, CLUSTER)                                                                                  \
     do {                                                                                                                \
         static std::atomic<unsigned long long> configured{0};                                                           \
-        if (first_use_on_this_device(configured))                                                                       \
-            SPEC_CUDA_TRY(cudaFuncSetAttribute(attention_mma_kernel<KV, DH, F, T>,                                      \
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,                             \
-                                               static_cast<int>(MmaSmem<DH, T>::kBytes)));                              \
+        status = allow_shared_memory(configured, attention_mma_kernel<KV, DH, F, T>, static_cast<int>(MmaSmem<DH, T>::kBytes)); \
+        if (status != SPEC_OK) return status;                                                                            \
         status = launch_attn(attention_mma_kernel<KV, DH, F, T>, grid, dim3(32 * kMmaWarps), MmaSmem<DH, T>::kBytes,    \
                              CLUSTER, stream, src.q, src.q_stride, rows.pos, rows.seq, m_rows, m.cfg.n_heads,           \
                              m.cfg.n_kv_heads, m_blocks, pool, src.pool.page_table, src.pool.pages_per_seq,            \
@@ -1411,13 +1407,12 @@ template <int DH, int TERMS>
 int launch_prompt_variant(const Model& m, const AttnSource& src, const PromptSegments& segs, const AttnOut& out, cudaStream_t stream) {
     const int group = m.cfg.n_heads / m.cfg.n_kv_heads;
     CUtensorMap kv_map;
-    const int status = cached_f16_rows_map(src.pool.kv, static_cast<unsigned long long>(src.pool.n_pages) * 2 * m.cfg.n_kv_heads *
+    int status = cached_f16_rows_map(src.pool.kv, static_cast<unsigned long long>(src.pool.n_pages) * 2 * m.cfg.n_kv_heads *
                                                             src.pool.page_size, DH, &kv_map);
     if (status != SPEC_OK) return status;
     static std::atomic<unsigned long long> configured{0};
-    if (first_use_on_this_device(configured))
-        SPEC_CUDA_TRY(cudaFuncSetAttribute(attention_prompt_kernel<DH, TERMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           static_cast<int>(PromptSmem<DH, TERMS>::kBytes)));
+    status = allow_shared_memory(configured, attention_prompt_kernel<DH, TERMS>, static_cast<int>(PromptSmem<DH, TERMS>::kBytes));
+    if (status != SPEC_OK) return status;
     const dim3 grid((group * segs.longest + kPromptQueries - 1) / kPromptQueries, m.cfg.n_kv_heads, segs.count);
     return launch_pdl(attention_prompt_kernel<DH, TERMS>, grid, dim3(32 * kPromptWarps), PromptSmem<DH, TERMS>::kBytes, stream, src.q, src.q_stride,
                       segs.table, m.cfg.n_heads, m.cfg.n_kv_heads, kv_map, src.pool.page_table, src.pool.pages_per_seq,

@@ -8,6 +8,7 @@
 
 #include <cstdarg>
 #include <cstdio>
+#include <mutex>
 
 #include "spec_decode.h"
 
@@ -55,14 +56,30 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // environment variable the library reads, documented in the public header).
 bool pdl_enabled();  // api.cu
 
-// True the first time it is called on the current device for this flag word (one bit per
-// device ordinal below 64): per-device one-time setup such as a kernel's shared-memory opt-in,
-// which a process that uses several GPUs has to repeat on each of them.
-inline bool first_use_on_this_device(std::atomic<unsigned long long>& seen) {
+// Does `configure` (which returns a status) unless it has been done on the current device for this flag word (one bit per
+// device ordinal below 64): per-device one-time setup such as a kernel's shared-memory opt-in, which a process that
+// uses several GPUs has to repeat on each of them.  Another thread that comes meanwhile waits for it; a failure is tried again.
+template <typename F>
+inline int once_on_this_device(std::atomic<unsigned long long>& done, F configure) {
     int device = 0;
-    if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return true;
+    if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return configure();
     const unsigned long long bit = 1ull << device;
-    return (seen.fetch_or(bit) & bit) == 0;
+    if (done.load(std::memory_order_acquire) & bit) return SPEC_OK;
+    static std::mutex mutex;
+    std::lock_guard<std::mutex> lock(mutex);
+    if (done.load(std::memory_order_relaxed) & bit) return SPEC_OK;
+    const int status = configure();
+    if (status == SPEC_OK) done.fetch_or(bit, std::memory_order_release);
+    return status;
+}
+
+// More than 48 KB of dynamic shared memory for a kernel.
+template <typename... KArgs>
+inline int allow_shared_memory(std::atomic<unsigned long long>& done, void (*kernel)(KArgs...), int bytes) {
+    return once_on_this_device(done, [&]() -> int {
+        SPEC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        return SPEC_OK;
+    });
 }
 
 // `cluster` > 0: in thread block clusters of that many CTAs along x.

@@ -385,9 +385,8 @@ template <int N_TOK>
 int launch_tc(const CUtensorMap& mw, const CUtensorMap& mhi, const CUtensorMap& mlo, float* partial, int n_out,
               int n_rows, int k_blocks, int splits, int packed, cudaStream_t stream, int drill = 0) {
     static std::atomic<unsigned long long> configured{0};
-    if (first_use_on_this_device(configured))
-        SPEC_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<N_TOK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           Smem<N_TOK>::kTotal));
+    const int status = allow_shared_memory(configured, gemm_tc_kernel<N_TOK>, Smem<N_TOK>::kTotal);
+    if (status != SPEC_OK) return status;
     const dim3 grid((n_out + kTileM - 1) / kTileM, splits, 1);
     return launch_pdl(gemm_tc_kernel<N_TOK>, grid, dim3(kThreads), Smem<N_TOK>::kTotal, stream, mw, mhi, mlo, partial,
                       n_out, n_rows, k_blocks, packed, drill);

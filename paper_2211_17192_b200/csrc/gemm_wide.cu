@@ -341,8 +341,8 @@ int launch_gemm_wide(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int hi_ro
     if (status == SPEC_OK) status = cached_bf16_map(lo, hi_rows, k, a.sub_rows, true, &mlo);
     if (status != SPEC_OK) return status;
     static std::atomic<unsigned long long> configured{0};
-    if (first_use_on_this_device(configured))
-        SPEC_CUDA_TRY(cudaFuncSetAttribute(gemm_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    status = allow_shared_memory(configured, gemm_wide_kernel, 227 * 1024);
+    if (status != SPEC_OK) return status;
     return launch_pdl(gemm_wide_kernel, dim3(2 * a.plan.pairs), dim3(kWideThreads), smem, stream, mw, mhi, mlo, partial, a);
 }
 

@@ -1062,8 +1062,8 @@ namespace {
 template <typename KV, int DH>
 int launch_variant(const MegaArgs& args, int ctas, cudaStream_t stream) {
     static std::atomic<unsigned long long> configured{0};
-    if (first_use_on_this_device(configured))
-        SPEC_CUDA_TRY(cudaFuncSetAttribute(pass_kernel<KV, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem::kTotal));
+    const int status = allow_shared_memory(configured, pass_kernel<KV, DH>, Smem::kTotal);
+    if (status != SPEC_OK) return status;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(kThreads);

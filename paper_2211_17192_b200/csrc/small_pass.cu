@@ -1043,10 +1043,13 @@ int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocation
     const spec_model_cfg& c = m.cfg;
     const int ki = c.d_model / 256, group = c.n_heads / c.n_kv_heads, units = c.d_ff / 16, gated = c.ffn != SPEC_FFN_GELU ? 1 : 0;
     static std::atomic<unsigned long long> configured{0};
-    if (first_use_on_this_device(configured))
+    const int status = once_on_this_device(configured, []() -> int {
         for (int k = 1; k <= kMaxKi; ++k)
             for (int rows = 2; rows <= 8; rows *= 2)
                 SPEC_CUDA_TRY(cudaFuncSetAttribute(pick(k, rows).fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+        return SPEC_OK;
+    });
+    if (status != SPEC_OK) return status;
     // all clusters have to be resident at once
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kC * kClusters);

@@ -10,11 +10,13 @@ use: there is no fallback of any kind.
 
 import ctypes
 import os
+import threading
 
 import torch
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "lib", "libspecdecode.so")
 _lib = None
+_loading = threading.Lock()
 
 STATUS_NAMES = {
     0: "SPEC_OK", -1: "SPEC_ERR_BAD_ARG", -2: "SPEC_ERR_BAD_CONFIG", -3: "SPEC_ERR_OOM", -4: "SPEC_ERR_CAPACITY",
@@ -36,13 +38,18 @@ def lib():
     """The loaded shared library (loads it on first call)."""
     global _lib
     if _lib is None:
-        if not os.path.exists(_LIB_PATH):
-            raise RuntimeError(
-                f"{_LIB_PATH} is missing: build it with `python -m paper_2211_17192_b200.build` "
-                "(there is no fallback path)")
-        handle = ctypes.CDLL(_LIB_PATH)
-        _declare(handle)
-        _lib = handle
+        with _loading:  # (one handle for all threads: what is declared on it has to be there for everyone)
+            if _lib is None:
+                if not os.path.exists(_LIB_PATH):
+                    raise RuntimeError(
+                        f"{_LIB_PATH} is missing: build it with `python -m paper_2211_17192_b200.build` "
+                        "(there is no fallback path)")
+                handle = ctypes.CDLL(_LIB_PATH)
+                _declare(handle)
+                # (declared where they are called: the function objects exist from here on, so that two threads declare the same one)
+                for name in ("choose_gamma", "linear_partials", "generate_adaptive", "set_gamma", "attention_plan", "pass_trace"):
+                    getattr(handle, "spec_" + name)
+                _lib = handle
     return _lib
 
 
@@ -338,8 +345,14 @@ _engine_declared = False
 
 def _declare_engine(h):
     global _engine_declared
-    if _engine_declared:
-        return
+    if not _engine_declared:
+        with _loading:
+            if not _engine_declared:
+                _declare_engine_calls(h)
+                _engine_declared = True
+
+
+def _declare_engine_calls(h):
     c = ctypes
     vp = c.c_void_p
     h.spec_init.restype = c.c_int
@@ -372,7 +385,6 @@ def _declare_engine(h):
     h.spec_time_forward.argtypes = [vp, c.c_int, c.c_int, c.c_int, c.c_int, c.POINTER(c.c_float)]
     h.spec_encode.restype = c.c_int
     h.spec_encode.argtypes = [vp, vp, vp, c.c_int, c.c_int]
-    _engine_declared = True
 
 
 def _cfg_struct(cfg):

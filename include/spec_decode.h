@@ -342,7 +342,9 @@ typedef struct spec_runtime_cfg {
                              inside the 2e-2 logit tolerance of bf16 models; bf16 keeps 8, which on
                              wide or deep models moves logits by more than that. */
     int max_src_len;      /* T5: longest source the encoders are given (0 for decoder-only models) */
-    int pass_kernel;      /* 0 (default): every pass is a chain of kernels.  1: passes of at most 16 rows of
+    int pass_kernel;      /* 0 (default): every pass is a chain of kernels, except that the blocks of a small bf16
+                             decoder (two or more, 256, 512 or 768 wide, heads of 64, fp16 K,V rows) are one kernel
+                             for up to eight rows.  1: passes of at most 16 rows of
                              a bf16 GPT- or Llama-shaped model run as one persistent cooperative kernel
                              (one CTA per SM, grid-wide barriers between the steps, weights streamed
                              ahead of the steps that wait); same results within the parity tolerances,

@@ -249,6 +249,27 @@ def weight_stream_bytes(cfg):
     return total
 
 
+def pass_launches(engine, which, cfg, batch, rows):
+    """Kernels of one pass over `rows` rows per sequence of this model, with its logits."""
+    if cfg["arch"] in ("bigram", "copy"):
+        return 1
+    n = batch * rows
+    bf16 = cfg["dtype"] == "bf16"
+    group = cfg["n_heads"] // cfg["n_kv_heads"]
+    if (bf16 and engine.kv_dtype == "fp16" and cfg["d_head"] == 64 and cfg["d_model"] in (256, 512, 768) and group <= 4 and
+            cfg["n_kv_heads"] <= 16 and cfg["d_ff"] % 16 == 0 and cfg["n_layers"] >= 2 and n * group <= 8):
+        return 4  # all blocks as one kernel; norm, head GEMM and its reduction
+    # attention, and the kernel that merges its key slices where no cluster does
+    attention = lambda cross: 1 if engine.attention_plan(which, batch, rows, cross)["cluster_merge"] else 2
+    t5 = cfg["arch"] == "t5"
+    if bf16:  # four GEMMs, two norms, rotary / append, attention, activation; cross-attention: norm, two GEMMs, queries, attention
+        block = 8 + attention(False) + (4 + attention(True) if t5 else 0)
+        return 1 + cfg["n_layers"] * block + 3
+    norm = 0 if n <= 8 or (n <= 64 and cfg["d_model"] <= 512) else 1  # (otherwise inside the GEMM behind it, as the activation always is)
+    block = 5 + 2 * norm + attention(False) + (2 + norm + attention(True) if t5 else 0)
+    return 1 + cfg["n_layers"] * block + norm + 1
+
+
 class GenerationWorkload:
     dtype = "bf16"
 
@@ -287,6 +308,7 @@ class GenerationWorkload:
         self.prompts = [workloads.make_prompt(1000 * rank + b, self.prompt_len, self.tcfg["vocab"]) for b in range(self.batch)]
         self.budget_tokens = grow
         self.kv_elem_bytes = 2 if self.engine.kv_dtype in ("fp16", "bf16") else 4
+        self.launches_per_iteration()
 
     def close(self):
         self.engine.close()
@@ -298,13 +320,14 @@ class GenerationWorkload:
         return self.batch * context * 2 * c["n_layers"] * c["n_kv_heads"] * c["d_head"] * self.kv_elem_bytes
 
     def launches_per_iteration(self):
-        # per block: 4 GEMMs, 2 norms, RoPE/append, attention, activation (+ the combine kernel when the
-        # key slices are not merged inside a cluster: long contexts); embed, final norm, head, its reduction
-        long_context = self.prompt_len > 256
-        fwd = lambda cfg, combine: 1 + (9 + combine) * cfg["n_layers"] + 3
-        draft = 1 if self.dcfg["arch"] in ("bigram", "copy") else fwd(self.dcfg, 0)  # (few slices: merged in the cluster)
-        target = fwd(self.tcfg, 1 if long_context else 0)
-        return 1 + self.gamma * (1 + draft + 1) + 1 + target + 2 + 1
+        """Kernels of one iteration, counted from how the library launches these shapes (while there is an engine to ask)."""
+        if self.engine is not None:
+            drafts = self.engine, 1, self.dcfg, self.batch
+            rows = [2] + [1] * (self.gamma - 1) if self.gamma else []  # (the first draft step feeds two rows per sequence)
+            # uniforms; rows, pass and draw per draft step; rows, pass, two sampling kernels; commit
+            self._launches = (1 + sum(1 + pass_launches(*drafts, r) + 1 for r in rows) +
+                              1 + pass_launches(self.engine, 0, self.tcfg, self.batch, self.gamma + 1) + 2 + 1)
+        return self._launches
 
     def timed_decode(self, warmup, steps, gamma):
         """Device time of `steps` iterations after `warmup` untimed ones (prompt pass untimed)."""
@@ -471,11 +494,7 @@ class EncDecWorkload(GenerationWorkload):
         self.prompts = [workloads.make_prompt(1000 * rank + b, self.prompt_len, self.tcfg["vocab"]) for b in range(self.batch)]
         self.budget_tokens = grow
         self.kv_elem_bytes = 2 if self.engine.kv_dtype in ("fp16", "bf16") else 4
-
-    def launches_per_iteration(self):
-        # per decoder block: 7 GEMMs, 3 norms, K/V append, cross-attention queries, 2 attentions, activation
-        fwd = lambda cfg: 1 + 15 * cfg["n_layers"] + 3
-        return 1 + self.gamma * (1 + fwd(self.dcfg) + 1) + 1 + fwd(self.tcfg) + 2 + 1
+        self.launches_per_iteration()
 
     def kv_bytes(self, context):
         c = self.tcfg

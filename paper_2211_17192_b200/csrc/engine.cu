@@ -996,12 +996,14 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     };
     const size_t before_rows = ctx->allocations.size();
     status = alloc_rows();
-    if (ctx->max_rows > pass_rows(256) && (status == SPEC_ERR_OOM || (status == SPEC_OK && !memory_to_spare(0)))) {
+    size_t spare = status == SPEC_OK ? memory_to_spare() : 0;
+    if (ctx->max_rows > pass_rows(256) && (status == SPEC_ERR_OOM || (status == SPEC_OK && !spare))) {
         cudaStreamSynchronize(ctx->stream);
         for (size_t i = before_rows; i < ctx->allocations.size(); ++i) cudaFree(ctx->allocations[i]);
         ctx->allocations.resize(before_rows);
         ctx->max_rows = pass_rows(256);
         status = alloc_rows();
+        if (status == SPEC_OK) spare = memory_to_spare();
     }
     if (status != SPEC_OK) return cleanup(status);
     // Page j of sequence b is pool page j * max_batch + b: consecutive pages of a
@@ -1034,7 +1036,7 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     ctx->cached[1].assign(B, 0);
     // (last: everything that a context cannot do without has its memory)
     for (int i = 0; i < n_models && !rt.pass_kernel; ++i)
-        if ((status = small_pass_init(ctx->small[i], ctx->model[i], ctx->allocations, ctx->stream)) != SPEC_OK) return cleanup(status);
+        if ((status = small_pass_init(ctx->small[i], ctx->model[i], ctx->allocations, spare, ctx->stream)) != SPEC_OK) return cleanup(status);
     *out = ctx;
     return SPEC_OK;
 }

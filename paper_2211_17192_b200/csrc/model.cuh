@@ -235,15 +235,16 @@ int launch_pass(const PassScratch& s, const Model& m, int which, const RowMeta& 
 void pass_scratch_release(PassScratch& s);
 int pass_take_error();
 
-// Whether `bytes` of device memory can be taken for something that only makes a context faster: 512 MB more stay free, for
-// the graphs that the context will capture and for what the caller allocates next.
-inline bool memory_to_spare(size_t bytes) {
+// Device memory that can be taken for what only makes a context faster: 512 MB stay free, for the graphs that the context will
+// capture and for what the caller allocates next.
+inline size_t memory_to_spare() {
     size_t free = 0, total = 0;
     if (cudaMemGetInfo(&free, &total) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return 0;
     }
-    return free >= bytes + (static_cast<size_t>(512) << 20);
+    const size_t reserve = static_cast<size_t>(512) << 20;
+    return free > reserve ? free - reserve : 0;
 }
 
 // small_pass.cu: the blocks of a small decoder over at most 8 rows as one cooperative kernel.
@@ -256,7 +257,7 @@ struct SmallPass {
     float* last_part = nullptr;
     size_t cta_bytes = 0;
 };
-int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocations, cudaStream_t stream);
+int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocations, size_t& spare, cudaStream_t stream);  // (`spare`: see above; what it takes comes off)
 bool small_pass_serves(const SmallPass& s, const Model& m, int batch, int m_rows);
 // Leaves the residual stream in h without the last FFN's result, whose partial sums are in s.last_part as small_pass_plan says.
 int launch_small_pass(const SmallPass& s, const Model& m, const RowMeta& rows, const PassTables& t, int batch, int m_rows, float* h,

@@ -1038,7 +1038,7 @@ bool shape_fits(const Model& m) {
 
 }  // namespace
 
-int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocations, cudaStream_t stream) {
+int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocations, size_t& spare, cudaStream_t stream) {
     s = SmallPass{};
     if (!shape_fits(m)) return SPEC_OK;
     const spec_model_cfg& c = m.cfg;
@@ -1091,11 +1091,12 @@ int small_pass_init(SmallPass& s, const Model& m, std::vector<void*>& allocation
     char* base = nullptr;
     const size_t bytes = gain_bytes + epoch_bytes + ll_bytes + part_bytes + s.cta_bytes * ctas;
     // a third copy of the weights, for speed alone: without room for it the chain of kernels serves the model
-    if (!memory_to_spare(bytes) || cudaMalloc(reinterpret_cast<void**>(&base), bytes) != cudaSuccess) {
+    if (bytes > spare || cudaMalloc(reinterpret_cast<void**>(&base), bytes) != cudaSuccess) {
         cudaGetLastError();
         return SPEC_OK;
     }
     allocations.push_back(base);
+    spare -= bytes;
     s.gains = reinterpret_cast<float*>(base);
     s.epoch = reinterpret_cast<unsigned*>(base + gain_bytes);
     s.exchanges = reinterpret_cast<unsigned long long*>(base + gain_bytes + epoch_bytes);

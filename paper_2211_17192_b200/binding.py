@@ -424,6 +424,8 @@ class Engine:
             structs.append(None if cfg is None else self._upload(cfg, weights))
         rt = _RuntimeCfg(max_batch, max_len, page_size, max_gamma, _DTYPE[kv_dtype], max_src_len, 1 if pass_kernel else 0)
         self.max_batch, self.max_len, self.max_gamma = max_batch, max_len, max_gamma
+        # (the context packs the weights on a stream of its own: what torch's stream still has to write of them comes first)
+        torch.cuda.current_stream(self.device).synchronize()
         ctx = ctypes.c_void_p()
         tc = _cfg_struct(target_cfg)
         dc = _cfg_struct(draft_cfg) if draft_cfg is not None else None

@@ -316,8 +316,9 @@ typedef struct spec_layer_weights {
 } spec_layer_weights;
 
 /* All pointers are DEVICE pointers that the caller keeps alive until
- * spec_free(); `layers` itself is a HOST array of n_layers entries that is
- * copied during spec_init. */
+ * spec_free(), with their contents complete when spec_init is called (it reads
+ * them on a stream of its own); `layers` itself is a HOST array of n_layers
+ * entries that is copied during spec_init. */
 typedef struct spec_weights {
     const void* tok_emb;  /* [vocab, d_model] */
     const void* pos_emb;  /* [max_positions, d_model], GPT only */

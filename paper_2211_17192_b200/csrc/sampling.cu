@@ -19,6 +19,7 @@
 // leaves the statistics (cut_floor_kernel).
 #include <algorithm>
 #include <cfloat>
+#include <cstddef>
 #include <mutex>
 
 #include <cooperative_groups.h>
@@ -312,14 +313,14 @@ __device__ int locate_in_range(const Weights& w, int r0, int r1, float rem, bool
 // positive weight if rounding leaves none.  The vocabulary is cut into WARPS
 // contiguous segments (one per warp); the segment holding the target is then
 // resolved by locate_in_range.  Returns the index to all threads, the total
-// through *total_out.
+// through *total_out.  `mine`: the sum over this warp's segment, where it is known already.
 template <int WARPS, class Weights>
-__device__ int block_inverse_cdf(const Weights& w, int vocab, float u, CdfScratch<WARPS>& s, float* total_out) {
+__device__ int block_inverse_cdf(const Weights& w, int vocab, float u, CdfScratch<WARPS>& s, float* total_out, const float* mine = nullptr) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int groups = w.groups();
     const int seg = (groups + WARPS - 1) / WARPS;
     const int g0 = min(groups, warp * seg), g1 = min(groups, g0 + seg);
-    const float acc = warp_range_sum<kCdfBatch>(w, g0, g1, lane);
+    const float acc = mine ? *mine : warp_range_sum<kCdfBatch>(w, g0, g1, lane);
     if (lane == 0) s.part[warp] = acc;
     __syncthreads();
     float total = 0.0f;
@@ -343,7 +344,7 @@ __device__ int block_inverse_cdf(const Weights& w, int vocab, float u, CdfScratc
 // target goes on to resolve it.  Returns the index in that CTA and -1 in the
 // others; the total is returned to all.
 template <int WARPS, class Weights>
-__device__ int cluster_inverse_cdf(const Weights& w, int vocab, float u, CdfScratch<WARPS>& s, float* total_out) {
+__device__ int cluster_inverse_cdf(const Weights& w, int vocab, float u, CdfScratch<WARPS>& s, float* total_out, const float* own = nullptr) {
     cg::cluster_group cluster = cg::this_cluster();
     const int nctas = static_cast<int>(cluster.num_blocks());
     const int rank = static_cast<int>(cluster.block_rank());
@@ -363,7 +364,7 @@ __device__ int cluster_inverse_cdf(const Weights& w, int vocab, float u, CdfScra
     const int b0 = seg_begin(mine), b1 = seg_end(mine);
     // When a warp's segment fits one batch of fetches, the weights stay in registers: the warp whose segment
     // holds the target then walks it without going back to memory.
-    const bool keep = seg <= 32 * kClusterCdfBatch;  // (uniform across the cluster)
+    const bool keep = !own && seg <= 32 * kClusterCdfBatch;  // (uniform across the cluster)
     float4 kept[kClusterCdfBatch];
     float acc;
     if (keep) {
@@ -381,7 +382,7 @@ __device__ int cluster_inverse_cdf(const Weights& w, int vocab, float u, CdfScra
         }
         acc = warp_sum(acc);
     } else {
-        acc = warp_range_sum<kClusterCdfBatch>(w, b0, b1, lane);
+        acc = own ? *own : warp_range_sum<kClusterCdfBatch>(w, b0, b1, lane);
     }
     if (lane == 0) s.part[warp] = acc;
     cluster.sync();
@@ -837,7 +838,6 @@ constexpr int kMostCtas = 4;    // per row
 static_assert(kSelSegments == 64, "two segments to a lane");
 
 struct SelShared {
-    unsigned cnt[kSelBins];
     unsigned mass_lo[kSelBins], mass_hi[kSelBins];  // a bin's mass, low and high word (apart: the low words then spread over all banks)
     float cand[kSelCap];
     unsigned long long cand_mass[kSelCap];
@@ -845,6 +845,7 @@ struct SelShared {
     unsigned long long warp_mass[kSelMostWarps];
     unsigned warp_cnt[kSelMostWarps];
     float warp_lo[kSelMostWarps], warp_hi[kSelMostWarps], warp_top[kSelMostWarps];
+    float below[kSelMostWarps];                     // mass that the warps have not listed (list_candidates)
     float cta_max[kMostCtas], cta_sum[kMostCtas];  // (in the CTA of rank 0)
     unsigned n_cand, n_hit, n_list;  // listed here; threads that reach the pivot; listed in all CTAs (in rank 0's)
     float floor;    // what rank 0 found
@@ -853,6 +854,7 @@ struct SelShared {
     int bin;
     unsigned in_bin;
     unsigned long long before, target;
+    unsigned cnt[kSelBins];  // (last: a nucleus from its candidates has no use for it)
 };
 
 // The CTAs that share a row.
@@ -947,6 +949,18 @@ __device__ __forceinline__ void for_each_logit(const Slice<VEC, LOADS>& s, F f) 
     });
 }
 
+// What a warp has listed of its row: at[0] .. at[n - 1].
+struct Listed {
+    const float* at;
+    int n;
+    float from, most;  // what is listed reaches `from`; the thread's largest logit
+    float ref;         // the reference of the weights in `SelShared::below`
+};
+template <int T, class F>
+__device__ __forceinline__ void for_each_logit(const Listed& s, F f) {
+    for (int i = threadIdx.x & 31; i < s.n; i += 32) f(s.at[i]);
+}
+
 __device__ __forceinline__ float warp_min(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -956,20 +970,28 @@ __device__ __forceinline__ float warp_min(float v) {
 // The floor among the finite logits >= kf: MASS = false, the k-th largest of
 // them; MASS = true, the nucleus of mass top_p with weights exp2((l - max) * c2).
 // Every thread of the team returns the same value; -inf means "keep everything".
-template <int T, bool MASS, bool VEC, int LOADS, bool SOLO>
-__device__ float select_floor(const Slice<VEC, LOADS>& s, const Team<SOLO>& team, float kf, unsigned k, float top_p, float c2, SelShared& sh) {
+// Of a Source that is not the row but its listed candidates: the nucleus of the row, NaN where the list does not decide it.
+template <int T, bool MASS, bool SOLO, class Source>
+__device__ float select_floor(const Source& s, const Team<SOLO>& team, float kf, unsigned k, float top_p, float c2, SelShared& sh) {
+    constexpr bool LIST = std::is_same<Source, Listed>::value;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // 1. range and number of the logits in play
     float lo = INFINITY, hi = -INFINITY, all = -INFINITY;
     unsigned n = 0;
-    for_each_logit<T>(s, [&](float v) {
-        all = fmaxf(all, v);
-        const bool in_play = fabsf(v) < INFINITY && v >= kf;
-        const float u = in_play ? v : __int_as_float(0x7fc00000);  // (fminf and fmaxf pass over a NaN operand)
-        lo = fminf(lo, u);
-        hi = fmaxf(hi, u);
-        n += in_play;
-    });
+    if constexpr (LIST) {
+        lo = s.from;
+        hi = all = s.most;
+        n = 1;
+    } else {
+        for_each_logit<T>(s, [&](float v) {
+            all = fmaxf(all, v);
+            const bool in_play = fabsf(v) < INFINITY && v >= kf;
+            const float u = in_play ? v : __int_as_float(0x7fc00000);  // (fminf and fmaxf pass over a NaN operand)
+            lo = fminf(lo, u);
+            hi = fmaxf(hi, u);
+            n += in_play;
+        });
+    }
     // what the warps of the whole team found
     auto of_all = [&](float& least, float& most, float& top, unsigned& count) {
         least = warp_min(least);
@@ -992,9 +1014,12 @@ __device__ float select_floor(const Slice<VEC, LOADS>& s, const Team<SOLO>& team
         top = warp_max(top);
         count = __reduce_add_sync(0xffffffffu, count);
     };
-    team.sync();  // (the shared arrays may still be read by a previous call)
+    if (!LIST) team.sync();  // (the shared arrays may still be read by a previous call)
     of_all(lo, hi, all, n);
     if (tid == 0) sh.row_top = all;
+    if constexpr (LIST) {
+        if (!(hi < INFINITY && hi >= lo)) return NAN;
+    }
     if (n == 0 || (!MASS && k > n)) return kf;  // nothing to cut
     // weight exp2((l - max) * c2) of a logit in units of 2^-32 (the largest float below 2^32, so that the row's
     // maximum still fits 32 bits): a bin's mass is then one 32-bit shared-memory atomic and, rarely, a carry
@@ -1003,7 +1028,7 @@ __device__ float select_floor(const Slice<VEC, LOADS>& s, const Team<SOLO>& team
 
     unsigned long long before = 0, target = k;  // counts, or masses
     for (int level = 0; level < kSelLevels; ++level) {
-        if (lo == hi) return hi;  // everything left is one value: it stays whole
+        if (lo == hi && !(LIST && level == 0)) return hi;  // everything left is one value: it stays whole
         const float top = hi, bottom = lo;
         // (top - v) * scale stays below kSelBins for every v >= bottom: the quarter bin absorbs the roundings
         const float scale = fminf((static_cast<float>(kSelBins) - 0.25f) / (top - bottom), FLT_MAX);
@@ -1061,8 +1086,17 @@ __device__ float select_floor(const Slice<VEC, LOADS>& s, const Team<SOLO>& team
                 b += from[1];
             }
             const unsigned long long upto = scan(a + b), all_of_it = __shfl_sync(0xffffffffu, upto, 31);
-            if (MASS && level == 0)  // the first level sees every logit in play: top_p of their mass is the target
-                target = static_cast<unsigned long long>(ceil(static_cast<double>(top_p) * static_cast<double>(all_of_it)));
+            if (MASS && level == 0) {  // the first level sees every logit in play: top_p of their mass is the target
+                double mass = static_cast<double>(all_of_it);
+                bool decided = true;
+                if constexpr (LIST) {  // .. and what is not listed
+                    float below = 0.0f;
+                    for (int i = lane; i < team.size * (T / 32); i += 32) below += team.of(sh, i / (T / 32)).below[i % (T / 32)];
+                    mass += static_cast<double>(warp_sum(below) * fast_exp2((s.ref - hi) * c2)) * 4294967040.0;
+                    decided = top_p * mass <= static_cast<double>(all_of_it);  // (not so for a NaN or infinite mass)
+                }
+                target = decided ? static_cast<unsigned long long>(ceil(static_cast<double>(top_p) * mass)) : 0ull;
+            }
             const unsigned long long above = before + upto - (a + b);
             const unsigned who = __ballot_sync(0xffffffffu, above < target && above + a + b >= target);
             if (who) {
@@ -1088,6 +1122,7 @@ __device__ float select_floor(const Slice<VEC, LOADS>& s, const Team<SOLO>& team
         const int bin = sh.bin;
         before = sh.before;
         target = sh.target;
+        if (LIST && target == 0) return NAN;
         // top-k knows how many logits the bin holds; the nucleus keeps no counts and finds out by copying them
         const bool few = MASS || sh.in_bin <= kSelCap;
         // a cheap test that no logit of the bin fails (its centre, half its width and the roundings of bin_of, with
@@ -1145,6 +1180,139 @@ __device__ float select_floor(const Slice<VEC, LOADS>& s, const Team<SOLO>& team
         hi = new_hi;
     }
     return lo;
+}
+
+template <int T>
+__device__ __forceinline__ float block_max(float v, float* per_warp) {
+    v = warp_max(v);
+    if ((threadIdx.x & 31) == 0) per_warp[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = per_warp[0];
+#pragma unroll
+    for (int w = 1; w < (T / 32); ++w) v = fmaxf(v, per_warp[w]);
+    return v;
+}
+// ---- the nucleus from a list of candidates ----
+// A nucleus is a few per cent of a row as a rule, so the row is read once: a sample of it, 32 groups per warp and spread over
+// the row, says above which logit its mass lies with room to spare; the pass lists what reaches that, every warp for
+// itself, and adds up the mass of the rest.  The selection, the statistics and the draw's sums then go over the list, in shared
+// memory.  A list that overflows or carries less than top_p of the mass decides nothing: the row is then binned as it lies.
+// The mass below is a float sum in a fixed order, so a row always gives the same floor, as with bins.
+// What bounded the bins was an atomic per logit and three passes over the row behind the one that read it; now it is issue of
+// the one pass (a dozen instructions per logit, over the same time as the loads) and the barriers of the selection.  Rows N(0, 3^2),
+// p = 0.9, with the draw, cold, between two events, binned against listed: 200 x 100000 80 us, 57; 64 x 100000 51, 35; 1 x
+// 50000 49, 23; 200 x 32000 35, 27; 24 x 9 rows of 50003, verified, 85, 50.  Short rows are all barriers, of which the list has
+// more: 16 x 8192 14, 16, but 96 x 17 rows of 8192, verified, 62, 54.  (Bins for the sampled range alone, no list: one pass over the row
+// fewer than bins, but its atomics, in a few lanes of every warp, cost as much as in all of them: 200 x 100000 72.)
+constexpr int kSampleBins = 256;
+constexpr float kSampleRange = 24.0f;  // of the bins, in powers of two below the largest
+// Of the sampled logits as many are listed as carry all but half of (1 - top_p) of their mass, but a tenth at least: a sample of
+// logits N(0, 3^2) holds few of those that carry the mass, and with a sixty-fourth as the least one row in 20 was listed too short.
+constexpr float kListLeast = 0.10f, kListShare = 0.15f;
+// Slots per warp: kListShare of its logits, 5 standard deviations (two CTAs with 100000 logits each then share an SM).
+inline int list_slots(int vocab, int ctas, int threads) {
+    const float most = kListShare * (32.0f * vocab / (ctas * threads) + 256.0f);
+    return static_cast<int>(most + 5.0f * sqrtf(most)) + 1;
+}
+
+// The logit from which on candidates are listed; +inf where the sample says that a list would not do.  *ref: the sample's
+// largest.  The same in all CTAs of a row.
+template <int T, bool VEC, int LOADS>
+__device__ float candidate_floor(const Slice<VEC, LOADS>& s, float top_p, float c2, SelShared& sh, float* ref) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, groups = s.row.groups();
+    const int g = static_cast<int>(static_cast<long long>(max(groups - 32, 0)) * warp / (T / 32 - 1)) + lane;
+    const float4 v = g < groups ? s.row.raw(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    for (int i = tid; i < kSampleBins; i += T) sh.mass_lo[i] = 0;
+    const float most = block_max<T>(fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)), sh.warp_hi);  // (the bins are clear)
+    *ref = most;
+    if (!(fabsf(most) < INFINITY)) return INFINITY;  // (uniform)
+    const float scale = c2 * (kSampleBins / kSampleRange);
+    auto count = [&](float x) {
+        const float b = (most - x) * scale;
+        if (b < static_cast<float>(kSampleBins)) atomicAdd(&sh.mass_lo[max(static_cast<int>(b), 0)], 1u);  // (not for a NaN)
+    };
+    count(v.x);
+    count(v.y);
+    count(v.z);
+    count(v.w);
+    __syncthreads();
+    if (warp == 0) {
+        constexpr int kEach = kSampleBins / 32;
+        float n[kEach], m[kEach], all_n = 0.0f, all_m = 0.0f;
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {
+            const int bin = lane * kEach + i;
+            n[i] = static_cast<float>(sh.mass_lo[bin]);
+            m[i] = n[i] * fast_exp2((static_cast<float>(bin) + 0.5f) * (-kSampleRange / kSampleBins));
+            all_n += n[i];
+            all_m += m[i];
+        }
+        float upto_n = warp_inclusive_scan(all_n, lane), upto_m = warp_inclusive_scan(all_m, lane);
+        const float total = __shfl_sync(kFullMask, upto_m, 31);
+        const float enough = (1.0f - 0.5f * (1.0f - top_p)) * total, least = (1.0f - 0.9f * (1.0f - top_p)) * total;
+        upto_n -= all_n;
+        upto_m -= all_m;
+        int bin = -1;
+        bool good = false;
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {  // the first bin down to which there is mass enough, or as many logits as can be listed
+            upto_n += n[i];
+            upto_m += m[i];
+            if (bin < 0 && ((upto_m >= enough && upto_n >= kListLeast * 4 * T) || upto_n > kListShare * 4 * T)) {
+                bin = lane * kEach + i;
+                good = upto_m >= least && upto_n <= 1.2f * kListShare * 4 * T;
+            }
+        }
+        const unsigned who = __ballot_sync(kFullMask, bin >= 0);
+        if (who == 0) {  // fewer logits within the bins than are listed at least
+            if (lane == 0) sh.floor = most - kSampleRange / c2;
+        } else if (lane == __ffs(who) - 1) {
+            sh.floor = good ? most - static_cast<float>(bin + 1) / scale : INFINITY;
+        }
+    }
+    __syncthreads();
+    return sh.floor;
+}
+
+// Lists the candidates of this warp's part of the slice, as the inverse CDF cuts it.
+template <int T, bool VEC, int LOADS>
+__device__ Listed list_candidates(const Slice<VEC, LOADS>& s, int each, float from, float ref, float c2, int slots, float* lists, SelShared& sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned before_me = (1u << lane) - 1;
+    const int seg = (each + T / 32 - 1) / (T / 32);
+    const int b0 = min(s.g1, s.g0 + warp * seg), b1 = min(s.g1, b0 + seg);
+    float* list = lists + warp * slots;
+    const float mc = fminf(-ref * c2, FLT_MAX);
+    float below = 0.0f, most = -INFINITY;
+    int n = 0;
+    const int last = slots - 1;  // (what does not fit goes to the last slot)
+    auto one = [&](float x) {
+        const bool in = x >= from;
+        const unsigned who = __ballot_sync(kFullMask, in);
+        if (in) list[min(n + __popc(who & before_me), last)] = x;
+        n += __popc(who);
+        below += in ? 0.0f : fast_exp2(fmaf(x, c2, mc));
+        most = fmaxf(most, x);
+    };
+    for (int base = b0; base < b1; base += 32 * LOADS) {
+        float4 v[LOADS];
+#pragma unroll
+        for (int i = 0; i < LOADS; ++i) {
+            const int g = base + 32 * i + lane;
+            v[i] = g < b1 ? s.row.raw(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        }
+#pragma unroll
+        for (int i = 0; i < LOADS; ++i) {
+            one(v[i].x);
+            one(v[i].y);
+            one(v[i].z);
+            one(v[i].w);
+        }
+    }
+    below = warp_sum(n > slots ? INFINITY : below);
+    if (lane == 0) sh.below[warp] = below;
+    __syncwarp();
+    return Listed{list, min(n, slots), from, most, ref};
 }
 
 // Top-k for k up to 128, without bins: every warp gives its largest lane maxima, 3 k of them in all; the k-th largest of
@@ -1252,16 +1420,6 @@ __device__ int list_row(const Slice<VEC, LOADS>& s, const Team<SOLO>& team, floa
     return gather_list<T>(team, false, sh);
 }
 
-template <int T>
-__device__ __forceinline__ float block_max(float v, float* per_warp) {
-    v = warp_max(v);
-    if ((threadIdx.x & 31) == 0) per_warp[threadIdx.x >> 5] = v;
-    __syncthreads();
-    v = per_warp[0];
-#pragma unroll
-    for (int w = 1; w < (T / 32); ++w) v = fmaxf(v, per_warp[w]);
-    return v;
-}
 template <int T>
 __device__ __forceinline__ unsigned long long block_sum(unsigned long long v, unsigned long long* per_warp) {
 #pragma unroll
@@ -1432,11 +1590,14 @@ constexpr int kFloorsOnly = 0, kWithStats = 1, kWithDraw = 2;
 // top-k they cost nothing, the list is there (24 x 9 rows of 50003, k = 40, p = 0.9: 66 us with kernels of their own, 40 so
 // with 1024 threads to a row, 32 with 512; 200 rows of 100000, k = 40, with the draw: 73, 28 and 22; one of 32000: 16, 9 and
 // 8), and after a nucleus one pass less and no second kernel (200 rows of 100000: 99, 91 and 70).
-template <int T, int LOADS, bool VEC, bool SOLO, int WORK>
-__global__ void __launch_bounds__(T, T == 256 ? 5 : LOADS == 8 ? 2 : 3)
+// LIST: the nucleus alone, from a list of `slots` candidates per warp.
+template <int T, int LOADS, bool VEC, bool SOLO, int WORK, bool LIST>
+__global__ void __launch_bounds__(T, LIST ? 1024 / T : T == 256 ? 5 : LOADS == 8 ? 2 : 3)
 cut_floor_kernel(const float* a, size_t a_stride, int a_rows, const float* b, size_t b_stride, int b_rows, int vocab, int top_k,
-                 float top_p, float c2, float* floors, CutWork work) {
-    __shared__ SelShared sh;
+                 float top_p, float c2, float* floors, CutWork work, int slots) {
+    extern __shared__ float lists[];
+    __shared__ __align__(16) unsigned char shared[LIST ? offsetof(SelShared, cnt) : sizeof(SelShared)];
+    SelShared& sh = *reinterpret_cast<SelShared*>(shared);
     pdl_wait();
     pdl_trigger();  // after the wait: the finishing kernel fetches inputs at once
     a = after_wait(a);
@@ -1456,7 +1617,18 @@ cut_floor_kernel(const float* a, size_t a_stride, int a_rows, const float* b, si
     float floor = -INFINITY, row_max = 0.0f, sum = 0.0f;
     int listed = -1;  // logits listed (the same in all CTAs; floor, row_max and sum of a listed row are the first one's)
     const bool nucleus = top_p > 0.0f && top_p < 1.0f;
-    if (top_k > 0 && top_k < vocab) {
+    Listed found{};
+    bool candidates = false;  // the nucleus came from them
+    if constexpr (LIST) {
+        float ref;
+        const float from = candidate_floor<T>(s, top_p, c2, sh, &ref);
+        if (from < INFINITY) {
+            found = list_candidates<T>(s, each, from, ref, c2, slots, lists, sh);
+            const float f = select_floor<T, true>(found, team, -INFINITY, 0u, top_p, c2, sh);
+            candidates = f == f;
+            if (candidates) floor = f;
+        }
+    } else if (top_k > 0 && top_k < vocab) {
         if constexpr (SOLO) listed = top_k_list<T>(s, static_cast<unsigned>(top_k), sh);
         if (listed >= 0) {
             if (first) floor = top_k_of_list<T>(static_cast<unsigned>(top_k), sh);
@@ -1467,12 +1639,25 @@ cut_floor_kernel(const float* a, size_t a_stride, int a_rows, const float* b, si
     }
     if (listed >= 0) {
         if (first) finish_list<T>(nucleus, top_p, c2, sh, &floor, &row_max, &sum);
-    } else if (nucleus) {
+    } else if (nucleus && !candidates) {
         floor = select_floor<T, true>(s, team, floor, 0u, top_p, c2, sh);
     }
     if (threadIdx.x == 0 && first && floors) floors[at] = floor;
+    float kept = 0.0f;  // the candidates that are kept, of this warp
+    if (LIST && WORK != kFloorsOnly && candidates) {
+        row_max = sh.row_top;
+        for_each_logit<T>(found, [&](float v) { kept += v >= floor ? fast_exp2((v - row_max) * c2) : 0.0f; });
+        kept = warp_sum(kept);
+    }
     if (WORK == kWithStats) {
-        if (listed < 0) row_statistics<T>(s, team, floor, c2, sh, &row_max, &sum);
+        if (LIST && candidates) {
+            if (threadIdx.x % 32 == 0) sh.below[threadIdx.x / 32] = kept;  // (read long ago)
+            team.sync();
+            if (threadIdx.x == 0 && first)
+                for (int i = 0; i < team.size * (T / 32); ++i) sum += team.of(sh, i / (T / 32)).below[i % (T / 32)];
+        } else if (listed < 0) {
+            row_statistics<T>(s, team, floor, c2, sh, &row_max, &sum);
+        }
         if (threadIdx.x == 0 && first) {
             float at_x = 0.0f;  // (none for p_{gamma+1})
             if (row != a_rows - 1) {
@@ -1504,7 +1689,8 @@ cut_floor_kernel(const float* a, size_t a_stride, int a_rows, const float* b, si
             pw.max_p = fmaxf(sh.row_top, -FLT_MAX);
             pw.c2 = c2;
             float total;
-            token = SOLO ? block_inverse_cdf<T / 32>(pw, vocab, u, cdf, &total) : cluster_inverse_cdf<T / 32>(pw, vocab, u, cdf, &total);
+            const float* mine = LIST && candidates ? &kept : nullptr;
+            token = SOLO ? block_inverse_cdf<T / 32>(pw, vocab, u, cdf, &total, mine) : cluster_inverse_cdf<T / 32>(pw, vocab, u, cdf, &total, mine);
         }
         // (of a cluster one CTA has drawn, and the others have -1)
         if (threadIdx.x == 0 && (SOLO || token >= 0)) work.tokens[static_cast<size_t>(at) * work.token_stride] = max(0, min(token, vocab - 1));
@@ -1572,6 +1758,10 @@ size_t verify_sample_workspace_bytes(int batch, int gamma, int vocab) {
     return stats_bytes(batch, gamma, vocab) + static_cast<size_t>(batch) * rows * sizeof(float) + 256;
 }
 
+constexpr size_t kMostListBytes = 160 * 1024;  // of candidates; a longer row is binned as it lies
+constexpr size_t kTwoListsBytes = 80 * 1024;   // of each of two CTAs on an SM
+size_t list_bytes(int vocab, int ctas, int threads) { return static_cast<size_t>(list_slots(vocab, ctas, threads)) * (threads / 32) * sizeof(float); }
+
 // How the rows of a cut are shared out.
 struct CutShape {
     int threads, loads, ctas;  // of a CTA; in flight per thread; CTAs per row
@@ -1584,11 +1774,16 @@ struct CutShape {
 // - a cluster pays where few rows are long and binned (4 x 512 threads against 512: 16 x 50003 26, 37; 16 x 128000 29, 53;
 //   64 x 100000 32, 50; 2 x 512: 128 x 100000 51, 66), not on more rows (200 x 100000 with two: 87, 70), shorter ones (16 x
 //   32000: 19, 18) or a list, whose passes are few (16 x 100000, k = 50: 13, 13).
+// - the nucleus from lists is as indifferent to its shape: 200 x 100000, a row to a CTA, two CTAs to an SM, with eight loads 64,
+// with four 57; with lists so long that one CTA fills the SM a pair (256 x 128000: 82, 512 threads alone 90).
 CutShape cut_shape(int rows, int vocab, int top_k) {
+    const bool listed = top_k <= 0 || top_k >= vocab;
     const bool binned = top_k <= 0 || top_k > 128 || top_k >= vocab, long_row = vocab >= 48 * 1024;
     if (rows > 4 * 148 && !long_row) return CutShape{256, 4, 1};
     if (binned && vocab < 12 * 1024) return CutShape{256, 4, 1};
     if (rows > 2 * 148) return CutShape{512, 4, 1};
+    if (listed && long_row && rows > 148)
+        return list_bytes(vocab, 1, 512) <= kTwoListsBytes ? CutShape{512, 4, 1} : CutShape{512, 8, 2};
     return CutShape{512, 8, binned && long_row ? (rows <= 74 ? 4 : rows <= 148 ? 2 : 1) : 1};
 }
 
@@ -1626,19 +1821,34 @@ int launch_cut(const float* a, size_t a_stride, int a_rows, const float* b, size
     }
     cfg.attrs = attr;
     cfg.numAttrs = n;
-#define SPEC_LAUNCH_CUT(T, L, S)                                                                                              \
-    do {                                                                                                                      \
-        if (vec) SPEC_CUDA_TRY(cudaLaunchKernelEx(&cfg, cut_floor_kernel<T, L, true, S, WORK>, a, a_stride, a_rows, b, b_stride,   \
-                                                  b_rows, vocab, top_k, top_p, c2, floors, work));                            \
-        else SPEC_CUDA_TRY(cudaLaunchKernelEx(&cfg, cut_floor_kernel<T, L, false, S, WORK>, a, a_stride, a_rows, b, b_stride, \
-                                              b_rows, vocab, top_k, top_p, c2, floors, work));                                \
+    const bool listed = !(top_k > 0 && top_k < vocab) && (vocab >= 12 * 1024 || total > 2 * 148) &&
+                        list_bytes(vocab, ctas, shape.threads) <= kMostListBytes;
+    int slots = 0;
+    if (listed) {
+        slots = list_slots(vocab, ctas, shape.threads);
+        cfg.dynamicSmemBytes = list_bytes(vocab, ctas, shape.threads);
+    }
+    auto launch = [&](auto kernel) -> int {
+        SPEC_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, a, a_stride, a_rows, b, b_stride, b_rows, vocab, top_k, top_p, c2, floors, work, slots));
+        return SPEC_OK;
+    };
+    auto launch_listed = [&](std::atomic<unsigned long long>& done, auto kernel) -> int {
+        const int status = allow_shared_memory(done, kernel, static_cast<int>(kMostListBytes));
+        return status != SPEC_OK ? status : launch(kernel);
+    };
+#define SPEC_LAUNCH_CUT(T, L, S)                                                                                                   \
+    do {                                                                                                                           \
+        static std::atomic<unsigned long long> done[2];                                                                            \
+        if (listed)                                                                                                                \
+            return vec ? launch_listed(done[0], cut_floor_kernel<T, L, true, S, WORK, true>)                                       \
+                       : launch_listed(done[1], cut_floor_kernel<T, L, false, S, WORK, true>);                                     \
+        return vec ? launch(cut_floor_kernel<T, L, true, S, WORK, false>) : launch(cut_floor_kernel<T, L, false, S, WORK, false>); \
     } while (0)
     if (ctas > 1) SPEC_LAUNCH_CUT(512, 8, false);
-    else if (shape.threads == 256) SPEC_LAUNCH_CUT(256, 4, true);
-    else if (shape.loads == 4) SPEC_LAUNCH_CUT(512, 4, true);
-    else SPEC_LAUNCH_CUT(512, 8, true);
+    if (shape.threads == 256) SPEC_LAUNCH_CUT(256, 4, true);
+    if (shape.loads == 4) SPEC_LAUNCH_CUT(512, 4, true);
+    SPEC_LAUNCH_CUT(512, 8, true);
 #undef SPEC_LAUNCH_CUT
-    return SPEC_OK;
 }
 
 int launch_verify_sample(const float* target_logits, const float* draft_logits, const int32_t* draft_tokens,

@@ -44,3 +44,41 @@ def test_floors_and_draws_do_not_depend_on_the_number_of_rows(vocab, top_k, top_
         # (weights are added in another order: 2^-20 of their sum at most, so a uniform number next to a step may fall on
         # the other side; of five, none is)
         assert torch.equal(drawn, tokens.repeat((rows + 4) // 5)[:rows]), rows
+
+
+@pytest.mark.parametrize("rows,vocab", [(1, 12288), (3, 12289), (2, 49152), (149, 50003), (150, 110000), (300, 12291), (600, 4099)])
+@pytest.mark.parametrize("top_p", [0.1, 0.9, 0.999])
+def test_nucleus_of_rows_whose_sample_misleads(rows, vocab, top_p):
+    """The nucleus is looked for among the logits that a sample of the row says to list.  Rows where that is wrong or no use: flat
+    ones, mass in a stretch that the sample misses, weight where it looks, more candidates in one stretch than a warp's list
+    holds, masked logits, few finite ones, ties."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(vocab)
+    base = torch.randn(10, vocab, device="cuda", generator=gen)
+    base[0] *= 3
+    base[1] *= 0.01
+    base[2] = 1.0
+    base[3, vocab // 2 + 300: vocab // 2 + 900] += 9
+    base[4, :128] += 5
+    base[5, vocab // 3: vocab // 3 + vocab // 8] += 6
+    base[6, 1::2] = -torch.inf
+    base[7, 17:] = -torch.inf
+    base[8] = base[8].mul(2).round()
+    base[9, : vocab // 2] -= 40
+    many = base.repeat((rows + 9) // 10, 1)[:rows].contiguous()
+    got = binding.spec_truncation_floors(many, 0.8, top_p=top_p)
+    again = binding.spec_truncation_floors(many, 0.8, top_p=top_p)
+    assert torch.equal(got, again)
+    u = torch.rand(rows, device="cuda", generator=gen)
+    tokens = binding.spec_sample(many, u, 0.8, top_p=top_p)
+    for i in range(min(rows, 10)):
+        row = np.sort(many[i].double().cpu().numpy())[::-1]
+        floor = float(got[i])
+        weight = np.exp((row - row[0]) / 0.8)
+        # (as above: 2^-32 of the largest per logit, a weight good to 2^-21, sums in fp32)
+        slack = vocab * 2.0 ** -31 + weight.sum() * 2.0 ** -20
+        assert weight[row >= floor].sum() >= top_p * weight.sum() - slack, i
+        assert weight[row > floor].sum() < top_p * weight.sum() + slack, i
+        assert float(many[i, int(tokens[i])]) >= floor, i
+    for i in range(10, rows):
+        assert float(got[i]) == float(got[i % 10]), i

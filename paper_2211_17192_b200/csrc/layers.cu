@@ -92,6 +92,10 @@ __global__ void embed_kernel(const void* tok_emb, const void* pos_emb, bool bf16
 // meanwhile.  The CTAs give one another their warps' sums of squares through distributed shared memory.
 constexpr int kNormMaxWidth = 4 * 1024 * 4;
 constexpr int kNormCtas = 8;  // of a cluster that shares a row
+// The elementwise kernels give a thread several rows where one each is more threads than the GPU holds at once: below that the
+// rows of a thread only lengthen it (96 rows of the 160M shape: a pass 625 us with a row each, 699 with four).
+constexpr long long kResidentThreads = 148 * 2048;
+constexpr int kNormFourRows = 296;  // at most for a cluster of four: eight CTAs of 256 threads to an SM
 constexpr int kNormClusterRows = 128;  // at most (launch_norm has both sides)
 
 template <int THREADS, int PER, int CTAS = 1>
@@ -203,65 +207,79 @@ __device__ __forceinline__ void store_cached4(KV* dst, const float (&v)[4]) {
     else *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(t);
 }
 
-// grid = (ceil(heads * d_head / 8 / block), rows), heads = n_heads + 2 n_kv_heads.  qkv row layout:
+// grid = (ceil(heads * d_head / 8 / block), ceil(rows / ROWS)), heads = n_heads + 2 n_kv_heads.  qkv row layout:
 // [q heads | k heads | v heads], d_head each.  A thread finishes elements j .. j+3 and
 // j + d_head/2 .. of one head of one row of the qkv GEMM (optional partial sums), applies
 // rotary positions (q and k heads; they pair j with j + d_head/2), leaves q in `qkv` for the
-// attention kernel, and appends K or V to the paged cache.
-template <typename KV>
+// attention kernel, and appends K or V to the paged cache.  ROWS as in ffn_act_kernel.
+constexpr int kQkvRows = 4;
+template <typename KV, int ROWS>
 __global__ void qkv_kernel(float* qkv, const float* partial, const PartialPlan plan, int n_rows,
                            const int32_t* pos, const int32_t* seq, int n_heads,
                            int n_kv_heads, int d_head, const float2* rope_table,
                            KV* kv_layer, const int32_t* page_table, int pages_per_seq,
-                           int page_size) {
+                           int page_shift) {
     pdl_trigger();
     pdl_wait();
     const int half = d_head / 2, per_head = half / 4;
-    const int task = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+    const int task = blockIdx.x * blockDim.x + threadIdx.x, r0 = ROWS * blockIdx.y;
     const int head = task / per_head, j = 4 * (task % per_head);
     if (head >= n_heads + 2 * n_kv_heads) return;
-    const int p = pos[r];
     const bool is_q = head < n_heads, is_k = !is_q && head < n_heads + n_kv_heads;
-    const bool rotate = rope_table && p >= 0 && (is_q || is_k);
-    float4 t0, t1;  // (cos, sin) of position p for the four pairs
-    if (rotate) {
-        const float4* t = reinterpret_cast<const float4*>(rope_table + static_cast<size_t>(p) * half + j);
-        t0 = t[0];
-        t1 = t[1];
-    }
     const int width = (n_heads + 2 * n_kv_heads) * d_head;
-    const size_t at = static_cast<size_t>(r) * width + head * d_head + j;
-    const size_t where[2] = {at, at + half};
-    float4 x[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    int p[ROWS];
+    float4 t[ROWS][2];  // (cos, sin) of the rows' positions for the four pairs
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) p[i] = pos[min(r0 + i, n_rows - 1)];
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i)
+        if (rope_table && p[i] >= 0 && (is_q || is_k)) {
+            const float4* at = reinterpret_cast<const float4*>(rope_table + static_cast<size_t>(p[i]) * half + j);
+            t[i][0] = at[0];
+            t[i][1] = at[1];
+        }
+    size_t where[2 * ROWS];
+    float4 x[2 * ROWS];
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+        where[2 * i] = static_cast<size_t>(min(r0 + i, n_rows - 1)) * width + head * d_head + j;
+        where[2 * i + 1] = where[2 * i] + half;
+        x[2 * i] = x[2 * i + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     if (partial) {
         // (a head of 64 or 128 columns lies inside one 256-column tile)
-        sum_partials<2, 4>(partial, partial_count(plan, r, head * d_head), static_cast<size_t>(n_rows) * width, where, x);
+        sum_partials<2 * ROWS, ROWS == 1 ? 4 : 1>(partial, partial_count(plan, r0, head * d_head), static_cast<size_t>(n_rows) * width, where, x);
     } else {
-        x[0] = *reinterpret_cast<const float4*>(qkv + where[0]);
-        x[1] = *reinterpret_cast<const float4*>(qkv + where[1]);
-    }
-    float a[4] = {x[0].x, x[0].y, x[0].z, x[0].w}, b[4] = {x[1].x, x[1].y, x[1].z, x[1].w};
-    if (rotate) {
-        const float c[4] = {t0.x, t0.z, t1.x, t1.z}, s[4] = {t0.y, t0.w, t1.y, t1.w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float y1 = a[e] * c[e] - b[e] * s[e], y2 = b[e] * c[e] + a[e] * s[e];
-            a[e] = y1;
-            b[e] = y2;
+        for (int i = 0; i < 2 * ROWS; ++i) x[i] = *reinterpret_cast<const float4*>(qkv + where[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+        if (ROWS > 1 && r0 + i >= n_rows) break;
+        const float4 xa = x[2 * i], xb = x[2 * i + 1];
+        float a[4] = {xa.x, xa.y, xa.z, xa.w}, b[4] = {xb.x, xb.y, xb.z, xb.w};
+        if (rope_table && p[i] >= 0 && (is_q || is_k)) {
+            const float c[4] = {t[i][0].x, t[i][0].z, t[i][1].x, t[i][1].z}, s[4] = {t[i][0].y, t[i][0].w, t[i][1].y, t[i][1].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float y1 = a[e] * c[e] - b[e] * s[e], y2 = b[e] * c[e] + a[e] * s[e];
+                a[e] = y1;
+                b[e] = y2;
+            }
         }
+        if (is_q) {
+            *reinterpret_cast<float4*>(qkv + where[2 * i]) = make_float4(a[0], a[1], a[2], a[3]);
+            *reinterpret_cast<float4*>(qkv + where[2 * i + 1]) = make_float4(b[0], b[1], b[2], b[3]);
+            continue;
+        }
+        if (p[i] < 0) continue;  // inactive row: nothing is cached
+        const int kv_head = is_k ? head - n_heads : head - n_heads - n_kv_heads;
+        const int page = page_table[seq[r0 + i] * pages_per_seq + (p[i] >> page_shift)];
+        const size_t block = (static_cast<size_t>(page) * 2 + (is_k ? 0 : 1)) * n_kv_heads + kv_head;
+        KV* dst = kv_layer + ((block << page_shift) + (p[i] & ((1 << page_shift) - 1))) * d_head + j;
+        store_cached4<KV>(dst, a);
+        store_cached4<KV>(dst + half, b);
     }
-    if (is_q) {
-        *reinterpret_cast<float4*>(qkv + where[0]) = make_float4(a[0], a[1], a[2], a[3]);
-        *reinterpret_cast<float4*>(qkv + where[1]) = make_float4(b[0], b[1], b[2], b[3]);
-        return;
-    }
-    if (p < 0) return;  // inactive row: nothing is cached
-    const int kv_head = is_k ? head - n_heads : head - n_heads - n_kv_heads;
-    const int page = page_table[seq[r] * pages_per_seq + p / page_size];
-    const size_t block = (static_cast<size_t>(page) * 2 + (is_k ? 0 : 1)) * n_kv_heads + kv_head;
-    KV* dst = kv_layer + (block * page_size + p % page_size) * d_head + j;
-    store_cached4<KV>(dst, a);
-    store_cached4<KV>(dst + half, b);
 }
 
 // logits[dst(i)] = table[token[src(i)]] for a table model: grid = (chunks, rows), block = 256.
@@ -316,42 +334,72 @@ __global__ void copy_logits_kernel(const int32_t* tokens, int max_len, const int
 }
 
 // f = gelu(u)  |  gelu(gate) * up  |  silu(gate) * up, with u the partial sums of the FFN-in GEMM, as two bf16 terms.
-// grid = (ceil(d_ff / 4 / block), rows): four columns per thread.
-template <int FFN>
+// grid = (ceil(d_ff / 4 / block), ceil(rows / ROWS)): four columns of ROWS rows per thread.  Of few rows each is a thread's own
+// (the kernel is then one trip to memory); of many ROWS share what is not arithmetic - how many partial sums there are takes
+// four integer divisions - and their loads are in flight together.  One row to a thread was bound by issue (940 instructions
+// a warp, 12.5 us behind the GEMM for 224 rows of the 7B shape, 9.8 with four).
+constexpr int kActRows = 4;  // (a tile's rows are a multiple of 16: these share their partial sums' number)
+template <int FFN, int ROWS>
 __global__ void ffn_act_kernel(const float* partial, const PartialPlan plan, int n_rows, int d_ff, __nv_bfloat16* f_hi,
                                __nv_bfloat16* f_lo) {
     pdl_trigger();
     pdl_wait();
-    const int c = 4 * (blockIdx.x * blockDim.x + threadIdx.x), r = blockIdx.y;
+    const int c = 4 * (blockIdx.x * blockDim.x + threadIdx.x), r0 = ROWS * blockIdx.y;
     if (c >= d_ff) return;
     constexpr bool kGated = FFN != SPEC_FFN_GELU;
     const int width = kGated ? 2 * d_ff : d_ff;
     const size_t stride = static_cast<size_t>(n_rows) * width;
-    const size_t at = static_cast<size_t>(r) * width + c;
-    float4 g = make_float4(0.f, 0.f, 0.f, 0.f), up = g;
-    const int n_gate = partial_count(plan, r, c), n_up = kGated ? partial_count(plan, r, c + d_ff) : n_gate;
-    if (kGated && n_gate == n_up) {
-        const size_t where[2] = {at, at + d_ff};
-        float4 both[2] = {g, g};
-        sum_partials<2, 4>(partial, n_gate, stride, where, both);
-        g = both[0];
-        up = both[1];
+    const int n_gate = partial_count(plan, r0, c), n_up = kGated ? partial_count(plan, r0, c + d_ff) : 0;
+    float4 g[ROWS], up[ROWS];
+    if constexpr (ROWS == 1) {
+        const size_t at = static_cast<size_t>(r0) * width + c;
+        g[0] = up[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (kGated && n_gate == n_up) {
+            const size_t where[2] = {at, at + d_ff};
+            float4 both[2] = {g[0], g[0]};
+            sum_partials<2, 4>(partial, n_gate, stride, where, both);
+            g[0] = both[0];
+            up[0] = both[1];
+        } else {
+            const size_t where[1] = {at};
+            sum_partials<1, 8>(partial, n_gate, stride, where, g);
+            if (kGated) {
+                const size_t where_up[1] = {at + d_ff};
+                sum_partials<1, 8>(partial, n_up, stride, where_up, up);
+            }
+        }
     } else {
-        const size_t where[1] = {at};
-        float4 one[1] = {g};
-        sum_partials<1, 8>(partial, n_gate, stride, where, one);
-        g = one[0];
-        if (kGated) {
-            const size_t where_up[1] = {at + d_ff};
-            sum_partials<1, 8>(partial, n_up, stride, where_up, one);
-            up = one[0];
+        const float* at[ROWS];
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+            at[i] = partial + static_cast<size_t>(min(r0 + i, n_rows - 1)) * width + c;
+            g[i] = up[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        for (int k = 0; k < max(n_gate, n_up); ++k) {
+            float4 p[ROWS], q[ROWS];
+#pragma unroll
+            for (int i = 0; i < ROWS; ++i) {
+                p[i] = k < n_gate ? *reinterpret_cast<const float4*>(at[i]) : make_float4(0.f, 0.f, 0.f, 0.f);
+                if (kGated) q[i] = k < n_up ? *reinterpret_cast<const float4*>(at[i] + d_ff) : make_float4(0.f, 0.f, 0.f, 0.f);
+                at[i] += stride;
+            }
+#pragma unroll
+            for (int i = 0; i < ROWS; ++i) {
+                g[i] = add4(g[i], p[i]);
+                if (kGated) up[i] = add4(up[i], q[i]);
+            }
         }
     }
-    float4 y;
-    if (FFN == SPEC_FFN_GELU) y = make_float4(gelu_tanh(g.x), gelu_tanh(g.y), gelu_tanh(g.z), gelu_tanh(g.w));
-    else if (FFN == SPEC_FFN_SWIGLU) y = make_float4(silu(g.x) * up.x, silu(g.y) * up.y, silu(g.z) * up.z, silu(g.w) * up.w);
-    else y = make_float4(gelu_tanh(g.x) * up.x, gelu_tanh(g.y) * up.y, gelu_tanh(g.z) * up.z, gelu_tanh(g.w) * up.w);
-    store_split4(f_hi, f_lo, static_cast<size_t>(r) * d_ff + c, y);
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+        if (ROWS > 1 && r0 + i >= n_rows) break;
+        const float4 x = g[i], u = up[i];
+        float4 y;
+        if (FFN == SPEC_FFN_GELU) y = make_float4(gelu_tanh(x.x), gelu_tanh(x.y), gelu_tanh(x.z), gelu_tanh(x.w));
+        else if (FFN == SPEC_FFN_SWIGLU) y = make_float4(silu(x.x) * u.x, silu(x.y) * u.y, silu(x.z) * u.z, silu(x.w) * u.w);
+        else y = make_float4(gelu_tanh(x.x) * u.x, gelu_tanh(x.y) * u.y, gelu_tanh(x.z) * u.z, gelu_tanh(x.w) * u.w);
+        store_split4(f_hi, f_lo, static_cast<size_t>(r0 + i) * d_ff + c, y);
+    }
 }
 
 }  // namespace
@@ -390,11 +438,15 @@ int launch_norm(float* h, const float* partial, const PartialPlan& plan, int row
     // Wide rows that leave SMs idle go to a cluster each.  Whole pass of the 7B shape at 500 cached tokens, a CTA of 1024
     // threads per row against a cluster, ms: 1 row 2.779 / 2.761, 3 rows 2.865 / 2.839, 7 rows 2.937 / 2.915, 16 rows
     // 3.111 / 3.123 (the runs of one side differ by as much), 32 rows 3.196 / 3.152, 64 rows 3.748 / 3.734, 126 rows
-    // 5.232 / 5.216; beyond, a CTA per row is enough for the GPU.
+    // 5.232 / 5.216; beyond, four larger CTAs (eight partial sums in flight, not two: 224 rows 11.0 -> 9.8 us behind the GEMM), and
+    // where those no longer fit side by side a CTA per row.
     const int groups = d / 4;
     if (groups > 512 && groups <= 128 * kNormCtas && n_rows <= kNormClusterRows)
         return launch_cluster(norm_kernel<128, 1, kNormCtas>, kNormCtas, dim3(n_rows * kNormCtas), dim3(128), 0, stream, h, partial,
                               plan, rows_total, gain, src_rows, d, eps, out, out_hi, out_lo);
+    if (groups > 512 && groups <= 1024 && n_rows <= kNormFourRows)
+        return launch_cluster(norm_kernel<256, 1, 4>, 4, dim3(n_rows * 4), dim3(256), 0, stream, h, partial, plan, rows_total, gain,
+                              src_rows, d, eps, out, out_hi, out_lo);
     if (groups <= 128) SPEC_LAUNCH_NORM(128, 1);
     if (groups <= 256) SPEC_LAUNCH_NORM(256, 1);
     if (groups <= 1024 && n_rows > 148) SPEC_LAUNCH_NORM(256, 4);
@@ -406,28 +458,31 @@ int launch_norm(float* h, const float* partial, const PartialPlan& plan, int row
 int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, const KvPool& pool, const RowMeta& rows,
                int n_rows, float* qkv, const float* partial, const PartialPlan& plan, cudaStream_t stream) {
     const int tasks = (n_heads + 2 * n_kv_heads) * (d_head / 8);
+    const bool many = static_cast<long long>(n_rows) * tasks > kResidentThreads;
     const int threads = n_rows <= 16 ? 64 : 256;
-    const dim3 grid((tasks + threads - 1) / threads, n_rows);
-    const dim3 block(threads);
-    if (pool.dtype == SPEC_DTYPE_FP16)
-        return launch_pdl(qkv_kernel<__half>, grid, block, 0, stream, qkv, partial, plan, n_rows, rows.pos, rows.seq, n_heads,
-                          n_kv_heads, d_head, rope, static_cast<__half*>(pool.kv), pool.page_table, pool.pages_per_seq,
-                          pool.page_size);
-    if (pool.dtype == SPEC_DTYPE_BF16)
-        return launch_pdl(qkv_kernel<__nv_bfloat16>, grid, block, 0, stream, qkv, partial, plan, n_rows, rows.pos,
-                          rows.seq, n_heads, n_kv_heads, d_head, rope, static_cast<__nv_bfloat16*>(pool.kv),
-                          pool.page_table, pool.pages_per_seq, pool.page_size);
-    return launch_pdl(qkv_kernel<float>, grid, block, 0, stream, qkv, partial, plan, n_rows, rows.pos, rows.seq,
-                      n_heads, n_kv_heads, d_head, rope, static_cast<float*>(pool.kv), pool.page_table,
-                      pool.pages_per_seq, pool.page_size);
+    const dim3 grid((tasks + threads - 1) / threads, many ? (n_rows + kQkvRows - 1) / kQkvRows : n_rows);
+    int page_shift = 0;  // (pages are a power of two)
+    while ((1 << page_shift) < pool.page_size) ++page_shift;
+#define SPEC_LAUNCH_QKV(KV, R)                                                                                                  \
+    return launch_pdl(qkv_kernel<KV, R>, grid, dim3(threads), 0, stream, qkv, partial, plan, n_rows, rows.pos, rows.seq, n_heads, \
+                      n_kv_heads, d_head, rope, static_cast<KV*>(pool.kv), pool.page_table, pool.pages_per_seq, page_shift)
+    if (pool.dtype == SPEC_DTYPE_FP16 && many) SPEC_LAUNCH_QKV(__half, kQkvRows);
+    if (pool.dtype == SPEC_DTYPE_FP16) SPEC_LAUNCH_QKV(__half, 1);
+    if (pool.dtype == SPEC_DTYPE_BF16 && many) SPEC_LAUNCH_QKV(__nv_bfloat16, kQkvRows);
+    if (pool.dtype == SPEC_DTYPE_BF16) SPEC_LAUNCH_QKV(__nv_bfloat16, 1);
+    if (many) SPEC_LAUNCH_QKV(float, kQkvRows);
+    SPEC_LAUNCH_QKV(float, 1);
+#undef SPEC_LAUNCH_QKV
 }
 
 int launch_ffn_act(const float* partial, const PartialPlan& plan, int n_rows, int d_ff, int ffn, __nv_bfloat16* f_hi,
                    __nv_bfloat16* f_lo, cudaStream_t stream) {
+    const bool many = static_cast<long long>(n_rows) * (d_ff / 4) > kResidentThreads;
     const int threads = n_rows <= 16 ? 64 : 256;
-    const dim3 grid((d_ff / 4 + threads - 1) / threads, n_rows);
-#define SPEC_LAUNCH_ACT(F) \
-    return launch_pdl(ffn_act_kernel<F>, grid, dim3(threads), 0, stream, partial, plan, n_rows, d_ff, f_hi, f_lo)
+    const dim3 grid((d_ff / 4 + threads - 1) / threads, many ? (n_rows + kActRows - 1) / kActRows : n_rows);
+#define SPEC_LAUNCH_ACT(F)                                                                                                     \
+    return many ? launch_pdl(ffn_act_kernel<F, kActRows>, grid, dim3(threads), 0, stream, partial, plan, n_rows, d_ff, f_hi, f_lo) \
+                : launch_pdl(ffn_act_kernel<F, 1>, grid, dim3(threads), 0, stream, partial, plan, n_rows, d_ff, f_hi, f_lo)
     if (ffn == SPEC_FFN_GELU) SPEC_LAUNCH_ACT(SPEC_FFN_GELU);
     if (ffn == SPEC_FFN_SWIGLU) SPEC_LAUNCH_ACT(SPEC_FFN_SWIGLU);
     SPEC_LAUNCH_ACT(SPEC_FFN_GATED_GELU);

@@ -1274,7 +1274,9 @@ __device__ float candidate_floor(const Slice<VEC, LOADS>& s, float top_p, float 
     return sh.floor;
 }
 
-// Lists the candidates of this warp's part of the slice, as the inverse CDF cuts it.
+// Lists the candidates of this warp's part of the slice, as the inverse CDF cuts it, two steps of two loads ahead (200 x 100000:
+// 47 us a call; one step of four at a time 50, of eight 53; four ahead of four 51, and eight ahead of eight spill: 70).
+constexpr int kListLoads = 2;
 template <int T, bool VEC, int LOADS>
 __device__ Listed list_candidates(const Slice<VEC, LOADS>& s, int each, float from, float ref, float c2, int slots, float* lists, SelShared& sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1286,27 +1288,37 @@ __device__ Listed list_candidates(const Slice<VEC, LOADS>& s, int each, float fr
     float below = 0.0f, most = -INFINITY;
     int n = 0;
     const int last = slots - 1;  // (what does not fit goes to the last slot)
-    auto one = [&](float x) {
-        const bool in = x >= from;
-        const unsigned who = __ballot_sync(kFullMask, in);
-        if (in) list[min(n + __popc(who & before_me), last)] = x;
-        n += __popc(who);
-        below += in ? 0.0f : fast_exp2(fmaf(x, c2, mc));
-        most = fmaxf(most, x);
-    };
-    for (int base = b0; base < b1; base += 32 * LOADS) {
-        float4 v[LOADS];
+    float4 v[kListLoads];
+    auto fetch = [&](int base) {
 #pragma unroll
-        for (int i = 0; i < LOADS; ++i) {
+        for (int i = 0; i < kListLoads; ++i) {
             const int g = base + 32 * i + lane;
             v[i] = g < b1 ? s.row.raw(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         }
+    };
+    if (b0 < b1) fetch(b0);
+    for (int base = b0; base < b1; base += 32 * kListLoads) {
+        float4 now[kListLoads];
 #pragma unroll
-        for (int i = 0; i < LOADS; ++i) {
-            one(v[i].x);
-            one(v[i].y);
-            one(v[i].z);
-            one(v[i].w);
+        for (int i = 0; i < kListLoads; ++i) now[i] = v[i];
+        if (base + 32 * kListLoads < b1) fetch(base + 32 * kListLoads);  // (on its way while these are looked at)
+#pragma unroll
+        for (int i = 0; i < kListLoads; ++i) {
+            const float x[4] = {now[i].x, now[i].y, now[i].z, now[i].w};
+            int at = 0, own = 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                at += __popc(__ballot_sync(kFullMask, x[j] >= from) & before_me);
+                most = fmaxf(most, x[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const bool in = x[j] >= from;
+                if (in) list[min(n + at + own, last)] = x[j];
+                own += in ? 1 : 0;
+                below += in ? 0.0f : fast_exp2(fmaf(x[j], c2, mc));
+            }
+            n += __shfl_sync(kFullMask, at + own, 31);
         }
     }
     below = warp_sum(n > slots ? INFINITY : below);

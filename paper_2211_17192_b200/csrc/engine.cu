@@ -47,6 +47,7 @@ struct spec_ctx {
     float* attn_part = nullptr;  // per key slice: (max, sum, accumulator) of every (row, head)
     int hi_rows = 0;
     spec::SmallPass small[2];  // per model: few-row passes of a small decoder as one kernel
+    spec::ClusterPass tiny[2];  // .. of a tiny fp32 decoder as one cluster
     spec::PassScratch pass;  // the persistent pass kernel's scratch (passes of at most 16 rows of a bf16 model)
     int32_t* row_block = nullptr;  // one allocation: the five row arrays below, a prompt chunk's packed rows and segments
     int32_t *row_token = nullptr, *row_pos = nullptr, *row_seq = nullptr, *logit_src = nullptr, *logit_dst = nullptr;
@@ -56,7 +57,7 @@ struct spec_ctx {
     char* report_dev = nullptr;
     std::vector<char> report_memory;
     std::vector<int32_t> staging;       // row descriptors on their way to row_block
-    int* error_words[5] = {};
+    int* error_words[6] = {};
 
     // Captured passes of spec_forward_logits: a shape is captured the third time it is asked for (the capture costs about
     // a launch-bound pass or two); the oldest of eight makes room.
@@ -249,12 +250,12 @@ struct Pass {
 // Non-zero (and cleared) if a kernel gave up on a bounded wait.
 int device_gave_up() {
     const int gemm = gemm_tc_take_error(), wide = gemm_wide_take_error(), pass = pass_take_error(), attn = attention_take_error(),
-              small = small_pass_take_error();
-    return gemm ? gemm : wide ? wide : pass ? pass : attn ? attn : small;
+              small = small_pass_take_error(), tiny = cluster_pass_take_error();
+    return gemm ? gemm : wide ? wide : pass ? pass : attn ? attn : small ? small : tiny;
 }
 
 struct ErrorWords {
-    int* word[5];
+    int* word[6];
 };
 
 // block = 128.  Leaves the state of the work before it in `out`.
@@ -263,7 +264,7 @@ __global__ void report_kernel(ErrorWords errors, int* nonfinite, const unsigned 
     pdl_wait();
     if (threadIdx.x == 0) {
         int code = 0;
-        for (int i = 0; i < 5; ++i)
+        for (int i = 0; i < 6; ++i)
             if (errors.word[i]) code |= *errors.word[i];
         out->gave_up = code;
         out->nonfinite = *nonfinite;
@@ -275,7 +276,8 @@ __global__ void report_kernel(ErrorWords errors, int* nonfinite, const unsigned 
 
 // Waits for everything on the context's stream; if it returns SPEC_OK, ctx->report describes it.
 int finish_work(spec_ctx* ctx, int batch) {
-    const ErrorWords errors{{ctx->error_words[0], ctx->error_words[1], ctx->error_words[2], ctx->error_words[3], ctx->error_words[4]}};
+    const ErrorWords errors{{ctx->error_words[0], ctx->error_words[1], ctx->error_words[2], ctx->error_words[3], ctx->error_words[4],
+                              ctx->error_words[5]}};
     SPEC_TRY(launch_pdl(report_kernel, dim3(1), dim3(128), 0, ctx->stream, errors, ctx->nonfinite, ctx->counters, ctx->length, batch,
                         reinterpret_cast<spec_report*>(ctx->report_dev)));
     SPEC_CUDA_TRY(cudaMemcpyAsync(ctx->report, ctx->report_dev, sizeof(spec_report) + batch * sizeof(int32_t), cudaMemcpyDeviceToHost,
@@ -331,7 +333,11 @@ int forward(spec_ctx* ctx, const Model& m, const RowMeta& rows, int batch, int m
     const float* bias = m.t5() ? m.dec_bias : nullptr;
 
     const bool small = !segs && small_pass_serves(ctx->small[which], m, batch, m_rows);
-    if (small) {
+    const bool tiny = !segs && cluster_pass_serves(ctx->tiny[which], batch, m_rows);
+    if (tiny) {
+        const PassTables tables{ctx->page_table, ctx->pages_per_seq, ctx->rt.page_size, nullptr, 0, nullptr, 0, 0};
+        SPEC_TRY(launch_cluster_pass(m, rows, tables, batch, m_rows, ctx->h, ctx->stream));
+    } else if (small) {
         const PassTables tables{ctx->page_table, ctx->pages_per_seq, ctx->rt.page_size, ctx->src_page_table,
                                 ctx->src_pages_per_seq, ctx->src_len, ctx->rt.max_len, ctx->rt.max_len - 1};
         SPEC_TRY(launch_small_pass(ctx->small[which], m, rows, tables, batch, m_rows, ctx->h, ctx->stream));
@@ -341,7 +347,7 @@ int forward(spec_ctx* ctx, const Model& m, const RowMeta& rows, int batch, int m
     } else {
         SPEC_TRY(launch_embed(m, rows, n_rows, ctx->h, ctx->stream));
     }
-    for (int l = 0; l < (small ? 0 : c.n_layers); ++l) {
+    for (int l = 0; l < (small || tiny ? 0 : c.n_layers); ++l) {
         const spec_layer_weights& w = m.layers[l];
         const spec_layer_weights& pw = pass.tc ? m.packed[l] : w;
         SPEC_TRY(pass.self_attention(w, pw, rows, batch, m_rows, layer_pool(ctx, m, l), nullptr, bias, ctx->rt.max_len,
@@ -1032,11 +1038,14 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     ctx->error_words[2] = pass_error_word();
     ctx->error_words[3] = attention_error_word();
     ctx->error_words[4] = small_pass_error_word();
+    ctx->error_words[5] = cluster_pass_error_word();
     ctx->cached[0].assign(B, 0);
     ctx->cached[1].assign(B, 0);
     // (last: everything that a context cannot do without has its memory)
     for (int i = 0; i < n_models && !rt.pass_kernel; ++i)
-        if ((status = small_pass_init(ctx->small[i], ctx->model[i], ctx->allocations, spare, ctx->stream)) != SPEC_OK) return cleanup(status);
+        if ((status = small_pass_init(ctx->small[i], ctx->model[i], ctx->allocations, spare, ctx->stream)) != SPEC_OK ||
+            (status = cluster_pass_init(ctx->tiny[i], ctx->model[i], ctx->rt.max_len)) != SPEC_OK)
+            return cleanup(status);
     *out = ctx;
     return SPEC_OK;
 }

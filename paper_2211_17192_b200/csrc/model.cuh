@@ -267,6 +267,16 @@ PartialPlan small_pass_plan(const SmallPass& s);
 int* small_pass_error_word();
 int small_pass_take_error();
 
+// cluster_pass.cu: the blocks of a tiny fp32 decoder over a few rows as one cluster.  Leaves the residual stream in h.
+struct ClusterPass {
+    int rows = 0;  // at most (0: not served)
+};
+int cluster_pass_init(ClusterPass& s, const Model& m, int max_len);
+bool cluster_pass_serves(const ClusterPass& s, int batch, int m_rows);
+int launch_cluster_pass(const Model& m, const RowMeta& rows, const PassTables& t, int batch, int m_rows, float* h, cudaStream_t stream);
+int* cluster_pass_error_word();
+int cluster_pass_take_error();
+
 // A tensor map over `rows` rows of `cols` (64 or 128) fp16 elements starting at `base`, fetched in boxes of 64 elements
 // by 32 rows with the 128-byte swizzle; maps are cached by (base, rows, cols).  gemm_tc.cu
 int cached_f16_rows_map(const void* base, unsigned long long rows, int cols, CUtensorMap* out);

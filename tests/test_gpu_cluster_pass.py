@@ -1,0 +1,40 @@
+"""Few-row passes of tiny fp32 decoders, which are one cluster of thread blocks: logits against the oracle for every number of
+rows it takes (and one more, which the chain of kernels takes), over ragged caches from none to the most keys it serves."""
+import numpy as np
+import pytest
+
+from oracle.decoder import Decoder
+from paper_2211_17192_b200 import binding, workloads
+
+pytestmark = pytest.mark.gpu
+
+# fp32 sums of up to 1024 products in another order (2^-24 each, a few times over per block): relative to the largest logit
+REL_TOL = 1e-4
+
+
+@pytest.mark.parametrize("d_model,layers,max_len", [(128, 1, 256), (128, 2, 100), (256, 1, 64), (256, 4, 256)])
+def test_cluster_pass_against_the_oracle(d_model, layers, max_len):
+    cfg = workloads.scaled_config(workloads.model_config("tiny_target"), d_model=d_model, n_heads=d_model // 64, n_kv_heads=d_model // 64,
+                                  d_ff=4 * d_model, n_layers=layers, vocab=500, max_positions=max_len)
+    w = workloads.make_weights(cfg, 9)
+    oracle = Decoder(cfg, w)
+    batch, most = 9, max_len - 10
+    tokens = np.stack([workloads.make_prompt(30 + b, most + 9, cfg["vocab"]) for b in range(batch)])
+    want = [oracle.forward_full(t) for t in tokens]
+    eng = binding.Engine(cfg, w, max_batch=batch, max_len=max_len, max_gamma=31, page_size=32)
+    for at in range(0, most, 32):
+        eng.forward_logits(0, np.ascontiguousarray(tokens[:, at:min(at + 32, most)]))
+    for n, rows in ((1, 1), (2, 1), (3, 1), (4, 1), (5, 1), (7, 1), (8, 1), (9, 1), (1, 2), (1, 3), (1, 4), (1, 5), (1, 7), (1, 8), (1, 9),
+                    (2, 2), (2, 3), (2, 4), (3, 2), (4, 2)):
+        for lengths in ([0] * n, [(7 * b + 31) % most for b in range(n)], [most - (b % 5) for b in range(n)], [min(128, most) + b % 3 - 2 for b in range(n)]):
+            eng.truncate(0, lengths + [most] * (batch - n))
+            new = np.stack([tokens[b, lengths[b]:lengths[b] + rows] for b in range(n)])
+            got = eng.forward_logits(0, new).cpu().numpy()
+            for b in range(n):
+                ref = want[b][lengths[b]:lengths[b] + rows]
+                assert np.abs(got[b] - ref).max() <= REL_TOL * np.abs(ref).max(), (n, rows, lengths, b)
+            # the cache whole again for the next case
+            eng.truncate(0, [0] * batch)
+            for at in range(0, most, 32):
+                eng.forward_logits(0, np.ascontiguousarray(tokens[:, at:min(at + 32, most)]))
+    eng.close()

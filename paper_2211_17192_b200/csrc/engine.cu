@@ -410,52 +410,46 @@ int encode(spec_ctx* ctx, const Model& m, int batch, int m_rows) {
 
 // ---- generation-loop kernels (one thread per sequence; tiny) ----------------
 
-// Uniforms of one iteration (the paper leaves the consumption of randomness
+// Rows of the passes below: a sequence that has its n_new tokens is frozen but stays in the batch, and its guesses may
+// then lie beyond the positions the context holds.  Such rows (position >= `limit`) are inactive: they are computed, and
+// neither cached nor looked at.
+__device__ __forceinline__ int held(int position, int limit) { return position < limit ? position : -1; }
+
+// The start of an iteration.
+// Its uniforms (the paper leaves the consumption of randomness
 // open; here every draw is keyed by the position it decides):
 //   draft_u[b, i]  draw of x_{i+1} at position L+i           (purpose 0)
 //   accept_u[b, i] accept test of x_{i+1} at position L+i     (purpose 1)
 //   final_u[b, n]  final draw t at position L+n, n = 0..gamma (purpose 2)
-__global__ void iteration_uniforms_kernel(const spec_ctx::Params* params,
-                                          const int32_t* length, int batch, int gamma,
-                                          float* draft_u, float* accept_u,
-                                          float* final_u) {
+// And the rows of its first draft step (`draft_rows`), two per sequence, positions L-2 and
+// L-1.  Position L-2 is already cached unless the previous iteration accepted
+// every guess (x_gamma was never fed to the draft); feeding it again rewrites
+// the same K,V row, so the shape of the step never changes.
+// One kernel: the second kernel of a graph starts 3 us after the first has ended, where one further on would take 1.
+__global__ void start_iteration_kernel(const spec_ctx::Params* params, const int32_t* tokens, const int32_t* length, int batch, int gamma,
+                                       int max_len, int limit, bool draft_rows, float* draft_u, float* accept_u, float* final_u,
+                                       int32_t* row_token, int32_t* row_pos, int32_t* row_seq, int32_t* logit_src, int32_t* logit_dst) {
     pdl_trigger();
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= batch * (gamma + 1)) return;
+    if (draft_rows && i < batch) {
+        const int L = length[i];
+        const int p0 = max(L - 2, 0), p1 = L - 1;
+        row_token[2 * i] = tokens[static_cast<size_t>(i) * max_len + p0];
+        row_token[2 * i + 1] = tokens[static_cast<size_t>(i) * max_len + p1];
+        row_pos[2 * i] = held(p0, limit);
+        row_pos[2 * i + 1] = held(p1, limit);
+        row_seq[2 * i] = row_seq[2 * i + 1] = i;
+        logit_src[i] = 2 * i + 1;
+        logit_dst[i] = i * gamma;  // q_1
+    }
     const int b = i / (gamma + 1), j = i % (gamma + 1);
     const uint32_t pos = static_cast<uint32_t>(length[b] + j);
     const unsigned long long seed = params->seed;
     final_u[i] = method_uniform(seed, pos, b, kPurposeFinal);
     accept_u[i] = method_uniform(seed, pos, b, kPurposeAccept);  // entry j = gamma is unused
     if (j < gamma) draft_u[b * gamma + j] = method_uniform(seed, pos, b, kPurposeDraft);
-}
-
-// Rows of the passes below: a sequence that has its n_new tokens is frozen but stays in the batch, and its guesses may
-// then lie beyond the positions the context holds.  Such rows (position >= `limit`) are inactive: they are computed, and
-// neither cached nor looked at.
-__device__ __forceinline__ int held(int position, int limit) { return position < limit ? position : -1; }
-
-// First draft step of an iteration: two rows per sequence, positions L-2 and
-// L-1.  Position L-2 is already cached unless the previous iteration accepted
-// every guess (x_gamma was never fed to the draft); feeding it again rewrites
-// the same K,V row, so the shape of the step never changes.
-__global__ void prep_draft_first_kernel(const int32_t* tokens, const int32_t* length,
-                                        int batch, int gamma, int max_len, int limit, int32_t* row_token, int32_t* row_pos,
-                                        int32_t* row_seq, int32_t* logit_src, int32_t* logit_dst) {
-    pdl_trigger();
-    pdl_wait();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= batch) return;
-    const int L = length[b];
-    const int p0 = max(L - 2, 0), p1 = L - 1;
-    row_token[2 * b] = tokens[static_cast<size_t>(b) * max_len + p0];
-    row_token[2 * b + 1] = tokens[static_cast<size_t>(b) * max_len + p1];
-    row_pos[2 * b] = held(p0, limit);
-    row_pos[2 * b + 1] = held(p1, limit);
-    row_seq[2 * b] = row_seq[2 * b + 1] = b;
-    logit_src[b] = 2 * b + 1;
-    logit_dst[b] = b * gamma;  // q_1
 }
 
 // Draft step i (2..gamma): one row per sequence, the previous guess x_{i-1} at position L+i-2.
@@ -529,21 +523,15 @@ int enqueue_iteration(spec_ctx* ctx, int batch, int gamma, float temperature) {
     if (gamma > 0) limit = std::min(limit, ctx->model[1].cfg.max_positions);
     const int blocks_b = (batch + threads - 1) / threads;
     const int blocks_bg = (batch * (gamma + 1) + threads - 1) / threads;
-    SPEC_TRY(launch_pdl(iteration_uniforms_kernel, dim3(blocks_bg), dim3(threads), 0, st, ctx->params, ctx->length,
-                        batch, gamma, ctx->draft_u, ctx->accept_u, ctx->final_u));
+    SPEC_TRY(launch_pdl(start_iteration_kernel, dim3(blocks_bg), dim3(threads), 0, st, ctx->params, ctx->tokens, ctx->length, batch, gamma,
+                        ctx->rt.max_len, limit, gamma > 0, ctx->draft_u, ctx->accept_u, ctx->final_u, ctx->row_token, ctx->row_pos,
+                        ctx->row_seq, ctx->logit_src, ctx->logit_dst));
     for (int step = 1; step <= gamma; ++step) {
-        int rows;
-        if (step == 1) {
-            SPEC_TRY(launch_pdl(prep_draft_first_kernel, dim3(blocks_b), dim3(threads), 0, st, ctx->tokens, ctx->length,
-                                batch, gamma, ctx->rt.max_len, limit, ctx->row_token, ctx->row_pos, ctx->row_seq,
-                                ctx->logit_src, ctx->logit_dst));
-            rows = 2 * batch;
-        } else {
+        if (step > 1)
             SPEC_TRY(launch_pdl(prep_draft_step_kernel, dim3(blocks_b), dim3(threads), 0, st, ctx->draft_tokens,
                                 ctx->length, batch, gamma, step, limit, ctx->row_token, ctx->row_pos, ctx->row_seq,
                                 ctx->logit_src, ctx->logit_dst));
-            rows = batch;
-        }
+        const int rows = step == 1 ? 2 * batch : batch;
         SPEC_TRY(forward(ctx, ctx->model[1], row_meta(ctx), batch, rows / batch, batch, ctx->logit_src, ctx->logit_dst, ctx->draft_logits));
         // x_step ~ q_step for every sequence
         SPEC_TRY(launch_sample_strided(ctx->draft_logits + static_cast<size_t>(step - 1) * vocab,

@@ -77,7 +77,7 @@ struct SmallArgs {
     int bias_span, bias_zero;
     float eps, inv_d;
     int per_group, per_rows, per_warp, warps_per_seq, page_shift;  // per_x: ceil(256 / x) of group, m_rows, warps_per_seq
-    unsigned long long* exchanges;        // [4][16][rows][d] pairs (value, epoch)
+    unsigned long long* exchanges;        // [4][16][8][d] pairs (value, epoch)
     unsigned* epoch;                      // exchanges of all passes so far
     float* last_part;                     // [clusters][rows][d]: the last FFN's partial sums
     float* h_out;
@@ -144,9 +144,10 @@ __device__ __forceinline__ void send4(const float* here, uint64_t* bar, int rank
 __device__ __forceinline__ void publish(unsigned long long* at, float v, unsigned epoch) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(at), "l"((static_cast<unsigned long long>(epoch) << 32) | __float_as_uint(v)) : "memory");
 }
-__device__ __forceinline__ unsigned long long peek(const unsigned long long* at) {
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(at) : "memory");
+// Two neighbouring words (each is whole, whichever of them is there first).
+__device__ __forceinline__ ulonglong2 peek2(const unsigned long long* at) {
+    ulonglong2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(at) : "memory");
     return v;
 }
 __device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t parity, uint32_t limit) {
@@ -263,17 +264,18 @@ struct Pass {
     __device__ __forceinline__ const int* row_at() const { return row_pos() + 16; }  // where a row goes in the cache
     __device__ __forceinline__ int by_group(int q) const { return q * a.per_group >> 8; }  // q / group, q < 8
 
-    // v + the `count` published values of one element, in cluster order.
-    __device__ __forceinline__ float gather(const unsigned long long* at, int count, unsigned when, float v) {
-        const int stride = a.rows * kD;
-        unsigned long long w[kClusters];
+    // v += the `count` published values of two neighbouring elements, in cluster order.
+    __device__ __forceinline__ void gather(const unsigned long long* at, int count, unsigned when, float2& v) {
+        constexpr int kStride = kRows * kD;  // (known here: the addresses take no registers)
+        const unsigned long long nobody = static_cast<unsigned long long>(when) << 32;  // 0.0f
+        ulonglong2 w[kClusters];
 #pragma unroll 1
         for (uint32_t spin = 0;; ++spin) {
             bool all = true;
 #pragma unroll
-            for (int c = 0; c < kClusters; ++c) w[c] = peek(at + min(c, count - 1) * stride);
+            for (int c = 0; c < kClusters; ++c) w[c] = c < count ? peek2(at + c * kStride) : make_ulonglong2(nobody, nobody);
 #pragma unroll
-            for (int c = 0; c < kClusters; ++c) all &= static_cast<unsigned>(w[c] >> 32) == when;
+            for (int c = 0; c < kClusters; ++c) all &= static_cast<unsigned>(w[c].x >> 32) == when && static_cast<unsigned>(w[c].y >> 32) == when;
             if (all) break;
             if (spin >= limit) {
                 limit = 1;
@@ -281,9 +283,10 @@ struct Pass {
             }
         }
 #pragma unroll
-        for (int c = 0; c < kClusters; ++c)
-            v += c < count ? __uint_as_float(static_cast<unsigned>(w[c])) : 0.0f;
-        return v;
+        for (int c = 0; c < kClusters; ++c) {
+            v.x += __uint_as_float(static_cast<unsigned>(w[c].x));
+            v.y += __uint_as_float(static_cast<unsigned>(w[c].y));
+        }
     }
     // The exchange buffer of an epoch.  Four take turns: whoever publishes an exchange has, since the one four before it,
     // waited for an FFN's sums of every cluster, and they have read what came before.
@@ -302,23 +305,29 @@ struct Pass {
                          : "memory");
         }
         if (n) {
+            // (two features to a thread, so that eight rows of 768 are one trip, not two: 128 tokens of the 97M shape at six rows a pass,
+            // with what else takes pairs below, 33.9 -> 32.1 ms)
+            const int items = a.rows * (kDs / 2);
 #pragma unroll 1
-            for (int i = tid; i < a.rows * kDs; i += kThreads) {  // (kDs is a multiple of 32: whole warps)
-                const int r = i / kDs, f = rank * kDs + i % kDs;
-                float v = h(cur)[r * kD + f];
+            for (int i = tid; (i & ~31) < items; i += kThreads) {  // (whole warps)
+                const bool on = i < items;
+                const int at = on ? i : 0, r = at / (kDs / 2), f = rank * kDs + at % (kDs / 2) * 2;
+                float2 v = *reinterpret_cast<const float2*>(h(cur) + r * kD + f);
+                if (on) {
 #pragma unroll 1
-                for (int k = 0; k < n; ++k) {
-                    const unsigned when = epoch - (n - 1 - k);
-                    v = gather(exchange(when) + r * kD + f, ffn_first && k == 0 ? a.clusters : a.n_kv_heads, when, v);
+                    for (int k = 0; k < n; ++k) {
+                        const unsigned when = epoch - (n - 1 - k);
+                        gather(exchange(when) + r * kD + f, ffn_first && k == 0 ? a.clusters : a.n_kv_heads, when, v);
+                    }
                 }
-                float4 q;  // four lanes' values: lane i of the four sends them to peers i and i + 4
-                q.x = __shfl_sync(kFullMask, v, lane & ~3);
-                q.y = __shfl_sync(kFullMask, v, (lane & ~3) + 1);
-                q.z = __shfl_sync(kFullMask, v, (lane & ~3) + 2);
-                q.w = __shfl_sync(kFullMask, v, (lane & ~3) + 3);
+                __syncwarp();
+                // two lanes' values: the even one sends them to peers 0 .. 3, the odd one to 4 .. 7
+                const float ox = __shfl_xor_sync(kFullMask, v.x, 1), oy = __shfl_xor_sync(kFullMask, v.y, 1);
+                const float4 q = lane & 1 ? make_float4(ox, oy, v.x, v.y) : make_float4(v.x, v.y, ox, oy);
                 const float* to = h(cur ^ 1) + r * kD + (f & ~3);
-                send4(to, bars + kBarH, lane & 3, q);
-                send4(to, bars + kBarH, (lane & 3) + 4, q);
+                if (on)
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) send4(to, bars + kBarH, 4 * (lane & 1) + p, q);
             }
             cur ^= 1;
         }
@@ -471,6 +480,13 @@ struct Pass {
             n_keys = cross ? a.src_len[s] : max(row_pos()[b * a.m_rows], 0);
             pages = cross ? a.src_page_table + s * a.src_pages_per_seq : a.page_table + s * a.pages_per_seq;
             if (key < n_keys) page = pages[key >> a.page_shift];
+            // on their way to L2 while the residual stream is awaited: a row of 128 bytes to a lane
+#pragma unroll 1
+            for (int at = key, p = page; at < n_keys; at += step, p = at < n_keys ? pages[at >> a.page_shift] : 0) {
+                const KeyRows r = key_rows(pool, p, n_keys, at);
+                const __half* row = r.at + min(lane & 15, r.last) * kDh + (lane < 16 ? 0 : a.n_kv_heads * a.page_size * kDh);
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(row));
+            }
         }
         collect(first_block ? 0 : 1, !cross, gain);
         ++epoch;
@@ -741,13 +757,30 @@ struct Pass {
         sync_consumers();
         refill();
 #pragma unroll 1
-        for (int i = tid; i < kDs * a.rows; i += kThreads) {
-            const int f = i % kDs, row = i / kDs;
-            float s = 0.0f;
+        for (int i = tid; i < kDs * ((a.rows + 1) / 2); i += kThreads) {  // (two rows to a thread)
+            const int f = i % kDs, row = i / kDs * 2;
+            float2 s = make_float2(0.0f, 0.0f);
+            const float* p = red() + (f >> 4) * 128 + (f & 15) * 8 + row;
 #pragma unroll 1
-            for (int k = 0; k < ks; ++k) s += red()[(k * kWo + (f >> 4)) * 128 + (f & 15) * 8 + row];
-            if (!a.mute) publish(exchange(epoch) + (cluster * a.rows + row) * kD + rank * kDs + f, s, epoch);
+            for (int k = 0; k < ks; k += 4, p += 4 * kWo * 128) {
+                float2 v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = *reinterpret_cast<const float2*>(p + j * kWo * 128);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    s.x += v[j].x;
+                    s.y += v[j].y;
+                }
+            }
+            publish_rows(row, rank * kDs + f, s);
         }
+    }
+    // The sums of rows `row` and `row` + 1 (if there is one) of a feature.
+    __device__ __forceinline__ void publish_rows(int row, int feature, const float2& v) {
+        if (a.mute) return;
+        unsigned long long* at = exchange(epoch) + (cluster * kRows + row) * kD + feature;
+        publish(at, v.x, epoch);
+        if (row + 1 < a.rows) publish(at + kD, v.y, epoch);
     }
 
     // The FFN of the rows: the cluster's share of W_out act(W_in x), published, or as plain sums after the last block.
@@ -760,7 +793,7 @@ struct Pass {
         for (int i = 0; i < KI; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) out[i][j] = 0.0f;
-        await_bytes(kBarF, kD * ((a.rows + 1) / 2 * 2) * 4);
+        await_bytes(kBarF, kD * (R > 2 ? (a.rows + 3) / 4 * 4 : 2) * 4);
         const int per = a.gated ? 2 : 1;
         __nv_bfloat16* ah = reinterpret_cast<__nv_bfloat16*>(sm + S::kAct);
         __nv_bfloat16* al = ah + 2 * kRows * 16;
@@ -808,27 +841,47 @@ struct Pass {
         }
         // to the owners of the feature slices: [rank][feature][8 rows]
         float* fred = reinterpret_cast<float*>(sm + S::kFred);
-        if (2 * t < a.rows) {
+        if constexpr (R > 2) {
+            // lanes t and t ^ 1 hold two rows each of features g and g + 8: the even one takes the four of g, the odd one of g + 8
+            const int odd = t & 1, quad = t >> 1 << 2;
+#pragma unroll
+            for (int i = 0; i < KI; ++i) {
+                const float x = __shfl_xor_sync(kFullMask, odd ? out[i][0] : out[i][2], 1), y = __shfl_xor_sync(kFullMask, odd ? out[i][1] : out[i][3], 1);
+                const float4 q = odd ? make_float4(x, y, out[i][2], out[i][3]) : make_float4(out[i][0], out[i][1], x, y);
+                const int f = (i * kWarps + warp) * 16 + g + 8 * odd;
+                if (quad < a.rows) send4(fred + (rank * kDs + f % kDs) * R + quad, bars + kBarF, f / kDs, q);
+            }
+        } else if (t == 0) {
 #pragma unroll
             for (int i = 0; i < KI; ++i)
 #pragma unroll
                 for (int up = 0; up < 2; ++up) {
-                    const int f = (i * kWarps + warp) * 16 + g + 8 * up, owner = f / kDs;
-                    send2(fred + (rank * kDs + f % kDs) * R + 2 * t, bars + kBarF, owner, out[i][2 * up], out[i][2 * up + 1]);
+                    const int f = (i * kWarps + warp) * 16 + g + 8 * up;
+                    send2(fred + (rank * kDs + f % kDs) * R, bars + kBarF, f / kDs, out[i][2 * up], out[i][2 * up + 1]);
                 }
         }
         sync_consumers();  // (every warp has read its fragments)
         refill();
         arrived(kBarF);
 #pragma unroll 1
-        for (int i = tid; i < kDs * a.rows; i += kThreads) {
-            const int row = i / kDs, f = i % kDs;
-            float s = fred[f * R + row];
+        for (int i = tid; i < kDs * ((a.rows + 1) / 2); i += kThreads) {
+            const int row = i / kDs * 2, f = i % kDs;
+            float2 v[kC];
 #pragma unroll
-            for (int c = 1; c < kC; ++c) s += fred[(c * kDs + f) * R + row];
-            const int at = (cluster * a.rows + row) * kD + rank * kDs + f;
-            if (plain) plain[at] = s;
-            else if (!a.mute) publish(exchange(epoch) + at, s, epoch);
+            for (int c = 0; c < kC; ++c) v[c] = *reinterpret_cast<const float2*>(fred + (c * kDs + f) * R + row);
+            float2 s = v[0];
+#pragma unroll
+            for (int c = 1; c < kC; ++c) {
+                s.x += v[c].x;
+                s.y += v[c].y;
+            }
+            if (plain) {
+                float* at = plain + (cluster * a.rows + row) * kD + rank * kDs + f;
+                at[0] = s.x;
+                if (row + 1 < a.rows) at[kD] = s.y;
+            } else {
+                publish_rows(row, rank * kDs + f, s);
+            }
         }
     }
 };

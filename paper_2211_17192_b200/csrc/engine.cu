@@ -38,6 +38,7 @@ struct spec_ctx {
 
     // activations (sized for the wider model)
     float *h = nullptr, *a = nullptr, *qkv = nullptr, *att = nullptr, *f = nullptr;
+    float* row_squares = nullptr;  // of a norm whose factor is applied later
     float *target_logits = nullptr, *draft_logits = nullptr;
     // tensor-core GEMM path: bf16 hi/lo copies of the GEMM input, split-K partial sums
     __nv_bfloat16 *x_hi = nullptr, *x_lo = nullptr;
@@ -173,21 +174,25 @@ struct Pass {
     PartialPlan closing{};  // of the last GEMM that closed a residual branch
     PartialPlan last{};     // of the last projection
     RowNorm normed{};       // fp32 path: the norm that the next projection applies itself
+    RowFactor factor{};     // of the last norm, where its projections' partial sums still want it
 
     __nv_bfloat16* hi() const { return ctx->x_hi; }
     __nv_bfloat16* lo() const { return ctx->x_lo; }
 
     // a (fp32) or hi/lo = rmsnorm(h[src(i)]) * gain for i < n
-    int norm(const float* gain, const int32_t* src_rows, int n) {
+    // (`projected`: the projection's sums go through launch_qkv or launch_ffn_act, which apply `factor`)
+    int norm(const float* gain, const int32_t* src_rows, int n, bool projected = false) {
         const int d = m.cfg.d_model;
         normed = RowNorm{};
+        factor = RowFactor{};
+        if (tc && projected && norm_defers(d, n)) factor = RowFactor{ctx->row_squares, static_cast<float>(d), m.cfg.rms_eps};
         // (on many rows of a wide model the squares and gains would be half as much work again as the products)
         if (!tc && !m.bf16() && (n <= 8 || (n <= kMostNormedRows && d <= 512))) {
             normed = RowNorm{gain, src_rows, m.cfg.rms_eps};
             return SPEC_OK;
         }
         const int status = tc ? launch_norm(ctx->h, pending ? branch : nullptr, closing, n_rows, gain, src_rows, n, d,
-                                            m.cfg.rms_eps, nullptr, hi(), lo(), st)
+                                            m.cfg.rms_eps, nullptr, hi(), lo(), st, factor.squares ? ctx->row_squares : nullptr)
                               : launch_norm(ctx->h, nullptr, PartialPlan{}, n_rows, gain, src_rows, n, d, m.cfg.rms_eps, ctx->a, nullptr,
                                             nullptr, st);
         pending = false;
@@ -217,10 +222,10 @@ struct Pass {
     // h += FFN(rmsnorm(h) * gain)
     int ffn(const spec_layer_weights& w, const spec_layer_weights& pw) {
         const spec_model_cfg& c = m.cfg;
-        SPEC_TRY(norm(w.ln2, nullptr, n_rows));
+        SPEC_TRY(norm(w.ln2, nullptr, n_rows, true));
         if (tc) {
             SPEC_TRY(proj(w.w_in, pw.w_in, m.ffn_in_dim(), c.d_model, nullptr));
-            SPEC_TRY(launch_ffn_act(ctx->partials, last, n_rows, c.d_ff, c.ffn, hi(), lo(), st));
+            SPEC_TRY(launch_ffn_act(ctx->partials, last, n_rows, c.d_ff, c.ffn, hi(), lo(), st, factor));
         } else {
             SPEC_TRY(proj(w.w_in, pw.w_in, c.d_ff, c.d_model, ctx->f, c.ffn));
         }
@@ -231,10 +236,10 @@ struct Pass {
                        const KvPool& pool, const int32_t* kv_len, const float* bias, int bias_span, int bias_zero,
                        int max_keys, const PromptSegments* segs = nullptr) {
         const spec_model_cfg& c = m.cfg;
-        SPEC_TRY(norm(w.ln1, nullptr, n_rows));
+        SPEC_TRY(norm(w.ln1, nullptr, n_rows, true));
         SPEC_TRY(proj(w.wqkv, pw.wqkv, m.qkv_dim(), c.d_model, ctx->qkv));
         SPEC_TRY(launch_qkv(c.n_heads, c.n_kv_heads, c.d_head, c.arch == SPEC_ARCH_LLAMA ? m.rope_table : nullptr, pool, rows,
-                            n_rows, ctx->qkv, partials(), last, st));
+                            n_rows, ctx->qkv, partials(), last, st, factor));
         const AttnSource src{ctx->qkv, m.qkv_dim(), pool, kv_len, bias, bias_span, bias_zero};
         if (segs) {
             SPEC_TRY(launch_prompt_attention(m, src, *segs, hi(), lo(), st));
@@ -353,14 +358,14 @@ int forward(spec_ctx* ctx, const Model& m, const RowMeta& rows, int batch, int m
         SPEC_TRY(pass.self_attention(w, pw, rows, batch, m_rows, layer_pool(ctx, m, l), nullptr, bias, ctx->rt.max_len,
                                      ctx->rt.max_len - 1, ctx->rt.max_len, segs));
         if (m.t5()) {  // cross-attention over the source's K,V (every row sees every source position)
-            SPEC_TRY(pass.norm(w.lnx, nullptr, n_rows));
+            SPEC_TRY(pass.norm(w.lnx, nullptr, n_rows, true));
             SPEC_TRY(pass.proj(w.wq_x, pw.wq_x, m.q_dim(), d, ctx->qkv));
             if (pass.tc)  // the partial sums become the query rows
                 SPEC_TRY(launch_qkv(c.n_heads, 0, c.d_head, nullptr, KvPool{}, rows, n_rows, ctx->qkv, ctx->partials,
-                                    pass.last, ctx->stream));
+                                    pass.last, ctx->stream, pass.factor));
             const KvPool pool = source_pool(ctx, m, static_cast<char*>(m.cross_kv) + static_cast<size_t>(l) * m.cross_stride);
             const int slices = attention_slices(m, batch, m_rows, ctx->rt.max_src_len);
-            const AttnSource src{ctx->qkv, m.q_dim(), pool, ctx->src_len, nullptr, 0, 0};
+            const AttnSource src{ctx->qkv, m.q_dim(), pool, ctx->src_len, nullptr, 0, 0, true};
             SPEC_TRY(launch_attention(m, src, rows, batch, m_rows, slices, ctx->rt.max_src_len, ctx->attn_part, pass.tc ? nullptr : ctx->att,
                                       pass.tc ? pass.hi() : nullptr, pass.tc ? pass.lo() : nullptr, ctx->stream));
             SPEC_TRY(pass.residual(w.wo_x, pw.wo_x, m.q_dim(), ctx->att));
@@ -939,6 +944,7 @@ extern "C" int spec_init(const spec_model_cfg* target_cfg, const spec_model_cfg*
     auto alloc_rows = [&]() -> int {
         const size_t R = ctx->max_rows;
         SPEC_TRY(dev_alloc(ctx, &ctx->h, R * d));
+        SPEC_TRY(dev_alloc(ctx, &ctx->row_squares, kDeferredRows * 32));
         SPEC_TRY(dev_alloc(ctx, &ctx->qkv, R * std::max(qkv, 2 * att)));
         if (any_fp32) {
             SPEC_TRY(dev_alloc(ctx, &ctx->a, R * d));

@@ -90,25 +90,29 @@ __global__ void embed_kernel(const void* tok_emb, const void* pos_emb, bool bf16
 // With CTAS > 1 a cluster of that many CTAs shares a row (d at most 4 * THREADS * CTAS, PER = 1, grid = rows * CTAS): a
 // row of 4096 with its eight partial sums is 147 KB, a microsecond of what one SM takes in, and nothing else runs
 // meanwhile.  The CTAs give one another their warps' sums of squares through distributed shared memory.
+// DEFER: they do not.  W . (rmsnorm(h) gain) is W . (h gain) times a factor per row, so the terms are of h * gain, the warps' sums of
+// squares go to `squares`, [row][32], and the kernel that adds up the GEMM's partial sums forms the factor (row_factor).  The
+// norm is a stop between two weight streams of which only the first 24 MB of the second is on its way meanwhile, and the
+// exchange between the CTAs was a fifth of it (7B shape, three rows: 7.0 -> 5.5 us behind the GEMM).
 constexpr int kNormMaxWidth = 4 * 1024 * 4;
 constexpr int kNormCtas = 8;  // of a cluster that shares a row
 // The elementwise kernels give a thread several rows where one each is more threads than the GPU holds at once: below that the
 // rows of a thread only lengthen it (96 rows of the 160M shape: a pass 625 us with a row each, 699 with four).
 constexpr long long kResidentThreads = 148 * 2048;
 constexpr int kNormFourRows = 296;  // at most for a cluster of four: eight CTAs of 256 threads to an SM
-constexpr int kNormClusterRows = 128;  // at most (launch_norm has both sides)
+constexpr int kNormClusterRows = kDeferredRows;  // at most (launch_norm has both sides)
 
-template <int THREADS, int PER, int CTAS = 1>
+template <int THREADS, int PER, int CTAS = 1, bool DEFER = false>
 __global__ void __launch_bounds__(THREADS)
 norm_kernel(float* h, const float* partial, const PartialPlan plan, int n_rows, const float* gain,
             const int32_t* src_rows, int d, float eps, float* out,
-            __nv_bfloat16* out_hi, __nv_bfloat16* out_lo) {
+            __nv_bfloat16* out_hi, __nv_bfloat16* out_lo, float* squares) {
     static_assert(CTAS == 1 || (PER == 1 && CTAS * THREADS / 32 == 32), "a lane per warp of the cluster");
     __shared__ float red[CTAS * THREADS / 32];
     const int r = blockIdx.x / CTAS;
     const int groups = d / 4;
     const int first = CTAS > 1 ? blockIdx.x % CTAS * THREADS + threadIdx.x : threadIdx.x;
-    if constexpr (CTAS > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // (its peers are there)
+    if constexpr (CTAS > 1 && !DEFER) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // (its peers are there)
     // the gains are constants: fetched while the kernel before this one is still finishing
     float4 gg[PER];
 #pragma unroll
@@ -165,7 +169,9 @@ norm_kernel(float* h, const float* partial, const PartialPlan plan, int n_rows, 
     for (int j = 0; j < PER; ++j) ss += (v[j].x * v[j].x + v[j].y * v[j].y) + (v[j].z * v[j].z + v[j].w * v[j].w);
     ss = warp_sum(ss);
     float total = 0.0f;
-    if constexpr (CTAS > 1) {
+    if constexpr (DEFER) {
+        if ((threadIdx.x & 31) == 0) squares[32 * r + (first >> 5)] = ss;
+    } else if constexpr (CTAS > 1) {
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         const int lane = threadIdx.x & 31;
         if (lane < CTAS) {
@@ -184,19 +190,29 @@ norm_kernel(float* h, const float* partial, const PartialPlan plan, int n_rows, 
 #pragma unroll
         for (int i = 0; i < THREADS / 32; ++i) total += red[i];
     }
-    const float scale = rsqrtf(total / static_cast<float>(d) + eps);
+    const float scale = DEFER ? 1.0f : rsqrtf(total / static_cast<float>(d) + eps);
     const size_t dst = static_cast<size_t>(r) * d;
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
         const int g = first + j * THREADS;
         if (g < groups) {
-            const float4 y = make_float4(v[j].x * scale * gg[j].x, v[j].y * scale * gg[j].y, v[j].z * scale * gg[j].z,
+            const float4 y = DEFER ? make_float4(v[j].x * gg[j].x, v[j].y * gg[j].y, v[j].z * gg[j].z, v[j].w * gg[j].w)
+                                   : make_float4(v[j].x * scale * gg[j].x, v[j].y * scale * gg[j].y, v[j].z * scale * gg[j].z,
                                          v[j].w * scale * gg[j].w);
             if (out) *reinterpret_cast<float4*>(out + dst + 4 * g) = y;
             if (out_hi) store_split4(out_hi, out_lo, dst + 4 * g, y);
         }
     }
 }
+
+// The factor of a deferred norm in row r (1 without one): what the norm kernel would have multiplied the row with.  All lanes.
+struct DeferredRow {
+    float square = 0.0f;  // this lane's, on its way while other loads are
+    __device__ __forceinline__ void fetch(const RowFactor& f, int r) {
+        if (f.squares) square = f.squares[32 * r + (threadIdx.x & 31)];
+    }
+    __device__ __forceinline__ float factor(const RowFactor& f) const { return f.squares ? rsqrtf(warp_sum(square) / f.width + f.eps) : 1.0f; }
+};
 
 template <typename KV>
 __device__ __forceinline__ void store_cached4(KV* dst, const float (&v)[4]) {
@@ -218,13 +234,17 @@ __global__ void qkv_kernel(float* qkv, const float* partial, const PartialPlan p
                            const int32_t* pos, const int32_t* seq, int n_heads,
                            int n_kv_heads, int d_head, const float2* rope_table,
                            KV* kv_layer, const int32_t* page_table, int pages_per_seq,
-                           int page_shift) {
+                           int page_shift, const RowFactor norm) {
     pdl_trigger();
     pdl_wait();
     const int half = d_head / 2, per_head = half / 4;
     const int task = blockIdx.x * blockDim.x + threadIdx.x, r0 = ROWS * blockIdx.y;
     const int head = task / per_head, j = 4 * (task % per_head);
-    if (head >= n_heads + 2 * n_kv_heads) return;
+    DeferredRow deferred[ROWS];
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) deferred[i].fetch(norm, min(r0 + i, n_rows - 1));
+    if (blockIdx.x * blockDim.x + (threadIdx.x & ~31) >= (n_heads + 2 * n_kv_heads) * per_head) return;  // (whole warps)
+    const bool out = head >= n_heads + 2 * n_kv_heads;
     const bool is_q = head < n_heads, is_k = !is_q && head < n_heads + n_kv_heads;
     const int width = (n_heads + 2 * n_kv_heads) * d_head;
     int p[ROWS];
@@ -242,22 +262,33 @@ __global__ void qkv_kernel(float* qkv, const float* partial, const PartialPlan p
     float4 x[2 * ROWS];
 #pragma unroll
     for (int i = 0; i < ROWS; ++i) {
-        where[2 * i] = static_cast<size_t>(min(r0 + i, n_rows - 1)) * width + head * d_head + j;
+        where[2 * i] = static_cast<size_t>(min(r0 + i, n_rows - 1)) * width + (out ? 0 : head * d_head + j);
         where[2 * i + 1] = where[2 * i] + half;
         x[2 * i] = x[2 * i + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     if (partial) {
         // (a head of 64 or 128 columns lies inside one 256-column tile)
-        sum_partials<2 * ROWS, ROWS == 1 ? 4 : 1>(partial, partial_count(plan, r0, head * d_head), static_cast<size_t>(n_rows) * width, where, x);
+        sum_partials<2 * ROWS, ROWS == 1 ? 4 : 1>(partial, partial_count(plan, r0, out ? 0 : head * d_head), static_cast<size_t>(n_rows) * width, where, x);
     } else {
 #pragma unroll
         for (int i = 0; i < 2 * ROWS; ++i) x[i] = *reinterpret_cast<const float4*>(qkv + where[i]);
     }
+    float factor[ROWS];
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) factor[i] = deferred[i].factor(norm);
+    if (out) return;
 #pragma unroll
     for (int i = 0; i < ROWS; ++i) {
         if (ROWS > 1 && r0 + i >= n_rows) break;
         const float4 xa = x[2 * i], xb = x[2 * i + 1];
         float a[4] = {xa.x, xa.y, xa.z, xa.w}, b[4] = {xb.x, xb.y, xb.z, xb.w};
+        if (norm.squares) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                a[e] *= factor[i];
+                b[e] *= factor[i];
+            }
+        }
         if (rope_table && p[i] >= 0 && (is_q || is_k)) {
             const float c[4] = {t[i][0].x, t[i][0].z, t[i][1].x, t[i][1].z}, s[4] = {t[i][0].y, t[i][0].w, t[i][1].y, t[i][1].w};
 #pragma unroll
@@ -341,11 +372,16 @@ __global__ void copy_logits_kernel(const int32_t* tokens, int max_len, const int
 constexpr int kActRows = 4;  // (a tile's rows are a multiple of 16: these share their partial sums' number)
 template <int FFN, int ROWS>
 __global__ void ffn_act_kernel(const float* partial, const PartialPlan plan, int n_rows, int d_ff, __nv_bfloat16* f_hi,
-                               __nv_bfloat16* f_lo) {
+                               __nv_bfloat16* f_lo, const RowFactor norm) {
     pdl_trigger();
     pdl_wait();
-    const int c = 4 * (blockIdx.x * blockDim.x + threadIdx.x), r0 = ROWS * blockIdx.y;
-    if (c >= d_ff) return;
+    const int mine = 4 * (blockIdx.x * blockDim.x + threadIdx.x), r0 = ROWS * blockIdx.y;
+    if (mine - 4 * static_cast<int>(threadIdx.x & 31) >= d_ff) return;  // (whole warps)
+    const bool beyond = mine >= d_ff;
+    const int c = beyond ? 0 : mine;
+    DeferredRow deferred[ROWS];
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) deferred[i].fetch(norm, min(r0 + i, n_rows - 1));
     constexpr bool kGated = FFN != SPEC_FFN_GELU;
     const int width = kGated ? 2 * d_ff : d_ff;
     const size_t stride = static_cast<size_t>(n_rows) * width;
@@ -390,6 +426,15 @@ __global__ void ffn_act_kernel(const float* partial, const PartialPlan plan, int
             }
         }
     }
+    if (norm.squares) {
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+            const float f = deferred[i].factor(norm);
+            g[i] = make_float4(g[i].x * f, g[i].y * f, g[i].z * f, g[i].w * f);
+            up[i] = make_float4(up[i].x * f, up[i].y * f, up[i].z * f, up[i].w * f);
+        }
+    }
+    if (beyond) return;
 #pragma unroll
     for (int i = 0; i < ROWS; ++i) {
         if (ROWS > 1 && r0 + i >= n_rows) break;
@@ -425,14 +470,17 @@ int launch_copy_logits(const int32_t* tokens, int max_len, const int32_t* length
                       gamma, rows.pos, rows.seq, src_rows, dst_rows, ngram, vocab, logits);
 }
 
+bool norm_defers(int d, int n_rows) { return d % 4 == 0 && d > 2048 && d <= 512 * kNormCtas && n_rows <= kNormClusterRows; }
+
 int launch_norm(float* h, const float* partial, const PartialPlan& plan, int rows_total, const float* gain, const int32_t* src_rows,
                 int n_rows, int d, float eps, float* out, __nv_bfloat16* out_hi, __nv_bfloat16* out_lo,
-                cudaStream_t stream) {
+                cudaStream_t stream, float* squares) {
     if (d % 4 || d > kNormMaxWidth)
         return fail(SPEC_ERR_BAD_CONFIG, "norm: width %d is not a multiple of 4 or exceeds %d", d, kNormMaxWidth);
 #define SPEC_LAUNCH_NORM(T, P)                                                                                              \
     return launch_pdl(norm_kernel<T, P>, dim3(n_rows), dim3(T), 0, stream, h, partial, plan, rows_total, gain, src_rows, d, \
-                      eps, out, out_hi, out_lo)
+                      eps, out, out_hi, out_lo, static_cast<float*>(nullptr))
+    if (squares && !norm_defers(d, n_rows)) return fail(SPEC_ERR_BAD_CONFIG, "norm: %d rows of %d are not deferred", n_rows, d);
     // a thread per 128-bit group of the row (fewer warps to reduce over where the row is narrow); with more rows than
     // SMs, small CTAs with several groups per thread, so that the CTAs of an SM wait for memory side by side.
     // Wide rows that leave SMs idle go to a cluster each.  Whole pass of the 7B shape at 500 cached tokens, a CTA of 1024
@@ -441,12 +489,15 @@ int launch_norm(float* h, const float* partial, const PartialPlan& plan, int row
     // 5.232 / 5.216; beyond, four larger CTAs (eight partial sums in flight, not two: 224 rows 11.0 -> 9.8 us behind the GEMM), and
     // where those no longer fit side by side a CTA per row.
     const int groups = d / 4;
+    if (squares)
+        return launch_cluster(norm_kernel<128, 1, kNormCtas, true>, 0, dim3(n_rows * kNormCtas), dim3(128), 0, stream, h, partial,
+                              plan, rows_total, gain, src_rows, d, eps, out, out_hi, out_lo, squares);
     if (groups > 512 && groups <= 128 * kNormCtas && n_rows <= kNormClusterRows)
         return launch_cluster(norm_kernel<128, 1, kNormCtas>, kNormCtas, dim3(n_rows * kNormCtas), dim3(128), 0, stream, h, partial,
-                              plan, rows_total, gain, src_rows, d, eps, out, out_hi, out_lo);
+                              plan, rows_total, gain, src_rows, d, eps, out, out_hi, out_lo, static_cast<float*>(nullptr));
     if (groups > 512 && groups <= 1024 && n_rows <= kNormFourRows)
         return launch_cluster(norm_kernel<256, 1, 4>, 4, dim3(n_rows * 4), dim3(256), 0, stream, h, partial, plan, rows_total, gain,
-                              src_rows, d, eps, out, out_hi, out_lo);
+                              src_rows, d, eps, out, out_hi, out_lo, static_cast<float*>(nullptr));
     if (groups <= 128) SPEC_LAUNCH_NORM(128, 1);
     if (groups <= 256) SPEC_LAUNCH_NORM(256, 1);
     if (groups <= 1024 && n_rows > 148) SPEC_LAUNCH_NORM(256, 4);
@@ -456,7 +507,7 @@ int launch_norm(float* h, const float* partial, const PartialPlan& plan, int row
 }
 
 int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, const KvPool& pool, const RowMeta& rows,
-               int n_rows, float* qkv, const float* partial, const PartialPlan& plan, cudaStream_t stream) {
+               int n_rows, float* qkv, const float* partial, const PartialPlan& plan, cudaStream_t stream, const RowFactor& norm) {
     const int tasks = (n_heads + 2 * n_kv_heads) * (d_head / 8);
     const bool many = static_cast<long long>(n_rows) * tasks > kResidentThreads;
     const int threads = n_rows <= 16 ? 64 : 256;
@@ -465,7 +516,7 @@ int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, cons
     while ((1 << page_shift) < pool.page_size) ++page_shift;
 #define SPEC_LAUNCH_QKV(KV, R)                                                                                                  \
     return launch_pdl(qkv_kernel<KV, R>, grid, dim3(threads), 0, stream, qkv, partial, plan, n_rows, rows.pos, rows.seq, n_heads, \
-                      n_kv_heads, d_head, rope, static_cast<KV*>(pool.kv), pool.page_table, pool.pages_per_seq, page_shift)
+                      n_kv_heads, d_head, rope, static_cast<KV*>(pool.kv), pool.page_table, pool.pages_per_seq, page_shift, norm)
     if (pool.dtype == SPEC_DTYPE_FP16 && many) SPEC_LAUNCH_QKV(__half, kQkvRows);
     if (pool.dtype == SPEC_DTYPE_FP16) SPEC_LAUNCH_QKV(__half, 1);
     if (pool.dtype == SPEC_DTYPE_BF16 && many) SPEC_LAUNCH_QKV(__nv_bfloat16, kQkvRows);
@@ -476,13 +527,13 @@ int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, cons
 }
 
 int launch_ffn_act(const float* partial, const PartialPlan& plan, int n_rows, int d_ff, int ffn, __nv_bfloat16* f_hi,
-                   __nv_bfloat16* f_lo, cudaStream_t stream) {
+                   __nv_bfloat16* f_lo, cudaStream_t stream, const RowFactor& norm) {
     const bool many = static_cast<long long>(n_rows) * (d_ff / 4) > kResidentThreads;
     const int threads = n_rows <= 16 ? 64 : 256;
     const dim3 grid((d_ff / 4 + threads - 1) / threads, many ? (n_rows + kActRows - 1) / kActRows : n_rows);
 #define SPEC_LAUNCH_ACT(F)                                                                                                     \
-    return many ? launch_pdl(ffn_act_kernel<F, kActRows>, grid, dim3(threads), 0, stream, partial, plan, n_rows, d_ff, f_hi, f_lo) \
-                : launch_pdl(ffn_act_kernel<F, 1>, grid, dim3(threads), 0, stream, partial, plan, n_rows, d_ff, f_hi, f_lo)
+    return many ? launch_pdl(ffn_act_kernel<F, kActRows>, grid, dim3(threads), 0, stream, partial, plan, n_rows, d_ff, f_hi, f_lo, norm) \
+                : launch_pdl(ffn_act_kernel<F, 1>, grid, dim3(threads), 0, stream, partial, plan, n_rows, d_ff, f_hi, f_lo, norm)
     if (ffn == SPEC_FFN_GELU) SPEC_LAUNCH_ACT(SPEC_FFN_GELU);
     if (ffn == SPEC_FFN_SWIGLU) SPEC_LAUNCH_ACT(SPEC_FFN_SWIGLU);
     SPEC_LAUNCH_ACT(SPEC_FFN_GATED_GELU);

@@ -96,7 +96,15 @@ int launch_copy_logits(const int32_t* tokens, int max_len, const int32_t* length
                        int vocab, float* logits, cudaStream_t stream);
 int launch_norm(float* h, const float* partial, const PartialPlan& plan, int rows_total, const float* gain, const int32_t* src_rows,
                 int n_rows, int d, float eps, float* out, __nv_bfloat16* out_hi, __nv_bfloat16* out_lo,
-                cudaStream_t stream);
+                cudaStream_t stream, float* squares = nullptr);
+// With `squares` ([n_rows][32] floats; only where norm_defers says so) the rows come without their factor, which whoever adds up
+// the projection's partial sums then applies: a RowFactor of these squares.
+bool norm_defers(int d, int n_rows);
+constexpr int kDeferredRows = 128;
+struct RowFactor {
+    const float* squares = nullptr;  // nullptr: the rows have it already
+    float width = 1.0f, eps = 0.0f;
+};
 
 // y[dst(r)] = x[r] . W^T (+ residual[r]) on the FMA pipes;  W is [n_out, k] row-major in fp32 or bf16.
 // dst(r) = dst_rows ? dst_rows[r] : r.  y and residual may alias.
@@ -161,7 +169,7 @@ struct KvPool {
 // active row appended to the pool.  n_kv_heads = 0: queries only; n_heads = 0:
 // K,V only.
 int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, const KvPool& pool, const RowMeta& rows,
-               int n_rows, float* qkv, const float* partial, const PartialPlan& plan, cudaStream_t stream);
+               int n_rows, float* qkv, const float* partial, const PartialPlan& plan, cudaStream_t stream, const RowFactor& norm = RowFactor{});
 void fill_rope_table(std::vector<float2>& table, int positions, int d_head, double base);
 
 // One attention call: head h of query row r is at q + r * q_stride + h * d_head.
@@ -177,6 +185,7 @@ struct AttnSource {
     const float* bias;
     int bias_span;
     int bias_zero;
+    bool fixed = false;  // the pool's rows are those of an earlier pass, all of them
 };
 
 // att[r, h] = softmax(scores) V for the rows of a pass; rows of sequence b are
@@ -204,7 +213,7 @@ int launch_prompt_attention(const Model& m, const AttnSource& src, const PromptS
 
 // f = gelu(u)  |  gelu(u[:, :F]) * u[:, F:]  |  silu(u[:, :F]) * u[:, F:], u the partial sums, f two bf16 terms.
 int launch_ffn_act(const float* partial, const PartialPlan& plan, int n_rows, int d_ff, int ffn, __nv_bfloat16* f_hi,
-                   __nv_bfloat16* f_lo, cudaStream_t stream);
+                   __nv_bfloat16* f_lo, cudaStream_t stream, const RowFactor& norm = RowFactor{});
 
 // mega.cu: one forward pass over at most 16 rows as one persistent cooperative kernel
 // (bf16 decoder-only models).

@@ -3,8 +3,9 @@
     python -m paper_2211_17192_b200.build [--force] [--verbose]
 
 Each `csrc/*.cu` is compiled to an object under `build/` and the objects are
-linked into `paper_2211_17192_b200/lib/libspecdecode.so`.  Nothing is cached
-outside the repository, so the shared object travels with the tree.
+linked into `paper_2211_17192_b200/lib/libspecdecode.so`; `csrc/calls.c`, the Python
+module of the calls that are made once per decision, becomes `lib/_calls.so`.  Nothing is cached
+outside the repository, so the shared objects travel with the tree.
 """
 
 import argparse
@@ -14,6 +15,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG_DIR)
@@ -22,6 +24,7 @@ INCLUDE = os.path.join(ROOT, "include")
 OBJ_DIR = os.path.join(ROOT, "build", "obj")
 LIB_DIR = os.path.join(PKG_DIR, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "libspecdecode.so")
+CALLS_PATH = os.path.join(LIB_DIR, "_calls.so")
 DIGEST_PATH = LIB_PATH + ".sha256"
 
 NVCC_FLAGS = [
@@ -57,7 +60,7 @@ def source_digest():
     h = hashlib.sha256(" ".join(NVCC_FLAGS[:8]).encode())
     for folder in (CSRC, INCLUDE):
         for name in sorted(os.listdir(folder)):
-            if name.endswith((".cu", ".cuh", ".h")):
+            if name.endswith((".cu", ".cuh", ".h", ".c")):
                 h.update(name.encode())
                 with open(os.path.join(folder, name), "rb") as f:
                     h.update(f.read())
@@ -68,7 +71,7 @@ def build(force=False, verbose=False):
     """Compile and link; returns the path of the shared library.  A library
     whose recorded source digest matches the tree is left alone."""
     digest = source_digest()
-    if not force and not verbose and os.path.exists(LIB_PATH) and os.path.exists(DIGEST_PATH):
+    if not force and not verbose and all(os.path.exists(p) for p in (LIB_PATH, CALLS_PATH, DIGEST_PATH)):
         with open(DIGEST_PATH) as f:
             if f.read().strip() == digest:
                 return LIB_PATH
@@ -102,6 +105,12 @@ def build(force=False, verbose=False):
         if res.returncode != 0:
             sys.stderr.write(res.stdout + res.stderr)
             raise RuntimeError("link failed")
+    cmd = [shutil.which("gcc") or "gcc", "-O2", "-std=c11", "-Wall", "-Wextra", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+           os.path.join(CSRC, "calls.c"), "-o", CALLS_PATH]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(" ".join(cmd) + "\n" + res.stdout + res.stderr)
+        raise RuntimeError("gcc failed for calls.c")
     with open(DIGEST_PATH, "w") as f:
         f.write(digest + "\n")
     return LIB_PATH

@@ -236,13 +236,12 @@ __global__ void qkv_kernel(float* qkv, const float* partial, const PartialPlan p
                            KV* kv_layer, const int32_t* page_table, int pages_per_seq,
                            int page_shift, const RowFactor norm) {
     pdl_trigger();
-    pdl_wait();
+    // (with partial sums the kernel in front is a tensor-core GEMM, which releases this one only after its own wait: the rows'
+    // positions, rotations and pages are older than that, and are fetched ahead of this kernel's)
+    if (!partial) pdl_wait();
     const int half = d_head / 2, per_head = half / 4;
     const int task = blockIdx.x * blockDim.x + threadIdx.x, r0 = ROWS * blockIdx.y;
     const int head = task / per_head, j = 4 * (task % per_head);
-    DeferredRow deferred[ROWS];
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i) deferred[i].fetch(norm, min(r0 + i, n_rows - 1));
     if (blockIdx.x * blockDim.x + (threadIdx.x & ~31) >= (n_heads + 2 * n_kv_heads) * per_head) return;  // (whole warps)
     const bool out = head >= n_heads + 2 * n_kv_heads;
     const bool is_q = head < n_heads, is_k = !is_q && head < n_heads + n_kv_heads;
@@ -258,6 +257,21 @@ __global__ void qkv_kernel(float* qkv, const float* partial, const PartialPlan p
             t[i][0] = at[0];
             t[i][1] = at[1];
         }
+    size_t cached[ROWS];  // where K or V of a row goes
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+        cached[i] = 0;
+        if (p[i] >= 0 && !is_q && !out) {
+            const int kv_head = is_k ? head - n_heads : head - n_heads - n_kv_heads;
+            const int page = page_table[seq[min(r0 + i, n_rows - 1)] * pages_per_seq + (p[i] >> page_shift)];
+            const size_t block = (static_cast<size_t>(page) * 2 + (is_k ? 0 : 1)) * n_kv_heads + kv_head;
+            cached[i] = ((block << page_shift) + (p[i] & ((1 << page_shift) - 1))) * d_head + j;
+        }
+    }
+    if (partial) pdl_wait();
+    DeferredRow deferred[ROWS];
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) deferred[i].fetch(norm, min(r0 + i, n_rows - 1));
     size_t where[2 * ROWS];
     float4 x[2 * ROWS];
 #pragma unroll
@@ -304,10 +318,7 @@ __global__ void qkv_kernel(float* qkv, const float* partial, const PartialPlan p
             continue;
         }
         if (p[i] < 0) continue;  // inactive row: nothing is cached
-        const int kv_head = is_k ? head - n_heads : head - n_heads - n_kv_heads;
-        const int page = page_table[seq[r0 + i] * pages_per_seq + (p[i] >> page_shift)];
-        const size_t block = (static_cast<size_t>(page) * 2 + (is_k ? 0 : 1)) * n_kv_heads + kv_head;
-        KV* dst = kv_layer + ((block << page_shift) + (p[i] & ((1 << page_shift) - 1))) * d_head + j;
+        KV* dst = kv_layer + cached[i];
         store_cached4<KV>(dst, a);
         store_cached4<KV>(dst + half, b);
     }

@@ -146,6 +146,9 @@ struct Worker {
     int tid, lane, warp, cta;
     uint32_t limit;  // of every wait; 1 after one ran out
     uint32_t turns;  // a bit per barrier: its parity
+    // what divisions by runtime numbers give, once for the pass: warps per sequence, this warp's sequence and place in it; the
+    // sequence of row `warp`; sequence and place in it of row tid / kDv
+    int wps, b, wi, warp_seq, out_seq, out_row;
 
     __device__ __forceinline__ void arrived(int which) {
         if (!bar_wait(bars + which, (turns >> which) & 1, limit)) limit = 1;
@@ -215,14 +218,14 @@ struct Worker {
         }
         return rsqrtf(sum_over_lanes(ss, lane) / static_cast<float>(D) + a.eps);
     }
-    // [rows][width] results in kRed go to peers first .. first + count - 1, row r at to + r * ld; the whole CTA, before and after
-    // a barrier.
-    __device__ __forceinline__ void share(int width, float* to, int ld, int which, int first, int count) {
-        const int groups = a.rows * (width / 4);
-#pragma unroll 1
-        for (int i = tid; i < groups * count; i += kThreads) {
-            const int peer = first + i / groups, at = i % groups, r = at / (width / 4), f = at % (width / 4) * 4;
-            send4(to + r * ld + f, bars + which, peer, *reinterpret_cast<const float4*>(sm + S::kRed + r * width + f));
+    // [rows][WIDTH] results in kRed go to everyone, row r to to + r * LD; the whole CTA, between two barriers.
+    template <int WIDTH, int LD>
+    __device__ __forceinline__ void share(float* to, int which) {
+        constexpr int kGroups = R * (WIDTH / 4);
+#pragma unroll
+        for (int i = tid; i < kGroups * kCtas; i += kThreads) {
+            const int peer = i / kGroups, at = i % kGroups, r = at / (WIDTH / 4), f = at % (WIDTH / 4) * 4;
+            if (r < a.rows) send4(to + r * LD + f, bars + which, peer, *reinterpret_cast<const float4*>(sm + S::kRed + r * WIDTH + f));
         }
     }
     __device__ __forceinline__ const int* row_pos() const { return reinterpret_cast<const int*>(sm + S::kMeta); }
@@ -240,7 +243,6 @@ struct Worker {
         float* red = sm + S::kRed;
         float* pool = a.kv + layer * a.layer_stride;
         // this warp's share of the keys: one sequence, every wps-th group of eight; the first are fetched ahead
-        const int wps = kWarps / a.batch, b = warp / wps, wi = warp % wps;
         const bool live = b < a.batch;
         int cached = 0;
         const int32_t* pages = nullptr;
@@ -290,8 +292,9 @@ struct Worker {
         {
             constexpr int kGroups = 3 * S::kDv / 4;
 #pragma unroll 1
-            for (int i = tid; i < a.rows * kGroups * S::kGroup; i += kThreads) {
-                const int peer = i / (a.rows * kGroups), at = i % (a.rows * kGroups), r = at / kGroups, f = at % kGroups * 4;
+            for (int i = tid; i < R * kGroups * S::kGroup; i += kThreads) {
+                const int peer = i / (R * kGroups), at = i % (R * kGroups), r = at / kGroups, f = at % kGroups * 4;
+                if (r >= a.rows) continue;
                 const int part = f / S::kDv, dim = j * S::kDv + f % S::kDv;
                 const float4 y = *reinterpret_cast<const float4*>(red + r * 3 * S::kDv + f);
                 send4(xq + r * 3 * kDh + part * kDh + dim, bars + kBarX, head * S::kGroup + peer, y);
@@ -334,8 +337,7 @@ struct Worker {
         }
         __syncthreads();
         if (warp < a.rows) {  // weights, a warp to a row
-            const int mine = warp / a.m_rows;
-            const int n = min(min(max(row_pos()[mine * a.m_rows], 0), kMaxKeys) + a.m_rows, kMaxKeys);
+            const int n = min(min(max(row_pos()[warp_seq * a.m_rows], 0), kMaxKeys) + a.m_rows, kMaxKeys);
             float* p = sc + warp * kMaxKeys;
             float top = -FLT_MAX;
             for (int i = lane; i < n; i += 32) top = fmaxf(top, p[i]);
@@ -380,8 +382,9 @@ struct Worker {
             const int r = tid / S::kDv, dim = tid % S::kDv;
             float o = 0.0f;
             if (r < a.rows) {
-                const int seq = r / a.m_rows, i = r % a.m_rows;
-                for (int w = 0; w < wps; ++w) o += red[((seq * wps + w) * R + i) * S::kDv + dim];
+                const float* p = red + (out_seq * wps * R + out_row) * S::kDv + dim;
+#pragma unroll 4
+                for (int w = 0; w < wps; ++w) o += p[w * R * S::kDv];
             }
             spread(o, r, sm + S::kOut + r * D + head * kDh + j * S::kDv + (dim & ~3), kBarO);
         }
@@ -404,7 +407,7 @@ struct Worker {
         }
         await_bytes(kBarH, a.rows * D * 4);
         __syncthreads();
-        share(S::kO, sm + S::kH + cta * S::kO, D, kBarH, 0, kCtas);
+        share<S::kO, D>(sm + S::kH + cta * S::kO, kBarH);
         arrived(kBarH);
         // ---- FFN ----
         arrived(kBarWi);
@@ -423,7 +426,7 @@ struct Worker {
         }
         await_bytes(kBarA, a.rows * S::kF * 4);
         __syncthreads();
-        share(S::kFc, sm + S::kAct + cta * S::kFc, S::kF, kBarA, 0, kCtas);
+        share<S::kFc, S::kF>(sm + S::kAct + cta * S::kFc, kBarA);
         arrived(kBarA);
         arrived(kBarW2);
         {  // a quarter of the inputs to a warp
@@ -483,7 +486,12 @@ __global__ void __launch_bounds__(kThreads, 1) cluster_pass_kernel(const __grid_
     }
     __syncthreads();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    W w{a, sm, bars, tid, tid & 31, tid >> 5, static_cast<int>(cta), a.limit, 0};
+    W w{a, sm, bars, tid, tid & 31, tid >> 5, static_cast<int>(cta), a.limit, 0, kWarps / a.batch, 0, 0, 0, 0, 0};
+    w.b = w.warp / w.wps;
+    w.wi = w.warp % w.wps;
+    w.warp_seq = w.warp / a.m_rows;
+    w.out_seq = tid / S::kDv / a.m_rows;
+    w.out_row = tid / S::kDv % a.m_rows;
     if (tid == 0) {  // (weights are constants)
         w.fetch_qkv(0);
         w.fetch_rest(0);

@@ -616,6 +616,14 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
                      const float* __restrict__ final_uniforms, float lenience, const float* floors,
                      int32_t* __restrict__ n_accepted, int32_t* __restrict__ next_token, int* __restrict__ nonfinite) {
     __shared__ FinishShared sh;
+    if (ALONE) {  // (all of its inputs may come from the kernel in front)
+        pdl_wait();
+        pdl_trigger();
+        target_logits = after_wait(target_logits);
+        draft_logits = after_wait(draft_logits);
+        draft_tokens = after_wait(draft_tokens);
+        uniforms = after_wait(uniforms);
+    }
     const int tid = threadIdx.x;
     const int b = blockIdx.x / cluster_size;
     const int rank = blockIdx.x % cluster_size;
@@ -627,7 +635,6 @@ verify_finish_kernel(const float* __restrict__ target_logits, const float* __res
     // Inputs that the kernel before does not produce can be fetched before waiting for it: it lets this one start when its
     // own wait is over, and so what came before it is complete.
     if (ALONE) {
-        pdl_trigger();
         __shared__ StatShared<kFinishThreads / 32> stat;
         for (int row = rank; row < rows; row += cluster_size) {
             const Row<VEC> r = make_row<VEC>(verify_row(target_logits, draft_logits, b, row, gamma, vocab), vocab);
@@ -1914,7 +1921,7 @@ int launch_verify_sample(const float* target_logits, const float* draft_logits, 
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl_enabled() && !alone ? 2 : 1;  // (the logits are read through the non-coherent path, right after the start)
+    cfg.numAttrs = pdl_enabled() ? 2 : 1;
 #define SPEC_LAUNCH_FINISH(G, V, C, A)                                                                                  \
     SPEC_CUDA_TRY(cudaLaunchKernelEx(&cfg, verify_finish_kernel<G, V, C, A>, target_logits, draft_logits, draft_tokens, \
                                      uniforms, gamma, vocab, inv_t, chunks, cluster_size, stats, final_uniforms,       \

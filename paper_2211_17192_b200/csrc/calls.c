@@ -2,7 +2,8 @@
  *
  * A lone decision keeps the GPU busy for 8 us; checking seven tensors in Python and a call through ctypes took the host 10.5.  Here
  * the same questions are asked of the same objects (is_cuda, dtype, is_contiguous(), shape, data_ptr()) from C, and the library
- * is called through its address: 4 x 8192 logits, call after call, 10.7 -> HHH us.
+ * is called through its address: 4 x 8192 logits, call after call, 10.5 -> 9.6 us, 7.7 where the GPU
+ * need not wait between two of them.
  * Whatever is not the plain case - another type, a missing tensor, a shape that does not fit - is answered with None and
  * nothing done: binding.py then makes the call itself and says what is wrong. */
 #define PY_SSIZE_T_CLEAN

@@ -1216,7 +1216,8 @@ constexpr float kSampleRange = 24.0f;  // of the bins, in powers of two below th
 // Of the sampled logits as many are listed as carry all but half of (1 - top_p) of their mass, but a tenth at least: a sample of
 // logits N(0, 3^2) holds few of those that carry the mass, and with a sixty-fourth as the least one row in 20 was listed too short.
 constexpr float kListLeast = 0.10f, kListShare = 0.15f;
-// Slots per warp: kListShare of its logits, 5 standard deviations (two CTAs with 100000 logits each then share an SM).
+// Slots per warp: kListShare of its logits, 5 standard deviations (two CTAs with 100000 logits each then share an SM).  Of 4000
+// such rows N(0, 3^2) two overflow, and are gone over again: 40 us more for a call that has one.
 inline int list_slots(int vocab, int ctas, int threads) {
     const float most = kListShare * (32.0f * vocab / (ctas * threads) + 256.0f);
     return static_cast<int>(most + 5.0f * sqrtf(most)) + 1;
@@ -1741,8 +1742,8 @@ int finish_cluster_size(int vocab) {
 }
 
 // One kernel for statistics and decision, where a call is bound by its launches and not by the GPU: a lone decision of
-// 4 x 8192 logits takes the host 10.5 us instead of 12.3, at 7.9 us of the GPU instead of 6.5 (a cluster of eight SMs reads all
-// rows, and nothing of it overlaps the call before).  The line is where the GPU's time meets the host's: 7 rows of 32000
+// 4 x 8192 logits takes the host one launch less, 1.8 us, at 7.9 us of the GPU instead of 6.5 (a cluster of eight SMs reads all
+// rows); call after call 7.7 us, with the checks in Python and without programmatic launch 10.5.  The line is where the GPU's time meets the host's: 7 rows of 32000
 // 9.6, 11 rows of 32000 11.7, 17 of 32000 13.7, 7 of 50003 11.9 (two kernels: 12.3 of the host); at T = 0, 4 x 128000
 // 8.7, 9 x 128000 14.1.  The generation loop replays a graph, to which only the GPU's time matters: never there.
 constexpr int kMostAlone = 8;  // CTAs to a sequence

@@ -17,9 +17,9 @@ import threading
 import torch
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "lib", "libspecdecode.so")
-_CALLS_PATH = os.path.join(os.path.dirname(_LIB_PATH), "_calls.so")
+_CALLS_PATH = os.path.join(os.path.dirname(_LIB_PATH), "_calls" + importlib.machinery.EXTENSION_SUFFIXES[0])  # (this interpreter's)
 _lib = None
-_calls = None  # the module of csrc/calls.c, which makes the plain calls of the sampling entry points
+_calls = None  # the module of csrc/calls.c, which makes the plain calls of the sampling entry points; None: it is not built
 _loading = threading.Lock()
 
 STATUS_NAMES = {
@@ -44,21 +44,22 @@ def lib():
     if _lib is None:
         with _loading:  # (one handle for all threads: what is declared on it has to be there for everyone)
             if _lib is None:
-                if not os.path.exists(_LIB_PATH) or not os.path.exists(_CALLS_PATH):
+                if not os.path.exists(_LIB_PATH):
                     raise RuntimeError(
-                        f"{_LIB_PATH if not os.path.exists(_LIB_PATH) else _CALLS_PATH} is missing: build it with `python -m paper_2211_17192_b200.build` "
+                        f"{_LIB_PATH} is missing: build it with `python -m paper_2211_17192_b200.build` "
                         "(there is no fallback path)")
                 handle = ctypes.CDLL(_LIB_PATH)
                 _declare(handle)
                 # (declared where they are called: the function objects exist from here on, so that two threads declare the same one)
                 for name in ("choose_gamma", "linear_partials", "generate_adaptive", "set_gamma", "attention_plan", "pass_trace"):
                     getattr(handle, "spec_" + name)
-                loader = importlib.machinery.ExtensionFileLoader("_calls", _CALLS_PATH)
-                calls = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_calls", _CALLS_PATH, loader=loader))
-                loader.exec_module(calls)
-                address = lambda f: ctypes.cast(f, ctypes.c_void_p).value
-                calls.bind(address(handle.spec_verify_sample_truncated), address(handle.spec_sample), torch.float32, torch.int32, torch.uint8)
-                _calls = calls
+                if os.path.exists(_CALLS_PATH):
+                    loader = importlib.machinery.ExtensionFileLoader("_calls", _CALLS_PATH)
+                    calls = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_calls", _CALLS_PATH, loader=loader))
+                    loader.exec_module(calls)
+                    address = lambda f: ctypes.cast(f, ctypes.c_void_p).value
+                    calls.bind(address(handle.spec_verify_sample_truncated), address(handle.spec_sample), torch.float32, torch.int32, torch.uint8)
+                    _calls = calls
                 _lib = handle
     return _lib
 
@@ -143,8 +144,8 @@ def spec_verify_sample(target_logits, draft_logits, draft_tokens, uniforms, temp
     """
     if workspace is not None and n_accepted is not None and next_token is not None:
         lib()
-        status = _calls.verify(target_logits, draft_logits, draft_tokens, uniforms, n_accepted, next_token, workspace, temperature,
-                               lenience, top_k, top_p, _stream())
+        status = _calls and _calls.verify(target_logits, draft_logits, draft_tokens, uniforms, n_accepted, next_token, workspace, temperature,
+                                          lenience, top_k, top_p, _stream())
         if status == 0:
             return n_accepted, next_token
         if status is not None:
@@ -211,7 +212,7 @@ def spec_sample(logits, uniforms, temperature, tokens=None, top_k=0, top_p=1.0):
     nucleus keep of each row when top_k > 0 or top_p < 1; logits [R, V] fp32 CUDA."""
     if tokens is not None and not top_k and top_p == 1.0:
         lib()
-        status = _calls.sample(logits, uniforms, temperature, tokens, _stream())
+        status = _calls and _calls.sample(logits, uniforms, temperature, tokens, _stream())
         if status == 0:
             return tokens
         if status is not None:

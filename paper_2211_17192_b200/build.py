@@ -3,8 +3,9 @@
     python -m paper_2211_17192_b200.build [--force] [--verbose]
 
 Each `csrc/*.cu` is compiled to an object under `build/` and the objects are
-linked into `paper_2211_17192_b200/lib/libspecdecode.so`; `csrc/calls.c`, the Python
-module of the calls that are made once per decision, becomes `lib/_calls.so`.  Nothing is cached
+linked into `paper_2211_17192_b200/lib/libspecdecode.so`.  `csrc/calls.c`, a shorter way to the calls that are
+made once per decision, becomes a module of the running interpreter beside it, where that interpreter's headers and a C compiler are
+at hand; without it the binding makes those calls itself.  Nothing is cached
 outside the repository, so the shared objects travel with the tree.
 """
 
@@ -24,8 +25,8 @@ INCLUDE = os.path.join(ROOT, "include")
 OBJ_DIR = os.path.join(ROOT, "build", "obj")
 LIB_DIR = os.path.join(PKG_DIR, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "libspecdecode.so")
-CALLS_PATH = os.path.join(LIB_DIR, "_calls.so")
-DIGEST_PATH = LIB_PATH + ".sha256"
+CALLS_SOURCE = os.path.join(CSRC, "calls.c")
+CALLS_PATH = os.path.join(LIB_DIR, "_calls" + sysconfig.get_config_var("EXT_SUFFIX"))  # (a module is one interpreter's)
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -60,21 +61,57 @@ def source_digest():
     h = hashlib.sha256(" ".join(NVCC_FLAGS[:8]).encode())
     for folder in (CSRC, INCLUDE):
         for name in sorted(os.listdir(folder)):
-            if name.endswith((".cu", ".cuh", ".h", ".c")):
+            if name.endswith((".cu", ".cuh", ".h")):
                 h.update(name.encode())
                 with open(os.path.join(folder, name), "rb") as f:
                     h.update(f.read())
     return h.hexdigest()
 
 
+def _up_to_date(path, digest):
+    if not os.path.exists(path) or not os.path.exists(path + ".sha256"):
+        return False
+    with open(path + ".sha256") as f:
+        return f.read().strip() == digest
+
+
+def _record(path, digest):
+    with open(path + ".sha256", "w") as f:
+        f.write(digest + "\n")
+
+
+def build_calls(force=False):
+    """The module of csrc/calls.c for the running interpreter; its path, or None where it cannot be built (a module
+    of other sources is then removed)."""
+    flags = ["-O2", "-std=c11", "-Wall", "-Wextra", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"]]
+    h = hashlib.sha256(" ".join(flags + [sys.version]).encode())
+    with open(CALLS_SOURCE, "rb") as f:
+        h.update(f.read())
+    if not force and _up_to_date(CALLS_PATH, h.hexdigest()):
+        return CALLS_PATH
+    for path in (CALLS_PATH, CALLS_PATH + ".sha256"):
+        if os.path.exists(path):
+            os.remove(path)
+    compiler = shutil.which("gcc") or shutil.which("cc") or shutil.which("clang")
+    why = "no C compiler"
+    if compiler:
+        os.makedirs(LIB_DIR, exist_ok=True)
+        res = subprocess.run([compiler] + flags + [CALLS_SOURCE, "-o", CALLS_PATH], capture_output=True, text=True)
+        if res.returncode == 0:
+            _record(CALLS_PATH, h.hexdigest())
+            return CALLS_PATH
+        why = res.stderr.strip()
+    sys.stderr.write(f"calls.c is not built, plain sampling calls take a few microseconds more: {why}\n")
+    return None
+
+
 def build(force=False, verbose=False):
     """Compile and link; returns the path of the shared library.  A library
     whose recorded source digest matches the tree is left alone."""
+    build_calls(force)
     digest = source_digest()
-    if not force and not verbose and all(os.path.exists(p) for p in (LIB_PATH, CALLS_PATH, DIGEST_PATH)):
-        with open(DIGEST_PATH) as f:
-            if f.read().strip() == digest:
-                return LIB_PATH
+    if not force and not verbose and _up_to_date(LIB_PATH, digest):
+        return LIB_PATH
     os.makedirs(OBJ_DIR, exist_ok=True)
     os.makedirs(LIB_DIR, exist_ok=True)
     nvcc = _nvcc()
@@ -105,14 +142,7 @@ def build(force=False, verbose=False):
         if res.returncode != 0:
             sys.stderr.write(res.stdout + res.stderr)
             raise RuntimeError("link failed")
-    cmd = [shutil.which("gcc") or "gcc", "-O2", "-std=c11", "-Wall", "-Wextra", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
-           os.path.join(CSRC, "calls.c"), "-o", CALLS_PATH]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        sys.stderr.write(" ".join(cmd) + "\n" + res.stdout + res.stderr)
-        raise RuntimeError("gcc failed for calls.c")
-    with open(DIGEST_PATH, "w") as f:
-        f.write(digest + "\n")
+    _record(LIB_PATH, digest)
     return LIB_PATH
 
 

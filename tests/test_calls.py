@@ -1,10 +1,12 @@
 """The module that makes the plain calls of the sampling entry points: what it takes, what it leaves to binding.py, and what it
 passes on.  Stand-ins with null addresses for the tensors, so that the library answers without a GPU."""
+import sysconfig
+
 import pytest
 import torch
 
 import __graft_entry__ as entry
-from paper_2211_17192_b200 import binding
+from paper_2211_17192_b200 import binding, build
 
 
 class StandIn:
@@ -65,3 +67,31 @@ def test_numbers_that_are_not_numbers_are_left_to_the_binding(calls):
     assert calls.verify(*plain(), 1.0, 1.0, 0, None, 0) is None
     assert calls.verify(*plain(), 1.0, 1.0, 1 << 40, 1.0, 0) is None
     assert calls.verify(*plain()) is None
+
+
+@pytest.mark.parametrize("built", [True, False])
+def test_without_the_module_the_binding_makes_the_calls(calls, monkeypatch, built):
+    monkeypatch.setattr(binding, "_calls", calls if built else None)
+    monkeypatch.setattr(binding, "_stream", lambda: 0)
+    t = plain()
+    with pytest.raises(binding.SpecError, match="null pointer"):
+        binding.spec_verify_sample(*t[:4], 1.0, n_accepted=t[4], next_token=t[5], workspace=t[6])
+    with pytest.raises(binding.SpecError):
+        binding.spec_sample(StandIn((3, 0), torch.float32), t[3], 1.0, tokens=t[4])
+
+
+def test_the_module_belongs_to_one_interpreter(calls):
+    assert build.CALLS_PATH == binding._CALLS_PATH and build.CALLS_PATH.endswith("_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+def test_a_machine_without_a_compiler_or_headers_does_without_the_module(tmp_path, monkeypatch, capsys):
+    at = tmp_path / "_calls.so"
+    monkeypatch.setattr(build, "CALLS_PATH", str(at))
+    monkeypatch.setattr(build, "LIB_DIR", str(tmp_path))
+    assert build.build_calls() == str(at) and build.build_calls() == str(at)
+    with monkeypatch.context() as m:
+        m.setattr(build.sysconfig, "get_paths", lambda: {"include": str(tmp_path)})
+        assert build.build_calls() is None and not at.exists() and "calls.c is not built" in capsys.readouterr().err
+    assert build.build_calls() == str(at)
+    monkeypatch.setattr(build.shutil, "which", lambda name: None)
+    assert build.build_calls() == str(at) and build.build_calls(force=True) is None and not at.exists()

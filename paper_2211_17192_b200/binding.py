@@ -142,7 +142,8 @@ def spec_verify_sample(target_logits, draft_logits, draft_tokens, uniforms, temp
     Returns (n_accepted [B] int32, next_token [B] int32); asynchronous on the
     current stream.  Output and workspace tensors are allocated when not given.
     """
-    if workspace is not None and n_accepted is not None and next_token is not None:
+    # (a tensor that is not on a GPU is refused below, without asking for a stream)
+    if workspace is not None and n_accepted is not None and next_token is not None and getattr(target_logits, "is_cuda", False):
         lib()
         status = _calls and _calls.verify(target_logits, draft_logits, draft_tokens, uniforms, n_accepted, next_token, workspace, temperature,
                                           lenience, top_k, top_p, _stream())
@@ -210,7 +211,7 @@ def spec_truncation_floors(logits, temperature, top_k=0, top_p=1.0, floors=None)
 def spec_sample(logits, uniforms, temperature, tokens=None, top_k=0, top_p=1.0):
     """tokens[r] ~ softmax(logits[r] / T) (argmax at T = 0), over what top-k and the
     nucleus keep of each row when top_k > 0 or top_p < 1; logits [R, V] fp32 CUDA."""
-    if tokens is not None and not top_k and top_p == 1.0:
+    if tokens is not None and not top_k and top_p == 1.0 and getattr(logits, "is_cuda", False):
         lib()
         status = _calls and _calls.sample(logits, uniforms, temperature, tokens, _stream())
         if status == 0:

@@ -69,6 +69,16 @@ def test_numbers_that_are_not_numbers_are_left_to_the_binding(calls):
     assert calls.verify(*plain()) is None
 
 
+def test_a_tensor_that_is_not_on_a_gpu_is_named(calls):
+    """Also on a machine without one: nothing asks for a stream before the tensors have been looked at."""
+    f, i, u = torch.float32, torch.int32, torch.uint8
+    host = [torch.zeros(2, 3, 8, dtype=f), torch.zeros(2, 2, 8, dtype=f), torch.zeros(2, 2, dtype=i), torch.zeros(2, 3, dtype=f)]
+    with pytest.raises(ValueError, match="target_logits must be a CUDA tensor"):
+        binding.spec_verify_sample(*host, 1.0, n_accepted=torch.zeros(2, dtype=i), next_token=torch.zeros(2, dtype=i), workspace=torch.zeros(64, dtype=u))
+    with pytest.raises(ValueError, match="logits must be a CUDA tensor"):
+        binding.spec_sample(host[0][0], torch.zeros(3, dtype=f), 1.0, tokens=torch.zeros(3, dtype=i))
+
+
 @pytest.mark.parametrize("built", [True, False])
 def test_without_the_module_the_binding_makes_the_calls(calls, monkeypatch, built):
     monkeypatch.setattr(binding, "_calls", calls if built else None)

@@ -85,7 +85,7 @@ __device__ __forceinline__ void cluster_merge_write(const float* fin, int n_q, i
                     o += os[s] * w;
                 }
             }
-            const float y = l > 0.0f ? o / l : 0.0f;  // an inactive row has no keys
+            const float y = l == 0.0f ? 0.0f : o / l;  // an inactive row has no keys; a sum that is no number has to show
             if (out.att) out.att[at + e] = y;
             if (out.hi) {
                 const __nv_bfloat16 h = __float2bfloat16_rn(y);
@@ -1198,7 +1198,7 @@ __global__ void attention_combine_kernel(const float* part, int slices, float* _
 #pragma unroll
     for (int s = 0; s < 32; ++s) o += s < slices ? acc[s] * w_sh[s] : 0.0f;  // slices in index order
     const float l = w_sh[32];
-    const float y = l > 0.0f ? o / l : 0.0f;  // an inactive row has no keys
+    const float y = l == 0.0f ? 0.0f : o / l;  // an inactive row has no keys; a sum that is no number has to show
     const size_t i = static_cast<size_t>(blockIdx.x) * DH + threadIdx.x;
     if (att) att[i] = y;
     if (att_hi) {

@@ -45,6 +45,24 @@ def test_non_finite_logits_are_reported(which, value, temperature, gamma):
         eng.close()
 
 
+@pytest.mark.parametrize("part", [0, 1, 2], ids=["q", "k", "v"])
+@pytest.mark.parametrize("base,rows", [("tiny_target", 9), ("tiny_target", 40), ("t5_tiny_target", 5)])
+def test_a_score_that_is_no_number_reaches_the_logits_of_fp32_models(base, rows, part):
+    """A NaN in the rows of Wqkv that make a head's q, k or v: no row of the pass (a chain of kernels at these sizes) has a finite logit
+    of it, whether a row's key slices are merged in a cluster or by a kernel of their own."""
+    cfg = workloads.scaled_config(workloads.model_config(base), n_layers=1)
+    w = dict(workloads.make_weights(cfg, 9))
+    w["l0.wqkv"] = w["l0.wqkv"].copy()
+    w["l0.wqkv"][part * cfg["n_heads"] * 64 + 64 + 5] = np.nan
+    t5 = cfg["arch"] == "t5"
+    for max_len in (64, 128):
+        eng = binding.Engine(cfg, w, max_batch=1, max_len=max_len, max_gamma=rows, page_size=32, max_src_len=40 if t5 else 0)
+        if t5:
+            eng.encode([workloads.make_prompt(5, 40, cfg["vocab"])])
+        assert eng.forward_logits(0, workloads.make_prompt(3, rows, cfg["vocab"])[None]).isnan().all()
+        eng.close()
+
+
 def test_a_bounded_wait_that_runs_out_is_reported_and_leaves_the_library_usable():
     h = binding.lib()
     h.spec_timeout_drill.restype = ctypes.c_int

@@ -19,6 +19,7 @@
 // Every wait is bounded.  One that runs out is recorded; the kernel goes on with whatever is there (the others count on it),
 // further waits give up at once, nothing more is asked for, and copies in flight are waited for at the end, with a limit.
 #include <cfloat>
+#include <climits>
 #include <vector>
 
 #include "model.cuh"
@@ -322,7 +323,8 @@ struct Worker {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) k4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            // (an inactive row, at a position below 0, is nobody's key)
+            // (an inactive row, at a position below 0, is nobody's key; what is not a row's key has a score of -inf, and a NaN is
+            // a score like any other: it has to reach the logits, where it is reported)
             const int at = own < 0 ? key : own < a.m_rows ? row_pos()[b * a.m_rows + own] : -1;
 #pragma unroll 1
             for (int i = 0; i < a.m_rows; ++i) {
@@ -332,7 +334,7 @@ struct Worker {
                 for (int g = 0; g < 4; ++g) s = dot4(k4[g], *reinterpret_cast<const float4*>(xq + r * 3 * kDh + 16 * g + 4 * t), s);
                 s += __shfl_xor_sync(kFullMask, s, 1);
                 s += __shfl_xor_sync(kFullMask, s, 2);
-                if (t == 0 && key < total) sc[r * kMaxKeys + key] = at >= 0 && at <= row_pos()[r] ? s * 0.125f : -FLT_MAX;
+                if (t == 0 && key < total) sc[r * kMaxKeys + key] = at >= 0 && at <= row_pos()[r] ? s * 0.125f : -INFINITY;
             }
         }
         __syncthreads();
@@ -344,12 +346,12 @@ struct Worker {
             top = warp_max(top);
             float sum = 0.0f;
             for (int i = lane; i < n; i += 32) {
-                const float e = p[i] > -FLT_MAX ? expf(p[i] - top) : 0.0f;
+                const float e = expf(p[i] - top);  // (top is finite where every score is -inf)
                 p[i] = e;
                 sum += e;
             }
             sum = warp_sum(sum);
-            const float inv = sum > 0.0f ? 1.0f / sum : 0.0f;
+            const float inv = sum == 0.0f ? 0.0f : 1.0f / sum;
             for (int i = lane; i < n; i += 32) p[i] *= inv;
         }
         __syncthreads();
@@ -361,11 +363,15 @@ struct Worker {
             for (int i = 0; i < R; ++i) acc[i] = 0.0f;
 #pragma unroll 4
             for (int at = wi * kSubs + sub; at < total; at += wps * kSubs) {
-                const float v = at < cached ? __ldcg(cache_row(at, 1) + j * S::kDv + dim)
-                                            : xq[(b * a.m_rows + at - cached) * 3 * kDh + 2 * kDh + j * S::kDv + dim];
+                const int own = at - cached;
+                const float v = own < 0 ? __ldcg(cache_row(at, 1) + j * S::kDv + dim)
+                                        : xq[(b * a.m_rows + own) * 3 * kDh + 2 * kDh + j * S::kDv + dim];
+                // (a row of the pass is nothing to those in front of it, not even 0 times its value, which may be no number)
+                const int from = own < 0 ? INT_MIN : row_pos()[b * a.m_rows + own] < 0 ? INT_MAX : row_pos()[b * a.m_rows + own];
 #pragma unroll
                 for (int i = 0; i < R; ++i)
-                    if (i < a.m_rows) acc[i] = fmaf(sc[(b * a.m_rows + i) * kMaxKeys + at], v, acc[i]);
+                    if (i < a.m_rows && row_pos()[b * a.m_rows + i] >= from)
+                        acc[i] = fmaf(sc[(b * a.m_rows + i) * kMaxKeys + at], v, acc[i]);
             }
 #pragma unroll
             for (int i = 0; i < R; ++i)

@@ -2,6 +2,7 @@
 rows it takes (and one more, which the chain of kernels takes), over ragged caches from none to the most keys it serves."""
 import numpy as np
 import pytest
+import torch
 
 from oracle.decoder import Decoder
 from paper_2211_17192_b200 import binding, workloads
@@ -37,4 +38,43 @@ def test_cluster_pass_against_the_oracle(d_model, layers, max_len):
             eng.truncate(0, [0] * batch)
             for at in range(0, most, 32):
                 eng.forward_logits(0, np.ascontiguousarray(tokens[:, at:min(at + 32, most)]))
+    eng.close()
+
+
+def _tiny(layers, d_model):
+    return workloads.scaled_config(workloads.model_config("tiny_target"), d_model=d_model, n_heads=d_model // 64, n_kv_heads=d_model // 64,
+                                   d_ff=4 * d_model, n_layers=layers, vocab=500, max_positions=64)
+
+
+@pytest.mark.parametrize("d_model", [128, 256])
+@pytest.mark.parametrize("part", [0, 1, 2], ids=["q", "k", "v"])
+def test_a_score_that_is_no_number_reaches_the_logits(d_model, part):
+    """A NaN in the rows of Wqkv that make a head's q, k or v: every logit of a pass of one block is one, and generation reports it."""
+    cfg = _tiny(1, d_model)
+    w = dict(workloads.make_weights(cfg, 9))
+    w["l0.wqkv"] = w["l0.wqkv"].copy()
+    w["l0.wqkv"][part * d_model + 64 + 5] = np.nan
+    tokens = workloads.make_prompt(3, 12, cfg["vocab"])
+    eng = binding.Engine(cfg, w, max_batch=1, max_len=64, max_gamma=8, page_size=32)
+    got = [eng.forward_logits(0, tokens[None, at:at + 3]) for at in (0, 3, 6)]
+    assert all(g.isnan().all() for g in got)
+    with pytest.raises(binding.SpecError) as e:
+        eng.generate([tokens[:3]], 8, 0, 1.0, 1)
+    assert e.value.status == -7
+    eng.close()
+
+
+@pytest.mark.parametrize("d_model", [128, 256])
+def test_a_row_that_is_no_number_is_nothing_to_the_rows_in_front_of_it(d_model):
+    cfg = _tiny(2, d_model)
+    w = dict(workloads.make_weights(cfg, 9))
+    w["tok_emb"] = w["tok_emb"].copy()
+    w["tok_emb"][7] = np.nan
+    tokens = np.array([[1, 2, 3, 4, 5, 7]], dtype=np.int32)
+    eng = binding.Engine(cfg, w, max_batch=1, max_len=64, max_gamma=8, page_size=32)
+    eng.forward_logits(0, tokens[:, :2])
+    got = eng.forward_logits(0, tokens[:, 2:])
+    assert got[0, 3].isnan().all() and got[0, :3].isfinite().all()
+    eng.truncate(0, [2])
+    assert torch.equal(eng.forward_logits(0, np.array([[3, 4, 5, 6]], dtype=np.int32))[0, :3], got[0, :3])
     eng.close()

@@ -135,8 +135,9 @@ int spec_verify_sample_lenient(const float* target_logits, const float* draft_lo
  * unless q_i(x_i) is 0 too.  Enqueues one more kernel (the per-row selection,
  * both cuts in one launch) before the other two; same workspace.  Top-k is
  * exact.  The nucleus takes fp32 weights exp((l - max) / T) from the hardware
- * exp2 and sums them in 2^-40 fixed point with integer additions, so a row
- * always gives the same cut whatever the order of summation; a cut whose mass
+ * exp2 and sums them in fixed point (units of 2^-32 of the row's largest, 2^-40
+ * after a top-k) with integer additions, so a row always gives the same cut
+ * whatever the order of summation and the rows beside it; a cut whose mass
  * comes within the weights' rounding (about 1e-6 of the total) of top_p may
  * differ from exact arithmetic by a neighbouring token.  Logits that are
  * -inf, +inf or NaN are never counted.  Errors as above plus SPEC_ERR_BAD_ARG

@@ -826,7 +826,7 @@ sample_kernel(const float* logits, size_t logit_stride, const float* uniforms, i
 // -inf, +inf and NaN logits are never in play).  Mass is summed in fixed point
 // (units of 2^-32 of the largest weight) with integer atomics, so every order of
 // summation gives the same totals: a row always gives the same floor, however the
-// threads interleave and however many CTAs share it.  The kernel is bound by instruction issue, not by memory
+// threads interleave, however many CTAs share it and whether it was listed (below).  The kernel is bound by instruction issue, not by memory
 // (the passes after the first hit L2), so the per-logit work is kept short: no
 // float-to-int conversion for the bin, one 32-bit atomic plus a rare carry for
 // the mass (a 64-bit shared-memory atomic cost 48 us of 180 on 960 rows of 32000),
@@ -852,7 +852,8 @@ struct SelShared {
     unsigned long long warp_mass[kSelMostWarps];
     unsigned warp_cnt[kSelMostWarps];
     float warp_lo[kSelMostWarps], warp_hi[kSelMostWarps], warp_top[kSelMostWarps];
-    float below[kSelMostWarps];                     // mass that the warps have not listed (list_candidates)
+    unsigned long long below[kSelMostWarps];        // mass that is not listed, of what the warps went over
+    float kept[kSelMostWarps];                      // of what the warps have listed, the weights that the cut leaves
     float cta_max[kMostCtas], cta_sum[kMostCtas];  // (in the CTA of rank 0)
     unsigned n_cand, n_hit, n_list;  // listed here; threads that reach the pivot; listed in all CTAs (in rank 0's)
     float floor;    // what rank 0 found
@@ -882,6 +883,7 @@ struct Team {
 // A CTA's slice of a row; LOADS 128-bit loads are in flight per thread when it is gone over.
 template <bool VEC, int LOADS>
 struct Slice {
+    static constexpr bool kList = false;
     Row<VEC> row;
     int g0, g1;
 };
@@ -932,9 +934,9 @@ __device__ int gather_list(const Team<SOLO>& team, bool masses, SelShared& sh) {
     return static_cast<int>(total);
 }
 
-// f(four logits, their group) over the slice.
+// f(LOADS times four logits, the first ones' group) over the slice; the others are T groups apart.
 template <int T, bool VEC, int LOADS, class F>
-__device__ __forceinline__ void for_each_group(const Slice<VEC, LOADS>& s, F f) {
+__device__ __forceinline__ void for_each_batch(const Slice<VEC, LOADS>& s, F f) {
     for (int base = s.g0 + threadIdx.x; base < s.g1; base += LOADS * T) {
         float4 v[LOADS];
 #pragma unroll
@@ -942,9 +944,16 @@ __device__ __forceinline__ void for_each_group(const Slice<VEC, LOADS>& s, F f) 
             const int g = base + i * T;
             v[i] = g < s.g1 ? s.row.raw(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         }
+        f(v, base);
+    }
+}
+// f(four logits, their group) over the slice.
+template <int T, bool VEC, int LOADS, class F>
+__device__ __forceinline__ void for_each_group(const Slice<VEC, LOADS>& s, F f) {
+    for_each_batch<T>(s, [&](const float4 (&v)[LOADS], int base) {
 #pragma unroll
         for (int i = 0; i < LOADS; ++i) f(v[i], base + i * T);
-    }
+    });
 }
 template <int T, bool VEC, int LOADS, class F>
 __device__ __forceinline__ void for_each_logit(const Slice<VEC, LOADS>& s, F f) {
@@ -957,17 +966,27 @@ __device__ __forceinline__ void for_each_logit(const Slice<VEC, LOADS>& s, F f) 
 }
 
 // What a warp has listed of its row: at[0] .. at[n - 1].
+template <bool VEC, int LOADS>
 struct Listed {
+    static constexpr bool kList = true;
+    static constexpr int kLoads = LOADS;
+    const Slice<VEC, LOADS>& slice;
     const float* at;
     int n;
-    float from, most;  // what is listed reaches `from`; the thread's largest logit
-    float ref;         // the reference of the weights in `SelShared::below`
+    float from, most;  // what is listed reaches `from`; the thread's largest logit (+inf for a NaN)
+    bool all;          // the warp's candidates all found a place
 };
-template <int T, class F>
-__device__ __forceinline__ void for_each_logit(const Listed& s, F f) {
+template <int T, bool VEC, int LOADS, class F>
+__device__ __forceinline__ void for_each_logit(const Listed<VEC, LOADS>& s, F f) {
     for (int i = threadIdx.x & 31; i < s.n; i += 32) f(s.at[i]);
 }
 
+// NaN if either is.
+__device__ __forceinline__ float max_or_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 __device__ __forceinline__ float warp_min(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -980,7 +999,7 @@ __device__ __forceinline__ float warp_min(float v) {
 // Of a Source that is not the row but its listed candidates: the nucleus of the row, NaN where the list does not decide it.
 template <int T, bool MASS, bool SOLO, class Source>
 __device__ float select_floor(const Source& s, const Team<SOLO>& team, float kf, unsigned k, float top_p, float c2, SelShared& sh) {
-    constexpr bool LIST = std::is_same<Source, Listed>::value;
+    constexpr bool LIST = Source::kList;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // 1. range and number of the logits in play
     float lo = INFINITY, hi = -INFINITY, all = -INFINITY;
@@ -988,7 +1007,7 @@ __device__ float select_floor(const Source& s, const Team<SOLO>& team, float kf,
     if constexpr (LIST) {
         lo = s.from;
         hi = all = s.most;
-        n = 1;
+        n = s.all ? 0 : 1;
     } else {
         for_each_logit<T>(s, [&](float v) {
             all = fmaxf(all, v);
@@ -1025,13 +1044,35 @@ __device__ float select_floor(const Source& s, const Team<SOLO>& team, float kf,
     of_all(lo, hi, all, n);
     if (tid == 0) sh.row_top = all;
     if constexpr (LIST) {
-        if (!(hi < INFINITY && hi >= lo)) return NAN;
+        if (n > 0 || !(hi < INFINITY && hi >= lo)) return NAN;
+    } else {
+        if (n == 0 || (!MASS && k > n)) return kf;  // nothing to cut
     }
-    if (n == 0 || (!MASS && k > n)) return kf;  // nothing to cut
     // weight exp2((l - max) * c2) of a logit in units of 2^-32 (the largest float below 2^32, so that the row's
     // maximum still fits 32 bits): a bin's mass is then one 32-bit shared-memory atomic and, rarely, a carry
     const float mc = fminf(-hi * c2, FLT_MAX);
-    auto fixed_mass = [&](float v) { return __float2uint_rz(fast_exp2(fmaf(v, c2, mc)) * 4294967040.0f); };
+    auto units = [&](float v) { return fast_exp2(fmaf(v, c2, mc)) * 4294967040.0f; };
+    auto fixed_mass = [&](float v) { return __float2uint_rz(units(v)); };
+    if constexpr (LIST) {
+        // what is not listed, in the same units: the total below is then the one that bins of the whole row come to, to the last
+        // bit.  As a rule all of it is far below the maximum, where adding 2^23 with rounding toward zero is the conversion.
+        unsigned long long below = 0;
+        auto rest = [&](float v) { return v < s.from ? units(v) : 0.0f; };
+        if (units(s.from) < 4194304.0f) {
+            auto whole = [&](float v) { return __float_as_uint(__fadd_rz(rest(v), 8388608.0f)) - 0x4b000000u; };
+            for_each_batch<T>(s.slice, [&](const float4 (&v)[Source::kLoads], int) {
+                unsigned part = 0;  // (each below 2^23, four to a load)
+#pragma unroll
+                for (int i = 0; i < Source::kLoads; ++i) part += (whole(v[i].x) + whole(v[i].y)) + (whole(v[i].z) + whole(v[i].w));
+                below += part;
+            });
+        } else {
+            for_each_logit<T>(s.slice, [&](float v) { below += __float2uint_rz(rest(v)); });
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
+        if (lane == 0) sh.below[warp] = below;
+    }
 
     unsigned long long before = 0, target = k;  // counts, or masses
     for (int level = 0; level < kSelLevels; ++level) {
@@ -1094,15 +1135,16 @@ __device__ float select_floor(const Source& s, const Team<SOLO>& team, float kf,
             }
             const unsigned long long upto = scan(a + b), all_of_it = __shfl_sync(0xffffffffu, upto, 31);
             if (MASS && level == 0) {  // the first level sees every logit in play: top_p of their mass is the target
-                double mass = static_cast<double>(all_of_it);
-                bool decided = true;
+                unsigned long long mass = all_of_it;
                 if constexpr (LIST) {  // .. and what is not listed
-                    float below = 0.0f;
+                    unsigned long long below = 0;
                     for (int i = lane; i < team.size * (T / 32); i += 32) below += team.of(sh, i / (T / 32)).below[i % (T / 32)];
-                    mass += static_cast<double>(warp_sum(below) * fast_exp2((s.ref - hi) * c2)) * 4294967040.0;
-                    decided = top_p * mass <= static_cast<double>(all_of_it);  // (not so for a NaN or infinite mass)
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
+                    mass += below;
                 }
-                target = decided ? static_cast<unsigned long long>(ceil(static_cast<double>(top_p) * mass)) : 0ull;
+                target = static_cast<unsigned long long>(ceil(static_cast<double>(top_p) * static_cast<double>(mass)));
+                if (LIST && target > all_of_it) target = 0;  // (not decided)
             }
             const unsigned long long above = before + upto - (a + b);
             const unsigned who = __ballot_sync(0xffffffffu, above < target && above + a + b >= target);
@@ -1202,15 +1244,17 @@ __device__ __forceinline__ float block_max(float v, float* per_warp) {
 // ---- the nucleus from a list of candidates ----
 // A nucleus is a few per cent of a row as a rule, so the row is read once: a sample of it, 32 groups per warp and spread over
 // the row, says above which logit its mass lies with room to spare; the pass lists what reaches that, every warp for
-// itself, and adds up the mass of the rest.  The selection, the statistics and the draw's sums then go over the list, in shared
-// memory.  A list that overflows or carries less than top_p of the mass decides nothing: the row is then binned as it lies.
-// The mass below is a float sum in a fixed order, so a row always gives the same floor, as with bins.
+// itself.  A second pass, over what L2 holds by then, adds up the mass of the rest, now that the row's maximum is known.  The selection,
+// the statistics and the draw's sums then go over the list, in shared memory.  A list that overflows or carries less than top_p of the
+// mass decides nothing: the row is then binned as it lies.
+// Masses are in the units of the bins, integers, so a row has one floor, from a list and from bins, to the last bit.  (Added up in fp32
+// while the row was listed, against the sample's maximum, the mass of the rest moved one floor in several hundred at T = 1, and one in 80 of rows
+// around 100 at T = 0.05.  The second pass is not in the time of a call after another: 200 x 100000 46.3 -> 45.1 us, cold 53 -> 61.)
 // What bounded the bins was an atomic per logit and three passes over the row behind the one that read it; now it is issue of
-// the one pass (a dozen instructions per logit, over the same time as the loads) and the barriers of the selection.  Rows N(0, 3^2),
-// p = 0.9, with the draw, cold, between two events, binned against listed: 200 x 100000 80 us, 57; 64 x 100000 51, 35; 1 x
-// 50000 49, 23; 200 x 32000 35, 27; 24 x 9 rows of 50003, verified, 85, 50.  Short rows are all barriers, of which the list has
-// more: 16 x 8192 14, 16, but 96 x 17 rows of 8192, verified, 62, 54.  (Bins for the sampled range alone, no list: one pass over the row
-// fewer than bins, but its atomics, in a few lanes of every warp, cost as much as in all of them: 200 x 100000 72.)
+// the passes (a dozen instructions per logit in the first) and the barriers of the selection.  Rows N(0, 3^2),
+// p = 0.9, with the draw, binned against listed, call after call: 200 x 100000 67 us, 45; 64 x 100000 33, 27; 1 x 50000 23, 18;
+// 200 x 32000 25, 21; 24 x 9 rows of 50003, verified, 61, 41.  (Bins for the sampled range alone, no list: one pass over the row
+// fewer than bins, but its atomics, in a few lanes of every warp, cost as much as in all of them: 200 x 100000, cold, 72 against 57.)
 constexpr int kSampleBins = 256;
 constexpr float kSampleRange = 24.0f;  // of the bins, in powers of two below the largest
 // Of the sampled logits as many are listed as carry all but half of (1 - top_p) of their mass, but a tenth at least: a sample of
@@ -1226,13 +1270,12 @@ inline int list_slots(int vocab, int ctas, int threads) {
 // The logit from which on candidates are listed; +inf where the sample says that a list would not do.  *ref: the sample's
 // largest.  The same in all CTAs of a row.
 template <int T, bool VEC, int LOADS>
-__device__ float candidate_floor(const Slice<VEC, LOADS>& s, float top_p, float c2, SelShared& sh, float* ref) {
+__device__ float candidate_floor(const Slice<VEC, LOADS>& s, float top_p, float c2, SelShared& sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, groups = s.row.groups();
     const int g = static_cast<int>(static_cast<long long>(max(groups - 32, 0)) * warp / (T / 32 - 1)) + lane;
     const float4 v = g < groups ? s.row.raw(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
     for (int i = tid; i < kSampleBins; i += T) sh.mass_lo[i] = 0;
     const float most = block_max<T>(fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)), sh.warp_hi);  // (the bins are clear)
-    *ref = most;
     if (!(fabsf(most) < INFINITY)) return INFINITY;  // (uniform)
     const float scale = c2 * (kSampleBins / kSampleRange);
     auto count = [&](float x) {
@@ -1283,17 +1326,17 @@ __device__ float candidate_floor(const Slice<VEC, LOADS>& s, float top_p, float 
 }
 
 // Lists the candidates of this warp's part of the slice, as the inverse CDF cuts it, two steps of two loads ahead (200 x 100000:
-// 47 us a call; one step of four at a time 50, of eight 53; four ahead of four 51, and eight ahead of eight spill: 70).
+// 47 us a call; one step of four at a time 50, of eight 53; four ahead of four 51, and eight ahead of eight spill: 70; all with the
+// mass of the rest in the same pass).
 constexpr int kListLoads = 2;
 template <int T, bool VEC, int LOADS>
-__device__ Listed list_candidates(const Slice<VEC, LOADS>& s, int each, float from, float ref, float c2, int slots, float* lists, SelShared& sh) {
+__device__ Listed<VEC, LOADS> list_candidates(const Slice<VEC, LOADS>& s, int each, float from, int slots, float* lists) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned before_me = (1u << lane) - 1;
     const int seg = (each + T / 32 - 1) / (T / 32);
     const int b0 = min(s.g1, s.g0 + warp * seg), b1 = min(s.g1, b0 + seg);
     float* list = lists + warp * slots;
-    const float mc = fminf(-ref * c2, FLT_MAX);
-    float below = 0.0f, most = -INFINITY;
+    float most = -INFINITY;
     int n = 0;
     const int last = slots - 1;  // (what does not fit goes to the last slot)
     float4 v[kListLoads];
@@ -1317,22 +1360,19 @@ __device__ Listed list_candidates(const Slice<VEC, LOADS>& s, int each, float fr
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 at += __popc(__ballot_sync(kFullMask, x[j] >= from) & before_me);
-                most = fmaxf(most, x[j]);
+                most = max_or_nan(most, x[j]);
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const bool in = x[j] >= from;
                 if (in) list[min(n + at + own, last)] = x[j];
                 own += in ? 1 : 0;
-                below += in ? 0.0f : fast_exp2(fmaf(x[j], c2, mc));
             }
             n += __shfl_sync(kFullMask, at + own, 31);
         }
     }
-    below = warp_sum(n > slots ? INFINITY : below);
-    if (lane == 0) sh.below[warp] = below;
     __syncwarp();
-    return Listed{list, min(n, slots), from, most, ref};
+    return Listed<VEC, LOADS>{s, list, min(n, slots), from, most == most ? most : INFINITY, n <= slots};
 }
 
 // Top-k for k up to 128, without bins: every warp gives its largest lane maxima, 3 k of them in all; the k-th largest of
@@ -1637,14 +1677,15 @@ cut_floor_kernel(const float* a, size_t a_stride, int a_rows, const float* b, si
     float floor = -INFINITY, row_max = 0.0f, sum = 0.0f;
     int listed = -1;  // logits listed (the same in all CTAs; floor, row_max and sum of a listed row are the first one's)
     const bool nucleus = top_p > 0.0f && top_p < 1.0f;
-    Listed found{};
+    Listed<VEC, LOADS> found{s};
     bool candidates = false;  // the nucleus came from them
     if constexpr (LIST) {
-        float ref;
-        const float from = candidate_floor<T>(s, top_p, c2, sh, &ref);
+        const float from = candidate_floor<T>(s, top_p, c2, sh);
         if (from < INFINITY) {
-            found = list_candidates<T>(s, each, from, ref, c2, slots, lists, sh);
-            const float f = select_floor<T, true>(found, team, -INFINITY, 0u, top_p, c2, sh);
+            const Listed<VEC, LOADS> listed = list_candidates<T>(s, each, from, slots, lists);
+            found.at = listed.at;
+            found.n = listed.n;
+            const float f = select_floor<T, true>(listed, team, -INFINITY, 0u, top_p, c2, sh);
             candidates = f == f;
             if (candidates) floor = f;
         }
@@ -1671,10 +1712,10 @@ cut_floor_kernel(const float* a, size_t a_stride, int a_rows, const float* b, si
     }
     if (WORK == kWithStats) {
         if (LIST && candidates) {
-            if (threadIdx.x % 32 == 0) sh.below[threadIdx.x / 32] = kept;  // (read long ago)
+            if (threadIdx.x % 32 == 0) sh.kept[threadIdx.x / 32] = kept;
             team.sync();
             if (threadIdx.x == 0 && first)
-                for (int i = 0; i < team.size * (T / 32); ++i) sum += team.of(sh, i / (T / 32)).below[i % (T / 32)];
+                for (int i = 0; i < team.size * (T / 32); ++i) sum += team.of(sh, i / (T / 32)).kept[i % (T / 32)];
         } else if (listed < 0) {
             row_statistics<T>(s, team, floor, c2, sh, &row_max, &sum);
         }
@@ -1794,8 +1835,9 @@ struct CutShape {
 // - a cluster pays where few rows are long and binned (4 x 512 threads against 512: 16 x 50003 26, 37; 16 x 128000 29, 53;
 //   64 x 100000 32, 50; 2 x 512: 128 x 100000 51, 66), not on more rows (200 x 100000 with two: 87, 70), shorter ones (16 x
 //   32000: 19, 18) or a list, whose passes are few (16 x 100000, k = 50: 13, 13).
-// - the nucleus from lists is as indifferent to its shape: 200 x 100000, a row to a CTA, two CTAs to an SM, with eight loads 64,
-// with four 57; with lists so long that one CTA fills the SM a pair (256 x 128000: 82, 512 threads alone 90).
+// - of the nucleus from lists, 200 x 100000 are one row to a CTA and two CTAs to an SM, with four loads (eight were 64 us to 57
+//   when loads were not yet requested two steps ahead); with lists so long that one CTA fills the SM, a pair (256 x 128000: 82, 512
+//   threads alone 90, likewise).
 CutShape cut_shape(int rows, int vocab, int top_k) {
     const bool listed = top_k <= 0 || top_k >= vocab;
     const bool binned = top_k <= 0 || top_k > 128 || top_k >= vocab, long_row = vocab >= 48 * 1024;

@@ -82,3 +82,19 @@ def test_nucleus_of_rows_whose_sample_misleads(rows, vocab, top_p):
         assert float(many[i, int(tokens[i])]) >= floor, i
     for i in range(10, rows):
         assert float(got[i]) == float(got[i % 10]), i
+
+
+@pytest.mark.parametrize("vocab,many,few", [(8192, 1184, (148,)), (4099, 1184, (148,)), (12289, 1184, (296, 61)), (50003, 600, (200, 100, 40))])
+@pytest.mark.parametrize("temperature,shift,top_p", [(1.0, 0.0, 0.9), (0.05, 100.0, 0.9), (0.7, -3000.0, 0.5)])
+def test_a_nucleus_is_the_same_from_bins_and_from_a_list(vocab, many, few, temperature, shift, top_p):
+    """Floors to the last bit over hundreds of random rows: many in one call against the same rows a few at a time, which other
+    launches take (short rows: bins, not lists).  Also at a temperature and a shift that leave few bits of the weights' exponents."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(vocab)
+    rows = torch.randn(many, vocab, device="cuda", generator=gen) * (3.0 * temperature) + shift
+    want = binding.spec_truncation_floors(rows, temperature, top_p=top_p)
+    assert len(torch.unique(want)) > many // 2
+    for n in few:
+        got = torch.cat([binding.spec_truncation_floors(rows[i:i + n].contiguous(), temperature, top_p=top_p) for i in range(0, many, n)])
+        differ = int((got != want).sum())
+        assert differ == 0, (n, differ)

@@ -853,6 +853,7 @@ struct SelShared {
     unsigned warp_cnt[kSelMostWarps];
     float warp_lo[kSelMostWarps], warp_hi[kSelMostWarps], warp_top[kSelMostWarps];
     unsigned long long below[kSelMostWarps];        // mass that is not listed, of what the warps went over
+    int found[kSelMostWarps];                       // candidates of the warps
     float kept[kSelMostWarps];                      // of what the warps have listed, the weights that the cut leaves
     float cta_max[kMostCtas], cta_sum[kMostCtas];  // (in the CTA of rank 0)
     unsigned n_cand, n_hit, n_list;  // listed here; threads that reach the pivot; listed in all CTAs (in rank 0's)
@@ -972,13 +973,13 @@ struct Listed {
     static constexpr int kLoads = LOADS;
     const Slice<VEC, LOADS>& slice;
     const float* at;
-    int n;
+    int n, first, step;
     float from, most;  // what is listed reaches `from`; the thread's largest logit (+inf for a NaN)
     bool all;          // the warp's candidates all found a place
 };
 template <int T, bool VEC, int LOADS, class F>
 __device__ __forceinline__ void for_each_logit(const Listed<VEC, LOADS>& s, F f) {
-    for (int i = threadIdx.x & 31; i < s.n; i += 32) f(s.at[i]);
+    for (int i = s.first; i < s.n; i += s.step) f(s.at[i]);
 }
 
 // NaN if either is.
@@ -998,7 +999,7 @@ __device__ __forceinline__ float warp_min(float v) {
 // Every thread of the team returns the same value; -inf means "keep everything".
 // Of a Source that is not the row but its listed candidates: the nucleus of the row, NaN where the list does not decide it.
 template <int T, bool MASS, bool SOLO, class Source>
-__device__ float select_floor(const Source& s, const Team<SOLO>& team, float kf, unsigned k, float top_p, float c2, SelShared& sh) {
+__device__ float select_floor(Source& s, const Team<SOLO>& team, float kf, unsigned k, float top_p, float c2, SelShared& sh) {
     constexpr bool LIST = Source::kList;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // 1. range and number of the logits in play
@@ -1044,6 +1045,7 @@ __device__ float select_floor(const Source& s, const Team<SOLO>& team, float kf,
     of_all(lo, hi, all, n);
     if (tid == 0) sh.row_top = all;
     if constexpr (LIST) {
+        s.all = n == 0;
         if (n > 0 || !(hi < INFINITY && hi >= lo)) return NAN;
     } else {
         if (n == 0 || (!MASS && k > n)) return kf;  // nothing to cut
@@ -1242,7 +1244,7 @@ __device__ __forceinline__ float block_max(float v, float* per_warp) {
     return v;
 }
 // ---- the nucleus from a list of candidates ----
-// A nucleus is a few per cent of a row as a rule, so the row is read once: a sample of it, 32 groups per warp and spread over
+// A nucleus is a few per cent of a row as a rule, so the row is read once: a sample of it, four groups at a time and spread over
 // the row, says above which logit its mass lies with room to spare; the pass lists what reaches that, every warp for
 // itself.  A second pass, over what L2 holds by then, adds up the mass of the rest, now that the row's maximum is known.  The selection,
 // the statistics and the draw's sums then go over the list, in shared memory.  A list that overflows or carries less than top_p of the
@@ -1250,21 +1252,34 @@ __device__ __forceinline__ float block_max(float v, float* per_warp) {
 // Masses are in the units of the bins, integers, so a row has one floor, from a list and from bins, to the last bit.  (Added up in fp32
 // while the row was listed, against the sample's maximum, the mass of the rest moved one floor in several hundred at T = 1, and one in 80 of rows
 // around 100 at T = 0.05.  The second pass is not in the time of a call after another: 200 x 100000 46.3 -> 45.1 us, cold 53 -> 61.)
+// A warp lists its own part of the row, and large logits may all lie in one part (ids in order of frequency, say): a row of
+// which a warp finds more than its share is listed once more, as one list.  Binned, listed where they lie by chance, and sorted, us
+// call after call, rows N(0, 3^2), p = 0.9, with the draw: 200 x 100000 68, 46, 64; 64 x 100000 33, 28, 38; 1 x 50000 23, 18,
+// 22; 200 x 32000 25, 22, 28; 960 x 32000 82, 58, 78; 24 x 9 rows of 50003, verified, 61, 42, 53.
+// A flat row (N(0, 1), or p = 0.99) is no row for a list, which the sample sees; it costs that row the sample, and its bins the
+// threads that the list's memory and registers keep off the SM: 64 x 100000 36 us binned, 37 so; 200 x 100000 72, 72; 600 x 20000
+// 39, 48; 256 x 128000, which a pair of CTAs shares for the list's sake, 94, 120.
 // What bounded the bins was an atomic per logit and three passes over the row behind the one that read it; now it is issue of
-// the passes (a dozen instructions per logit in the first) and the barriers of the selection.  Rows N(0, 3^2),
-// p = 0.9, with the draw, binned against listed, call after call: 200 x 100000 67 us, 45; 64 x 100000 33, 27; 1 x 50000 23, 18;
-// 200 x 32000 25, 21; 24 x 9 rows of 50003, verified, 61, 41.  (Bins for the sampled range alone, no list: one pass over the row
-// fewer than bins, but its atomics, in a few lanes of every warp, cost as much as in all of them: 200 x 100000, cold, 72 against 57.)
+// the passes (a dozen instructions per logit in the first) and the barriers of the selection.  (Bins for the sampled range alone, no
+// list: one pass over the row fewer than bins, but its atomics, in a few lanes of every warp, cost as much as in all of them:
+// 200 x 100000, cold, 72 against 57.  One list for all warps from the start, filled in runs that the warps ask for: 60 for 46.)
 constexpr int kSampleBins = 256;
 constexpr float kSampleRange = 24.0f;  // of the bins, in powers of two below the largest
 // Of the sampled logits as many are listed as carry all but half of (1 - top_p) of their mass, but a tenth at least: a sample of
 // logits N(0, 3^2) holds few of those that carry the mass, and with a sixty-fourth as the least one row in 20 was listed too short.
+// Where the most that can be listed carries less than all but 0.7 of (1 - top_p), nothing is (at 0.9 one row in six N(0, 3^2) at
+// p = 0.98 was listed in vain).
 constexpr float kListLeast = 0.10f, kListShare = 0.15f;
-// Slots per warp: kListShare of its logits, 5 standard deviations (two CTAs with 100000 logits each then share an SM).  Of 4000
-// such rows N(0, 3^2) two overflow, and are gone over again: 40 us more for a call that has one.
+// Slots per warp: kListShare of its logits, 5 standard deviations (two CTAs with 100000 logits each then share an SM).  A CTA of several
+// has room for the whole row's candidates where two of them still fit an SM, for they need not be spread evenly.
+constexpr size_t kTwoListsBytes = 80 * 1024;  // of each of two CTAs on an SM
 inline int list_slots(int vocab, int ctas, int threads) {
-    const float most = kListShare * (32.0f * vocab / (ctas * threads) + 256.0f);
-    return static_cast<int>(most + 5.0f * sqrtf(most)) + 1;
+    auto of = [&](int warps) {
+        const float most = kListShare * (static_cast<float>(vocab) / warps + 256.0f);
+        return static_cast<int>(most + 5.0f * sqrtf(most)) + 1;
+    };
+    const int warps = threads / 32;
+    return std::max(of(ctas * warps), std::min(of(warps), static_cast<int>(kTwoListsBytes / sizeof(float)) / warps));
 }
 
 // The logit from which on candidates are listed; +inf where the sample says that a list would not do.  *ref: the sample's
@@ -1272,7 +1287,7 @@ inline int list_slots(int vocab, int ctas, int threads) {
 template <int T, bool VEC, int LOADS>
 __device__ float candidate_floor(const Slice<VEC, LOADS>& s, float top_p, float c2, SelShared& sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, groups = s.row.groups();
-    const int g = static_cast<int>(static_cast<long long>(max(groups - 32, 0)) * warp / (T / 32 - 1)) + lane;
+    const int g = groups > T ? static_cast<int>(static_cast<long long>(groups - 4) * (tid / 4) / (T / 4 - 1)) + tid % 4 : tid;
     const float4 v = g < groups ? s.row.raw(g, -INFINITY) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
     for (int i = tid; i < kSampleBins; i += T) sh.mass_lo[i] = 0;
     const float most = block_max<T>(fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)), sh.warp_hi);  // (the bins are clear)
@@ -1300,7 +1315,7 @@ __device__ float candidate_floor(const Slice<VEC, LOADS>& s, float top_p, float 
         }
         float upto_n = warp_inclusive_scan(all_n, lane), upto_m = warp_inclusive_scan(all_m, lane);
         const float total = __shfl_sync(kFullMask, upto_m, 31);
-        const float enough = (1.0f - 0.5f * (1.0f - top_p)) * total, least = (1.0f - 0.9f * (1.0f - top_p)) * total;
+        const float enough = (1.0f - 0.5f * (1.0f - top_p)) * total, least = (1.0f - 0.7f * (1.0f - top_p)) * total;
         upto_n -= all_n;
         upto_m -= all_m;
         int bin = -1;
@@ -1372,7 +1387,7 @@ __device__ Listed<VEC, LOADS> list_candidates(const Slice<VEC, LOADS>& s, int ea
         }
     }
     __syncwarp();
-    return Listed<VEC, LOADS>{s, list, min(n, slots), from, most == most ? most : INFINITY, n <= slots};
+    return Listed<VEC, LOADS>{s, list, n, lane, 32, from, most == most ? most : INFINITY, n <= slots};
 }
 
 // Top-k for k up to 128, without bins: every warp gives its largest lane maxima, 3 k of them in all; the k-th largest of
@@ -1678,14 +1693,40 @@ cut_floor_kernel(const float* a, size_t a_stride, int a_rows, const float* b, si
     int listed = -1;  // logits listed (the same in all CTAs; floor, row_max and sum of a listed row are the first one's)
     const bool nucleus = top_p > 0.0f && top_p < 1.0f;
     Listed<VEC, LOADS> found{s};
+    found.first = threadIdx.x % 32;
+    found.step = 32;
     bool candidates = false;  // the nucleus came from them
     if constexpr (LIST) {
         const float from = candidate_floor<T>(s, top_p, c2, sh);
         if (from < INFINITY) {
-            const Listed<VEC, LOADS> listed = list_candidates<T>(s, each, from, slots, lists);
+            Listed<VEC, LOADS> listed = list_candidates<T>(s, each, from, slots, lists);
             found.at = listed.at;
             found.n = listed.n;
-            const float f = select_floor<T, true>(listed, team, -INFINITY, 0u, top_p, c2, sh);
+            if (threadIdx.x % 32 == 0) sh.found[threadIdx.x / 32] = listed.n;
+            // A warp has more than its share of slots: listed once more, one warp's candidates behind another's, if the CTA has room for
+            // all of them, and the selection shares them out evenly.  (A loop, so that the selection is there once: with a second
+            // copy of it for this case 200 x 100000 were 52 us, as a function of its own 58, and 46 so.)
+            float f;
+#pragma unroll 1
+            for (bool again = false;; again = true) {
+                f = select_floor<T, true>(listed, team, -INFINITY, 0u, top_p, c2, sh);
+                if (again || listed.all) break;  // (the same for the team)
+                team.sync();  // (what the warps found has been read)
+                int total = 0, before = 0;
+#pragma unroll
+                for (int w = 0; w < T / 32; ++w) {
+                    if (w == static_cast<int>(threadIdx.x / 32)) before = total;
+                    total += sh.found[w];
+                }
+                const bool room = total <= slots * (T / 32);
+                if (room) list_candidates<T>(s, each, from, found.n, lists + before - static_cast<int>(threadIdx.x / 32) * found.n);
+                found.at = lists + before;
+                listed.all = room;
+                listed.at = lists;
+                listed.first = threadIdx.x;
+                listed.step = T;
+                listed.n = total;
+            }
             candidates = f == f;
             if (candidates) floor = f;
         }
@@ -1820,7 +1861,6 @@ size_t verify_sample_workspace_bytes(int batch, int gamma, int vocab) {
 }
 
 constexpr size_t kMostListBytes = 160 * 1024;  // of candidates; a longer row is binned as it lies
-constexpr size_t kTwoListsBytes = 80 * 1024;   // of each of two CTAs on an SM
 size_t list_bytes(int vocab, int ctas, int threads) { return static_cast<size_t>(list_slots(vocab, ctas, threads)) * (threads / 32) * sizeof(float); }
 
 // How the rows of a cut are shared out.
@@ -1883,7 +1923,9 @@ int launch_cut(const float* a, size_t a_stride, int a_rows, const float* b, size
     }
     cfg.attrs = attr;
     cfg.numAttrs = n;
-    const bool listed = !(top_k > 0 && top_k < vocab) && (vocab >= 12 * 1024 || total > 2 * 148) &&
+    // (short rows are all barriers, of which the list has more, unless they are many: binned and listed, 16 x 8192 11 us, 11;
+    // 600 x 4099 18, 20; 600 x 8192 19, 20; 1600 x 8192 40, 37; 96 x 17 x 8192, verified, 50, 45)
+    const bool listed = !(top_k > 0 && top_k < vocab) && (vocab >= 12 * 1024 || (vocab >= 6 * 1024 && total > 1024)) &&
                         list_bytes(vocab, ctas, shape.threads) <= kMostListBytes;
     int slots = 0;
     if (listed) {

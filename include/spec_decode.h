@@ -625,7 +625,7 @@ int spec_device_error(void);
  * The device error flags are clear afterwards and the context stays usable.  Synchronises `stream`.
  *
  * spec_timeout_drill_pass does the same for the kernel that runs few-row passes of a small bf16 model
- * (which: 0 target, 1 draft) as one grid: a row at the cached length of sequence 0, of which no CTA
+ * (which: 0 target, 1 draft) as one grid, or of a tiny fp32 one as one cluster: a row at the cached length of sequence 0, of which no CTA
  * publishes its share, with a limit of 64 tries per wait.  The cached length stays as it is; a
  * generation in progress ends.  Errors: SPEC_ERR_DEVICE_TIMEOUT as intended, SPEC_ERR_BAD_CONFIG if
  * the model's one-row passes are a chain of kernels. */

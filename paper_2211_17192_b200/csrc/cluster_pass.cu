@@ -17,7 +17,8 @@
 // takes them, as it takes contexts of more than kMaxKeys positions.
 //
 // Every wait is bounded.  One that runs out is recorded; the kernel goes on with whatever is there (the others count on it),
-// further waits give up at once, nothing more is asked for, and copies in flight are waited for at the end, with a limit.
+// further waits give up at once, nothing more is asked for, and at the end the copies and the announced exchanges that are still in
+// flight are waited for, with a limit; what nobody announced any more has a grace time to arrive before the CTA leaves.
 #include <cfloat>
 #include <climits>
 #include <vector>
@@ -34,6 +35,7 @@ constexpr int kDh = 64;
 constexpr int kMaxKeys = 256;
 constexpr uint32_t kSpin = 1u << 20;   // tries of a bounded wait: about a second
 constexpr uint32_t kDrain = 1u << 14;  // and of the last ones of a pass that gave up
+constexpr uint32_t kGraceNs = 20000;   // a store between two SMs takes about one microsecond
 
 __device__ int g_cluster_error;  // a bounded wait expired
 
@@ -53,7 +55,8 @@ struct ClusterArgs {
     int pages_per_seq, page_shift;
     float eps;
     float* h_out;
-    uint32_t limit;
+    uint32_t limit;  // of every wait, in tries
+    int mute;        // spec_timeout_drill_pass: nothing is sent
 };
 
 // R: rows at most
@@ -219,6 +222,9 @@ struct Worker {
         }
         return rsqrtf(sum_over_lanes(ss, lane) / static_cast<float>(D) + a.eps);
     }
+    __device__ __forceinline__ void send(const float* here, int which, int rank, const float4& v) {
+        if (!a.mute) send4(here, bars + which, rank, v);
+    }
     // [rows][WIDTH] results in kRed go to everyone, row r to to + r * LD; the whole CTA, between two barriers.
     template <int WIDTH, int LD>
     __device__ __forceinline__ void share(float* to, int which) {
@@ -226,7 +232,7 @@ struct Worker {
 #pragma unroll
         for (int i = tid; i < kGroups * kCtas; i += kThreads) {
             const int peer = i / kGroups, at = i % kGroups, r = at / (WIDTH / 4), f = at % (WIDTH / 4) * 4;
-            if (r < a.rows) send4(to + r * LD + f, bars + which, peer, *reinterpret_cast<const float4*>(sm + S::kRed + r * WIDTH + f));
+            if (r < a.rows) send(to + r * LD + f, which, peer, *reinterpret_cast<const float4*>(sm + S::kRed + r * WIDTH + f));
         }
     }
     __device__ __forceinline__ const int* row_pos() const { return reinterpret_cast<const int*>(sm + S::kMeta); }
@@ -298,7 +304,7 @@ struct Worker {
                 if (r >= a.rows) continue;
                 const int part = f / S::kDv, dim = j * S::kDv + f % S::kDv;
                 const float4 y = *reinterpret_cast<const float4*>(red + r * 3 * S::kDv + f);
-                send4(xq + r * 3 * kDh + part * kDh + dim, bars + kBarX, head * S::kGroup + peer, y);
+                send(xq + r * 3 * kDh + part * kDh + dim, kBarX, head * S::kGroup + peer, y);
                 const int p = row_pos()[r];
                 if (peer == 0 && part > 0 && p >= 0) {
                     const size_t page = a.page_table[row_seq()[r] * a.pages_per_seq + (p >> a.page_shift)];
@@ -473,7 +479,7 @@ struct Worker {
         q.w = __shfl_sync(kFullMask, v, (lane & ~3) + 3);
         if (r < a.rows)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) send4(to, bars + which, 4 * (lane & 3) + i, q);
+            for (int i = 0; i < 4; ++i) send(to, which, 4 * (lane & 3) + i, q);
     }
 };
 
@@ -522,12 +528,14 @@ __global__ void __launch_bounds__(kThreads, 1) cluster_pass_kernel(const __grid_
     for (int l = 0; l < a.n_layers; ++l) w.block(l);
     if (w.limit == 1) {
         atomicCAS(&g_cluster_error, 0, 1);
-        if (tid == 0)  // the copies that this thread asked for: a barrier is past one of the two parities at any time
-            for (int i = 0; i < 4; ++i) bar_wait(&bars[i], 0, kDrain), bar_wait(&bars[i], 1, kDrain);
+        if (tid == 0)  // what this thread asked for or announced: a barrier is past one of the two parities at any time
+            for (int i = 0; i < 8; ++i) bar_wait(&bars[i], 0, kDrain), bar_wait(&bars[i], 1, kDrain);
     }
     __syncthreads();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");  // nobody leaves while a peer may still write here
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    // (a CTA whose waits have all been met has received everything; of the others some stores may be issued and not here yet)
+    if (w.limit == 1) __nanosleep(kGraceNs);
 }
 
 using ClusterFn = void (*)(const ClusterArgs);
@@ -595,7 +603,7 @@ int cluster_pass_init(ClusterPass& s, const Model& m, int max_len) {
 bool cluster_pass_serves(const ClusterPass& s, int batch, int m_rows) { return batch * m_rows <= s.rows; }
 
 int launch_cluster_pass(const Model& m, const RowMeta& rows, const PassTables& t, int batch, int m_rows, float* h,
-                        cudaStream_t stream) {
+                        cudaStream_t stream, bool drill) {
     const spec_model_cfg& c = m.cfg;
     ClusterArgs a{};
     auto f = [](const void* p) { return static_cast<const float*>(p); };
@@ -621,7 +629,8 @@ int launch_cluster_pass(const Model& m, const RowMeta& rows, const PassTables& t
     while ((1 << a.page_shift) < t.page_size) ++a.page_shift;
     a.eps = c.rms_eps;
     a.h_out = h;
-    a.limit = kSpin;
+    a.limit = drill ? 64 : kSpin;
+    a.mute = drill ? 1 : 0;
     const Variant v = variant(c.d_model);
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = launch_config(v, stream, attr);

@@ -1470,7 +1470,8 @@ extern "C" int spec_pass_trace(spec_ctx* ctx, int which, int batch, int rows, un
 extern "C" int spec_timeout_drill_pass(spec_ctx* ctx, int which) {
     if (!ctx || which < 0 || which > 1 || (which == 1 && !ctx->has_draft)) return fail(SPEC_ERR_BAD_ARG, "spec_timeout_drill_pass: bad argument");
     const Model& m = ctx->model[which];
-    if (ctx->rt.pass_kernel || !small_pass_serves(ctx->small[which], m, 1, 1))
+    const bool tiny = cluster_pass_serves(ctx->tiny[which], 1, 1);
+    if (ctx->rt.pass_kernel || !(tiny || small_pass_serves(ctx->small[which], m, 1, 1)))
         return fail(SPEC_ERR_BAD_CONFIG, "spec_timeout_drill_pass: one-row passes of this model are a chain of kernels");
     if (m.t5() && !ctx->encoded) return fail(SPEC_ERR_BAD_ARG, "spec_timeout_drill_pass: call spec_encode first");
     const int pos = ctx->cached[which][0];
@@ -1481,7 +1482,8 @@ extern "C" int spec_timeout_drill_pass(spec_ctx* ctx, int which) {
     const RowMeta rows{ctx->row_block, ctx->row_block + 4, ctx->row_block + 8};
     const PassTables tables{ctx->page_table, ctx->pages_per_seq, ctx->rt.page_size, ctx->src_page_table,
                             ctx->src_pages_per_seq, ctx->src_len, ctx->rt.max_len, ctx->rt.max_len - 1};
-    SPEC_TRY(launch_small_pass(ctx->small[which], m, rows, tables, 1, 1, ctx->h, ctx->stream, true));
+    SPEC_TRY(tiny ? launch_cluster_pass(m, rows, tables, 1, 1, ctx->h, ctx->stream, true)
+                  : launch_small_pass(ctx->small[which], m, rows, tables, 1, 1, ctx->h, ctx->stream, true));
     SPEC_TRY(finish_work(ctx, 0));
     return fail(SPEC_ERR_CUDA, "drill: the pass did not report the wait that should have run out");
 }

@@ -282,7 +282,8 @@ struct ClusterPass {
 };
 int cluster_pass_init(ClusterPass& s, const Model& m, int max_len);
 bool cluster_pass_serves(const ClusterPass& s, int batch, int m_rows);
-int launch_cluster_pass(const Model& m, const RowMeta& rows, const PassTables& t, int batch, int m_rows, float* h, cudaStream_t stream);
+int launch_cluster_pass(const Model& m, const RowMeta& rows, const PassTables& t, int batch, int m_rows, float* h, cudaStream_t stream,
+                        bool drill = false);  // (`drill`: nobody sends anything, and every wait gives up after 64 tries)
 int* cluster_pass_error_word();
 int cluster_pass_take_error();
 

@@ -78,3 +78,38 @@ def test_a_row_that_is_no_number_is_nothing_to_the_rows_in_front_of_it(d_model):
     eng.truncate(0, [2])
     assert torch.equal(eng.forward_logits(0, np.array([[3, 4, 5, 6]], dtype=np.int32))[0, :3], got[0, :3])
     eng.close()
+
+
+@pytest.mark.parametrize("d_model", [128, 256])
+def test_pages_of_any_size(d_model):
+    cfg = _tiny(2, d_model)
+    w = workloads.make_weights(cfg, 9)
+    tokens = np.stack([workloads.make_prompt(b, 60, cfg["vocab"]) for b in range(2)])
+    want = None
+    for page_size in (32, 64, 256):
+        eng = binding.Engine(cfg, w, max_batch=2, max_len=64, max_gamma=8, page_size=page_size)
+        got = torch.cat([eng.forward_logits(0, np.ascontiguousarray(tokens[:, at:at + 2])) for at in range(0, 60, 2)], dim=1)
+        eng.close()
+        want = got if want is None else want
+        assert torch.equal(got, want), page_size
+
+
+def test_rows_beyond_what_the_context_holds():
+    """One sequence takes more guesses than the other and is frozen early, at lengths whose guesses lie beyond the last position
+    among others.  Each gets the tokens it gets alone."""
+    cfg = _tiny(2, 128)
+    w = workloads.make_weights(cfg, 9)
+    d = dict(w)
+    d["pos_emb"] = w["pos_emb"].copy()
+    d["pos_emb"][:20] = np.random.default_rng(1).standard_normal((20, 128), dtype=np.float32)
+    prompts = [workloads.make_prompt(1, 30, cfg["vocab"]), workloads.make_prompt(2, 3, cfg["vocab"])]
+    gamma, frozen = 3, 0
+    for n_new in range(8, 17):
+        eng = binding.Engine(cfg, w, cfg, d, max_batch=2, max_len=30 + n_new + gamma + 1, max_gamma=gamma, page_size=32)
+        alone = [eng.generate([p], n_new, gamma, 0.0, 1) for p in prompts]
+        frozen += alone[0][1]["iterations"] < alone[1][1]["iterations"]
+        both, _ = eng.generate(prompts, n_new, gamma, 0.0, 1)
+        eng.close()
+        for b in range(2):
+            assert (both[b] == alone[b][0][0]).all(), n_new
+    assert frozen

@@ -656,6 +656,6 @@ extern "C" int spec_timeout_drill(void* stream) {
 
 extern "C" int spec_device_error(void) {
     const int gemm = spec::gemm_tc_take_error(), wide = spec::gemm_wide_take_error(), pass = spec::pass_take_error(), attn = spec::attention_take_error(),
-              small = spec::small_pass_take_error();
-    return gemm ? gemm : wide ? wide : pass ? pass : attn ? attn : small;
+              small = spec::small_pass_take_error(), tiny = spec::cluster_pass_take_error();
+    return gemm ? gemm : wide ? wide : pass ? pass : attn ? attn : small ? small : tiny;
 }

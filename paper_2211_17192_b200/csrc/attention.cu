@@ -165,12 +165,11 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 
 constexpr int kTileKeys = 16;  // keys per staged tile of the tensor-core kernel
 
-// Which K,V rows a tensor-core kernel may fetch before its pdl_wait().  The kernel in front (launch_qkv) writes this pass's rows
-// and releases this one at its start; the GEMM in front of that has released it only after its own wait, so what lies further back -
-// the rows' positions, the page table, the K,V rows of earlier passes - is complete when this kernel starts, and an SM that
+// The rows that the caller says are settled are fetched before the pdl_wait().  The kernel in front (launch_qkv) writes this pass's
+// rows and releases this one at its start; the GEMM in front of that has released it only after its own wait, so what lies further
+// back - the rows' positions, the page table, the K,V rows of earlier passes - is complete when this kernel starts, and an SM that
 // the GEMM has left can fetch them while the projection is finished (7B shape behind the projection, with the queries read 16 bytes at a
 // time: one sequence of three rows at 1024 keys 11.4 -> 7.9 us, 32 of seven at 512 36 -> 28).
-constexpr int kNoneSettled = 0, kOldSettled = 1, kAllSettled = 2;  // (kOldSettled: in front of the sequence's first row)
 
 // A 16-key tile of one KV head ([key][DH] in the pool) into shared memory rows of
 // DH + 4 floats; keys at or beyond n_valid become zeros.
@@ -233,13 +232,13 @@ attention_mma_kernel(const float* qkv, int q_stride, const int32_t* pos,
                      const int32_t* seq, int m_rows, int n_heads, int n_kv_heads, int m_blocks,
                      const KV* kv_layer, const int32_t* __restrict__ page_table, int pages_per_seq,
                      int page_size, const int32_t* kv_len, const float* __restrict__ bias, int bias_span,
-                     int bias_zero, float scale, int settled, float* __restrict__ part, const AttnOut out) {
+                     int bias_zero, float scale, Settled settled, float* __restrict__ part, const AttnOut out) {
     using S = MmaSmem<DH, IN_TURN>;
     extern __shared__ __align__(16) float smem_f[];
     __shared__ int q_pos[16], q_row[16], q_head[16];
     __shared__ float merge_w[16][kMmaWarps], merge_m[16];
     pdl_trigger();
-    if (settled == kNoneSettled) pdl_wait();
+    if (settled == Settled::kNone) pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, t = lane & 3;
     const int slice = blockIdx.x, slices = gridDim.x, b = blockIdx.z;
@@ -306,10 +305,10 @@ attention_mma_kernel(const float* qkv, int q_stride, const int32_t* pos,
         cp_async_commit();
     };
     // the first tiles are requested before the queries are staged, those that are settled before the queries are there
-    const int old = settled == kAllSettled ? INT_MAX : settled == kOldSettled ? max(pos[b * m_rows], 0) : 0;
+    const int old = settled == Settled::kAll ? INT_MAX : settled == Settled::kOld ? max(pos[b * m_rows], 0) : 0;
     int early = 0;
     while (early < kMmaStages && early < my_tiles && first_key(early) + kTileKeys <= old) issue(early++);
-    if (settled != kNoneSettled) pdl_wait();
+    if (settled != Settled::kNone) pdl_wait();
     for (; early < kMmaStages; ++early) issue(early);
     {
         constexpr int kEach = 16 * DH / 4 / (32 * kMmaWarps);
@@ -597,7 +596,7 @@ attention_f16_kernel(const float* qkv, int q_stride, const int32_t* pos,
                      const int32_t* seq, int m_rows, int n_heads, int n_kv_heads, int q_blocks,
                      const __grid_constant__ CUtensorMap kv_map, const int32_t* __restrict__ page_table, int pages_per_seq,
                      int page_size, const int32_t* kv_len, const float* __restrict__ bias, int bias_span,
-                     int bias_zero, float scale, int settled, float* __restrict__ part, const AttnOut out) {
+                     int bias_zero, float scale, Settled settled, float* __restrict__ part, const AttnOut out) {
     using S = F16Smem<DH, MB>;
     constexpr int KP = kF16Warps / MB;        // key parts of a tile
     constexpr int KW = kF16TileKeys / KP;     // keys of a tile that one warp multiplies (16 MB)
@@ -618,7 +617,7 @@ attention_f16_kernel(const float* qkv, int q_stride, const int32_t* pos,
     }
     __syncthreads();
     pdl_trigger();
-    if (settled == kNoneSettled) pdl_wait();
+    if (settled == Settled::kNone) pdl_wait();
     const int g = lane >> 2, t = lane & 3;
     const int mb = warp % MB, kw0 = (warp / MB) * KW;
     const int slice = blockIdx.x, slices = gridDim.x, b = blockIdx.z;
@@ -687,8 +686,8 @@ attention_f16_kernel(const float* qkv, int q_stride, const int32_t* pos,
     };
     int pg_next[2] = {0, 0};
     // the first tiles are requested before the queries are staged, those that are settled before the queries are there
-    const int old = settled == kAllSettled ? INT_MAX : settled == kOldSettled ? max(pos[b * m_rows], 0) : 0;
-    bool waited = settled == kNoneSettled;
+    const int old = settled == Settled::kAll ? INT_MAX : settled == Settled::kOld ? max(pos[b * m_rows], 0) : 0;
+    bool waited = settled == Settled::kNone;
 #pragma unroll
     for (int t = 0; t < S::kStages - 1; ++t) {
         if (!waited && !(t < my_tiles && kF16TileKeys * (t0 + t + 1) <= old)) {
@@ -1380,7 +1379,6 @@ int launch_attention_variant(const Model& m, const AttnSource& src, const RowMet
     const bool fused = attention_merges_in_cluster(m, batch, m_rows, max_keys) && slices <= kMaxClusterSlices;
     const KV* pool = static_cast<const KV*>(src.pool.kv);
     int status;
-    const int settled = src.fixed ? kAllSettled : src.kv_len ? kNoneSettled : kOldSettled;
     if constexpr (std::is_same<KV, __half>::value) {
         if (attention_uses_f16(m, batch, m_rows, max_keys)) {
             const int q_blocks = (queries + kF16MaxQueries - 1) / kF16MaxQueries;
@@ -1398,7 +1396,7 @@ int launch_attention_variant(const Model& m, const AttnSource& src, const RowMet
         status = launch_attn(attention_f16_kernel<DH, MB, F>, grid, dim3(32 * kF16Warps), F16Smem<DH, MB>::kBytes,      \
                              CLUSTER, stream, src.q, src.q_stride, rows.pos, rows.seq, m_rows, m.cfg.n_heads,           \
                              m.cfg.n_kv_heads, q_blocks, kv_map, src.pool.page_table, src.pool.pages_per_seq,           \
-                             src.pool.page_size, src.kv_len, src.bias, src.bias_span, src.bias_zero, scale, settled, part, out); \
+                             src.pool.page_size, src.kv_len, src.bias, src.bias_span, src.bias_zero, scale, src.settled, part, out); \
     } while (0)
             if (per_cta <= 16) { if (fused) SPEC_LAUNCH_F16(1, true, slices); else SPEC_LAUNCH_F16(1, false, 0); }
             else if (per_cta <= 32) { if (fused) SPEC_LAUNCH_F16(2, true, slices); else SPEC_LAUNCH_F16(2, false, 0); }
@@ -1423,7 +1421,7 @@ int launch_attention_variant(const Model& m, const AttnSource& src, const RowMet
         status = launch_attn(attention_mma_kernel<KV, DH, F, T>, grid, dim3(32 * kMmaWarps), MmaSmem<DH, T>::kBytes,    \
                              CLUSTER, stream, src.q, src.q_stride, rows.pos, rows.seq, m_rows, m.cfg.n_heads,           \
                              m.cfg.n_kv_heads, m_blocks, pool, src.pool.page_table, src.pool.pages_per_seq,            \
-                             src.pool.page_size, src.kv_len, src.bias, src.bias_span, src.bias_zero, scale, settled, part, out); \
+                             src.pool.page_size, src.kv_len, src.bias, src.bias_span, src.bias_zero, scale, src.settled, part, out); \
     } while (0)
         if (fused && in_turn) SPEC_LAUNCH_MMA(true, true, slices);
         else if (fused) SPEC_LAUNCH_MMA(true, false, slices);

@@ -42,6 +42,11 @@ inline int fail(int status, const char* fmt, ...) {
 // streaming the first weight tiles).  pdl_wait() returns once the predecessor
 // grid has completed and its writes are visible; because every kernel waits,
 // completion is transitive along the stream.
+// One exception.  The tensor-core GEMMs (gemm_tc.cu, gemm_wide.cu) trigger only after their own wait: whatever lies in front of such
+// a GEMM is complete when a kernel behind it starts, and so it is for the kernel behind that one, whatever the first of the two does.
+// qkv_kernel with partial sums (first behind the GEMM) and the tensor-core attention kernels told so by AttnSource::settled (second)
+// read what is older than the GEMM - positions, page tables, K,V rows of earlier passes - before they wait.  Every other kernel may
+// trigger before its wait, so behind none of them is anything known to be complete.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // A load through a const __restrict__ pointer, or by __ldg, may be moved in front of pdl_wait(), where what the kernel before
 // writes is not there yet.  A pointer that has come through here after the wait holds it back.

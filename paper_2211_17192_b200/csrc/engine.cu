@@ -240,7 +240,8 @@ struct Pass {
         SPEC_TRY(proj(w.wqkv, pw.wqkv, m.qkv_dim(), c.d_model, ctx->qkv));
         SPEC_TRY(launch_qkv(c.n_heads, c.n_kv_heads, c.d_head, c.arch == SPEC_ARCH_LLAMA ? m.rope_table : nullptr, pool, rows,
                             n_rows, ctx->qkv, partials(), last, st, factor));
-        const AttnSource src{ctx->qkv, m.qkv_dim(), pool, kv_len, bias, bias_span, bias_zero};
+        // (an encoder's rows are all of this pass)
+        const AttnSource src{ctx->qkv, m.qkv_dim(), pool, kv_len, bias, bias_span, bias_zero, tc && !kv_len ? Settled::kOld : Settled::kNone};
         if (segs) {
             SPEC_TRY(launch_prompt_attention(m, src, *segs, hi(), lo(), st));
             return residual(w.wo, pw.wo, m.q_dim(), ctx->att);
@@ -365,7 +366,7 @@ int forward(spec_ctx* ctx, const Model& m, const RowMeta& rows, int batch, int m
                                     pass.last, ctx->stream, pass.factor));
             const KvPool pool = source_pool(ctx, m, static_cast<char*>(m.cross_kv) + static_cast<size_t>(l) * m.cross_stride);
             const int slices = attention_slices(m, batch, m_rows, ctx->rt.max_src_len);
-            const AttnSource src{ctx->qkv, m.q_dim(), pool, ctx->src_len, nullptr, 0, 0, true};
+            const AttnSource src{ctx->qkv, m.q_dim(), pool, ctx->src_len, nullptr, 0, 0, pass.tc ? Settled::kAll : Settled::kNone};
             SPEC_TRY(launch_attention(m, src, rows, batch, m_rows, slices, ctx->rt.max_src_len, ctx->attn_part, pass.tc ? nullptr : ctx->att,
                                       pass.tc ? pass.hi() : nullptr, pass.tc ? pass.lo() : nullptr, ctx->stream));
             SPEC_TRY(pass.residual(w.wo_x, pw.wo_x, m.q_dim(), ctx->att));

@@ -196,7 +196,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
                 ++it;
                 if (++s == stages) { s = 0; ++use; }
             }
-        pdl_trigger();
+        pdl_trigger();  // (after the wait: kernels behind this one count on what lies in front of it, common.cuh)
         if (!ok && rank == 0)  // nothing may still be on its way when the CTAs leave
             for (int i = 0; i < stages; ++i) {
                 mbar_wait(&full_bar[i], 0, kDrainLimit);

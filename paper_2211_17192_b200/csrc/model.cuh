@@ -172,6 +172,9 @@ int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, cons
                int n_rows, float* qkv, const float* partial, const PartialPlan& plan, cudaStream_t stream, const RowFactor& norm = RowFactor{});
 void fill_rope_table(std::vector<float2>& table, int positions, int d_head, double base);
 
+// Which K,V rows of a pool are complete although kernels in front may still be running (common.cuh has the rule): none; those in front
+// of each sequence's first row of the pass; all of them.
+enum class Settled { kNone, kOld, kAll };
 // One attention call: head h of query row r is at q + r * q_stride + h * d_head.
 // kv_len == nullptr: causal over the pool (row at position p sees keys 0..p);
 // otherwise every active row of sequence slot s sees keys 0..kv_len[s]-1.
@@ -185,7 +188,7 @@ struct AttnSource {
     const float* bias;
     int bias_span;
     int bias_zero;
-    bool fixed = false;  // the pool's rows are those of an earlier pass, all of them
+    Settled settled = Settled::kNone;  // (anything else only behind a tensor-core GEMM and its launch_qkv)
 };
 
 // att[r, h] = softmax(scores) V for the rows of a pass; rows of sequence b are

@@ -38,6 +38,7 @@
 
 #include <cuda_fp16.h>
 
+#include "cluster_util.cuh"
 #include "model.cuh"
 
 namespace spec {
@@ -121,25 +122,6 @@ struct Smem {
     static_assert(kStages >= 4, "what a phase reads fits");
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-__device__ __forceinline__ uint32_t peer_u32(uint32_t addr, int rank) {
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-// Stores into a peer's shared memory that are counted in bytes on the peer's barrier.
-__device__ __forceinline__ void send2(const float* here, uint64_t* bar, int rank, float x, float y) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(peer_u32(smem_u32(here), rank)),
-                 "r"(__float_as_uint(x)), "r"(__float_as_uint(y)), "r"(peer_u32(smem_u32(bar), rank))
-                 : "memory");
-}
-__device__ __forceinline__ void send4(const float* here, uint64_t* bar, int rank, const float4& v) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
-                     peer_u32(smem_u32(here), rank)),
-                 "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)), "r"(__float_as_uint(v.w)),
-                 "r"(peer_u32(smem_u32(bar), rank))
-                 : "memory");
-}
 // A value and the exchange it belongs to in one 8-byte word.
 __device__ __forceinline__ void publish(unsigned long long* at, float v, unsigned epoch) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(at), "l"((static_cast<unsigned long long>(epoch) << 32) | __float_as_uint(v)) : "memory");
@@ -149,23 +131,6 @@ __device__ __forceinline__ ulonglong2 peek2(const unsigned long long* at) {
     ulonglong2 v;
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(at) : "memory");
     return v;
-}
-__device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t parity, uint32_t limit) {
-#pragma unroll 1
-    for (uint32_t spin = 0; spin < limit; ++spin) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t"
-            ".reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t"
-            "}"
-            : "=r"(done)
-            : "r"(smem_u32(bar)), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
 }
 __device__ __forceinline__ void sync_consumers() { __syncthreads(); }
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1) {

@@ -96,7 +96,7 @@ __global__ void embed_kernel(const void* tok_emb, const void* pos_emb, bool bf16
 // exchange between the CTAs was a fifth of it (7B shape, three rows: 7.0 -> 5.5 us behind the GEMM).
 constexpr int kNormMaxWidth = 4 * 1024 * 4;
 constexpr int kNormCtas = 8;  // of a cluster that shares a row
-// The elementwise kernels give a thread several rows where one each is more threads than the GPU holds at once: below that the
+// The activation kernel gives a thread several rows where one each is more threads than the GPU holds at once: below that the
 // rows of a thread only lengthen it (96 rows of the 160M shape: a pass 625 us with a row each, 699 with four).
 constexpr long long kResidentThreads = 148 * 2048;
 constexpr int kNormFourRows = 296;  // at most for a cluster of four: eight CTAs of 256 threads to an SM
@@ -223,13 +223,14 @@ __device__ __forceinline__ void store_cached4(KV* dst, const float (&v)[4]) {
     else *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(t);
 }
 
-// grid = (ceil(heads * d_head / 8 / block), ceil(rows / ROWS)), heads = n_heads + 2 n_kv_heads.  qkv row layout:
+// grid = (ceil(heads * d_head / 8 / block), rows), heads = n_heads + 2 n_kv_heads.  qkv row layout:
 // [q heads | k heads | v heads], d_head each.  A thread finishes elements j .. j+3 and
 // j + d_head/2 .. of one head of one row of the qkv GEMM (optional partial sums), applies
 // rotary positions (q and k heads; they pair j with j + d_head/2), leaves q in `qkv` for the
-// attention kernel, and appends K or V to the paged cache.  ROWS as in ffn_act_kernel.
-constexpr int kQkvRows = 4;
-template <typename KV, int ROWS>
+// attention kernel, and appends K or V to the paged cache.  A row to a thread at any number of rows: four, as in ffn_act_kernel, changed
+// nothing (a block of the 7B shape, us: 448 rows 372 with four, 370; 1024 rows 782, 783; 16 prompts of 500 to 1000 tokens with their
+// answers 1.5 % longer with four in one run, 0.8 % shorter in another).
+template <typename KV>
 __global__ void qkv_kernel(float* qkv, const float* partial, const PartialPlan plan, int n_rows,
                            const int32_t* pos, const int32_t* seq, int n_heads,
                            int n_kv_heads, int d_head, const float2* rope_table,
@@ -240,88 +241,68 @@ __global__ void qkv_kernel(float* qkv, const float* partial, const PartialPlan p
     // positions, rotations and pages are older than that, and are fetched ahead of this kernel's)
     if (!partial) pdl_wait();
     const int half = d_head / 2, per_head = half / 4;
-    const int task = blockIdx.x * blockDim.x + threadIdx.x, r0 = ROWS * blockIdx.y;
+    const int task = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
     const int head = task / per_head, j = 4 * (task % per_head);
     if (blockIdx.x * blockDim.x + (threadIdx.x & ~31) >= (n_heads + 2 * n_kv_heads) * per_head) return;  // (whole warps)
     const bool out = head >= n_heads + 2 * n_kv_heads;
     const bool is_q = head < n_heads, is_k = !is_q && head < n_heads + n_kv_heads;
     const int width = (n_heads + 2 * n_kv_heads) * d_head;
-    int p[ROWS];
-    float4 t[ROWS][2];  // (cos, sin) of the rows' positions for the four pairs
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i) p[i] = pos[min(r0 + i, n_rows - 1)];
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i)
-        if (rope_table && p[i] >= 0 && (is_q || is_k)) {
-            const float4* at = reinterpret_cast<const float4*>(rope_table + static_cast<size_t>(p[i]) * half + j);
-            t[i][0] = at[0];
-            t[i][1] = at[1];
-        }
-    size_t cached[ROWS];  // where K or V of a row goes
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i) {
-        cached[i] = 0;
-        if (p[i] >= 0 && !is_q && !out) {
-            const int kv_head = is_k ? head - n_heads : head - n_heads - n_kv_heads;
-            const int page = page_table[seq[min(r0 + i, n_rows - 1)] * pages_per_seq + (p[i] >> page_shift)];
-            const size_t block = (static_cast<size_t>(page) * 2 + (is_k ? 0 : 1)) * n_kv_heads + kv_head;
-            cached[i] = ((block << page_shift) + (p[i] & ((1 << page_shift) - 1))) * d_head + j;
-        }
+    const int p = pos[r];
+    const bool rotate = rope_table && p >= 0 && (is_q || is_k);
+    float4 t0, t1;  // (cos, sin) of position p for the four pairs
+    if (rotate) {
+        const float4* at = reinterpret_cast<const float4*>(rope_table + static_cast<size_t>(p) * half + j);
+        t0 = at[0];
+        t1 = at[1];
+    }
+    size_t cached = 0;  // where K or V goes
+    if (p >= 0 && !is_q && !out) {
+        const int kv_head = is_k ? head - n_heads : head - n_heads - n_kv_heads;
+        const int page = page_table[seq[r] * pages_per_seq + (p >> page_shift)];
+        const size_t block = (static_cast<size_t>(page) * 2 + (is_k ? 0 : 1)) * n_kv_heads + kv_head;
+        cached = ((block << page_shift) + (p & ((1 << page_shift) - 1))) * d_head + j;
     }
     if (partial) pdl_wait();
-    DeferredRow deferred[ROWS];
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i) deferred[i].fetch(norm, min(r0 + i, n_rows - 1));
-    size_t where[2 * ROWS];
-    float4 x[2 * ROWS];
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i) {
-        where[2 * i] = static_cast<size_t>(min(r0 + i, n_rows - 1)) * width + (out ? 0 : head * d_head + j);
-        where[2 * i + 1] = where[2 * i] + half;
-        x[2 * i] = x[2 * i + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    DeferredRow deferred;
+    deferred.fetch(norm, r);
+    const size_t at = static_cast<size_t>(r) * width + (out ? 0 : head * d_head + j);
+    const size_t where[2] = {at, at + half};
+    float4 x[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
     if (partial) {
         // (a head of 64 or 128 columns lies inside one 256-column tile)
-        sum_partials<2 * ROWS, ROWS == 1 ? 4 : 1>(partial, partial_count(plan, r0, out ? 0 : head * d_head), static_cast<size_t>(n_rows) * width, where, x);
+        sum_partials<2, 4>(partial, partial_count(plan, r, out ? 0 : head * d_head), static_cast<size_t>(n_rows) * width, where, x);
     } else {
-#pragma unroll
-        for (int i = 0; i < 2 * ROWS; ++i) x[i] = *reinterpret_cast<const float4*>(qkv + where[i]);
+        x[0] = *reinterpret_cast<const float4*>(qkv + where[0]);
+        x[1] = *reinterpret_cast<const float4*>(qkv + where[1]);
     }
-    float factor[ROWS];
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i) factor[i] = deferred[i].factor(norm);
+    const float factor = deferred.factor(norm);
     if (out) return;
+    float a[4] = {x[0].x, x[0].y, x[0].z, x[0].w}, b[4] = {x[1].x, x[1].y, x[1].z, x[1].w};
+    if (norm.squares) {
 #pragma unroll
-    for (int i = 0; i < ROWS; ++i) {
-        if (ROWS > 1 && r0 + i >= n_rows) break;
-        const float4 xa = x[2 * i], xb = x[2 * i + 1];
-        float a[4] = {xa.x, xa.y, xa.z, xa.w}, b[4] = {xb.x, xb.y, xb.z, xb.w};
-        if (norm.squares) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                a[e] *= factor[i];
-                b[e] *= factor[i];
-            }
+        for (int e = 0; e < 4; ++e) {
+            a[e] *= factor;
+            b[e] *= factor;
         }
-        if (rope_table && p[i] >= 0 && (is_q || is_k)) {
-            const float c[4] = {t[i][0].x, t[i][0].z, t[i][1].x, t[i][1].z}, s[4] = {t[i][0].y, t[i][0].w, t[i][1].y, t[i][1].w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float y1 = a[e] * c[e] - b[e] * s[e], y2 = b[e] * c[e] + a[e] * s[e];
-                a[e] = y1;
-                b[e] = y2;
-            }
-        }
-        if (is_q) {
-            *reinterpret_cast<float4*>(qkv + where[2 * i]) = make_float4(a[0], a[1], a[2], a[3]);
-            *reinterpret_cast<float4*>(qkv + where[2 * i + 1]) = make_float4(b[0], b[1], b[2], b[3]);
-            continue;
-        }
-        if (p[i] < 0) continue;  // inactive row: nothing is cached
-        KV* dst = kv_layer + cached[i];
-        store_cached4<KV>(dst, a);
-        store_cached4<KV>(dst + half, b);
     }
+    if (rotate) {
+        const float c[4] = {t0.x, t0.z, t1.x, t1.z}, s[4] = {t0.y, t0.w, t1.y, t1.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float y1 = a[e] * c[e] - b[e] * s[e], y2 = b[e] * c[e] + a[e] * s[e];
+            a[e] = y1;
+            b[e] = y2;
+        }
+    }
+    if (is_q) {
+        *reinterpret_cast<float4*>(qkv + where[0]) = make_float4(a[0], a[1], a[2], a[3]);
+        *reinterpret_cast<float4*>(qkv + where[1]) = make_float4(b[0], b[1], b[2], b[3]);
+        return;
+    }
+    if (p < 0) return;  // inactive row: nothing is cached
+    KV* dst = kv_layer + cached;
+    store_cached4<KV>(dst, a);
+    store_cached4<KV>(dst + half, b);
 }
 
 // logits[dst(i)] = table[token[src(i)]] for a table model: grid = (chunks, rows), block = 256.
@@ -520,20 +501,16 @@ int launch_norm(float* h, const float* partial, const PartialPlan& plan, int row
 int launch_qkv(int n_heads, int n_kv_heads, int d_head, const float2* rope, const KvPool& pool, const RowMeta& rows,
                int n_rows, float* qkv, const float* partial, const PartialPlan& plan, cudaStream_t stream, const RowFactor& norm) {
     const int tasks = (n_heads + 2 * n_kv_heads) * (d_head / 8);
-    const bool many = static_cast<long long>(n_rows) * tasks > kResidentThreads;
     const int threads = n_rows <= 16 ? 64 : 256;
-    const dim3 grid((tasks + threads - 1) / threads, many ? (n_rows + kQkvRows - 1) / kQkvRows : n_rows);
+    const dim3 grid((tasks + threads - 1) / threads, n_rows);
     int page_shift = 0;  // (pages are a power of two)
     while ((1 << page_shift) < pool.page_size) ++page_shift;
-#define SPEC_LAUNCH_QKV(KV, R)                                                                                                  \
-    return launch_pdl(qkv_kernel<KV, R>, grid, dim3(threads), 0, stream, qkv, partial, plan, n_rows, rows.pos, rows.seq, n_heads, \
+#define SPEC_LAUNCH_QKV(KV)                                                                                                      \
+    return launch_pdl(qkv_kernel<KV>, grid, dim3(threads), 0, stream, qkv, partial, plan, n_rows, rows.pos, rows.seq, n_heads,   \
                       n_kv_heads, d_head, rope, static_cast<KV*>(pool.kv), pool.page_table, pool.pages_per_seq, page_shift, norm)
-    if (pool.dtype == SPEC_DTYPE_FP16 && many) SPEC_LAUNCH_QKV(__half, kQkvRows);
-    if (pool.dtype == SPEC_DTYPE_FP16) SPEC_LAUNCH_QKV(__half, 1);
-    if (pool.dtype == SPEC_DTYPE_BF16 && many) SPEC_LAUNCH_QKV(__nv_bfloat16, kQkvRows);
-    if (pool.dtype == SPEC_DTYPE_BF16) SPEC_LAUNCH_QKV(__nv_bfloat16, 1);
-    if (many) SPEC_LAUNCH_QKV(float, kQkvRows);
-    SPEC_LAUNCH_QKV(float, 1);
+    if (pool.dtype == SPEC_DTYPE_FP16) SPEC_LAUNCH_QKV(__half);
+    if (pool.dtype == SPEC_DTYPE_BF16) SPEC_LAUNCH_QKV(__nv_bfloat16);
+    SPEC_LAUNCH_QKV(float);
 #undef SPEC_LAUNCH_QKV
 }
 

@@ -1,6 +1,6 @@
 """Many rows of a wide block, against the oracle, on either side of the lines at which the small kernels between the GEMMs change:
-four rows to a thread of the activation (from 111 rows of this shape on) and of the projection's (from 395 on), a norm that leaves
-its factor to them (up to 128), a cluster of four thread blocks to a row (up to 296) and one (beyond); row counts that are no multiple of four."""
+four rows to a thread of the activation (from 111 rows of this shape on), a norm that leaves its factor to it and to the
+projection's (up to 128), a cluster of four thread blocks to a row (up to 296) and one (beyond); row counts that are no multiple of four."""
 import numpy as np
 import pytest
 

@@ -91,9 +91,10 @@ __global__ void embed_kernel(const void* tok_emb, const void* pos_emb, bool bf16
 // row of 4096 with its eight partial sums is 147 KB, a microsecond of what one SM takes in, and nothing else runs
 // meanwhile.  The CTAs give one another their warps' sums of squares through distributed shared memory.
 // DEFER: they do not.  W . (rmsnorm(h) gain) is W . (h gain) times a factor per row, so the terms are of h * gain, the warps' sums of
-// squares go to `squares`, [row][32], and the kernel that adds up the GEMM's partial sums forms the factor (row_factor).  The
+// squares go to `squares`, [row][32], and the kernel that adds up the GEMM's partial sums forms the factor (DeferredRow).  The
 // norm is a stop between two weight streams of which only the first 24 MB of the second is on its way meanwhile, and the
-// exchange between the CTAs was a fifth of it (7B shape, three rows: 7.0 -> 5.5 us behind the GEMM).
+// exchange between the CTAs was a fifth of it (7B shape, three rows: 7.0 -> 5.5 us behind the GEMM).  The terms have the same 16 bits
+// either way: logits of nine shapes of pass are off 64 bits by 6.87e-4 (mean; 6.88e-4 with the factor applied here).
 constexpr int kNormMaxWidth = 4 * 1024 * 4;
 constexpr int kNormCtas = 8;  // of a cluster that shares a row
 // The activation kernel gives a thread several rows where one each is more threads than the GPU holds at once: below that the
@@ -479,7 +480,8 @@ int launch_norm(float* h, const float* partial, const PartialPlan& plan, int row
     // threads per row against a cluster, ms: 1 row 2.779 / 2.761, 3 rows 2.865 / 2.839, 7 rows 2.937 / 2.915, 16 rows
     // 3.111 / 3.123 (the runs of one side differ by as much), 32 rows 3.196 / 3.152, 64 rows 3.748 / 3.734, 126 rows
     // 5.232 / 5.216; beyond, four larger CTAs (eight partial sums in flight, not two: 224 rows 11.0 -> 9.8 us behind the GEMM), and
-    // where those no longer fit side by side a CTA per row.
+    // where those no longer fit side by side a CTA per row (us a block, a CTA per row against four: 160 rows 177 / 173, 224 rows
+    // 212 / 211, 259 rows 292 / 292, 296 rows 296 / 297).
     const int groups = d / 4;
     if (squares)
         return launch_cluster(norm_kernel<128, 1, kNormCtas, true>, 0, dim3(n_rows * kNormCtas), dim3(128), 0, stream, h, partial,

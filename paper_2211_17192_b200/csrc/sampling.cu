@@ -1251,7 +1251,8 @@ __device__ __forceinline__ float block_max(float v, float* per_warp) {
 // mass decides nothing: the row is then binned as it lies.
 // Masses are in the units of the bins, integers, so a row has one floor, from a list and from bins, to the last bit.  (Added up in fp32
 // while the row was listed, against the sample's maximum, the mass of the rest moved one floor in several hundred at T = 1, and one in 80 of rows
-// around 100 at T = 0.05.  The second pass is not in the time of a call after another: 200 x 100000 46.3 -> 45.1 us, cold 53 -> 61.)
+// around 100 at T = 0.05.  The second pass costs
+// nothing where L2 holds the rows already, 200 x 100000 46.3 -> 45.1 us, with other rows at every call 46.4 -> 50.2, cold 53 -> 61.)
 // A warp lists its own part of the row, and large logits may all lie in one part (ids in order of frequency, say): a row of
 // which a warp finds more than its share is listed once more, as one list.  Binned, listed where they lie by chance, and sorted, us
 // call after call, rows N(0, 3^2), p = 0.9, with the draw: 200 x 100000 68, 46, 64; 64 x 100000 33, 28, 38; 1 x 50000 23, 18,
